@@ -189,9 +189,10 @@ size_t bigcn_layer_workspace_bytes(int64_t N, int32_t K, int32_t F);
  * calls above within fp32 rounding; it runs the kernels of bigcn_pack_rows,
  * bigcn_pack_weights, bigcn_xnor_gemm_degscaled and bigcn_spmm_prescaled on
  * `stream`, except that when K <= 32767 the product keeps Z' factored in the
- * workspace -- the integer dots (as uint16 with a bias of 32768) and each
- * row's alpha_i / sqrt(dhat_i) -- and the aggregation applies the row factor
- * per neighbour and beta_j per column, gathering half the bytes. No
+ * workspace -- the integer dots (in byte planes where K <= 3072, else as uint16
+ * with a bias of 32768) and each row's alpha_i / sqrt(dhat_i) -- and the
+ * aggregation applies the row factor per neighbour and beta_j per column,
+ * gathering a quarter or half of the bytes. No
  * activation follows (Sec. 4.1.2).
  *
  * X N x K (ldx), Wt K x F (ldw), CSR as in bigcn_spmm_norm, H N x F (ldh).
@@ -218,7 +219,7 @@ bigcn_status bigcn_layer_forward(const float *X, int64_t N, int32_t K, int64_t l
  * layer's kernel q (pack rows, pack weights, XNOR product, aggregation) and
  * event 4 after the last (as external events while the stream is being
  * captured); entries beyond 5 are not touched. When the rows are few and
- * long (fewer than a wave of warps), the rows are packed inside the product's
+ * long, or too few for a tensor-core product, they are packed inside the product's
  * kernel and the first interval is empty. Everything else is
  * bigcn_layer_forward's.
  */
@@ -248,8 +249,8 @@ bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int32_t K, int
  * goes through memory. When K <= 32767, layer 1's Z' stays factored in the
  * workspace (integer dots as biased uint16 and a row scale, as in
  * bigcn_layer_forward), so its aggregation gathers half-size rows. When
- * K <= 2048 (the dots exact in fp16), Fh <= 128 and Fo <= 64, both products
- * stay factored as fp16 dots and a row scale and both aggregations run on the
+ * K <= 2048, Fh <= 128 and Fo <= 64, both products
+ * stay factored as byte dots and a row scale and both aggregations run on the
  * tensor cores (bigcn_forward_2layer_aggregation); layer 1's aggregation then
  * binarizes H1 and computes layer 2's dots for any Fh <= 128. The call
  * launches 4 to 7 kernels (bigcn_forward_2layer_launches).
@@ -275,7 +276,7 @@ size_t bigcn_forward_2layer_workspace_bytes(int64_t N, int32_t K, int32_t Fh, in
 int32_t bigcn_forward_2layer_launches(int64_t N, int32_t K, int32_t Fh, int32_t Fo);
 
 /* Which aggregation bigcn_forward_2layer runs for these widths: 1 = both on
- * the tensor cores over fp16 dots, 0 = on the CUDA cores, -1 = invalid sizes.
+ * the tensor cores over byte dots, 0 = on the CUDA cores, -1 = invalid sizes.
  * An interface query with no counterpart in the paper (it selects how the
  * sums of Eq. 13 are evaluated, not what they are); needs no device. */
 int32_t bigcn_forward_2layer_aggregation(int32_t K, int32_t Fh, int32_t Fo);

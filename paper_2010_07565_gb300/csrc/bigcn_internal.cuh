@@ -133,12 +133,30 @@ class EventMarks {
     bool failed_ = false;
 };
 
-// A dot of Eqs. 11-12 in the compressed forms of a factored product: uint16
-// with a bias of 32768 (|dot| <= 32767), or fp16 bits when `f16` (exact for
-// |dot| <= 2048); `valid` false gives the zero dot of a padding column.
-__device__ __forceinline__ uint16_t encode_dot(int dot, bool valid, bool f16) {
-    if (f16) return valid ? __half_as_ushort(__int2half_rn(dot)) : uint16_t(0);
+// A dot of Eqs. 11-12 as uint16 with a bias of 32768 (|dot| <= 32767);
+// `valid` false gives the zero dot of a padding column.
+__device__ __forceinline__ uint16_t encode_dot(int dot, bool valid) {
     return uint16_t(valid ? dot + 32768 : 32768);
+}
+
+// A dot in byte planes. A dot has the parity of K, so it is 2 v + (K & 1) with
+// |v| <= K / 2 <= 16383, and v = lo + 256 hi with lo in [-128, 127]. The low plane
+// holds lo + 128, the high plane hi + 128. For dots of about sqrt(K) (signs
+// that agree about half the time) v fits the low byte alone: only a row in
+// which some dot does not -- a wide row -- has its high plane written and read,
+// and the sign bit of its row scale (the scale itself is never negative) says
+// so. Half the bytes of a 16-bit dot, and nothing is rounded.
+struct ByteDot {
+    int b;                                          // v + 128
+    __device__ __forceinline__ ByteDot(int dot, int K) : b(((dot - (K & 1)) >> 1) + 128) {}
+    __device__ __forceinline__ bool wide() const { return unsigned(b) > 255u; }
+    __device__ __forceinline__ uint32_t lo() const { return uint32_t(b) & 255u; }
+    __device__ __forceinline__ uint32_t hi() const { return uint32_t((b >> 8) + 128); }
+};
+
+// A row scale with its row's wide flag in the sign bit.
+__device__ __forceinline__ float flag_scale(float s, bool wide) {
+    return __uint_as_float(__float_as_uint(s) | (wide ? 0x80000000u : 0u));
 }
 
 // 1 / sqrt(1 + row length): the D^-1/2 factor of A + I (Sec. 3.1, Eq. 1),

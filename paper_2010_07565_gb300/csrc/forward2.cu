@@ -15,10 +15,10 @@
 // not fit the fused kernel (hidden width not a multiple of 4 or above 128, or
 // more than 64 outputs). Every step runs on the GPU either way.
 //
-// When K <= 2048 (layer 1's dots exact in fp16), Fh <= 128 and Fo <= 64, the
-// products stay factored as fp16 dots with a row scale and both
-// aggregations run on the tensor cores (spmm_tc.cu): step 2 writes layer 2's
-// dots D2 and row scale s2 instead of fp32 Z2', and step 3 multiplies by beta2.
+// When K <= 2048, Fh <= 128 and Fo <= 64, the products stay factored as byte
+// planes of dots (ByteDot) with a row scale and both aggregations run on the
+// tensor cores (spmm_tc.cu): step 2 writes layer 2's dots D2 and row scale s2
+// instead of fp32 Z2', and step 3 multiplies by beta2.
 //
 // Every kernel after the first is launched with programmatic serialization:
 // it may start while its predecessor drains, and waits (griddepcontrol) only
@@ -34,13 +34,14 @@ size_t round_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 // Largest K (or Fh) whose dots the compressed uint16 form holds.
 constexpr int32_t kMaxDots16K = 32767;
-// Largest K whose dots fp16 holds exactly: the tensor-core aggregation's input.
-constexpr int32_t kMaxDotsF16K = 2048;
+// Largest K of the tensor-core path: the front kernel that then always runs
+// (Fh <= 128) has all of a row's dots in one block.
+constexpr int32_t kMaxTcK = 2048;
 
-// The tensor-core path: layer 1's dots as fp16, both aggregations on
-// spmm_tc.cu, layer 2's product kept factored as fp16 dots as well.
+// The tensor-core path: layer 1's dots in byte planes, both aggregations on
+// spmm_tc.cu, layer 2's product kept factored in byte planes as well.
 bool forward2_tc(int32_t K, int32_t Fh, int32_t Fo) {
-    return K <= kMaxDotsF16K && spmm_tc_pack_gemm_supported(Fh, Fo);
+    return K <= kMaxTcK && spmm_tc_pack_gemm_supported(Fh, Fo);
 }
 
 // Workspace carve-up. Layer 1's Z' is fp32 (N x Fh) or, when K <= 32767,
@@ -79,7 +80,7 @@ bool forward2_workspace(int64_t N, int32_t K, int32_t Fh, int32_t Fo, Forward2Wo
     w->h1 = take(size_t(N) * Fh * 4);
     w->bits2 = take(size_t(N) * w2 * 8);
     w->alpha2 = take(size_t(N) * 4);
-    w->d2 = take(w->tc ? size_t(N) * Fo16 * 2 : 0);
+    w->d2 = take(w->tc ? size_t(N) * Fo16 : 0);      // (no wide dots: Fh <= 128)
     w->s2 = take(w->tc ? size_t(N) * 4 : 0);
     w->total = off;
     return true;
@@ -168,9 +169,9 @@ extern "C" bigcn_status bigcn_forward_2layer(
     const int words1 = bigcn_words(K), words2 = bigcn_words(Fh);
     const int64_t Fh8 = (Fh + 7) / 8 * 8, Fo4 = (Fo + 3) / 4 * 4;
     const int64_t Fh16 = (Fh + 15) / 16 * 16, Fo16 = (Fo + 15) / 16 * 16;
-    const int64_t ldd1 = w.tc ? Fh16 : Fh8;     // layer 1's compressed row stride
-    const bool fused = spmm_pack_gemm_supported(Fh, Fo);
+        const bool fused = spmm_pack_gemm_supported(Fh, Fo);
     uint16_t *D1 = w.c16 ? static_cast<uint16_t *>(Z1) : nullptr;
+    uint8_t *P1 = static_cast<uint8_t *>(Z1);       // the tensor-core path's byte planes
     float *Z1f = w.c16 ? nullptr : static_cast<float *>(Z1);
     cudaStream_t s = as_stream(stream);
     EventMarks marks(events, n_events, s);
@@ -184,11 +185,14 @@ extern "C" bigcn_status bigcn_forward_2layer(
     mark();
     if (front_supported(N, K, Fh, dev)) {
         FrontArgs fr{X, N, K, ldx, scale, shift, wbits1, beta1, Fh, words1, rowptr, Z1f, Fh};
-        if (w.c16) {
-            fr.D16 = D1;
-            fr.ldd16 = ldd1;
+        if (w.tc) {
+            fr.dots8 = P1;
+            fr.ldd8 = Fh16;
             fr.rowscale = s1;
-            fr.dots_f16 = w.tc;
+        } else if (w.c16) {
+            fr.D16 = D1;
+            fr.ldd16 = Fh8;
+            fr.rowscale = s1;
         }
         launch_front(fr, dev, s, true);
         mark();
@@ -196,25 +200,26 @@ extern "C" bigcn_status bigcn_forward_2layer(
         launch_pack_rows(X, N, K, ldx, scale, shift, bits1, words1, alpha1, dev, s, true, false);
         mark();
         GemmArgs g1{bits1, alpha1, N, wbits1, beta1, Fh, K, words1, Z1f, Fh, nullptr, rowptr};
-        if (w.c16) {
+        if (w.c16) {        // (the tensor-core path always has the fused front)
             g1.dots16 = D1;
-            g1.ldd16 = ldd1;
+            g1.ldd16 = Fh8;
             g1.rowscale = s1;
-            g1.dots_f16 = w.tc;
         }
         launch_xnor_gemm(g1, dev, s, true);
         mark();
     }
     if (w.tc) {
         // Both aggregations on the tensor cores: layer 1's fused with layer 2's
-        // binarization and product (fp16 dots D2 and row scale s2), then layer 2's.
-        uint16_t *D2 = static_cast<uint16_t *>(at(w.d2));
-        float *s2 = static_cast<float *>(at(w.s2));
-        SpmmTcPackGemmArgs f{rowptr, colidx, N, nnz, D1, ldd1, s1, Fh, beta1, H1, ldh1,
+        // binarization and product (byte dots D2 and row scale s2), then layer 2's.
+        uint8_t *D2 = static_cast<uint8_t *>(at(w.d2));
+        // Row scales in the rows' padding where it has room: one gather per entry
+        // less for layer 2's aggregation.
+        float *s2 = Fo16 - Fo >= 4 ? nullptr : static_cast<float *>(at(w.s2));
+        SpmmTcPackGemmArgs f{rowptr, colidx, N, nnz, P1, Fh16, s1, Fh, K, beta1, H1, ldh1,
                              wbits2, Fo, D2, Fo16, s2};
         launch_spmm_tc_pack_gemm(f, dev, s, true);
         mark();
-        SpmmTcArgs a2{rowptr, colidx, N, nnz, D2, Fo16, s2, Fo, out, ldo, beta2, pred};
+        SpmmTcArgs a2{rowptr, colidx, N, nnz, D2, Fo16, s2, Fo, Fh, out, ldo, beta2, pred};
         launch_spmm_tc(a2, dev, s, true);
         mark();
         const bigcn_status ls = launch_status();

@@ -14,10 +14,12 @@
 // memory (odd row pitch: conflict-free). Several blocks per SM overlap one
 // block's HBM-bound phase A with another's POPC-bound phase B.
 //
-// Either kernel can leave Z' factored instead (D16 non-null, K <= 32767):
-// the integer dots as uint16 with a bias of 32768 (rows padded to a multiple
-// of 4 with zero dots) and the row scale alpha_i / sqrt(dhat_i), for an
-// aggregation that gathers half-size rows and applies beta per column.
+// Either kernel can leave Z' factored instead (K <= 32767), for an aggregation
+// that gathers smaller rows and applies beta per column: the integer dots and
+// the row scale alpha_i / sqrt(dhat_i), the dots as uint16 with a bias of 32768
+// (D16 non-null: rows padded to a multiple of 4 with zero dots) or in byte
+// planes (dots8 non-null: ByteDot; the row's threads agree on its wide flag
+// before its scale and its high plane are written).
 //
 // The packed weight columns and beta come from the weight-packing kernel
 // that runs first. This whole-row kernel is used when there are enough rows
@@ -37,9 +39,12 @@ constexpr int kFrontUnroll = 8;
 constexpr int kFrontMaxK = 2048;
 constexpr size_t kFrontMaxSmem = 160 * 1024;
 
+// Columns per 16 threads of the product phase: F rounded up to 16, 32, 64 or 128.
+int front_cols(int F) { return F <= 16 ? 16 : F <= 32 ? 32 : F <= 64 ? 64 : 128; }
+
 size_t front_smem(int BM, int F, int words) {
     const size_t pitch = size_t(words) + 1;   // odd pitch in 64-bit words
-    return (size_t(BM) + size_t(F)) * pitch * 8 + size_t(BM) * 4;
+    return (size_t(BM) + size_t(front_cols(F))) * pitch * 8 + size_t(BM) * 4;
 }
 
 template <int RI, int CJ>
@@ -48,13 +53,20 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
              const float *__restrict__ scale, const float *__restrict__ shift,
              const uint64_t *__restrict__ wbits, const float *__restrict__ beta, int F, int words,
              const int64_t *__restrict__ rowptr, float *__restrict__ Z, int64_t ldz,
-             uint16_t *__restrict__ D16, int64_t ldd16, float *__restrict__ rowscale, bool f16) {
+             uint16_t *__restrict__ D16, int64_t ldd16, float *__restrict__ rowscale,
+             uint8_t *__restrict__ dots8, int64_t ldd8) {
     constexpr int BM = 16 * RI;
+    // Thread cg owns V neighbouring columns (and the V that lie 64 further on),
+    // so that a row's byte dots are stored V to a word; column c is staged at
+    // row cg + 16 j of Bs, which keeps the product's reads free of conflicts.
+    constexpr int V = CJ < 4 ? CJ : 4;
+    auto column = [](int cg, int j) { return V * cg + j % V + 16 * V * (j / V); };
+    auto slot = [](int c) { return c % (16 * V) / V + 16 * (c % V + V * (c / (16 * V))); };
     extern __shared__ __align__(16) unsigned char smem[];
     const int pitch = words + 1;
     uint64_t *As = reinterpret_cast<uint64_t *>(smem);             // BM x pitch
-    uint64_t *Bs = As + size_t(BM) * pitch;                          // F x pitch
-    float *sAlpha = reinterpret_cast<float *>(Bs + size_t(F) * pitch);
+    uint64_t *Bs = As + size_t(BM) * pitch;                          // 16 CJ x pitch
+    float *sAlpha = reinterpret_cast<float *>(Bs + size_t(16 * CJ) * pitch);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t m0 = int64_t(blockIdx.x) * BM;
@@ -82,7 +94,7 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
     // once per block).
     grid_dependency_wait();
     for (int q = tid; q < F * words; q += kFrontThreads)
-        Bs[(q / words) * pitch + (q % words)] = __ldg(wbits + q);
+        Bs[slot(q / words) * pitch + (q % words)] = __ldg(wbits + q);
     __syncthreads();
 
     // Phase B: XNOR-popcount against every column.
@@ -97,10 +109,7 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
 #pragma unroll
         for (int i = 0; i < RI; ++i) a[i] = As[size_t(rg + 16 * i) * pitch + w];
 #pragma unroll
-        for (int j = 0; j < CJ; ++j) {
-            const int c = cg + 16 * j;
-            b[j] = c < F ? Bs[size_t(c) * pitch + w] : 0ull;
-        }
+        for (int j = 0; j < CJ; ++j) b[j] = Bs[size_t(cg + 16 * j) * pitch + w];
 #pragma unroll
         for (int i = 0; i < RI; ++i)
 #pragma unroll
@@ -110,23 +119,54 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
 #pragma unroll
     for (int i = 0; i < RI; ++i) {
         const int64_t row = m0 + rg + 16 * i;
+        bool wide = false;
+        if (dots8 != nullptr) {             // the row's 16 lanes agree on its flag
+#pragma unroll
+            for (int j = 0; j < CJ; ++j)
+                if (column(cg, j) < F) wide |= ByteDot(K - 2 * mism[i][j], K).wide();
+            wide = (__ballot_sync(kFullMask, wide) >> (tid & 16) & 0xffffu) != 0u;
+        }
         if (row >= N) continue;
         const float ai = rowptr == nullptr
                              ? sAlpha[rg + 16 * i]
                              : sAlpha[rg + 16 * i] *
                                    inv_sqrt_degree(__ldg(rowptr + row + 1) - __ldg(rowptr + row));
+        if (dots8 != nullptr) {             // byte planes + row scale, V columns per store
+            if (cg == 0) rowscale[row] = flag_scale(ai, wide);
+#pragma unroll
+            for (int j0 = 0; j0 < CJ; j0 += V) {
+                const int col = column(cg, j0);
+                if (col >= ldd8) continue;
+                uint32_t lo = 0, hi = 0;
+#pragma unroll
+                for (int e = 0; e < V; ++e) {
+                    const ByteDot d(K - 2 * mism[i][j0 + e], K);
+                    lo |= d.lo() << (8 * e);
+                    hi |= (d.hi() & 255u) << (8 * e);
+                }
+                uint8_t *p = dots8 + row * ldd8 + col;
+                auto put = [&](uint8_t *q, uint32_t v) {
+                    if (V == 4) *reinterpret_cast<uint32_t *>(q) = v;
+                    else if (V == 2) *reinterpret_cast<uint16_t *>(q) = uint16_t(v);
+                    else *q = uint8_t(v);
+                };
+                put(p, lo);
+                if (wide) put(p + N * ldd8, hi);
+            }
+            continue;
+        }
         if (D16 != nullptr) {               // compressed output: biased dots + row scale
             if (cg == 0) rowscale[row] = ai;
 #pragma unroll
             for (int j = 0; j < CJ; ++j) {
-                const int col = cg + 16 * j;
-                if (col < ldd16) D16[row * ldd16 + col] = encode_dot(K - 2 * mism[i][j], col < F, f16);
+                const int col = column(cg, j);
+                if (col < ldd16) D16[row * ldd16 + col] = encode_dot(K - 2 * mism[i][j], col < F);
             }
             continue;
         }
 #pragma unroll
         for (int j = 0; j < CJ; ++j) {
-            const int col = cg + 16 * j;
+            const int col = column(cg, j);
             if (col < F) Z[row * ldz + col] = ai * (__ldg(beta + col) * float(K - 2 * mism[i][j]));
         }
     }
@@ -139,7 +179,7 @@ void launch_ri_cj(const FrontArgs &a, int BM, size_t smem, cudaStream_t s, bool 
                          int(smem));
     launch_kernel(front_kernel<RI, CJ>, dim3(grid), dim3(kFrontThreads), smem, s, pdl,
                   dim3(1, 1, 1), a.X, a.N, a.K, a.ldx, a.scale, a.shift, a.wbits, a.beta, a.F,
-                  a.words, a.rowptr, a.Z, a.ldz, a.D16, a.ldd16, a.rowscale, a.dots_f16);
+                  a.words, a.rowptr, a.Z, a.ldz, a.D16, a.ldd16, a.rowscale, a.dots8, a.ldd8);
 }
 
 template <int RI>
@@ -217,9 +257,11 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
                    const uint64_t *__restrict__ wbits, const float *__restrict__ beta, int F,
                    int words, const int64_t *__restrict__ rowptr, float *__restrict__ Z,
                    int64_t ldz, uint16_t *__restrict__ D16, int64_t ldd16,
-                   float *__restrict__ rowscale, int P, int pitch, bool f16) {
+                   float *__restrict__ rowscale, int P, int pitch, uint8_t *__restrict__ dots8,
+                   int64_t ldd8) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float part[kSplitWarps];
+    __shared__ int wide_s[kSplitWarps];      // byte planes: row r of the group holds a wide dot
     constexpr int R = kSplitWarps / G;       // rows per group
     constexpr int T = 32 * G;                // threads per row in the product
     constexpr Affine kA = kAffine ? Affine::kShared : Affine::kNone;
@@ -231,7 +273,7 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
     const int rr = tid / T, tt = tid % T, sub = tt % P;
     const int cstep = T / P;                 // columns per pass
     const int Fw = D16 != nullptr ? int(ldd16) : F;   // columns written (with padding)
-    const int passes = (Fw + cstep - 1) / cstep;
+    const int passes = (Fw + cstep - 1) / cstep;      // at most 2 without padding (F <= 128)
     if (kAffine) {
         for (int k0 = tid; k0 < K; k0 += 4 * kSplitThreads) {
             float2 v[4];
@@ -257,6 +299,7 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
                                                                      warp % G)
                                    : 0.0f;
         if (lane == 0) part[warp] = l1;
+        if (tid < R) wide_s[tid] = 0;
         if (!staged) {
             grid_dependency_wait();     // the packed weight columns come from the previous kernel
             const int n = F * words;
@@ -279,15 +322,16 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
         }
         __syncthreads();
         const int64_t row2 = group * R + rr;
+        float ai = 0.0f;
+        int mine[2];                         // byte planes: this lane's dots
         if (row2 < N) {                      // uniform over each warp (T is a multiple of 32)
             float t = 0.0f;
 #pragma unroll
             for (int g = 0; g < G; ++g) t += part[rr * G + g];
-            const float ai =
-                rowptr == nullptr
-                    ? t / float(K)
-                    : (t / float(K)) *
-                          inv_sqrt_degree(__ldg(rowptr + row2 + 1) - __ldg(rowptr + row2));
+            ai = rowptr == nullptr
+                     ? t / float(K)
+                     : (t / float(K)) *
+                           inv_sqrt_degree(__ldg(rowptr + row2 + 1) - __ldg(rowptr + row2));
             if (D16 != nullptr && tt == 0) rowscale[row2] = ai;
             const uint64_t *a = As + size_t(rr) * pitch;
             const ulonglong2 *a2 = reinterpret_cast<const ulonglong2 *>(a);
@@ -309,14 +353,31 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
                     }
                 }
                 for (int o = 1; o < P; o <<= 1) mism += __shfl_xor_sync(kFullMask, mism, o);
+                if (j < 2) mine[j] = K - 2 * mism;
                 if (sub != 0 || c >= Fw) continue;
-                if (D16 != nullptr)
-                    D16[row2 * ldd16 + c] = encode_dot(K - 2 * mism, c < F, f16);
+                if (dots8 != nullptr) {
+                    const ByteDot d(K - 2 * mism, K);
+                    dots8[row2 * ldd8 + c] = uint8_t(d.lo());
+                    if (d.wide()) wide_s[rr] = 1;
+                } else if (D16 != nullptr)
+                    D16[row2 * ldd16 + c] = encode_dot(K - 2 * mism, c < F);
                 else
                     Z[row2 * ldz + c] = ai * (__ldg(beta + c) * float(K - 2 * mism));
             }
         }
         __syncthreads();                     // As and part are rewritten by the next rows
+        if (dots8 != nullptr) {              // the row's flag is known: its scale and high plane
+            const bool wide = wide_s[rr] != 0;
+            if (row2 < N && tt == 0) rowscale[row2] = flag_scale(ai, wide);
+            if (row2 < N && wide && sub == 0)
+                for (int j = 0; j < passes; ++j) {
+                    const int c = tt / P + j * cstep;
+                    if (c < F)
+                        dots8[(N + row2) * ldd8 + c] =
+                            uint8_t(ByteDot(j == 0 ? mine[0] : mine[1], K).hi());
+                }
+            __syncthreads();                 // wide_s is cleared for the next rows
+        }
     }
     if (!staged) grid_dependency_wait();
 }
@@ -342,7 +403,7 @@ void launch_split(const FrontArgs &a, const DeviceInfo &dev, cudaStream_t s, boo
     const size_t smem = split_smem(a.F, a.K, pitch, affine);
     void (*kernel)(const float *, int64_t, int, int64_t, const float *, const float *,
                    const uint64_t *, const float *, int, int, const int64_t *, float *, int64_t,
-                   uint16_t *, int64_t, float *, int, int, bool);
+                   uint16_t *, int64_t, float *, int, int, uint8_t *, int64_t);
     if (G == 2) kernel = affine ? front_split_kernel<2, true> : front_split_kernel<2, false>;
     else if (G == 4) kernel = affine ? front_split_kernel<4, true> : front_split_kernel<4, false>;
     else kernel = affine ? front_split_kernel<8, true> : front_split_kernel<8, false>;
@@ -357,7 +418,7 @@ void launch_split(const FrontArgs &a, const DeviceInfo &dev, cudaStream_t s, boo
     launch_kernel(kernel, dim3(unsigned(groups < resident ? groups : resident)),
                   dim3(kSplitThreads), smem, s, pdl, dim3(1, 1, 1), a.X, a.N, a.K, a.ldx, a.scale,
                   a.shift, a.wbits, a.beta, a.F, a.words, a.rowptr, a.Z, a.ldz, a.D16, a.ldd16,
-                  a.rowscale, P, pitch, a.dots_f16);
+                  a.rowscale, P, pitch, a.dots8, a.ldd8);
 }
 
 }  // namespace

@@ -60,9 +60,14 @@ struct GemmArgs {
     uint16_t *dots16 = nullptr;
     int64_t ldd16 = 0;
     float *rowscale = nullptr;
-    // With dots_f16 the compressed dots are fp16 bits instead (exact for
-    // K <= 2048), padding columns zero: the input of launch_spmm_tc.
-    bool dots_f16 = false;
+    // Compressed output in byte planes instead (nullable; replaces Z and
+    // dots16): the low plane (N rows of ldd8 bytes, a multiple of 16 >= F) and,
+    // N * ldd8 bytes on, the high plane, of which only the rows whose scale in
+    // rowscale carries the wide flag are written (ByteDot, flag_scale); padding
+    // columns hold anything. The input of launch_spmm_tc. Needs
+    // xnor_gemm_bytes_supported.
+    uint8_t *dots8 = nullptr;
+    int64_t ldd8 = 0;
     // Nullable device scratch of xnor_gemm_tc_bexp_bytes(K, F) bytes (16-byte
     // aligned): the tensor-core product then expands B's signs to FP8 once
     // into it, and each CTA copies its tiles instead of expanding them.
@@ -80,6 +85,11 @@ bool xnor_gemm_tc_supported(int64_t N, int K, int F, const DeviceInfo &dev);
 struct GemmArgs;
 void launch_xnor_gemm_tc(const GemmArgs &args, const DeviceInfo &dev, cudaStream_t stream,
                          bool pdl);
+
+// Whether launch_xnor_gemm can write byte planes: a row's wide flag needs all
+// of the row's dots in one block (256 columns on the tensor cores, 64 on the
+// CUDA cores), unless K <= 254, where no dot is wide.
+bool xnor_gemm_bytes_supported(int64_t N, int K, int F, const DeviceInfo &dev);
 
 // Step 4: the XNOR-popcount product and its scaling (Eqs. 11-12).
 void launch_xnor_gemm(const GemmArgs &args, const DeviceInfo &dev, cudaStream_t stream,
@@ -162,7 +172,8 @@ struct FrontArgs {
     uint16_t *D16 = nullptr;
     int64_t ldd16 = 0;
     float *rowscale = nullptr;
-    bool dots_f16 = false;   // as in GemmArgs
+    uint8_t *dots8 = nullptr;    // byte planes, as in GemmArgs
+    int64_t ldd8 = 0;
 };
 
 // Whether the fused pack + XNOR-GEMM kernel fits (F <= 128, packed tiles in
@@ -212,51 +223,52 @@ void launch_spmm_pack_gemm(const SpmmPackGemmArgs &args, const DeviceInfo &dev,
                            cudaStream_t stream, bool pdl = false);
 
 // Step 5 on the tensor cores (spmm_tc.cu) over a product kept factored as
-// fp16 integer dots (exact for |dot| <= 2048): H_if = colscale_f *
-// (1/sqrt(dhat_i)) * sum_{j in N(i) u {i}} rowscale_j * D[j, f], with
-// rowscale_j carrying 1/sqrt(dhat_j). D's rows hold ldd halves (a multiple of
-// 8, at least F rounded up to 16); features F .. round_up(F, 16) must hold
-// zero dots. F <= 128.
+// integer dots in byte planes: H_if = colscale_f * (1/sqrt(dhat_i)) *
+// sum_{j in N(i) u {i}} rowscale_j * dot[j, f], with rowscale_j carrying
+// 1/sqrt(dhat_j) and, in its sign bit, row j's wide flag. D's low plane has
+// rows of ldd bytes (a multiple of 16 >= F), the high plane follows N * ldd
+// bytes on. K's parity is that of every dot.
 struct SpmmTcArgs {
     const int64_t *rowptr;
     const int32_t *colidx;
     int64_t N;
     int64_t nnz;
-    const uint16_t *D;       // fp16 bits
+    const uint8_t *D;
     int64_t ldd;
-    const float *rowscale;   // N
+    const float *rowscale;   // N; nullptr: the last four bytes of D's rows (ldd - F >= 4, F <= 128)
     int F;
+    int K;
     float *H;                // N x F (row stride ldh)
     int64_t ldh;
     const float *colscale;   // nullable: 1
-    int32_t *pred;           // nullable: each row's argmax (lowest index on ties)
+    int32_t *pred;           // nullable: each row's argmax (lowest index on ties; F <= 128)
 };
-bool spmm_tc_supported(int F);
 void launch_spmm_tc(const SpmmTcArgs &args, const DeviceInfo &dev, cudaStream_t stream,
                     bool pdl = false);
 
 // Layer 1's tensor-core aggregation fused with layer 2's binarization and
-// XNOR product (spmm_tc.cu): from layer 1's fp16 dots D1 (row scale s1,
-// column scale beta1) to layer 2's fp16 dots D2 (rows of ldd2 halves, a
-// multiple of 8 >= Fo rounded up to 16, zeros past Fo) and row scale s2
+// XNOR product (spmm_tc.cu): from layer 1's byte planes D1 (row scale s1,
+// column scale beta1) to layer 2's D2 (low plane only, rows of ldd2 bytes, a
+// multiple of 16 >= Fo: with Fh <= 128 no dot is wide) and row scale s2
 // (alpha2_i / sqrt(dhat_i)); H1 (nullable) receives layer 1's output.
 struct SpmmTcPackGemmArgs {
     const int64_t *rowptr;
     const int32_t *colidx;
     int64_t N;
     int64_t nnz;
-    const uint16_t *D1;
+    const uint8_t *D1;
     int64_t ldd1;
     const float *s1;
     int Fh;
+    int K;                   // layer 1's input features
     const float *beta1;
     float *H1;
     int64_t ldh1;
     const uint64_t *wbits2;  // Fo x ceil(Fh / 64)
     int Fo;
-    uint16_t *D2;
+    uint8_t *D2;
     int64_t ldd2;
-    float *s2;
+    float *s2;               // nullptr: the last four bytes of D2's rows (ldd2 - Fo >= 4)
 };
 bool spmm_tc_pack_gemm_supported(int Fh, int Fo);
 void launch_spmm_tc_pack_gemm(const SpmmTcPackGemmArgs &args, const DeviceInfo &dev,

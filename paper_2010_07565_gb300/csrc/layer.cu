@@ -13,9 +13,10 @@
 // fit 16 bits (K <= 32767) the product leaves Z factored: the integer dots
 // and the row scale s_j = alpha_j / sqrt(dhat_j), and the aggregation applies
 // s_j per neighbour and beta_f per column, so each gathered row is half the
-// bytes. With K <= 2048 the dots are fp16 (exact) and the aggregation runs on
-// the tensor cores (spmm_tc.cu); else they are biased uint16 and it runs on
-// the CUDA cores (spmm.cu).
+// bytes. Where a row's dots lie in one block of the product the dots are kept
+// in byte planes (ByteDot) and the aggregation runs on the tensor cores
+// (spmm_tc.cu); else they are biased uint16 and it runs on the CUDA cores
+// (spmm.cu).
 #include <mutex>
 
 #include "launch.cuh"
@@ -53,18 +54,25 @@ constexpr int32_t kMaxDots16K = 32767;
 
 // Workspace carve-up of the fused layer; every piece 256-byte aligned. Z is
 // either fp32 (N x F) or compressed: uint16 dots (N x round_up(F, 8), so that
-// the aggregation can load eight dots at a time) and a row scale (N); then the
+// the aggregation can load eight dots at a time) or two byte planes (N x
+// round_up(F, 16) each), and a row scale (N); then the
 // FP8 tiles of the weight signs for the tensor-core product (about F x K bytes
 // when K >= 128 and F >= 32).
 struct LayerWorkspace {
     size_t a_bits, alpha, b_bits, beta, z, rowscale, bexp, bexp_bytes, total;
     bool compressed;
-    bool f16;                // dots as fp16 (K <= 2048): the tensor-core aggregation
-    int64_t ldd;             // halves per compressed row
+    bool planes;             // both byte planes fit the Z piece
+    int64_t ldd;             // uint16 dots per compressed row
+    int64_t ldd8;            // bytes per row of a byte plane
 };
 
-// Largest K whose dots fp16 holds exactly.
-constexpr int32_t kMaxDotsF16K = 2048;
+// Largest K whose dots are kept in byte planes. Signs that agree half the time
+// give dots of standard deviation sqrt(K): at K = 3072 one in 10^6 does not fit
+// the low byte, at 4096 one in 15000, so that of 256-feature rows one in 60 is
+// wide and most blocks of 32 need their second pass (2^20 rows, F = 256: K =
+// 3000 at 664 us for half the rows, K = 4096 at 2013 us against 2011 us for
+// uint16 dots on the CUDA cores).
+constexpr int32_t kMaxPlanesK = 3072;
 
 bool layer_workspace(int64_t N, int32_t K, int32_t F, LayerWorkspace *w) {
     if (N < 0 || K < 1 || F < 1) return false;
@@ -72,12 +80,12 @@ bool layer_workspace(int64_t N, int32_t K, int32_t F, LayerWorkspace *w) {
     const int64_t F8 = (int64_t(F) + 7) / 8 * 8;
     if (N > kMaxElems / (words > F8 ? words : F8)) return false;
     w->compressed = K <= kMaxDots16K;
-    // fp16 dots and the tensor-core aggregation for rows of up to 128 features
-    // (wider rows would walk their index lists once per 128-feature slab; the
-    // CUDA-core aggregation was measured faster at 256: 2047 vs 2567 us on
-    // 2^20 nodes of mean degree 16).
-    w->f16 = K <= kMaxDotsF16K && F <= 128;
-    w->ldd = w->f16 ? (int64_t(F) + 15) / 16 * 16 : F8;
+    w->ldd8 = (int64_t(F) + 15) / 16 * 16;
+    // Rows of uint16 dots are padded to 16 features where F <= 128 and K <= 2048,
+    // to 8 elsewhere; two byte planes (padded to 16) take the same bytes when
+    // the paddings agree, and no others are used: the workspace does not grow.
+    w->ldd = K <= 2048 && F <= 128 ? w->ldd8 : F8;
+    w->planes = K <= kMaxPlanesK && w->ldd == w->ldd8;
     size_t off = 0;
     w->a_bits = off; off = round_up(off + size_t(N) * size_t(words) * 8);
     w->alpha = off;  off = round_up(off + size_t(N) * 4);
@@ -191,9 +199,12 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     EventMarks marks(events, n_events, s);
     if (!marks.ok()) return BIGCN_ERR_CUDA;
 
-    // Few long rows: centring, packing and the product in one kernel (the
-    // split front), after the weights are packed.
-    const bool fused = front_split_supported(N, K, F, dev);
+    // Few long rows, or rows too few for a tensor-core product: centring, packing
+    // and the product in one kernel (the front), after the weights are packed.
+    const bool small = F <= 128 && K <= 2048 && N < 128 * int64_t(dev.sm_count);
+    const bool fused =
+        front_split_supported(N, K, F, dev) || (small && front_supported(N, K, F, dev));
+    const bool bytes = w.planes && (fused || xnor_gemm_bytes_supported(N, K, F, dev));
     marks.mark();
     if (!fused) launch_pack_rows(X, N, K, ldx, scale, shift, a_bits, words, alpha, dev, s);
     marks.mark();
@@ -202,14 +213,18 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     GemmArgs g{a_bits, alpha, N, b_bits, beta, F, K, words, Zs, F, nullptr, rowptr};
     if (w.bexp_bytes > 0) g.b_e4m3 = reinterpret_cast<uint8_t *>(ws + w.bexp);
     SpmmArgs a{rowptr, colidx, N, nnz, Zs, F, F, H, ldh, true, false};
-    if (w.compressed) {
+    if (bytes) {
+        g.Z = nullptr;
+        g.dots8 = reinterpret_cast<uint8_t *>(ws + w.z);
+        g.ldd8 = w.ldd8;
+        g.rowscale = reinterpret_cast<float *>(ws + w.rowscale);
+    } else if (w.compressed) {
         uint16_t *D16 = reinterpret_cast<uint16_t *>(ws + w.z);
         float *rowscale = reinterpret_cast<float *>(ws + w.rowscale);
         g.Z = nullptr;
         g.dots16 = D16;
         g.ldd16 = w.ldd;
         g.rowscale = rowscale;
-        g.dots_f16 = w.f16;
         a.Z = nullptr;
         a.ldz = w.ldd;
         a.D16 = D16;
@@ -218,14 +233,14 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     }
     if (fused) {
         FrontArgs fr{X, N, K, ldx, scale, shift, b_bits, beta, F, words, rowptr, g.Z, g.ldz,
-                     g.dots16, g.ldd16, g.rowscale, g.dots_f16};
+                     g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8};
         launch_front(fr, dev, s);
     } else {
         launch_xnor_gemm(g, dev, s);
     }
     marks.mark();
-    if (w.f16) {        // fp16 dots: the aggregation on the tensor cores
-        SpmmTcArgs t{rowptr, colidx, N, nnz, a.D16, w.ldd, a.rowscale, F, H, ldh, beta, nullptr};
+    if (bytes) {        // byte planes: the aggregation on the tensor cores
+        SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, w.ldd8, g.rowscale, F, K, H, ldh, beta, nullptr};
         launch_spmm_tc(t, dev, s);
     } else {
         launch_spmm_norm(a, dev, s);

@@ -4,45 +4,64 @@
 //   H_if = c_f * (1/sqrt(dhat_i)) * sum_{j in N(i) u {i}} s_j * dot_jf
 //
 // with s_j = alpha_j / sqrt(dhat_j) the row scale and c_f = beta_f the column
-// scale of Eqs. 11-12. The dots are stored as fp16 (exact: |dot| <= K <= 2048)
-// in rows of 16 * FT features (padding features hold zero dots).
+// scale of Eqs. 11-12. The dots come in byte planes (ByteDot): one byte per
+// dot, rows of 16 * FT features, and a second byte for the rows marked wide.
 //
 // Why tensor cores: the aggregation reads one row of dots per CSR entry. Done
 // on CUDA cores, every gathered dot costs a decode and an FMA, and the kernel
 // is bound by instruction issue well below what L2 delivers to random row
 // gathers. Here the sum over a run of 16 CSR entries is one
-// mma.sync.m16n8k16 per 16 features: A = the 16 gathered rows (features x
-// entries, read from shared memory with ldmatrix.trans), B = the entries'
-// weights s_j, D = fp32 accumulators. The MMA consumes the fp16 dots as they
-// are, so no decode instruction remains.
+// mma.sync.m16n8k16 per 16 features: A = the gathered rows (features x
+// entries), B = the entries' weights s_j, D = fp32 accumulators.
+//
+// Why bytes: the walk is bound by latency -- rows in flight per SM, that is
+// shared memory per gathered row, and the dependent steps between a block's
+// arrival and the next -- not by L2's bandwidth (20 TB/s for such gathers). A
+// byte per dot halves a staged row against fp16, which buys deeper rings and
+// half as many copies, for one permute and one packed fma per two dots. On
+// 232,965 nodes of mean degree 492 (114.8 M gathered rows): layer 1, 128
+// features, 2600 -> 1880 us (7.8 TB/s of 128-byte rows; issue 51 %, ALU and the
+// copies' latency bind); layer 2, 41 features, 1475 -> 1160 us. On 2^20 nodes of
+// mean degree 16, 64 features: 787 -> 464 us.
+//
+// A staged row is read with ldmatrix.trans as pairs of neighbouring features:
+// a lane's register then holds features 2g and 2g + 1 of two entries, which a
+// byte permute turns into two A registers (even features in matrix rows 0-7,
+// odd ones in rows 8-15). The bytes u = lo + 128 enter as fp16 subnormals u
+// 2^-24, and one packed fma, u 2^-24 * 2^15 + ((K & 1) - 256) 2^-10, makes
+// them dot * 2^-10: every step exact, and no entry's value ever leaves fp16.
+// Rows marked wide add hi * 2^-1 (dot = 2 lo + (K & 1) + 512 hi) in a second
+// walk over the blocks that hold any, with the weights of the other entries
+// zero: as long as the first where every row is wide.
 //
 // B carries the weights as two fp16 parts, hi = fp16(s' ) and lo = fp16(s' -
 // hi) with s' = s_j * 2^(14 - E) (an exact power-of-two scaling that puts the
 // row's largest weight just below 2^15), so the product keeps 22 bits of each
-// weight; hi and lo land in separate accumulator columns and are added in
-// fp32 at the end. E is the largest exponent among the weights seen so far for
+// weight. E is the largest exponent among the weights seen so far for
 // that output row: when a later entry raises it, the row's accumulators are
 // multiplied by the exact power of two that keeps them consistent.
 //
-// A warp takes a window of up to 4 consecutive output rows: their lists
-// (self entry first, then the CSR neighbours) are walked as one stream of
-// positions, 16 at a time, and output row r of the window owns B columns
-// 2r (hi) and 2r + 1 (lo). Lane (g, t) of the MMA's fragment layout then
-// holds row t's sums for features 16 T + g and 16 T + g + 8 of every tile T.
+// A warp takes a window of consecutive output rows whose lists (self entry
+// first, then the CSR neighbours) it walks as one stream of positions, 32 to a
+// block. One-row windows (long rows) put hi and lo in columns 0 and 1 of B;
+// eight-row windows (short rows, so that a block is not mostly padding) give
+// column r to output row r and multiply twice, by the hi and by the lo parts,
+// into sums of their own (added to the same sums, the lo products would be
+// rounded at the hi sums' last place: 1.3e-7 from 64 bits instead of 1.0e-7).
 // Gathered rows are staged by cp.async (16 bytes per copy; positions past the
-// end of the stream and out-of-range column indices copy zeros and carry zero
-// weight) in a per-warp ring of two (or three) blocks, XOR-swizzled so that
-// ldmatrix reads are free of bank conflicts without padding the rows: the
-// copies of the next block(s) are in flight while block n is multiplied, and
-// the column indices, copied two blocks further ahead, and the row scales go
-// through shared memory too, so the loop never waits on a register loaded
-// from global memory.
+// end of the stream and out-of-range column indices copy nothing and carry
+// zero weight: any stale byte is a finite fp16) in a per-warp ring,
+// XOR-swizzled so that ldmatrix reads are free of bank conflicts: the copies
+// of the next block(s) are in flight while block n is multiplied. The column
+// indices are loaded one block ahead of the copies they name and the row scales
+// along with their rows, both into registers (a lane owns one position of a
+// block), so that neither is waited for.
 //
-// Rows with more than `heavy_degree` neighbours are each walked by all 8 warps
+// Rows with more than `heavy_degree` neighbours are each walked by all warps
 // of one block, whose fp32 partial rows are added in warp order
 // (deterministic); light windows go one per warp, or, when there are many,
-// in turn to the warps of one wave of persistent blocks that first walk the
-// heavy rows.
+// to the warps of one wave of persistent blocks, which first walk the heavy rows
+// and then take the windows of their block's share as they become free.
 #include <cuda_fp16.h>
 
 #include "launch.cuh"
@@ -50,53 +69,62 @@
 namespace bigcn {
 namespace {
 
-constexpr int kTcThreads = 256;
+constexpr int kTcThreads = 128;
 constexpr int kTcWarps = kTcThreads / 32;
-constexpr int kTcRows = 4;          // output rows per light window
+constexpr int kTcRows = 8;          // output rows per window of short rows
+constexpr int EB = 32;              // positions per sub-block: one per lane
 
-// Entries per block: 32 for narrow rows in one-row windows (every lane owns
-// an entry, and the per-block work -- index copies, waits, scales, B
-// fragments -- covers twice the entries; two MMA k-steps per block; layer 2 on
-// the Reddit-shaped graph: 2.04 -> 1.93 ms), else 16 (wide rows would leave one
-// block per SM; in four-row windows 32 was measured slower: 835 -> 1215 us on
-// 2^20 nodes of mean degree 16).
-constexpr int tc_entries_per_block(int FT, int ROWS) { return ROWS == 1 && FT <= 4 ? 32 : 16; }
+// Per width and window form: sub-blocks per block, blocks in a warp's ring, and
+// the blocks (of 4 warps) per SM that the registers are held to. Fewer warps with
+// more registers and rows in flight beat more warps: 128 features in one-row
+// windows, 16 warps and three stages of 4 KB 1873 us, 20 warps and two 2245 us, 24
+// warps and two 2368 us (24 in blocks of eight warps, whose windows their warps
+// share less evenly, 2369 us), 12 warps and four 2084 us; 41 features, 20 warps
+// and two stages of 64 rows 1160 us, 24 warps and four of 32 1249 us. Eight-row
+// windows of 33 to 64 features spill at 96 registers (20 warps: 548 us, 16 warps
+// 464 us on 2^20 rows).
+constexpr int tc_sub(int FT, int ROWS) { return FT > 4 || ROWS > 1 ? 1 : 2; }
+constexpr int tc_stages(int FT, int ROWS) { return FT > 4 ? 3 : 2; }
+constexpr int tc_blocks(int FT, int ROWS) { return FT > 4 || (FT > 2 && ROWS > 1) ? 4 : 5; }
 
-template <int FT, int NSTAGES, int EBLOCK>
+// Tiles of 16 features, sub-blocks per block, blocks in the ring.
+template <int FT, int SUB, int NSTAGES>
 struct TcGeom {
-    static constexpr int FP = 16 * FT;             // features per staged row
-    static constexpr int CH = 2 * FT;              // 16-byte copies per row
-    // Bytes per staged row: the row's 32 FT bytes rounded up to a multiple of
-    // 128, its 16-byte chunk c stored at slot c ^ (r & 7) of staged row r. The
-    // eight rows an ldmatrix reads then fall in eight different bank groups,
-    // and the two halves of every 32-byte sector of a gathered row stay in one
-    // aligned 32-byte slot pair (a padded pitch of 32 FT + 16 bytes split a
-    // sector over two shared-memory lines on every other row: 256-byte rows
-    // gathered at 13.7 TB/s instead of 20.6 TB/s, 96-byte rows at 8.8 instead
-    // of 13.0 TB/s, 24 warps per SM).
-    static constexpr int PITCH = (FP * 2 + 127) / 128 * 128;
-    static constexpr int EB = EBLOCK;              // entries per block (16 or 32)
-    static constexpr int KCH = EB * CH / 32;       // 16-byte row copies per lane and block
-    static constexpr int STAGE = EB * PITCH;       // one block of EB entries
+    static constexpr int P2 = FT <= 1 ? 1 : FT <= 2 ? 2 : FT <= 4 ? 4 : 8;   // chunks per staged row
+    // Bytes per staged row, 16 P2: 8 / P2 rows to a 128-byte line, the row's
+    // 16-byte chunk c stored at slot c ^ (row / (8 / P2)) mod P2. The eight rows
+    // an ldmatrix reads then fall in eight different bank groups, and the two
+    // halves of every 32-byte sector of a gathered row stay in one aligned
+    // 32-byte slot pair (a padded pitch that splits sectors over two
+    // shared-memory lines fetches them twice: 256-byte rows gathered at 13.7
+    // TB/s instead of 20.6 TB/s, 96-byte rows at 8.8 instead of 13.0 TB/s).
+    static constexpr int PITCH = 16 * P2;
+    static constexpr int LINE = 8 / P2;            // staged rows per 128-byte line
+    static constexpr int STEP = 32 / P2;           // rows covered by one copy per lane
+    static constexpr int PART = EB * PITCH;        // one sub-block
+    static constexpr int STAGE = SUB * PART;       // one block
     static constexpr int NS = NSTAGES;             // row ring depth (blocks)
     static constexpr int D = NS - 1;               // blocks of rows copied ahead
-    static constexpr int DI = 2;                   // groups between a block's index copy and its row copy
-    static constexpr int NI = DI + 1;              // index slots
-    // one warp's ring: NS row stages, NS x EB row scales, NI x EB column
-    // indices (a multiple of 128 bytes, so that every stage starts on a
-    // 128-byte line)
-    static constexpr int WARP = (NS * STAGE + NS * EB * 4 + NI * EB * 4 + 127) / 128 * 128;
+    // One warp's ring: NS row stages (each starting on a 128-byte line), then the
+    // checked columns of the block being copied and the weights of the block
+    // being multiplied (per sub-block EB hi and EB lo halves).
+    static constexpr int CHECKED = NS * STAGE;
+    static constexpr int HALVES = CHECKED + SUB * EB * 4;
+    static constexpr int WARP = HALVES + SUB * EB * 4;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
     return uint32_t(__cvta_generic_to_shared(p));
 }
 
-// 16-byte global -> shared copy; copies zeros when `live` is false.
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool live) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
-                 "r"(live ? 16 : 0)
-                 : "memory");
+// 16-byte global -> shared copy, skipped for j < 0 (a predicate, not a branch).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, int j) {
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "setp.ge.s32 p, %2, 0;\n"
+        "@p cp.async.cg.shared.global [%0], [%1], 16;\n}" ::"r"(dst),
+        "l"(src), "r"(j)
+        : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() {
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -122,6 +150,23 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// Two low bytes (as fp16 subnormals u 2^-24) to two dots times 2^-10.
+__device__ __forceinline__ uint32_t bytes_to_half2(uint32_t h, uint32_t offset) {
+    uint32_t r;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(h), "r"(0x78007800u), "r"(offset));
+    return r;
+}
+// Two high bytes (hi + 128, the same way) to hi * 2^-1.
+__device__ __forceinline__ uint32_t high_to_half2(uint32_t h) {
+    uint32_t r;     // (u 2^-24 2^15 - 2^-2) 2^8 = (u - 128) 2^-1
+    asm("{\n.reg .b32 t;\n"
+        "fma.rn.f16x2 t, %1, %2, %3;\n"
+        "mul.rn.f16x2 %0, t, %4;\n}"
+        : "=r"(r)
+        : "r"(h), "r"(0x78007800u), "r"(0xB400B400u), "r"(0x5C005C00u));
+    return r;
+}
+
 // 2^e as a float for e in [-126, 127].
 __device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) << 23); }
 
@@ -129,359 +174,483 @@ __device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) 
 __device__ __forceinline__ int exponent_of(uint32_t bits) { return int(bits >> 23) - 127; }
 
 constexpr int kNoScale = -126;      // exponent of a row that has seen no weight yet
+constexpr int kDotShift = 10;       // the A operands are dots times 2^-10
 
 struct TcParams {
     const int64_t *rowptr;
     const int32_t *colidx;
     int64_t N;
     int64_t nnz;
-    const uint16_t *D;       // N x ldd fp16 dots
-    int64_t ldd;             // halves; a multiple of 8, >= 16 * FT
-    const float *rowscale;   // s_j
+    const uint8_t *D;        // low plane, N x ldd bytes; the high plane follows
+    int64_t ldd;             // bytes; a multiple of 16
+    const float *rowscale;   // s_j, negative for a wide row; nullptr: kept in D's rows
+    uint32_t offset;         // ((K & 1) - 256) 2^-10, twice, in fp16
     int64_t heavy_degree;    // rows with more neighbours are walked by whole blocks
-    bool off32;              // N * ldd * 2 < 2^32: row byte offsets fit 32 bits
-    int f_base;              // first feature of this launch (column slab y: f_base + 16 FT y)
     int heavy_blocks;        // blocks [0, heavy_blocks) walk the heavy rows
     int light_first;         // blocks [light_first, grid) walk the light windows
 };
 
-// A window: up to ROWS output rows, each contributing the list entries
-// [q0, q0 + len) of its list (entry 0 = the self-loop, entry q > 0 = CSR
-// neighbour q - 1), laid out one after the other as positions. Position p of
-// row r is the row's self-loop when p == selfp[r], else CSR entry cbase[r] + p.
+// A window: ROWS consecutive output rows, each contributing its list (entry 0 =
+// the self-loop, entry q > 0 = CSR neighbour q - 1) or, for a part of a heavy
+// row, entries [q0, q1) of it, laid out one after the other as positions.
+// Row r covers positions [off[r], off[r + 1]); position p of it is the self-loop
+// when p == its self position, else CSR entry cbase + p. With eight rows,
+// lane r holds row r's cbase.
 template <int ROWS>
 struct Window {
-    int64_t row[ROWS];       // -1: inactive (no positions)
-    int64_t cbase[ROWS];
-    int selfp[ROWS];
-    int off[ROWS + 1];       // first position of each row; off[ROWS] = stream length
+    int64_t first;           // output row of r = 0
+    int64_t cbase;           // ROWS == 1: the row's; else of row (lane & 7)
+    bool self0;              // ROWS == 1: position 0 is the self-loop (else off[r] are)
+    int off[ROWS + 1];       // off[ROWS] = stream length
 };
 
-// a[r] for a row r known only at run time, as a chain of selects (indexing the
-// array dynamically would place the window in local memory).
-template <int ROWS, class T>
-__device__ __forceinline__ T pick(const T *a, int r) {
-    T v = a[0];
-#pragma unroll
-    for (int k = 1; k < ROWS; ++k)
-        if (r == k) v = a[k];
-    return v;
-}
-
+// The row that position p belongs to (zero-length rows hold none).
 template <int ROWS>
-__device__ __forceinline__ int tag_of(const Window<ROWS> &w, int p) {
+__device__ __forceinline__ int row_of(const Window<ROWS> &w, int p) {
     int r = 0;
 #pragma unroll
     for (int k = 1; k < ROWS; ++k) r += int(p >= w.off[k]);
     return r;
 }
 
-// Column index of the entry at position p, or -1 (past the end, or out of range).
+// The column that position p of the stream gathers: the CSR's (unchecked), the
+// output row's own for a self-loop, -1 past the end. Called by all lanes
+// together.
 template <int ROWS>
-__device__ __forceinline__ int fetch_col(const TcParams &P, const Window<ROWS> &w, int p) {
-    if (p >= w.off[ROWS]) return -1;
-    const int r = tag_of(w, p);
-    const int64_t j = p == pick<ROWS>(w.selfp, r) ? pick<ROWS>(w.row, r)
-                                                   : int64_t(__ldg(P.colidx + pick<ROWS>(w.cbase, r) + p));
-    return (j >= 0 && j < P.N) ? int(j) : -1;
+__device__ __forceinline__ int fetch_column(const TcParams &P, const Window<ROWS> &w, int p) {
+    int j = -1;
+    if constexpr (ROWS == 1) {
+        if (p < w.off[1])
+            j = w.self0 && p == 0 ? int(w.first) : __ldg(P.colidx + (w.cbase + p));
+    } else {
+        const int r = row_of<ROWS>(w, p);
+        int start = w.off[0];
+#pragma unroll
+        for (int k = 1; k < ROWS; ++k) start = r >= k ? w.off[k] : start;
+        const int64_t entry = __shfl_sync(kFullMask, w.cbase, r) + p;
+        if (p < w.off[ROWS]) j = p == start ? int(w.first) + r : __ldg(P.colidx + entry);
+    }
+    return j;
 }
 
-// Per-lane sums of a window after its walk: row t = lane & 3, features
-// 16 T + g and 16 T + g + 8 (g = lane >> 2), scaled back to fp32 values.
-template <int FT>
+// Per-lane sums of a window after its walk: R2 output rows (ROWS == 1: lanes
+// with t = 0 hold the row; else lane (g, t) holds rows 2t and 2t + 1), features
+// 16 T + 2g and 16 T + 2g + 1 (g = lane >> 2, t = lane & 3), as fp32 values.
+template <int FT, int R2>
 struct TcRowSums {
-    float v[FT][2];
+    float v[R2][FT][2];
 };
 
-// Walks a window's position stream and leaves its sums in `out`. The warp's
-// ring `ring` (shared, TcGeom<FT, NS, EB>::WARP bytes) is free on entry and on exit.
-//
-// Pipeline (blocks of EB positions; lane e = lane mod EB owns position e of a
-// block; with EB = 16 lanes 16-31 repeat lanes 0-15). Group m of cp.async
-// copies holds block m + D's rows and row scales and block m + D + DI's column
-// indices. Iteration n first waits for group n - DI (block n + D's indices),
-// issues group n -- so that its rows are in flight while the warp waits for
-// block n -- then waits for group n - D (block n's rows) and multiplies. No
-// register of the loop waits on a global load. Block b uses row stage b mod NS
-// and index slot b mod NI.
-template <int FT, int ROWS, int NS, int EBLOCK>
-__device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS> &w,
-                                           uint8_t *ring, TcRowSums<FT> &out) {
-    using G = TcGeom<FT, NS, EBLOCK>;
+// A lane's column j (-1: copies nothing) for copy_plane, in shared memory
+// (`checked`), permuted so that a lane there reads the columns of its P2 rows at
+// once: one store and one or two loads instead of P2 shuffles.
+template <class G>
+__device__ __forceinline__ void put_column(int *checked, int j) {
+    const int lane = threadIdx.x & 31;
+    checked[(lane % G::STEP) * G::P2 + lane / G::STEP] = j;
+}
+
+// The copy of one sub-block's rows of a plane to shared address `stage`.
+// Copy k of a lane moves chunk `piece` of staged row r0 + k STEP to its slot,
+// which for P2 = 8 alternates between two (4 rows on, bit 2 of the row flips),
+// else is the same for every k. `plane` points at chunk `piece` of row 0; `mine`:
+// the lane's chunk exists.
+template <class G>
+__device__ __forceinline__ void copy_plane(uint32_t stage, const int *checked,
+                                           const uint8_t *plane, uint32_t row_bytes, bool mine) {
+    constexpr int P2 = G::P2;
+    const int lane = threadIdx.x & 31;
+    const int r0 = lane / P2, piece = lane % P2;
+    const uint32_t base =
+        stage + uint32_t(r0 * G::PITCH + ((piece ^ ((r0 / G::LINE) & (P2 - 1))) << 4));
+    int jj[P2];
+    if constexpr (P2 == 1) {
+        jj[0] = checked[lane];
+    } else {
+        if constexpr (P2 == 2) {
+            const int2 v = *reinterpret_cast<const int2 *>(checked + r0 * 2);
+            jj[0] = v.x, jj[1] = v.y;
+        } else {
+#pragma unroll
+            for (int q = 0; q < P2 / 4; ++q) {
+                const int4 v = *reinterpret_cast<const int4 *>(checked + r0 * P2 + 4 * q);
+                jj[4 * q] = v.x, jj[4 * q + 1] = v.y, jj[4 * q + 2] = v.z, jj[4 * q + 3] = v.w;
+            }
+        }
+    }
+    if (mine)
+#pragma unroll
+        for (int k = 0; k < P2; ++k)
+            cp_async16((base ^ (P2 == 8 && (k & 1) ? 64u : 0u)) + uint32_t(k * G::STEP * G::PITCH),
+                       plane + uint64_t(uint32_t(jj[k])) * row_bytes, jj[k]);
+}
+
+// A window's sums in the MMA's accumulator layout: ROWS == 1 hi and lo in columns
+// 0 and 1; else hi (v[0]) and lo (v[1]) with a column per row.
+template <int FT, int ROWS>
+struct TcSums {
+    static constexpr int PARTS = ROWS == 1 ? 1 : 2;
+    float v[PARTS][FT][4];
+    // Multiplies all sums of a lane's even and odd columns.
+    __device__ __forceinline__ void scale(float even, float odd) {
+#pragma unroll
+        for (int p = 0; p < PARTS; ++p)
+#pragma unroll
+            for (int T = 0; T < FT; ++T)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[p][T][q] *= (q & 1) ? odd : even;
+    }
+};
+
+// A lane's weight on its row's scale as its two fp16 parts in shared memory (`halves`:
+// EB hi parts, then EB lo parts), entries 2t, 2t + 1, and those 8, 16 and 24 on,
+// next to one another, so that a lane's B fragments are one load.
+__device__ __forceinline__ void put_weight(uint16_t *halves, float ws) {
+    const int lane = threadIdx.x & 31;
+    const __half hi = __float2half_rn(ws);
+    const __half lo = __float2half_rn(ws - __half2float(hi));
+    const int at = ((lane >> 1) & 3) * 8 + (lane >> 3) * 2 + (lane & 1);
+    halves[at] = __half_as_ushort(hi);
+    halves[EB + at] = __half_as_ushort(lo);
+}
+
+// One pass over a staged sub-block (shared address `rows` = the sub-block + this
+// lane's ldmatrix row) with the weights in `halves`. ROWS == 1: hi in column 0
+// and lo in column 1 of B; else column g holds the hi (b) or lo (c) parts of row
+// g, whose positions are those with 0 <= position - glo < glen (rel = the
+// sub-block's first position - glo). Per 16 features one ldmatrix (four 8-entry
+// groups) feeds the MMAs of both k-steps.
+template <int FT, int ROWS, class Convert>
+__device__ __forceinline__ void multiply(TcSums<FT, ROWS> &acc, uint32_t rows,
+                                         const uint16_t *halves, int rel, uint32_t glen,
+                                         Convert convert) {
     const int lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
-    constexpr int EB = G::EB;
-    const int e16 = lane & (EB - 1);        // this lane's entry of a block
-    const int total = w.off[ROWS];
-    const int nblk = (total + EB - 1) / EB;
-    const uint32_t rows_s = smem_addr(ring);
-    float *wslot = reinterpret_cast<float *>(ring + G::NS * G::STAGE);   // NS x EB scales
-    int *cslot = reinterpret_cast<int *>(wslot + G::NS * EB);            // NI x EB indices
-    const uint32_t wslot_s = smem_addr(wslot), cslot_s = smem_addr(cslot);
-    const uint32_t n32 = uint32_t(P.N);     // N <= INT32_MAX
-    // Copy plan of one block's rows: chunk q = lane + 32 k -> row q / CH, piece
-    // q % CH, stored at slot piece ^ (row & 7) of the staged row. For CH a power
-    // of two a lane's rows are r0 + k S (S = 32 / CH) and its slots repeat with
-    // period 8 / S, so only that many destinations are kept.
-    constexpr bool kPow2 = (G::CH & (G::CH - 1)) == 0;
-    constexpr int kStep = kPow2 ? 32 / G::CH : 0;
-    constexpr int kPer = kPow2 ? (kStep >= 8 ? 1 : 8 / kStep) : G::KCH;
-    constexpr int kArr = kPow2 ? 1 : G::KCH;
-    int crow[kArr], cpo[kArr];
-    uint32_t cdst[kPer];
-    if constexpr (kPow2) {
-        const int r0 = lane / G::CH, piece = lane % G::CH;
-        crow[0] = r0;
-        cpo[0] = piece * 16;
-#pragma unroll
-        for (int m = 0; m < kPer; ++m)
-            cdst[m] = uint32_t(r0 * G::PITCH + ((piece ^ ((r0 + m * kStep) & 7)) * 16));
+    uint4 b = make_uint4(0u, 0u, 0u, 0u), c = b;
+    if constexpr (ROWS == 1) {
+        if (g < 2) b = *reinterpret_cast<const uint4 *>(halves + g * EB + t * 8);
     } else {
+        b = *reinterpret_cast<const uint4 *>(halves + t * 8);
+        c = *reinterpret_cast<const uint4 *>(halves + EB + t * 8);
+        auto mask = [&](int e) {
+            const uint32_t p = uint32_t(rel + 2 * t + e);
+            return (p < glen ? 0xffffu : 0u) | (p + 1 < glen ? 0xffff0000u : 0u);
+        };
+        const uint32_t m0 = mask(0), m1 = mask(8), m2 = mask(16), m3 = mask(24);
+        b = make_uint4(b.x & m0, b.y & m1, b.z & m2, b.w & m3);
+        c = make_uint4(c.x & m0, c.y & m1, c.z & m2, c.w & m3);
+    }
+    const uint32_t b0[2] = {b.x, b.z}, b1[2] = {b.y, b.w};
+    const uint32_t c0[2] = {c.x, c.z}, c1[2] = {c.y, c.w};
 #pragma unroll
-        for (int k = 0; k < G::KCH; ++k) {
-            const int piece = (lane + 32 * k) % G::CH;
-            crow[k] = (lane + 32 * k) / G::CH;
-            cpo[k] = piece * 16;
-            cdst[k] = uint32_t(crow[k] * G::PITCH + ((piece ^ (crow[k] & 7)) * 16));
+    for (int T = 0; T < FT; ++T) {
+        uint32_t x[4];
+        ldsm_x4_trans(rows ^ uint32_t(T << 4), x);
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {
+            // even features (bytes 0, 2) in matrix rows 0-7, odd in 8-15
+            const uint32_t a[4] = {convert(__byte_perm(x[2 * kk], 0u, 0x4240)),
+                                   convert(__byte_perm(x[2 * kk], 0u, 0x4341)),
+                                   convert(__byte_perm(x[2 * kk + 1], 0u, 0x4240)),
+                                   convert(__byte_perm(x[2 * kk + 1], 0u, 0x4341))};
+            mma_16816(acc.v[0][T], a, b0[kk], b1[kk]);
+            if constexpr (ROWS > 1) mma_16816(acc.v[1][T], a, c0[kk], c1[kk]);
         }
     }
-    auto plan_row = [&](int k) { return kPow2 ? crow[0] + k * kStep : crow[k]; };
-    auto plan_src = [&](int k) { return kPow2 ? cpo[0] : cpo[k]; };
-    auto plan_dst = [&](int k) {
-        return kPow2 ? cdst[k % kPer] + uint32_t(k * kStep * G::PITCH) : cdst[k];
-    };
-    const char *Dbytes = reinterpret_cast<const char *>(P.D) +
-                         2 * (int64_t(P.f_base) + int64_t(blockIdx.y) * G::FP);
-    const uint32_t row_bytes = uint32_t(P.ldd) * 2u;
-    // ldmatrix addresses of this lane: matrices (entries 0-7 | 8-15) x
-    // (features 0-7 | 8-15) of a tile; lane l supplies entry e = (l & 7) +
-    // 8 (l >> 4), chunk c = 2 T + b with b = (l >> 3) & 1, stored at slot
-    // c ^ (e & 7) = 2 (T ^ y) + (b ^ x0) with x0 = l & 1, y = (l >> 1) & 3.
-    // Stages start on 128-byte lines and the row pitch is a multiple of 128,
-    // so the address is ((stage + tl) ^ 32 (T & 3)) + 128 (T >> 2) with
-    // tl = e PITCH + 16 (b ^ x0) + 32 y.
-    constexpr int kTq = FT < 4 ? FT : 4;
-    const uint32_t tl = uint32_t(((lane & 7) + 8 * (lane >> 4)) * G::PITCH +
-                                 16 * (((lane >> 3) & 1) ^ (lane & 1)) + 32 * ((lane >> 1) & 3));
+}
 
-    // Block b's column indices -> index slot `st` (zeros for self / dead entries).
-    auto copy_cols = [&](int b, int st) {
-        const int p = b * EB + e16;
-        const int tg = tag_of(w, p);
-        const bool live = p < total && p != pick<ROWS>(w.selfp, tg);
-        const int32_t *src = P.colidx + (live ? pick<ROWS>(w.cbase, tg) + p : 0);
-        if (lane < EB)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
-                             cslot_s + uint32_t((st * EB + e16) * 4)),
-                         "l"(src), "r"(live ? 4 : 0)
-                         : "memory");
-    };
-    // Column of block b's entry of this lane, from its landed index slot `st`.
-    auto column = [&](int b, int st) -> int {
-        const int p = b * EB + e16;
-        if (p >= total) return -1;
-        const int tg = tag_of(w, p);
-        const int j = p == pick<ROWS>(w.selfp, tg) ? int(pick<ROWS>(w.row, tg))
-                                                    : cslot[st * EB + e16];
-        return uint32_t(j) < n32 ? j : -1;
-    };
-    // A block's rows and row scales (column j per lane; -1: dead) -> stage `st`.
-    // Dead entries copy zeros and read nothing (pointing them all at one real
-    // row instead made that row's L2 line a hot spot: 2.7 -> 4.5 ms on the
-    // Reddit-shaped graph).
-    auto copy_rows = [&](int st, int j) {
-        const uint32_t base = rows_s + uint32_t(st * G::STAGE);
-        if (P.off32) {          // each lane's row byte offset, shuffled once per copy
-            const uint32_t ro = j >= 0 ? uint32_t(j) * row_bytes : 0xffffffffu;
+// The columns of a window's first NS blocks, loaded before its walk begins.
+template <int ROWS, int SUB, int NS>
+__device__ __forceinline__ void fetch_first(const TcParams &P, const Window<ROWS> &w,
+                                            int (&c)[NS][SUB]) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-            for (int k = 0; k < G::KCH; ++k) {
-                const uint32_t r = __shfl_sync(kFullMask, ro, plan_row(k));
-                const bool live = r != 0xffffffffu;
-                cp_async16(base + plan_dst(k), Dbytes + (live ? r : 0u) + plan_src(k), live);
-            }
-        } else {
+    for (int b = 0; b < NS; ++b)
 #pragma unroll
-            for (int k = 0; k < G::KCH; ++k) {
-                const int jj = __shfl_sync(kFullMask, j, plan_row(k));
-                cp_async16(base + plan_dst(k),
-                           Dbytes + int64_t(jj >= 0 ? jj : 0) * row_bytes + plan_src(k), jj >= 0);
-            }
-        }
-        if (lane < EB)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
-                             wslot_s + uint32_t((st * EB + e16) * 4)),
-                         "l"(P.rowscale + (j >= 0 ? j : 0)), "r"(j >= 0 ? 4 : 0)
-                         : "memory");
-    };
+        for (int u = 0; u < SUB; ++u) c[b][u] = fetch_column<ROWS>(P, w, (b * SUB + u) * EB + lane);
+}
 
-    float acc[FT][4];
-#pragma unroll
-    for (int T = 0; T < FT; ++T)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[T][c] = 0.0f;
-    int E[ROWS];
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) E[r] = kNoScale;
+// The row of a window (its scale's exponent E: see walk_window) as the weight 2^(14
+// - E) that its entries' scales are multiplied by; tg = the lane's row.
+template <int ROWS>
+__device__ __forceinline__ float row_unit(int E, int tg) {
+    return exp2i(min(14 - (ROWS == 1 ? E : __shfl_sync(kFullMask, E, tg)), 127));
+}
 
-    // Prologue: groups -DI .. -1 (the index copies of blocks D .. D + DI - 1;
-    // from group -D on also the rows of blocks 0 .. D - 1, whose indices are
-    // read directly).
+// Where lane (g, t) finds the positions of row g (its column of B) in an
+// eight-row window.
+template <int ROWS>
+struct Column {
+    int lo = 0;
+    uint32_t len = 0;
+    __device__ __forceinline__ explicit Column(const Window<ROWS> &w) {
+        if constexpr (ROWS > 1) {
+            const int g = (threadIdx.x & 31) >> 2;
+            int hi = w.off[1];
+            lo = w.off[0];
 #pragma unroll
-    for (int m = -G::DI; m < 0; ++m) {
-        if (m + G::D >= 0) copy_rows(m + G::D, fetch_col(P, w, EB * (m + G::D) + e16));
-        copy_cols(m + G::D + G::DI, (m + G::D + G::DI) % G::NI);
-        cp_async_commit();
-    }
-
-    int st = 0;                             // row stage of block n (n mod NS)
-    int si = G::D % G::NI;                  // index slot of block n + D
-    for (int n = 0; n < nblk; ++n) {
-        const int stD = st == 0 ? G::NS - 1 : st - 1;       // row stage of block n + D (= n - 1)
-        const int siI = si == 0 ? G::NI - 1 : si - 1;       // index slot of block n + D + DI
-        cp_async_wait<G::DI - 1>();     // group n - DI: block n + D's indices
-        __syncwarp();
-        const int jD = column(n + G::D, si);
-        __syncwarp();           // every lane has read index slot si before it is reused
-        copy_rows(stD, jD);
-        copy_cols(n + G::D + G::DI, siI);
-        cp_async_commit();
-        cp_async_wait<G::D>();          // group n - D: block n's rows and scales
-        __syncwarp();
-
-        // This block's weights and the scale exponent of each row they belong to.
-        const float w0 = wslot[st * EB + e16];      // 0 for dead entries
-        uint32_t b0[EB / 16], b1[EB / 16];
-        if constexpr (ROWS == 1) {
-            const int e = exponent_of(__reduce_max_sync(kFullMask, __float_as_uint(w0)));
-            if (e > E[0]) {     // keep the sums on the row's current scale
-                const float f = exp2i(max(E[0] - e, -126));
-#pragma unroll
-                for (int T = 0; T < FT; ++T)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[T][c] *= f;
-                E[0] = e;
-            }
-            const float ws = w0 * exp2i(min(14 - E[0], 127));
-            const __half hi = __float2half_rn(ws);
-            const __half lo = __float2half_rn(ws - __half2float(hi));
-            const uint32_t pw = uint32_t(__half_as_ushort(hi)) | (uint32_t(__half_as_ushort(lo)) << 16);
-            // B fragment: column 0 = hi, column 1 = lo, columns 2-7 zero; entries
-            // 2t, 2t+1 (b0) and 2t+8, 2t+9 (b1).
-            const uint32_t sel = g == 0 ? 0x5410u : 0x7632u;
-#pragma unroll
-            for (int kk = 0; kk < EB / 16; ++kk) {
-                const uint32_t v0 = __shfl_sync(kFullMask, pw, 16 * kk + 2 * t);
-                const uint32_t v1 = __shfl_sync(kFullMask, pw, 16 * kk + 2 * t + 1);
-                const uint32_t v2 = __shfl_sync(kFullMask, pw, 16 * kk + 2 * t + 8);
-                const uint32_t v3 = __shfl_sync(kFullMask, pw, 16 * kk + 2 * t + 9);
-                b0[kk] = g < 2 ? __byte_perm(v0, v1, sel) : 0u;
-                b1[kk] = g < 2 ? __byte_perm(v2, v3, sel) : 0u;
-            }
-        } else {
-            const int pos = n * EB + e16;
-            const int tg = pos < total ? tag_of(w, pos) : ROWS;
-            const int tlo = tag_of(w, n * EB);
-            const int thi = tag_of(w, min(n * EB + EB - 1, total - 1));
-            bool grew = false;
-            int Enew[ROWS];
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                Enew[r] = E[r];
-                if (r >= tlo && r <= thi) {
-                    const int e = exponent_of(
-                        __reduce_max_sync(kFullMask, tg == r ? __float_as_uint(w0) : 0u));
-                    if (e > Enew[r]) {
-                        Enew[r] = e;
-                        grew = true;
-                    }
+            for (int k = 1; k < ROWS; ++k)
+                if (g == k) {
+                    lo = w.off[k];
+                    hi = w.off[k + 1];
                 }
-            }
-            if (grew) {         // keep every row's sums on its current scale
-                const float f = exp2i(max(pick<ROWS>(E, t) - pick<ROWS>(Enew, t), -126));
-#pragma unroll
-                for (int T = 0; T < FT; ++T)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[T][c] *= f;
-#pragma unroll
-                for (int r = 0; r < ROWS; ++r) E[r] = Enew[r];
-            }
-            uint32_t pw = 0u;
-            if (tg < ROWS) {
-                const float ws = w0 * exp2i(min(14 - pick<ROWS>(E, tg), 127));
-                const __half hi = __float2half_rn(ws);
-                const __half lo = __float2half_rn(ws - __half2float(hi));
-                pw = uint32_t(__half_as_ushort(hi)) | (uint32_t(__half_as_ushort(lo)) << 16);
-            }
-            // B fragment: column g = 2 r + part, entries 2t, 2t+1, 2t+8, 2t+9.
-            const int sel_row = g >> 1;
-            const uint32_t sel = (g & 1) ? 0x7632u : 0x5410u;
-            auto pair = [&](int e) -> uint32_t {   // entries e, e + 1 of column g
-                const uint32_t va = __shfl_sync(kFullMask, pw, e);
-                const uint32_t vb = __shfl_sync(kFullMask, pw, e + 1);
-                const int ta = __shfl_sync(kFullMask, tg, e);
-                const int tb = __shfl_sync(kFullMask, tg, e + 1);
-                const uint32_t h = __byte_perm(va, vb, sel);
-                return (ta == sel_row ? (h & 0xffffu) : 0u) | (tb == sel_row ? (h & 0xffff0000u) : 0u);
-            };
-#pragma unroll
-            for (int kk = 0; kk < EB / 16; ++kk) {
-                b0[kk] = pair(16 * kk + 2 * t);
-                b1[kk] = pair(16 * kk + 2 * t + 8);
-            }
+            len = uint32_t(hi - lo);
         }
+    }
+};
 
-        const uint32_t sl = rows_s + uint32_t(st * G::STAGE) + tl;
-        uint32_t tq[kTq];
+// The second walk of a window that has wide rows: adds their high plane (weights
+// on the scales that the first walk ended with; other entries weigh nothing) for
+// the 32-position sub-blocks marked in `marks` (bit q: sub-blocks q << shift ..
+// ((q + 1) << shift) - 1). Two stages: the next sub-block's rows are copied
+// while one is multiplied. A function of its own, so that the first walk's
+// registers need not hold both.
+template <int FT, int ROWS, class G>
+__device__ __noinline__ void high_walk(TcParams P, Window<ROWS> w, uint8_t *ring,
+                                       TcSums<FT, ROWS> &sums, int E, uint32_t marks, int shift) {
+    const int lane = threadIdx.x & 31;
+    const int piece = lane % G::P2, slab = int(blockIdx.y) * FT;
+    const bool mine = piece < FT && (slab + piece) * 16 < int(P.ldd);
+    const uint8_t *plane = P.D + P.N * P.ldd + (slab + piece) * 16;
+    const uint32_t tl =
+        uint32_t(lane * G::PITCH) | uint32_t(((lane / G::LINE) & (G::P2 - 1)) << 4);
+    int *checked = reinterpret_cast<int *>(ring + G::CHECKED);
+    uint16_t *halves = reinterpret_cast<uint16_t *>(ring + G::HALVES);
+    const Column<ROWS> col(w);
+    const int nsub = (w.off[ROWS] + EB - 1) / EB;
+    TcSums<FT, ROWS> acc = sums;
+    // The first marked sub-block from b on (nsub: none).
+    auto next = [&](int b) {
+        while (b < nsub && !((marks >> (b >> shift)) & 1u)) ++b;
+        return b;
+    };
+    auto start = [&](int b, int st) -> float {      // copies; the lane's scale if wide, else 0
+        const int j = b < nsub ? fetch_column<ROWS>(P, w, b * EB + lane) : -1;
+        float s = uint32_t(j) < uint32_t(P.N) ? __ldg(P.rowscale + j) : 0.0f;
+        s = s < 0.0f ? -s : 0.0f;
+        __syncwarp();
+        put_column<G>(checked, s > 0.0f ? j : -1);
+        __syncwarp();
+        copy_plane<G>(smem_addr(ring) + uint32_t(st * G::PART), checked, plane, uint32_t(P.ldd), mine);
+        cp_async_commit();
+        return s;
+    };
+    int b = next(0), st = 0;
+    float s = start(b, 0);
+    while (b < nsub) {
+        const int b2 = next(b + 1);
+        const float s2 = start(b2, st ^ 1);
+        cp_async_wait<1>();
+        put_weight(halves, s * row_unit<ROWS>(E, row_of<ROWS>(w, b * EB + lane)));
+        __syncwarp();
+        multiply<FT, ROWS>(acc, smem_addr(ring) + uint32_t(st * G::PART) + tl, halves,
+                           b * EB - col.lo, col.len, [](uint32_t h) { return high_to_half2(h); });
+        __syncwarp();
+        b = b2;
+        s = s2;
+        st ^= 1;
+    }
+    cp_async_wait<0>();
+    __syncwarp();
+    sums = acc;
+}
+
+// Walks a window's position stream and leaves its sums in `out`; c holds the
+// columns of its first blocks (fetch_first). The warp's ring `ring` (shared,
+// TcGeom<FT, SUB, NS>::WARP bytes) is free on entry and on exit.
+//
+// Pipeline (blocks of SUB x 32 positions; lane e owns position e of each
+// sub-block; D = NS - 1): iteration n starts the row copies of block n + D, whose
+// columns were loaded an iteration ago, loads the columns of block n + D + 1,
+// then waits for block n's rows and multiplies. Block b uses row stage b mod NS.
+template <int FT, int ROWS, int SUB, int NS>
+__device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS> &w,
+                                           uint8_t *ring, int (&c)[NS][SUB],
+                                           TcRowSums<FT, ROWS == 1 ? 1 : 2> &out) {
+    using G = TcGeom<FT, SUB, NS>;
+    constexpr int P2 = G::P2, D = G::D;
+    constexpr int BLOCK = SUB * EB;
+    const int lane = threadIdx.x & 31;
+    const int t = lane & 3;
+    const int total = w.off[ROWS];
+    const int nblk = (total + BLOCK - 1) / BLOCK;
+    const uint32_t rows_s = smem_addr(ring);
+    int *checked = reinterpret_cast<int *>(ring + G::CHECKED);
+    uint16_t *halves = reinterpret_cast<uint16_t *>(ring + G::HALVES);
+    const uint32_t n32 = uint32_t(P.N);     // N <= INT32_MAX
+    const int piece = lane % P2;                            // this lane's chunk of a row
+    const int slab = int(blockIdx.y) * FT;                  // first chunk of this column slab
+    const bool mine = piece < FT && (slab + piece) * 16 < int(P.ldd);
+    const uint8_t *Dbytes = P.D + (slab + piece) * 16;
+    const uint32_t row_bytes = uint32_t(P.ldd);
+    // ldmatrix: lane l supplies chunk T of staged row l, at slot T ^ x of it.
+    const uint32_t tl =
+        uint32_t(lane * G::PITCH) | uint32_t(((lane / G::LINE) & (P2 - 1)) << 4);
+    // Row scales kept in D's rows: the last four bytes of the slab's last chunk.
+    const uint32_t in_row = uint32_t(lane * G::PITCH) +
+                            uint32_t(((FT - 1) ^ ((lane / G::LINE) & (P2 - 1))) << 4) + 12u;
+    // Starts the copies of a block's rows to the stage at `stage`; s receives this
+    // lane's row scales (0 for a dead position; 1 for a live one when scales are
+    // kept in the rows).
+    auto start_block = [&](uint32_t stage, const int (&col)[SUB], float (&s)[SUB]) {
 #pragma unroll
-        for (int m = 0; m < kTq; ++m) tq[m] = sl ^ uint32_t(32 * m);
+        for (int u = 0; u < SUB; ++u) {
+            const bool live = uint32_t(col[u]) < n32;
+            put_column<G>(checked + u * EB, live ? col[u] : -1);
+            s[u] = !live ? 0.0f : P.rowscale == nullptr ? 1.0f : __ldg(P.rowscale + col[u]);
+        }
+        __syncwarp();
 #pragma unroll
-        for (int kk = 0; kk < EB / 16; ++kk)
+        for (int u = 0; u < SUB; ++u)
+            copy_plane<G>(stage + uint32_t(u * G::PART), checked + u * EB, Dbytes, row_bytes, mine);
+    };
+
+    TcSums<FT, ROWS> acc;
 #pragma unroll
-            for (int T = 0; T < FT; ++T) {
-                uint32_t a[4];
-                ldsm_x4_trans(tq[T & 3] + uint32_t(kk * 16 * G::PITCH + 128 * (T >> 2)), a);
-                mma_16816(acc[T], a, b0[kk], b1[kk]);
+    for (int p = 0; p < TcSums<FT, ROWS>::PARTS; ++p)
+#pragma unroll
+        for (int T = 0; T < FT; ++T)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc.v[p][T][q] = 0.0f;
+    // Sub-blocks that hold wide rows, as high_walk takes them.
+    uint32_t marks = 0;
+    const int shift = max(0, 27 - __clz(max(nblk * SUB - 1, 0)));
+    int E = kNoScale;           // ROWS == 1: the row's; else of row (lane & 7)
+    uint32_t bound = 0;         // ROWS == 1: the largest scale (bits) that E covers
+    float unit = 0.0f;          // ROWS == 1: 2^(14 - E)
+    const Column<ROWS> col(w);
+
+    float sq[NS][SUB];          // the row scales of blocks n .. n + D
+#pragma unroll
+    for (int b = 0; b < NS; ++b)
+#pragma unroll
+        for (int u = 0; u < SUB; ++u) sq[b][u] = 0.0f;
+#pragma unroll
+    for (int b = 0; b < D; ++b) {
+        if (b < nblk) start_block(rows_s + uint32_t(b * G::STAGE), c[b], sq[b]);
+        cp_async_commit();
+        __syncwarp();           // `checked` is free again
+    }
+    int cnext[SUB];
+#pragma unroll
+    for (int u = 0; u < SUB; ++u) cnext[u] = c[D][u];
+    uint32_t stage = rows_s;                                // block n's
+    uint32_t stage_d = rows_s + uint32_t(D * G::STAGE);     // block n + D's
+#pragma unroll 1
+    for (int n = 0; n < nblk; ++n) {
+        if (n + D < nblk) {
+            start_block(stage_d, cnext, sq[D]);
+#pragma unroll
+            for (int u = 0; u < SUB; ++u)
+                cnext[u] = fetch_column<ROWS>(P, w, ((n + D + 1) * SUB + u) * EB + lane);
+        }
+        cp_async_commit();              // (the count of groups goes on past the end)
+        cp_async_wait<D>();             // block n's rows
+        __syncwarp();
+
+        // This block's weights (0 for dead entries) on the scale of the row they
+        // belong to; a sign bit marks a wide row.
+        uint32_t sb[SUB], top = 0;
+#pragma unroll
+        for (int u = 0; u < SUB; ++u) {
+            if (P.rowscale == nullptr && sq[0][u] != 0.0f)
+                sq[0][u] = *reinterpret_cast<const float *>(ring + (stage - rows_s) + u * G::PART +
+                                                            in_row);
+            sb[u] = __float_as_uint(sq[0][u]);
+            top = max(top, sb[u]);
+        }
+        float ws[SUB];
+        if constexpr (ROWS == 1) {
+            if (__any_sync(kFullMask, top > bound)) {   // a wide row, or a larger weight
+                uint32_t wb = 0;
+#pragma unroll
+                for (int u = 0; u < SUB; ++u) {
+                    if (__any_sync(kFullMask, sb[u] >> 31)) marks |= 1u << ((n * SUB + u) >> shift);
+                    wb = max(wb, sb[u] & 0x7fffffffu);
+                }
+                const int e = exponent_of(__reduce_max_sync(kFullMask, wb));
+                if (e > E) {            // keep the sums on the row's current scale
+                    const float f = exp2i(max(E - e, -126));
+                    acc.scale(f, f);
+                    E = e;
+                    bound = (uint32_t(E + 127) << 23) | 0x7fffffu;
+                }
+                unit = row_unit<ROWS>(E, 0);
             }
-        __syncwarp();           // stage st is refilled in iteration n + 1
-        st = st == G::NS - 1 ? 0 : st + 1;
-        si = si == G::NI - 1 ? 0 : si + 1;
+#pragma unroll
+            for (int u = 0; u < SUB; ++u) ws[u] = __uint_as_float(sb[u] & 0x7fffffffu) * unit;
+        } else {
+            static_assert(ROWS == 1 || SUB == 1, "");
+            const uint32_t wb = sb[0] & 0x7fffffffu;
+            const int tg = row_of<ROWS>(w, n * EB + lane);
+            const int Et = __shfl_sync(kFullMask, E, tg);
+            if (__any_sync(kFullMask, sb[0] > ((uint32_t(Et + 127) << 23) | 0x7fffffu))) {
+                if (__any_sync(kFullMask, sb[0] >> 31)) marks |= 1u << (n >> shift);
+                const int tlo = row_of<ROWS>(w, n * EB);
+                const int thi = row_of<ROWS>(w, min(n * EB + EB, total) - 1);
+                int Enew = E;
+                for (int r = tlo; r <= thi; ++r) {
+                    const int e = exponent_of(__reduce_max_sync(kFullMask, tg == r ? wb : 0u));
+                    if ((lane & 7) == r) Enew = max(Enew, e);
+                }
+                const float f = exp2i(max(E - Enew, -126));
+                acc.scale(__shfl_sync(kFullMask, f, 2 * t), __shfl_sync(kFullMask, f, 2 * t + 1));
+                E = Enew;
+            }
+            ws[0] = __uint_as_float(wb) * row_unit<ROWS>(E, tg);
+        }
+#pragma unroll
+        for (int u = 0; u < SUB; ++u) put_weight(halves + u * 2 * EB, ws[u]);
+        __syncwarp();
+        const uint32_t offset = P.offset;
+#pragma unroll
+        for (int u = 0; u < SUB; ++u)
+            multiply<FT, ROWS>(acc, stage + uint32_t(u * G::PART) + tl, halves + u * 2 * EB,
+                               (n * SUB + u) * EB - col.lo, col.len,
+                               [&](uint32_t h) { return bytes_to_half2(h, offset); });
+        __syncwarp();           // this stage is refilled in iteration n + 1
+#pragma unroll
+        for (int b = 0; b < D; ++b)
+#pragma unroll
+            for (int u = 0; u < SUB; ++u) sq[b][u] = sq[b + 1][u];
+        stage_d = stage;
+        stage = stage == rows_s + uint32_t(D * G::STAGE) ? rows_s : stage + uint32_t(G::STAGE);
     }
     cp_async_wait<0>();         // the ring is idle before the next window
     __syncwarp();
+    if (marks != 0u && P.rowscale != nullptr) {     // (scales kept in the rows have no wide rows)
+        TcSums<FT, ROWS> sums = acc;
+        high_walk<FT, ROWS, G>(P, w, ring, sums, E, marks, shift);
+        acc = sums;
+    }
 
-    const int Et = pick<ROWS>(E, t);
-    const float back = exp2i(max(min(Et - 14, 127), -126));
+    if constexpr (ROWS == 1) {
+        const float back = exp2i(max(min(E - 14 + kDotShift, 127), -126));
 #pragma unroll
-    for (int T = 0; T < FT; ++T) {
-        out.v[T][0] = (acc[T][0] + acc[T][1]) * back;
-        out.v[T][1] = (acc[T][2] + acc[T][3]) * back;
+        for (int T = 0; T < FT; ++T) {
+            out.v[0][T][0] = (acc.v[0][T][0] + acc.v[0][T][1]) * back;
+            out.v[0][T][1] = (acc.v[0][T][2] + acc.v[0][T][3]) * back;
+        }
+    } else {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int Er = __shfl_sync(kFullMask, E, 2 * t + r);
+            const float back = exp2i(max(min(Er - 14 + kDotShift, 127), -126));
+#pragma unroll
+            for (int T = 0; T < FT; ++T) {
+                constexpr int L = TcSums<FT, ROWS>::PARTS - 1;
+                out.v[r][T][0] = (acc.v[0][T][r] + acc.v[L][T][r]) * back;
+                out.v[r][T][1] = (acc.v[0][T][2 + r] + acc.v[L][T][2 + r]) * back;
+            }
+        }
     }
 }
 
-// The output rows of a walk as the epilogues see them: lane (g, t) holds the
-// sums of row rows[t] (-1: none) with the normalisation dinv[t].
-struct TcRows {
-    int64_t row[4];
-    float dinv[4];
-    __device__ __forceinline__ int64_t of(int t) const {
-        int64_t i = row[0];
-#pragma unroll
-        for (int r = 1; r < 4; ++r)
-            if (t == r) i = row[r];
-        return i;
-    }
-    __device__ __forceinline__ float dinv_of(int t) const {
-        float d = dinv[0];
-#pragma unroll
-        for (int r = 1; r < 4; ++r)
-            if (t == r) d = dinv[r];
-        return d;
-    }
-};
-
 // Epilogue of the plain aggregation: H_if = dinv_i * (c_f * sum_f) for f < F
 // (features f0 .. f0 + 16 FT - 1 of the block's column slab), with an
-// optional argmax of each row (lowest index on ties; one slab only).
+// optional argmax of each row (lowest index on ties; one slab only). Called by
+// all lanes for one output row per group of eight lanes (lane bits 2..4); i is
+// -1 where a lane's group has none. `alone`: one row, in the lanes with t = 0.
 template <int FT>
 struct TcStore {
     float *H;
@@ -489,33 +658,45 @@ struct TcStore {
     int F;
     const float *colscale;   // nullable: 1
     int32_t *pred;           // nullable (one column slab only)
-    int f_base;              // first feature of the launch's slab 0
-    static constexpr size_t kSmemFloats = 0;
-    __device__ __forceinline__ void prologue(float *) {}
-    __device__ __forceinline__ void operator()(const TcRows &rows, const TcRowSums<FT> &s) const {
-        const int lane = threadIdx.x & 31;
-        const int g = lane >> 2, t = lane & 3;
-        const int64_t i = rows.of(t);
-        const float di = rows.dinv_of(t);
-        const int f0 = f_base + int(blockIdx.y) * 16 * FT;
+    bool vec2;               // feature pairs of H are 8-byte aligned
+    const float *sScale = nullptr;      // shared: the slab's column scales, set by prologue()
+    static constexpr size_t kSmemFloats = 16 * FT;
+    __device__ __forceinline__ void prologue(float *smem) {
+        const int f = int(blockIdx.y) * 16 * FT + int(threadIdx.x);
+        if (threadIdx.x < 16 * FT)
+            smem[threadIdx.x] = colscale == nullptr ? 1.0f : f < F ? __ldg(colscale + f) : 0.0f;
+        sScale = smem;
+    }
+    template <bool kAlone>
+    __device__ __forceinline__ void row(int64_t i, float di, const float (&v)[FT][2]) const {
+        const int g = (threadIdx.x & 31) >> 2;
+        const int f0 = int(blockIdx.y) * 16 * FT + 2 * g;
         float bestv = 0.0f;
         int best = -1;
         if (i >= 0) {
+            float *h = H + i * ldh;
 #pragma unroll
-            for (int T = 0; T < FT; ++T)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int f = f0 + 16 * T + g + 8 * h;
-                    if (f < F) {
-                        const float c = colscale != nullptr ? __ldg(colscale + f) : 1.0f;
-                        const float o = di * (c * s.v[T][h]);
-                        H[i * ldh + f] = o;
-                        if (best < 0 || o > bestv) {
-                            bestv = o;
-                            best = f;
-                        }
-                    }
+            for (int T = 0; T < FT; ++T) {
+                const int f = f0 + 16 * T;
+                if (f >= F) continue;
+                const bool two = f + 1 < F;
+                const float2 cs = *reinterpret_cast<const float2 *>(sScale + 16 * T + 2 * g);
+                const float o0 = di * (cs.x * v[T][0]), o1 = di * (cs.y * v[T][1]);
+                if (two && vec2) {
+                    *reinterpret_cast<float2 *>(h + f) = make_float2(o0, o1);
+                } else {
+                    h[f] = o0;
+                    if (two) h[f + 1] = o1;
                 }
+                if (best < 0 || o0 > bestv) {
+                    bestv = o0;
+                    best = f;
+                }
+                if (two && o1 > bestv) {
+                    bestv = o1;
+                    best = f + 1;
+                }
+            }
         }
         if (pred != nullptr) {          // over the 8 lanes of the row (lane bits 2..4)
 #pragma unroll
@@ -535,8 +716,9 @@ struct TcStore {
 // Epilogue of layer 1 fused with layer 2's binarization and product: H1_i =
 // dinv_i * beta1 . sums (optionally stored), its signs packed LSB-first,
 // alpha2_i = mean |H1_i| (Eqs. 7-8), and the XNOR-popcount dots against W2's
-// packed columns (Eqs. 11-12), stored as fp16 rows of ldd2 halves (zeros past
-// Fo) with the row scale s2_i = alpha2_i * dinv_i -- layer 2's factored product.
+// packed columns (Eqs. 11-12), stored as byte dots in rows of ldd2 bytes
+// (|dot| <= Fh <= 128: no row is wide) with the row scale s2_i = alpha2_i *
+// dinv_i, in s2 or in the row's last four bytes -- layer 2's factored product.
 template <int FT>
 struct TcPackGemm {
     float *H1;               // nullable N x Fh (row stride ldh1)
@@ -546,9 +728,9 @@ struct TcPackGemm {
     const uint64_t *wbits2;  // Fo x words2
     int Fo;
     int words2;              // 1 or 2
-    uint16_t *D2;            // N x ldd2 fp16 dots
+    uint8_t *D2;             // N x ldd2 byte dots
     int64_t ldd2;
-    float *s2;               // N
+    float *s2;               // N; nullptr: the last four bytes of D2's rows
     const float *sBeta1 = nullptr;     // shared copies, set by prologue()
     const uint64_t *sW2 = nullptr;
 
@@ -556,102 +738,151 @@ struct TcPackGemm {
     __device__ __forceinline__ void prologue(float *smem) {
         float *b1 = smem;
         uint64_t *w2 = reinterpret_cast<uint64_t *>(smem + 128);
-        for (int q = threadIdx.x; q < Fh; q += kTcThreads) b1[q] = __ldg(beta1 + q);
+        for (int q = threadIdx.x; q < 128; q += kTcThreads) b1[q] = q < Fh ? __ldg(beta1 + q) : 0.0f;
         for (int q = threadIdx.x; q < Fo * words2; q += kTcThreads) w2[q] = __ldg(wbits2 + q);
         sBeta1 = b1;
         sW2 = w2;
     }
-    __device__ __forceinline__ void operator()(const TcRows &rows, const TcRowSums<FT> &s) const {
+    template <bool kAlone>
+    __device__ __forceinline__ void row(int64_t i, float di, const float (&v)[FT][2]) const {
+        constexpr int NW = (FT + 1) / 2;        // 32-feature words
         const int lane = threadIdx.x & 31;
-        const int g = lane >> 2, t = lane & 3;
-        const int64_t i = rows.of(t);
-        const float di = rows.dinv_of(t);
-        uint64_t w0 = 0, w1 = 0;
+        const int g = lane >> 2;
+        uint32_t w[NW];
         float l1 = 0.0f;
 #pragma unroll
-        for (int T = 0; T < FT; ++T)
+        for (int q = 0; q < NW; ++q) w[q] = 0u;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int f = 16 * T + g + 8 * h;
-                if (f < Fh) {
-                    const float v = di * (sBeta1[f] * s.v[T][h]);
-                    if (H1 != nullptr && i >= 0) H1[i * ldh1 + f] = v;
-                    l1 += fabsf(v);
-                    if (v >= 0.0f) {
-                        if (f < 64) w0 |= 1ull << f;
-                        else w1 |= 1ull << (f - 64);
-                    }
-                }
+        for (int T = 0; T < FT; ++T) {
+            const int f = 16 * T + 2 * g;
+            const float2 b = *reinterpret_cast<const float2 *>(sBeta1 + f);     // 0 past Fh
+            const float x0 = di * (b.x * v[T][0]), x1 = di * (b.y * v[T][1]);
+            if (H1 != nullptr && i >= 0) {
+                if (f < Fh) H1[i * ldh1 + f] = x0;
+                if (f + 1 < Fh) H1[i * ldh1 + f + 1] = x1;
             }
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {     // the row's 8 lanes
-            w0 |= __shfl_xor_sync(kFullMask, w0, o);
-            w1 |= __shfl_xor_sync(kFullMask, w1, o);
-            l1 += __shfl_xor_sync(kFullMask, l1, o);
+            if (f < Fh) l1 += fabsf(x0);
+            if (f + 1 < Fh) l1 += fabsf(x1);
+            if (x0 >= 0.0f && f < Fh) w[T / 2] |= 1u << (16 * (T & 1));
+            if (x1 >= 0.0f && f + 1 < Fh) w[T / 2] |= 2u << (16 * (T & 1));
         }
-        if (i < 0) return;
-        if (g == 0) s2[i] = (l1 / float(Fh)) * di;
-        for (int o = g; o < ldd2; o += 8) {
-            uint16_t d = 0;
-            if (o < Fo) {
-                int mism = __popcll(w0 ^ sW2[o * words2]);
-                if (words2 > 1) mism += __popcll(w1 ^ sW2[o * words2 + 1]);
-                d = __half_as_ushort(__int2half_rn(Fh - 2 * mism));
+        // Over the row's 8 lanes; the one row of a one-row window goes to all lanes.
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            w[q] <<= 2 * g;
+            if (kAlone) {
+                w[q] = __reduce_or_sync(kFullMask, (lane & 3) == 0 ? w[q] : 0u);
+            } else {
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) w[q] |= __shfl_xor_sync(kFullMask, w[q], o);
             }
-            D2[i * ldd2 + o] = d;
+        }
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) l1 += __shfl_xor_sync(kFullMask, l1, o);
+        if (i >= 0 && g == 0) {
+            const float s = (l1 / float(Fh)) * di;
+            if (s2 != nullptr) s2[i] = s;
+            else *reinterpret_cast<float *>(D2 + (i + 1) * ldd2 - 4) = s;
+        }
+        if (kAlone) i = __shfl_sync(kFullMask, i, 0);
+        if (i < 0) return;
+        const uint64_t w0 = uint64_t(w[0]) | (NW > 1 ? uint64_t(w[NW > 1 ? 1 : 0]) << 32 : 0);
+        const uint64_t w1 = NW > 2 ? uint64_t(w[NW > 2 ? 2 : 0]) |
+                                         (NW > 3 ? uint64_t(w[NW > 3 ? 3 : 0]) << 32 : 0)
+                                   : 0;
+        uint8_t *d = D2 + i * ldd2;
+        for (int o = kAlone ? lane : g; o < Fo; o += kAlone ? 32 : 8) {
+            int mism = __popcll(w0 ^ sW2[o * words2]);
+            if (words2 > 1) mism += __popcll(w1 ^ sW2[o * words2 + 1]);
+            d[o] = uint8_t(ByteDot(Fh - 2 * mism, Fh).lo());
         }
     }
 };
 
-// One light window: rows first .. first + ROWS - 1, leaving out heavy ones.
-template <int FT, int ROWS, int NS, int EBLOCK, class Epi>
-__device__ __forceinline__ void light_window(const TcParams &P, const Epi &epi, uint8_t *ring,
-                                             int64_t first) {
+// Light windows (heavy rows left out): the block's share is windows first, first +
+// step, ..., which its warps take in turn as they become free (`next` counts
+// those taken), so that no warp waits for the one with the longest rows. A
+// warp draws its next window and loads its row pointers when it begins the one
+// before, and that window's first columns before it writes the results.
+template <int FT, int ROWS, int SUB, int NS, class Epi>
+__device__ __forceinline__ void light_windows(const TcParams &P, const Epi &epi, uint8_t *ring,
+                                              int *next, int64_t first, int64_t step) {
+    const int lane = threadIdx.x & 31;
+    const int64_t windows = (P.N + ROWS - 1) / ROWS;
+    const int64_t mine = first < windows ? (windows - first + step - 1) / step : 0;
+    auto draw = [&]() -> int64_t {          // the output row of the next window, or -1
+        int k = 0;
+        if (lane == 0) k = atomicAdd(next, 1);
+        k = __shfl_sync(kFullMask, k, 0);
+        return k < mine ? (first + k * step) * ROWS : -1;
+    };
+    // Row pointer `lane` of a window (rows past the end repeat the last pointer).
+    auto pointer = [&](int64_t row0) -> int64_t {
+        return lane <= ROWS ? __ldg(P.rowptr + min(row0 + lane, P.N)) : 0;
+    };
     Window<ROWS> w;
-    TcRows out;
-    int pos = 0;
+    int64_t row0 = draw();
+    if (row0 < 0) return;
+    int64_t ptr = pointer(row0);
+    int c[NS][SUB];
+    int deg;                                // of row (lane mod ROWS); -1: none, or a heavy block's
+    auto enter = [&]() {                    // row0's window from its row pointers
+        w.first = row0;
+        const int r = ROWS == 1 ? 0 : lane & 7;
+        const int64_t b = min(max(__shfl_sync(kFullMask, ptr, r), int64_t(0)), P.nnz);
+        const int64_t e = min(max(__shfl_sync(kFullMask, ptr, r + 1), b), P.nnz);
+        deg = row0 + r < P.N && e - b <= P.heavy_degree ? int(e - b) : -1;
+        int end = deg + 1;                  // inclusive prefix sum over the window's rows
+        if constexpr (ROWS > 1) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        out.row[r] = -1;
-        out.dinv[r] = 0.0f;
-    }
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-        const int64_t i = first + r;
-        w.off[r] = pos;
-        w.row[r] = -1;
-        w.cbase[r] = 0;
-        w.selfp[r] = -1;
-        if (i < P.N) {
-            const int64_t rb = __ldg(P.rowptr + i), re = __ldg(P.rowptr + i + 1);
-            const int64_t b = min(max(rb, int64_t(0)), P.nnz);
-            const int64_t e = min(max(re, b), P.nnz);
-            const int64_t deg = e - b;
-            out.row[r] = i;
-            out.dinv[r] = inv_sqrt_degree(deg);
-            if (deg <= P.heavy_degree) {
-                w.row[r] = i;
-                w.selfp[r] = pos;
-                w.cbase[r] = b - pos - 1;
-                pos += int(deg + 1);
-            } else {
-                out.row[r] = -1;    // a heavy block's row
+            for (int o = 1; o < ROWS; o <<= 1) {
+                const int v = __shfl_up_sync(kFullMask, end, o, ROWS);
+                if (r >= o) end += v;
             }
         }
+        w.off[0] = 0;
+        if constexpr (ROWS == 1) {
+            w.off[1] = end;
+        } else {
+#pragma unroll
+            for (int k = 0; k < ROWS; ++k) w.off[k + 1] = __shfl_sync(kFullMask, end, k);
+        }
+        w.cbase = b - (end - (deg + 1)) - 1;
+        w.self0 = true;
+        fetch_first<ROWS, SUB, NS>(P, w, c);
+    };
+    enter();
+    while (true) {
+        const int64_t row = row0;
+        row0 = draw();
+        if (row0 >= 0) ptr = pointer(row0);
+        const float dinv = inv_sqrt_degree(deg);
+        const int dg = deg;
+        TcRowSums<FT, ROWS == 1 ? 1 : 2> s;
+        walk_window<FT, ROWS, SUB, NS>(P, w, ring, c, s);
+        if (row0 >= 0) enter();
+        if constexpr (ROWS == 1) {
+            if (dg >= 0) epi.template row<true>((lane & 3) == 0 ? row : -1, dinv, s.v[0]);
+        } else {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int q = 2 * (lane & 3) + r;
+                const bool has = __shfl_sync(kFullMask, dg, q) >= 0;
+                const float di = __shfl_sync(kFullMask, dinv, q);
+                epi.template row<false>(has ? row + q : -1, di, s.v[r]);
+            }
+        }
+        if (row0 < 0) return;
     }
-    w.off[ROWS] = pos;
-    TcRowSums<FT> s;
-    walk_window<FT, ROWS, NS, EBLOCK>(P, w, ring, s);
-    epi(out, s);
 }
 
 // Heavy rows (blocks take chunks of 32 rows in turn): every warp of the block
-// walks an eighth of the row's list (a one-row window), and warp 0 adds the
-// eight partial rows in warp order. A warp's partial row goes to the start of
+// walks an equal part of the row's list (a one-row window), and warp 0 adds the
+// partial rows in warp order. A warp's partial row goes to the start of
 // its own ring, which is idle between walks.
-template <int FT, int NS, int EBLOCK, class Epi>
+template <int FT, int SUB, int NS, class Epi>
 __device__ __forceinline__ void heavy_rows(const TcParams &P, const Epi &epi, uint8_t *rings) {
-    using G = TcGeom<FT, NS, EBLOCK>;
+    using G = TcGeom<FT, SUB, NS>;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     uint8_t *ring = rings + warp * G::WARP;
@@ -677,19 +908,20 @@ __device__ __forceinline__ void heavy_rows(const TcParams &P, const Epi &epi, ui
             const int64_t span = dg + 1;
             const int64_t q0 = span * warp / kTcWarps, q1 = span * (warp + 1) / kTcWarps;
             Window<1> w;
-            w.row[0] = i;
-            w.selfp[0] = int(-q0);          // position of entry 0 (outside unless q0 == 0)
-            w.cbase[0] = cb + q0 - 1;
+            w.first = i;
+            w.self0 = q0 == 0;
+            w.cbase = cb + q0 - 1;
             w.off[0] = 0;
             w.off[1] = int(q1 - q0);
-            TcRowSums<FT> s;
-            walk_window<FT, 1, NS, EBLOCK>(P, w, ring, s);
+            TcRowSums<FT, 1> s;
+            int c[NS][SUB];
+            fetch_first<1, SUB, NS>(P, w, c);
+            walk_window<FT, 1, SUB, NS>(P, w, ring, c, s);
             if (t == 0) {
 #pragma unroll
-                for (int T = 0; T < FT; ++T) {
-                    part(warp)[16 * T + g] = s.v[T][0];
-                    part(warp)[16 * T + g + 8] = s.v[T][1];
-                }
+                for (int T = 0; T < FT; ++T)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) part(warp)[16 * T + 2 * g + h] = s.v[0][T][h];
             }
             __syncthreads();
             if (warp == 0) {
@@ -698,34 +930,23 @@ __device__ __forceinline__ void heavy_rows(const TcParams &P, const Epi &epi, ui
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         float a = 0.0f;
-                        for (int q = 0; q < kTcWarps; ++q) a += part(q)[16 * T + g + 8 * h];
-                        s.v[T][h] = a;
+                        for (int q = 0; q < kTcWarps; ++q) a += part(q)[16 * T + 2 * g + h];
+                        s.v[0][T][h] = a;
                     }
-                TcRows out;
-                out.row[0] = i;
-                out.dinv[0] = inv_sqrt_degree(dg);
-#pragma unroll
-                for (int k = 1; k < 4; ++k) {
-                    out.row[k] = -1;
-                    out.dinv[k] = 0.0f;
-                }
-                epi(out, s);
+                epi.template row<true>(t == 0 ? i : -1, inv_sqrt_degree(dg), s.v[0]);
             }
             __syncthreads();    // the rings are walked again by the next heavy row
         }
     }
 }
 
-// Blocks per SM the kernel is compiled for: three with two-stage rings (at
-// most 80 registers a thread), two with three stages.
-constexpr int tc_min_blocks(int NS) { return NS == 2 ? 3 : 2; }
-
-template <int FT, int ROWS, int NS, class Epi>
-__global__ void __launch_bounds__(kTcThreads, tc_min_blocks(NS))
+template <int FT, int ROWS, int SUB, int NS, class Epi>
+__global__ void __launch_bounds__(kTcThreads, tc_blocks(FT, ROWS))
 spmm_tc_kernel(TcParams P, Epi epi) {
-    constexpr int EB = tc_entries_per_block(FT, ROWS);
-    using G = TcGeom<FT, NS, EB>;
+    using G = TcGeom<FT, SUB, NS>;
     extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ int next;        // windows of the block's share that its warps have taken
+    if (threadIdx.x == 0) next = 0;
     // The rings start on a 128-byte line (the ldmatrix addressing relies on it).
     uint8_t *rings = smem + ((128u - (smem_addr(smem) & 127u)) & 127u);
     float *extra = reinterpret_cast<float *>(rings + kTcWarps * G::WARP);
@@ -735,30 +956,23 @@ spmm_tc_kernel(TcParams P, Epi epi) {
     const int warp = threadIdx.x >> 5;
     uint8_t *ring = rings + warp * G::WARP;
     // Blocks [0, heavy_blocks) walk the heavy rows; blocks from light_first on
-    // then walk light windows, warp by warp in turn. Many windows: one wave of
+    // then walk light windows. Many windows: one wave of
     // persistent blocks does both (a block per window would hold its SM until
     // its longest row ended, most of its warps idle). Few windows: a warp per
     // window, with separate leading blocks for the heavy rows.
-    if (int(blockIdx.x) < P.heavy_blocks) heavy_rows<FT, NS, EB>(P, epi, rings);
+    if (int(blockIdx.x) < P.heavy_blocks) heavy_rows<FT, SUB, NS>(P, epi, rings);
     if (int(blockIdx.x) < P.light_first) return;
-    const int64_t windows = (P.N + ROWS - 1) / ROWS;
-    for (int64_t wi = int64_t(int(blockIdx.x) - P.light_first) * kTcWarps + warp; wi < windows;
-         wi += int64_t(int(gridDim.x) - P.light_first) * kTcWarps)
-        light_window<FT, ROWS, NS, EB>(P, epi, ring, wi * ROWS);
+    light_windows<FT, ROWS, SUB, NS>(P, epi, ring, &next, int(blockIdx.x) - P.light_first,
+                                int(gridDim.x) - P.light_first);
 }
 
-template <int FT, int NS, int EB>
+template <int FT, int SUB, int NS>
 size_t tc_smem(size_t extra_floats) {
-    using G = TcGeom<FT, NS, EB>;
-    static_assert(G::FP * 4 <= G::WARP, "a warp's partial row must fit its ring");
-    static_assert(G::WARP % 16 == 0, "rings must keep 16-byte alignment");
+    using G = TcGeom<FT, SUB, NS>;
+    static_assert(16 * FT * 4 <= G::WARP, "a warp's partial row must fit its ring");
+    static_assert(G::WARP % 128 == 0, "stages must start on 128-byte lines");
     return 128 + size_t(kTcWarps) * G::WARP + extra_floats * 4;
 }
-
-// Rows per light window: one when rows are long (a window's blocks then all
-// belong to one row), four for short rows (so that a block of 16 entries
-// spans several rows instead of mostly padding).
-int tc_rows(int64_t N, int64_t nnz) { return N > 0 && nnz >= 24 * N ? 1 : kTcRows; }
 
 // Heavy-row threshold: rows above max(64, 4 x the mean degree) take a whole block.
 int64_t tc_heavy_degree(int64_t N, int64_t nnz) {
@@ -766,13 +980,14 @@ int64_t tc_heavy_degree(int64_t N, int64_t nnz) {
     return 4 * mean > 64 ? 4 * mean : 64;
 }
 
-template <int FT, int ROWS, int NS, class Epi>
+template <int FT, int ROWS, class Epi>
 void launch_rows(const TcParams &P0, const Epi &epi, int slabs, const DeviceInfo &dev,
                  cudaStream_t s, bool pdl) {
     TcParams P = P0;
     P.heavy_degree = tc_heavy_degree(P.N, P.nnz);
-    const size_t smem = tc_smem<FT, NS, tc_entries_per_block(FT, ROWS)>(Epi::kSmemFloats);
-    auto kernel = spmm_tc_kernel<FT, ROWS, NS, Epi>;
+    constexpr int SUB = tc_sub(FT, ROWS), NS = tc_stages(FT, ROWS);
+    const size_t smem = tc_smem<FT, SUB, NS>(Epi::kSmemFloats);
+    auto kernel = spmm_tc_kernel<FT, ROWS, SUB, NS, Epi>;
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     // One wave of resident blocks, or fewer when the windows do not need them.
     int per_sm = 0;
@@ -801,43 +1016,46 @@ void launch_rows(const TcParams &P0, const Epi &epi, int slabs, const DeviceInfo
     launch_kernel(kernel, grid, dim3(kTcThreads), smem, s, pdl, dim3(1, 1, 1), P, epi);
 }
 
+// Rows per window: one when rows are long (a window's blocks then all belong to
+// one row; at a mean degree of 50 and 41 features 122 us against 113 us for eight
+// rows, at 120 and 100 features 301 against 366 us), or too few to give many
+// warps eight (1001 rows: 6.3 us against 7.8 us; 5000 rows: 11.0 against 10.0 us),
+// else eight (2^20 rows of mean degree 16, 64 features: 442 us against 894 us).
+constexpr int64_t kOneRowDegree = 64;
+constexpr int64_t kFewRows = 16;        // per SM
+
+bool tc_one_row(int64_t N, int64_t nnz, const DeviceInfo &dev) {
+    return nnz >= kOneRowDegree * N || N < kFewRows * int64_t(dev.sm_count);
+}
+
 template <int FT, class Epi>
 void launch_ft(const TcParams &P, const Epi &epi, const DeviceInfo &dev, cudaStream_t s,
                bool pdl, int slabs = 1) {
-    // Two-stage rings and three blocks (24 warps) per SM: on the Reddit-shaped
-    // graph 3109 -> 3000 us (layer 1) and 1927 -> 1869 us (layer 2) against
-    // three stages at two blocks per SM; four-row windows 846 -> 782 us (2^20
-    // nodes of mean degree 16, 64 features). Four-row windows of more than 64
-    // features keep three stages: at 80 registers they would spill.
-    constexpr int kNs4 = FT <= 4 ? 2 : 3;
-    if (tc_rows(P.N, P.nnz) == 1) launch_rows<FT, 1, 2>(P, epi, slabs, dev, s, pdl);
-    else launch_rows<FT, kTcRows, kNs4>(P, epi, slabs, dev, s, pdl);
+    if (tc_one_row(P.N, P.nnz, dev)) launch_rows<FT, 1>(P, epi, slabs, dev, s, pdl);
+    else launch_rows<FT, kTcRows>(P, epi, slabs, dev, s, pdl);
+}
+
+TcParams tc_params(const int64_t *rowptr, const int32_t *colidx, int64_t N, int64_t nnz,
+                   const uint8_t *D, int64_t ldd, const float *rowscale, int K) {
+    // ((K & 1) - 256) 2^-10 in fp16: -2^-2, or -255/1024
+    const uint32_t off = (K & 1) != 0 ? 0xB3F8u : 0xB400u;
+    return TcParams{rowptr, colidx, N, nnz, D, ldd, rowscale, off | (off << 16), 0, 0,
+                    0};
 }
 
 }  // namespace
 
-bool spmm_tc_supported(int F) { return F >= 1; }
-
-// Column slabs of 128 features (FT = 8) in one launch, then the remaining
-// F mod 128 features in a second launch with as many 16-feature tiles as they
-// need (or one launch of ceil(F / 16) tiles when F <= 128).
+// Column slabs of at most 128 features, of equal width.
 void launch_spmm_tc(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bool pdl) {
     if (a.N == 0) return;
-    TcParams P{a.rowptr, a.colidx, a.N, a.nnz, a.D, a.ldd, a.rowscale, 0,
-               a.N * a.ldd * 2 < (int64_t(1) << 32), 0, 0, 0};
-    const int full = a.F > 128 ? a.F / 128 : 0;
-    if (full > 0) {
-        launch_ft<8>(P, TcStore<8>{a.H, a.ldh, a.F, a.colscale, nullptr, 0}, dev, s, pdl, full);
-        pdl = true;         // the remainder launch follows on the same stream
-    }
-    const int rest = a.F - 128 * full;
-    if (rest == 0) return;
-    P.f_base = 128 * full;
-    int32_t *pred = full == 0 ? a.pred : nullptr;
-    switch ((rest + 15) / 16) {
+    const TcParams P = tc_params(a.rowptr, a.colidx, a.N, a.nnz, a.D, a.ldd, a.rowscale, a.K);
+    const bool vec2 = a.ldh % 2 == 0 && aligned_to(a.H, 8);
+    const int tiles = (a.F + 15) / 16, slabs = (tiles + 7) / 8;
+    switch ((tiles + slabs - 1) / slabs) {
 #define BIGCN_TC_CASE(ft)                                                                     \
     case ft:                                                                                  \
-        launch_ft<ft>(P, TcStore<ft>{a.H, a.ldh, a.F, a.colscale, pred, P.f_base}, dev, s, pdl); \
+        launch_ft<ft>(P, TcStore<ft>{a.H, a.ldh, a.F, a.colscale, a.pred, vec2}, dev, s, pdl, \
+                      slabs);                                                                 \
         break;
         BIGCN_TC_CASE(1)
         BIGCN_TC_CASE(2)
@@ -859,8 +1077,7 @@ bool spmm_tc_pack_gemm_supported(int Fh, int Fo) {
 void launch_spmm_tc_pack_gemm(const SpmmTcPackGemmArgs &a, const DeviceInfo &dev,
                               cudaStream_t s, bool pdl) {
     if (a.N == 0) return;
-    TcParams P{a.rowptr, a.colidx, a.N, a.nnz, a.D1, a.ldd1, a.s1, 0,
-               a.N * a.ldd1 * 2 < (int64_t(1) << 32), 0, 0, 0};
+    const TcParams P = tc_params(a.rowptr, a.colidx, a.N, a.nnz, a.D1, a.ldd1, a.s1, a.K);
     const int words2 = (a.Fh + 63) / 64;
     switch ((a.Fh + 15) / 16) {
 #define BIGCN_TCPG_CASE(ft)                                                                 \

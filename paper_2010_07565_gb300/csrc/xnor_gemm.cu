@@ -44,7 +44,7 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
                       int K, int words, float *__restrict__ Z, int64_t ldz,
                       int32_t *__restrict__ dots, const int64_t *__restrict__ rowptr,
                       uint16_t *__restrict__ dots16, int64_t ldd16, float *__restrict__ rowscale,
-                      bool f16) {
+                      uint8_t *__restrict__ dots8, int64_t ldd8) {
     constexpr int BN = 16 * TN;
     constexpr int kALoads = kBM * kBKW / kThreads;                         // 4
     constexpr int kBLoads = (BN * kBKW + kThreads - 1) / kThreads;          // 1..2
@@ -141,6 +141,28 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
     for (int i = 0; i < kTM; ++i) {
         if (kSplit && i % S != rank) continue;
         const int64_t row = m0 + ty + 16 * i;
+        if (dots8 != nullptr) {             // byte planes: the row's 16 lanes agree on its flag
+            bool wide = false;
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                if (n0 + tx + 16 * j < F) wide |= ByteDot(K - 2 * mism[i][j], K).wide();
+            wide = (__ballot_sync(kFullMask, wide) >> (tid & 16) & 0xffffu) != 0u;
+            if (row >= N) continue;
+            if (n0 == 0 && tx == 0) {
+                float s = __ldg(alpha + row);
+                if (kDegreeScale) s *= inv_sqrt_degree(__ldg(rowptr + row + 1) - __ldg(rowptr + row));
+                rowscale[row] = flag_scale(s, wide);
+            }
+            uint8_t *lo = dots8 + row * ldd8 + n0 + tx;
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                if (n0 + tx + 16 * j < F) {
+                    const ByteDot d(K - 2 * mism[i][j], K);
+                    lo[16 * j] = uint8_t(d.lo());
+                    if (wide) lo[N * ldd8 + 16 * j] = uint8_t(d.hi());
+                }
+            continue;
+        }
         if (row >= N) continue;
         float ai = __ldg(alpha + row);
         if (kDegreeScale) ai *= inv_sqrt_degree(__ldg(rowptr + row + 1) - __ldg(rowptr + row));
@@ -149,7 +171,7 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
 #pragma unroll
             for (int j = 0; j < TN; ++j) {
                 const int col = n0 + tx + 16 * j;
-                if (col < ldd16) dots16[row * ldd16 + col] = encode_dot(K - 2 * mism[i][j], col < F, f16);
+                if (col < ldd16) dots16[row * ldd16 + col] = encode_dot(K - 2 * mism[i][j], col < F);
             }
             continue;
         }
@@ -182,12 +204,12 @@ void launch_tn(const GemmArgs &g, const DeviceInfo &dev, cudaStream_t s, bool pd
     if (S == 1) {
         launch_kernel(xnor_gemm_popc_kernel<TN, kDeg, false>, dim3(gx, gy), dim3(kThreads), 0, s,
                       pdl, dim3(1, 1, 1), g.A, g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z,
-                      g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots_f16);
+                      g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8);
         return;
     }
     launch_kernel(xnor_gemm_popc_kernel<TN, kDeg, true>, dim3(gx, gy, S), dim3(kThreads), 0, s,
                   pdl, dim3(1, 1, S), g.A, g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z,
-                  g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots_f16);
+                  g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8);
 }
 
 template <bool kDeg>
@@ -198,6 +220,10 @@ void launch_deg(const GemmArgs &g, const DeviceInfo &dev, cudaStream_t s, bool p
 }
 
 }  // namespace
+
+bool xnor_gemm_bytes_supported(int64_t N, int K, int F, const DeviceInfo &dev) {
+    return K <= 32767 && F <= (xnor_gemm_tc_supported(N, K, F, dev) ? 256 : K <= 254 ? 256 : 64);
+}
 
 void launch_xnor_gemm(const GemmArgs &g, const DeviceInfo &dev, cudaStream_t stream, bool pdl) {
     if (g.N == 0) return;

@@ -48,6 +48,62 @@ constexpr int kTcThreads = 256;
 constexpr int kTcKBytes = 128;
 constexpr int kTcStages = 2;
 
+// Byte-plane epilogue of a product tile (rows and warps as in tc_epilogue
+// below): each thread writes its row's low bytes, 16 columns to a 16-byte
+// store, and notes whether any of its dots is wide; the warps sharing a row
+// meet in shared memory, and only a warp that holds a wide row reads tensor
+// memory again to write that row's high plane.
+template <int NT, int kHalves, int kWarps, bool kDeg>
+__device__ __forceinline__ void tc_epilogue_bytes(uint32_t tmem, int warp, int lane, int64_t m0,
+                                                  int n0, int64_t N,
+                                                  const float *__restrict__ alpha,
+                                                  const int64_t *__restrict__ rowptr, int F,
+                                                  float *__restrict__ rowscale,
+                                                  uint8_t *__restrict__ dots8, int64_t ldd8, int K) {
+    constexpr int kSplit = kWarps / (4 * kHalves);     // warps sharing a row
+    __shared__ uint8_t wide_s[kSplit][kUmmaM * kHalves];
+    const int quad = warp & 3;
+    const int hsel = (warp >> 2) % kHalves;
+    const int cs = warp / (4 * kHalves);
+    const int r = kUmmaM * hsel + 32 * quad + lane;
+    const int64_t row = m0 + r;
+    const uint32_t taddr = tmem + (uint32_t(32 * quad) << 16) + uint32_t(hsel * NT);
+    const int cols = min(F - n0, NT);                  // columns of this tile
+    uint8_t *dr = dots8 + row * ldd8 + n0;
+    auto slice = [&](int c0, bool high) -> bool {      // 16 columns: store, any wide?
+        uint32_t acc[16];
+        tmem_ld16(taddr + uint32_t(c0), acc);
+        bool w = false;
+        uint32_t u[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const ByteDot d(__float2int_rn(__uint_as_float(acc[e])), K);
+            w |= d.wide() && c0 + e < cols;
+            u[e / 4] |= (high ? d.hi() & 255u : d.lo()) << (8 * (e % 4));
+        }
+        if (row < N)
+            *reinterpret_cast<uint4 *>(dr + (high ? N * ldd8 : 0) + c0) =
+                make_uint4(u[0], u[1], u[2], u[3]);
+        return w;
+    };
+    bool wide = false;
+#pragma unroll 1
+    for (int c0 = 16 * cs; c0 < cols; c0 += 16 * kSplit) wide |= slice(c0, false);
+    wide_s[cs][r] = uint8_t(wide && row < N);
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kWarps) : "memory");     // the epilogue's warps
+    wide = false;
+#pragma unroll
+    for (int q = 0; q < kSplit; ++q) wide |= wide_s[q][r] != 0;
+    if (row < N && n0 == 0 && cs == 0) {
+        float ai = __ldg(alpha + row);
+        if (kDeg) ai *= inv_sqrt_degree(__ldg(rowptr + row + 1) - __ldg(rowptr + row));
+        rowscale[row] = flag_scale(ai, wide);
+    }
+    if (__any_sync(kFullMask, wide))
+#pragma unroll 1
+        for (int c0 = 16 * cs; c0 < cols; c0 += 16 * kSplit) slice(c0, true);
+}
+
 // Epilogue of a product tile by kWarps warps: warp w reads tensor-memory lanes
 // 32 (w % 4) .. (its rows) of accumulator h = (w / 4) % kHalves (rows 128 h
 // on, NT columns further on) with tcgen05.ld, converts the exact fp32 dots to
@@ -62,7 +118,13 @@ __device__ __forceinline__ void tc_epilogue(uint32_t tmem, int warp, int lane, i
                                             float *__restrict__ Z, int64_t ldz,
                                             int32_t *__restrict__ dots,
                                             uint16_t *__restrict__ dots16, int64_t ldd16,
-                                            float *__restrict__ rowscale, bool f16) {
+                                            float *__restrict__ rowscale,
+                                            uint8_t *__restrict__ dots8, int64_t ldd8, int K) {
+    if (dots8 != nullptr) {     // byte planes (one column tile, or no wide dots)
+        tc_epilogue_bytes<NT, kHalves, kWarps, kDeg>(tmem, warp, lane, m0, n0, N, alpha, rowptr, F,
+                                                     rowscale, dots8, ldd8, K);
+        return;
+    }
     const bool vec_z = (ldz & 3) == 0 && (reinterpret_cast<uintptr_t>(Z) & 15) == 0;
     const bool vec_d = (F & 3) == 0 && (reinterpret_cast<uintptr_t>(dots) & 15) == 0;
     {
@@ -93,8 +155,7 @@ __device__ __forceinline__ void tc_epilogue(uint32_t tmem, int warp, int lane, i
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const int col = col0 + 4 * q + e;
-                        u[e] = encode_dot(__float2int_rn(__uint_as_float(acc[4 * q + e])), col < F,
-                                          f16);
+                        u[e] = encode_dot(__float2int_rn(__uint_as_float(acc[4 * q + e])), col < F);
                     }
                     *reinterpret_cast<uint2 *>(dr + 4 * q) =
                         make_uint2(u[0] | (u[1] << 16), u[2] | (u[3] << 16));
@@ -144,8 +205,8 @@ xnor_gemm_tc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ al
                     const uint64_t *__restrict__ B, const float *__restrict__ beta, int F, int K,
                     int words, float *__restrict__ Z, int64_t ldz, int32_t *__restrict__ dots,
                     const int64_t *__restrict__ rowptr, uint16_t *__restrict__ dots16,
-                    int64_t ldd16, float *__restrict__ rowscale, bool f16,
-                    const uint8_t *__restrict__ bexp) {
+                    int64_t ldd16, float *__restrict__ rowscale, uint8_t *__restrict__ dots8,
+                    int64_t ldd8, const uint8_t *__restrict__ bexp) {
     constexpr int kStageA = kUmmaM * kTcKBytes;
     constexpr int kStageB = NT * kTcKBytes;
     constexpr int kStage = kStageA + kStageB;
@@ -308,8 +369,8 @@ xnor_gemm_tc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ al
 
     if (ok)
         tc_epilogue<NT, 1, kTcThreads / 32, kDeg>(tmem, warp, lane, m0, n0, N, alpha, rowptr, beta, F,
-                                                  Z, ldz, dots,
-                                 dots16, ldd16, rowscale, f16);
+                                                  Z, ldz, dots, dots16, ldd16, rowscale, dots8, ldd8,
+                                                  K);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
@@ -350,8 +411,8 @@ xnor_gemm_tc_ws_kernel(const uint64_t *__restrict__ A, const float *__restrict__
                        const float *__restrict__ beta, int F, int K, int words,
                        float *__restrict__ Z, int64_t ldz, int32_t *__restrict__ dots,
                        const int64_t *__restrict__ rowptr, uint16_t *__restrict__ dots16,
-                       int64_t ldd16, float *__restrict__ rowscale, bool f16,
-                       const uint8_t *__restrict__ bexp) {
+                       int64_t ldd16, float *__restrict__ rowscale, uint8_t *__restrict__ dots8,
+                       int64_t ldd8, const uint8_t *__restrict__ bexp) {
     constexpr int NT = kWsCols;
     constexpr int kStageA = kWsRows * kTcKBytes;        // two 128-row halves
     constexpr int kStageB = NT * kTcKBytes;
@@ -528,8 +589,7 @@ xnor_gemm_tc_ws_kernel(const uint64_t *__restrict__ A, const float *__restrict__
     if (!ok && tid == 0) atomicAdd(&g_tc_timeouts, 1u);
     if (ok && warp < kWsExpWarps)
         tc_epilogue<NT, 2, kWsExpWarps, kDeg>(tmem, warp, lane, m0, n0, N, alpha, rowptr, beta, F, Z,
-                                              ldz, dots,
-                                 dots16, ldd16, rowscale, f16);
+                                              ldz, dots, dots16, ldd16, rowscale, dots8, ldd8, K);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == kMmaWarp)
@@ -592,7 +652,7 @@ void launch_nt2(const GemmArgs &g, cudaStream_t s, bool pdl) {
     }
     launch_kernel(kernel, grid, dim3(kTcThreads), smem, s, pdl || kBexp, dim3(1, 1, 1), g.A,
                   g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z, g.ldz, g.dots, g.rowptr,
-                  g.dots16, g.ldd16, g.rowscale, g.dots_f16, static_cast<const uint8_t *>(g.b_e4m3));
+                  g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, static_cast<const uint8_t *>(g.b_e4m3));
 }
 
 template <bool kDeg>
@@ -606,7 +666,7 @@ void launch_ws(const GemmArgs &g, cudaStream_t s, bool pdl) {
                   pdl, dim3(1, 1, 1), g.B, g.F, g.K, g.words, KB, g.b_e4m3);
     launch_kernel(kernel, grid, dim3(kWsThreads), smem, s, true, dim3(1, 1, 1), g.A, g.alpha, g.N,
                   g.beta, g.F, g.K, g.words, g.Z, g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16,
-                  g.rowscale, g.dots_f16, static_cast<const uint8_t *>(g.b_e4m3));
+                  g.rowscale, g.dots8, g.ldd8, static_cast<const uint8_t *>(g.b_e4m3));
 }
 
 template <int NT, bool kDeg>
