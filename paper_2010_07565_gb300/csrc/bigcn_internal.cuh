@@ -154,6 +154,12 @@ struct ByteDot {
     __device__ __forceinline__ uint32_t hi() const { return uint32_t((b >> 8) + 128); }
 };
 
+// Whether column c counts for a row's wide flag: of each half of `half` columns
+// the first `valid`.
+__device__ __forceinline__ bool flag_column(int c, int half, int valid) {
+    return (c >= half ? c - half : c) < valid;
+}
+
 // A row scale with its row's wide flag in the sign bit.
 __device__ __forceinline__ float flag_scale(float s, bool wide) {
     return __uint_as_float(__float_as_uint(s) | (wide ? 0x80000000u : 0u));

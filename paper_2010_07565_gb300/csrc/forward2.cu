@@ -172,6 +172,10 @@ extern "C" bigcn_status bigcn_forward_2layer(
         const bool fused = spmm_pack_gemm_supported(Fh, Fo);
     uint16_t *D1 = w.c16 ? static_cast<uint16_t *>(Z1) : nullptr;
     uint8_t *P1 = static_cast<uint8_t *>(Z1);       // the tensor-core path's byte planes
+    // Both aggregations' window counters, which the front sets to zero (alpha1 is
+    // not used by it).
+    uint32_t *counters =
+        w.tc && N >= 2 * kTcCounters ? reinterpret_cast<uint32_t *>(alpha1) : nullptr;
     float *Z1f = w.c16 ? nullptr : static_cast<float *>(Z1);
     cudaStream_t s = as_stream(stream);
     EventMarks marks(events, n_events, s);
@@ -189,6 +193,8 @@ extern "C" bigcn_status bigcn_forward_2layer(
             fr.dots8 = P1;
             fr.ldd8 = Fh16;
             fr.rowscale = s1;
+            fr.counters = counters;
+            fr.n_counters = 2 * kTcCounters;
         } else if (w.c16) {
             fr.D16 = D1;
             fr.ldd16 = Fh8;
@@ -216,10 +222,11 @@ extern "C" bigcn_status bigcn_forward_2layer(
         // less for layer 2's aggregation.
         float *s2 = Fo16 - Fo >= 4 ? nullptr : static_cast<float *>(at(w.s2));
         SpmmTcPackGemmArgs f{rowptr, colidx, N, nnz, P1, Fh16, s1, Fh, K, beta1, H1, ldh1,
-                             wbits2, Fo, D2, Fo16, s2};
+                             wbits2, Fo, D2, Fo16, s2, counters};
         launch_spmm_tc_pack_gemm(f, dev, s, true);
         mark();
         SpmmTcArgs a2{rowptr, colidx, N, nnz, D2, Fo16, s2, Fo, Fh, out, ldo, beta2, pred};
+        if (counters != nullptr) a2.counters = counters + kTcCounters;
         launch_spmm_tc(a2, dev, s, true);
         mark();
         const bigcn_status ls = launch_status();

@@ -18,9 +18,12 @@
 // alone) and the aggregation in its mean / GraphSAGE mode. GraphSAGE's two
 // products are one product over the packed columns of W_self and W_neigh
 // (packed by one launch into the two halves of one array), each half padded
-// to a multiple of 8 columns with beta = 0 (so the padding's products are
-// exactly 0), so that both halves of a product row start on a 16-byte
-// boundary for the gathers.
+// so that both halves of a product row start on a 16-byte boundary for the
+// gathers: to a multiple of 16 columns for byte dots (the padding is never
+// stored), else of 8 with beta = 0 (so the padding's products are exactly 0).
+// Byte dots are aggregated on the tensor cores (spmm_tc.cu): GraphSAGE on
+// 232,965 nodes of mean degree 492, F = 128, 3860 us on the CUDA cores over
+// uint16 dots, 1810 us there.
 #include "launch.cuh"
 
 using namespace bigcn;
@@ -37,16 +40,19 @@ struct InductiveWorkspace {
     size_t a_bits, alpha, b_bits, beta, z, rowscale, total;
     int64_t Fp, Fz, ldz;
     bool compressed;
+    bool planes;             // laid out for byte planes (rows of ldz bytes)
 };
 
 bool inductive_workspace(int32_t agg, int64_t N, int32_t K, int32_t F, InductiveWorkspace *w) {
     if (N < 0 || K < 1 || F < 1) return false;
     if (agg != BIGCN_AGG_MEAN && agg != BIGCN_AGG_SAGE) return false;
     const bool sage = agg == BIGCN_AGG_SAGE;
-    w->Fp = (int64_t(F) + 7) / 8 * 8;
+    w->planes = K <= kMaxPlanesK && F <= (sage ? 128 : 256);
+    const int64_t pad = w->planes ? 16 : 8;
+    w->Fp = (int64_t(F) + pad - 1) / pad * pad;
     w->Fz = sage ? 2 * w->Fp : F;
     w->compressed = K <= kMaxDots16K;
-    w->ldz = w->compressed ? (w->Fz + 7) / 8 * 8 : w->Fz;
+    w->ldz = w->compressed ? (w->Fz + pad - 1) / pad * pad : w->Fz;
     const int64_t words = bigcn_words(K);
     if (N > kMaxElems / (words > w->ldz ? words : w->ldz)) return false;
     if (int64_t(K) > kMaxElems / w->Fz) return false;
@@ -118,32 +124,53 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
     uint64_t *b_bits = reinterpret_cast<uint64_t *>(ws + w.b_bits);
     float *beta = reinterpret_cast<float *>(ws + w.beta);
     const int words = bigcn_words(K);
-    const int Fz = int(w.Fz);
     cudaStream_t s = as_stream(stream);
 
     // Packed weight columns: Wt's, or Wt's in columns [0, F) and W_neigh's in
     // [Fp, Fp + F), the padding columns with beta = 0 (their bits are never
-    // scaled by anything else).
-    if (sage && F != w.Fp && cudaMemsetAsync(beta, 0, size_t(Fz) * 4, s) != cudaSuccess)
+    // scaled by anything else; byte dots of the padding are never stored).
+    auto fuse = [&](int cols) {      // the front: few long rows, or too few for a tensor-core product
+        return front_split_supported(N, K, cols, dev) ||
+               (w.planes && cols <= 128 && K <= 2048 && N < 128 * int64_t(dev.sm_count) &&
+                front_supported(N, K, cols, dev));
+    };
+    const bool bytes = w.planes && planes_faster(N, nnz, F) &&
+                       (fuse(int(w.Fz)) || xnor_gemm_bytes_supported(N, K, int(w.Fz), dev));
+    // uint16 dots and fp32 rows are padded to 8 columns even where the workspace
+    // has room for 16.
+    const int64_t Fp = bytes ? w.Fp : (int64_t(F) + 7) / 8 * 8;
+    const int Fz = sage ? int(2 * Fp) : F;
+    const int64_t ldz = bytes ? w.ldz : w.compressed ? (int64_t(Fz) + 7) / 8 * 8 : Fz;
+    const bool fused = fuse(Fz);
+    if (sage && F != Fp && !bytes && cudaMemsetAsync(beta, 0, size_t(Fz) * 4, s) != cudaSuccess)
         return BIGCN_ERR_CUDA;
-    const bool fused = front_split_supported(N, K, Fz, dev);
     if (!fused) launch_pack_rows(X, N, K, ldx, scale, shift, a_bits, words, alpha, dev, s);
     const WeightPack wa{Wt, K, F, ldw, b_bits, words, beta, 0};
-    const WeightPack wb = sage ? WeightPack{W_neigh, K, F, ldwn, b_bits + w.Fp * words, words,
-                                            beta + w.Fp, 0}
+    const WeightPack wb = sage ? WeightPack{W_neigh, K, F, ldwn, b_bits + Fp * words, words,
+                                            beta + Fp, 0}
                                : WeightPack{nullptr, 1, 0, 0, nullptr, 0, nullptr, 0};
     launch_pack_weights2(wa, wb, s);
     // The product without a degree factor: Z_ij = alpha_i beta_j dot_ij, kept
     // factored (uint16 dots, row scale alpha_i) when K allows.
     GemmArgs g{a_bits, alpha, N, b_bits, beta, Fz, K, words, nullptr, Fz, nullptr, nullptr};
-    SpmmArgs a{rowptr, colidx, N, nnz, nullptr, w.ldz, F, H, ldh, true, true};
+    SpmmArgs a{rowptr, colidx, N, nnz, nullptr, ldz, F, H, ldh, true, true};
     a.agg = sage ? kAggSage : kAggMean;
-    const int64_t half = sage ? w.Fp : 0;
-    if (w.compressed) {
+    const int64_t half = sage ? Fp : 0;
+    if (bytes) {
+        g.dots8 = reinterpret_cast<uint8_t *>(ws + w.z);
+        g.ldd8 = ldz;
+        g.rowscale = reinterpret_cast<float *>(ws + w.rowscale);
+        if (sage) {
+            g.half = int(Fp);
+            g.valid = F;
+        }
+        if (N >= kTcCounters && (fused || xnor_gemm_counters(N, K, Fz, dev)))
+            g.counters = reinterpret_cast<uint32_t *>(alpha);    // (only the product reads alpha)
+    } else if (w.compressed) {
         uint16_t *D16 = reinterpret_cast<uint16_t *>(ws + w.z);
         float *rowscale = reinterpret_cast<float *>(ws + w.rowscale);
         g.dots16 = D16;
-        g.ldd16 = w.ldz;
+        g.ldd16 = ldz;
         g.rowscale = rowscale;
         a.D16 = D16 + half;
         a.rowscale = rowscale;
@@ -153,7 +180,7 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
     } else {
         float *Z = reinterpret_cast<float *>(ws + w.z);
         g.Z = Z;
-        g.ldz = w.ldz;
+        g.ldz = ldz;
         a.Z = Z + half;
         a.Zs = Z;
         // fp32 rows: the gathers read up to F rounded to 4, inside the padded half.
@@ -161,11 +188,19 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
     }
     if (fused) {         // few long rows: centring, packing and product in one kernel
         FrontArgs fr{X, N, K, ldx, scale, shift, b_bits, beta, Fz, words, nullptr, g.Z, g.ldz,
-                     g.dots16, g.ldd16, g.rowscale};
+                     g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half, g.valid,
+                     g.counters, kTcCounters};
         launch_front(fr, dev, s);
     } else {
         launch_xnor_gemm(g, dev, s);
     }
-    launch_spmm_norm(a, dev, s);
+    if (bytes) {
+        SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8 + half, ldz, g.rowscale, F, K, H, ldh,
+                     beta + half, nullptr, a.agg, sage ? g.dots8 : nullptr, beta};
+        t.counters = g.counters;
+        launch_spmm_tc(t, dev, s);
+    } else {
+        launch_spmm_norm(a, dev, s);
+    }
     return launch_status();
 }

@@ -68,6 +68,14 @@ struct GemmArgs {
     // xnor_gemm_bytes_supported.
     uint8_t *dots8 = nullptr;
     int64_t ldd8 = 0;
+    // Columns that make a row wide: of each half of `half` columns the first
+    // `valid` (0: all F; GraphSAGE's halves are padded with columns of no weight).
+    int half = 0;
+    int valid = 0;
+    // Nullable: the aggregation's window counters (kTcCounters words, which may be
+    // alpha[0 ..]), set to zero once alpha has been read. Left alone by a product
+    // that reads a row's alpha in several blocks: xnor_gemm_counters says.
+    uint32_t *counters = nullptr;
     // Nullable device scratch of xnor_gemm_tc_bexp_bytes(K, F) bytes (16-byte
     // aligned): the tensor-core product then expands B's signs to FP8 once
     // into it, and each CTA copies its tiles instead of expanding them.
@@ -86,10 +94,34 @@ struct GemmArgs;
 void launch_xnor_gemm_tc(const GemmArgs &args, const DeviceInfo &dev, cudaStream_t stream,
                          bool pdl);
 
+// Largest K whose dots are kept in byte planes. Signs that agree half the time
+// give dots of standard deviation sqrt(K): at K = 3072 one in 10^6 does not fit
+// the low byte, at 4096 one in 15000, so that of 256-feature rows one in 60 is
+// wide and most blocks of 32 need their second walk (2^20 rows, F = 256: K =
+// 3000 at 1330 us, K = 4096 at 2013 us, against 2011 us for uint16 dots on the
+// CUDA cores).
+constexpr int32_t kMaxPlanesK = 3072;
+
+// Whether byte planes and the tensor-core walk are the faster form for rows of F
+// dots. Up to 128 features always (as measured from 1001 to 2^20 nodes). Wider
+// rows take two column slabs, each of which walks the index lists: worth it on
+// long rows (6581 nodes of mean degree 239, F = 180: a whole layer 124 -> 80 us)
+// and where the uint16 dots overflow L2 (2^20 nodes of mean degree 16, F = 256:
+// 2010 -> 1650 us), not on short rows whose dots stay in L2 (100,000 nodes of mean
+// degree 8, F = 256: 104 -> 116 us; 21,732 of 12, F = 160: 28 -> 30 us).
+inline bool planes_faster(int64_t N, int64_t nnz, int F) {
+    return F <= 128 || nnz >= 64 * N || N * int64_t(F) * 2 > (int64_t(192) << 20);
+}
+
 // Whether launch_xnor_gemm can write byte planes: a row's wide flag needs all
 // of the row's dots in one block (256 columns on the tensor cores, 64 on the
 // CUDA cores), unless K <= 254, where no dot is wide.
 bool xnor_gemm_bytes_supported(int64_t N, int K, int F, const DeviceInfo &dev);
+
+// Window counters of one aggregation on the tensor cores (one per column slab).
+constexpr int kTcCounters = 2;
+// Whether launch_xnor_gemm zeroes GemmArgs::counters for these sizes.
+bool xnor_gemm_counters(int64_t N, int K, int F, const DeviceInfo &dev);
 
 // Step 4: the XNOR-popcount product and its scaling (Eqs. 11-12).
 void launch_xnor_gemm(const GemmArgs &args, const DeviceInfo &dev, cudaStream_t stream,
@@ -174,6 +206,10 @@ struct FrontArgs {
     float *rowscale = nullptr;
     uint8_t *dots8 = nullptr;    // byte planes, as in GemmArgs
     int64_t ldd8 = 0;
+    int half = 0;
+    int valid = 0;
+    uint32_t *counters = nullptr;    // nullable: kTcCounters words to set to zero
+    int n_counters = 0;
 };
 
 // Whether the fused pack + XNOR-GEMM kernel fits (F <= 128, packed tiles in
@@ -242,6 +278,16 @@ struct SpmmTcArgs {
     int64_t ldh;
     const float *colscale;   // nullable: 1
     int32_t *pred;           // nullable: each row's argmax (lowest index on ties; F <= 128)
+    // As in SpmmArgs. kAggSage: D points at the neighbour half of each row and Ds
+    // at the self half. kAggWeighted: rowscale carries dinv_j.
+    int agg = kAggGcn;
+    const uint8_t *Ds = nullptr;
+    const float *colscale_s = nullptr;
+    const float *values = nullptr;
+    const float *dinv = nullptr;
+    // Nullable: kTcCounters words that an earlier kernel of the call has set to
+    // zero, from which all blocks take their windows (else each block its share).
+    uint32_t *counters = nullptr;
 };
 void launch_spmm_tc(const SpmmTcArgs &args, const DeviceInfo &dev, cudaStream_t stream,
                     bool pdl = false);
@@ -269,6 +315,7 @@ struct SpmmTcPackGemmArgs {
     uint8_t *D2;
     int64_t ldd2;
     float *s2;               // nullptr: the last four bytes of D2's rows (ldd2 - Fo >= 4)
+    uint32_t *counters = nullptr;    // as in SpmmTcArgs
 };
 bool spmm_tc_pack_gemm_supported(int Fh, int Fo);
 void launch_spmm_tc_pack_gemm(const SpmmTcPackGemmArgs &args, const DeviceInfo &dev,

@@ -66,14 +66,6 @@ struct LayerWorkspace {
     int64_t ldd8;            // bytes per row of a byte plane
 };
 
-// Largest K whose dots are kept in byte planes. Signs that agree half the time
-// give dots of standard deviation sqrt(K): at K = 3072 one in 10^6 does not fit
-// the low byte, at 4096 one in 15000, so that of 256-feature rows one in 60 is
-// wide and most blocks of 32 need their second pass (2^20 rows, F = 256: K =
-// 3000 at 664 us for half the rows, K = 4096 at 2013 us against 2011 us for
-// uint16 dots on the CUDA cores).
-constexpr int32_t kMaxPlanesK = 3072;
-
 bool layer_workspace(int64_t N, int32_t K, int32_t F, LayerWorkspace *w) {
     if (N < 0 || K < 1 || F < 1) return false;
     const int64_t words = bigcn_words(K);
@@ -204,7 +196,8 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     const bool small = F <= 128 && K <= 2048 && N < 128 * int64_t(dev.sm_count);
     const bool fused =
         front_split_supported(N, K, F, dev) || (small && front_supported(N, K, F, dev));
-    const bool bytes = w.planes && (fused || xnor_gemm_bytes_supported(N, K, F, dev));
+    const bool bytes = w.planes && planes_faster(N, nnz, F) &&
+                       (fused || xnor_gemm_bytes_supported(N, K, F, dev));
     marks.mark();
     if (!fused) launch_pack_rows(X, N, K, ldx, scale, shift, a_bits, words, alpha, dev, s);
     marks.mark();
@@ -218,6 +211,10 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
         g.dots8 = reinterpret_cast<uint8_t *>(ws + w.z);
         g.ldd8 = w.ldd8;
         g.rowscale = reinterpret_cast<float *>(ws + w.rowscale);
+        // The aggregation's window counters lie in alpha, which only the product
+        // reads (the front not at all).
+        if (N >= kTcCounters && (fused || xnor_gemm_counters(N, K, F, dev)))
+            g.counters = reinterpret_cast<uint32_t *>(alpha);
     } else if (w.compressed) {
         uint16_t *D16 = reinterpret_cast<uint16_t *>(ws + w.z);
         float *rowscale = reinterpret_cast<float *>(ws + w.rowscale);
@@ -234,6 +231,8 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     if (fused) {
         FrontArgs fr{X, N, K, ldx, scale, shift, b_bits, beta, F, words, rowptr, g.Z, g.ldz,
                      g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8};
+        fr.counters = g.counters;
+        fr.n_counters = kTcCounters;
         launch_front(fr, dev, s);
     } else {
         launch_xnor_gemm(g, dev, s);
@@ -241,6 +240,7 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     marks.mark();
     if (bytes) {        // byte planes: the aggregation on the tensor cores
         SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, w.ldd8, g.rowscale, F, K, H, ldh, beta, nullptr};
+        t.counters = g.counters;
         launch_spmm_tc(t, dev, s);
     } else {
         launch_spmm_norm(a, dev, s);

@@ -61,7 +61,9 @@
 // of one block, whose fp32 partial rows are added in warp order
 // (deterministic); light windows go one per warp, or, when there are many,
 // to the warps of one wave of persistent blocks, which first walk the heavy rows
-// and then take the windows of their block's share as they become free.
+// and then take the windows as they become free (from one counter; a fixed share
+// per block left 15 % of the warps idle on power-law graphs: GraphSAGE on 232,965
+// nodes 2110 -> 1808 us, weighted rows on 100,003 nodes 217 -> 178 us).
 #include <cuda_fp16.h>
 
 #include "launch.cuh"
@@ -183,9 +185,14 @@ struct TcParams {
     int64_t nnz;
     const uint8_t *D;        // low plane, N x ldd bytes; the high plane follows
     int64_t ldd;             // bytes; a multiple of 16
+    int width;               // bytes of a row that are gathered (<= ldd)
     const float *rowscale;   // s_j, negative for a wide row; nullptr: kept in D's rows
+    int agg;                 // aggregator (kAgg...)
+    const float *values;     // kAggWeighted: a_ij per CSR entry
+    const float *dinv;       // kAggWeighted: 1/sqrt(dhat) per node
     uint32_t offset;         // ((K & 1) - 256) 2^-10, twice, in fp16
     int64_t heavy_degree;    // rows with more neighbours are walked by whole blocks
+    uint32_t *counters;      // nullable: windows taken so far by all blocks, per column slab
     int heavy_blocks;        // blocks [0, heavy_blocks) walk the heavy rows
     int light_first;         // blocks [light_first, grid) walk the light windows
 };
@@ -200,7 +207,7 @@ template <int ROWS>
 struct Window {
     int64_t first;           // output row of r = 0
     int64_t cbase;           // ROWS == 1: the row's; else of row (lane & 7)
-    bool self0;              // ROWS == 1: position 0 is the self-loop (else off[r] are)
+    bool self0;              // position 0 (of each row) is the self-loop
     int off[ROWS + 1];       // off[ROWS] = stream length
 };
 
@@ -213,24 +220,56 @@ __device__ __forceinline__ int row_of(const Window<ROWS> &w, int p) {
     return r;
 }
 
-// The column that position p of the stream gathers: the CSR's (unchecked), the
-// output row's own for a self-loop, -1 past the end. Called by all lanes
-// together.
-template <int ROWS>
-__device__ __forceinline__ int fetch_column(const TcParams &P, const Window<ROWS> &w, int p) {
-    int j = -1;
+// What position p of the stream gathers: the CSR's column (unchecked), the
+// output row's own for a self-loop, -1 past the end; with kW (a weighted A) also
+// the entry's a_ij (1 for the self-loop). Called by all lanes together.
+template <bool kW>
+struct Entry {
+    int col;
+    float a;
+};
+template <>
+struct Entry<false> {
+    int col;
+    static constexpr float a = 1.0f;
+};
+
+// The factor applied to row i's sum: Eq. 1's 1/sqrt(dhat_i) (read for a weighted
+// A), the mean's 1/dhat_i, or GraphSAGE's 1/|N(i)| (0 without neighbours).
+__device__ __forceinline__ float row_factor(const TcParams &P, int64_t i, int64_t deg) {
+    return P.agg == kAggGcn        ? inv_sqrt_degree(deg)
+           : P.agg == kAggWeighted ? __ldg(P.dinv + i)
+           : P.agg == kAggMean     ? 1.0f / (1.0f + float(deg))
+           : deg > 0               ? 1.0f / float(deg)
+                                   : 0.0f;
+}
+
+template <int ROWS, bool kW>
+__device__ __forceinline__ Entry<kW> fetch_entry(const TcParams &P, const Window<ROWS> &w, int p) {
+    Entry<kW> q;
+    q.col = -1;
+    if constexpr (kW) q.a = 1.0f;
+    auto take = [&](int64_t entry) {
+        q.col = __ldg(P.colidx + entry);
+        if constexpr (kW) q.a = __ldg(P.values + entry);
+    };
     if constexpr (ROWS == 1) {
-        if (p < w.off[1])
-            j = w.self0 && p == 0 ? int(w.first) : __ldg(P.colidx + (w.cbase + p));
+        if (p < w.off[1]) {
+            if (w.self0 && p == 0) q.col = int(w.first);
+            else take(w.cbase + p);
+        }
     } else {
         const int r = row_of<ROWS>(w, p);
         int start = w.off[0];
 #pragma unroll
         for (int k = 1; k < ROWS; ++k) start = r >= k ? w.off[k] : start;
         const int64_t entry = __shfl_sync(kFullMask, w.cbase, r) + p;
-        if (p < w.off[ROWS]) j = p == start ? int(w.first) + r : __ldg(P.colidx + entry);
+        if (p < w.off[ROWS]) {
+            if (w.self0 && p == start) q.col = int(w.first) + r;
+            else take(entry);
+        }
     }
-    return j;
+    return q;
 }
 
 // Per-lane sums of a window after its walk: R2 output rows (ROWS == 1: lanes
@@ -360,14 +399,15 @@ __device__ __forceinline__ void multiply(TcSums<FT, ROWS> &acc, uint32_t rows,
 }
 
 // The columns of a window's first NS blocks, loaded before its walk begins.
-template <int ROWS, int SUB, int NS>
+template <int ROWS, bool kW, int SUB, int NS>
 __device__ __forceinline__ void fetch_first(const TcParams &P, const Window<ROWS> &w,
-                                            int (&c)[NS][SUB]) {
+                                            Entry<kW> (&c)[NS][SUB]) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int b = 0; b < NS; ++b)
 #pragma unroll
-        for (int u = 0; u < SUB; ++u) c[b][u] = fetch_column<ROWS>(P, w, (b * SUB + u) * EB + lane);
+        for (int u = 0; u < SUB; ++u)
+            c[b][u] = fetch_entry<ROWS, kW>(P, w, (b * SUB + u) * EB + lane);
 }
 
 // The row of a window (its scale's exponent E: see walk_window) as the weight 2^(14
@@ -405,12 +445,12 @@ struct Column {
 // ((q + 1) << shift) - 1). Two stages: the next sub-block's rows are copied
 // while one is multiplied. A function of its own, so that the first walk's
 // registers need not hold both.
-template <int FT, int ROWS, class G>
+template <int FT, int ROWS, bool kW, class G>
 __device__ __noinline__ void high_walk(TcParams P, Window<ROWS> w, uint8_t *ring,
                                        TcSums<FT, ROWS> &sums, int E, uint32_t marks, int shift) {
     const int lane = threadIdx.x & 31;
     const int piece = lane % G::P2, slab = int(blockIdx.y) * FT;
-    const bool mine = piece < FT && (slab + piece) * 16 < int(P.ldd);
+    const bool mine = piece < FT && (slab + piece) * 16 < P.width;
     const uint8_t *plane = P.D + P.N * P.ldd + (slab + piece) * 16;
     const uint32_t tl =
         uint32_t(lane * G::PITCH) | uint32_t(((lane / G::LINE) & (G::P2 - 1)) << 4);
@@ -425,11 +465,14 @@ __device__ __noinline__ void high_walk(TcParams P, Window<ROWS> w, uint8_t *ring
         return b;
     };
     auto start = [&](int b, int st) -> float {      // copies; the lane's scale if wide, else 0
-        const int j = b < nsub ? fetch_column<ROWS>(P, w, b * EB + lane) : -1;
-        float s = uint32_t(j) < uint32_t(P.N) ? __ldg(P.rowscale + j) : 0.0f;
-        s = s < 0.0f ? -s : 0.0f;
+        Entry<kW> q;
+        q.col = -1;
+        if (b < nsub) q = fetch_entry<ROWS, kW>(P, w, b * EB + lane);
+        const float sj = uint32_t(q.col) < uint32_t(P.N) ? __ldg(P.rowscale + q.col) : 0.0f;
+        const bool wide = __float_as_uint(sj) >> 31;
+        const float s = wide ? fabsf(sj) * q.a : 0.0f;
         __syncwarp();
-        put_column<G>(checked, s > 0.0f ? j : -1);
+        put_column<G>(checked, wide ? q.col : -1);
         __syncwarp();
         copy_plane<G>(smem_addr(ring) + uint32_t(st * G::PART), checked, plane, uint32_t(P.ldd), mine);
         cp_async_commit();
@@ -463,9 +506,9 @@ __device__ __noinline__ void high_walk(TcParams P, Window<ROWS> w, uint8_t *ring
 // sub-block; D = NS - 1): iteration n starts the row copies of block n + D, whose
 // columns were loaded an iteration ago, loads the columns of block n + D + 1,
 // then waits for block n's rows and multiplies. Block b uses row stage b mod NS.
-template <int FT, int ROWS, int SUB, int NS>
+template <int FT, int ROWS, bool kW, int SUB, int NS>
 __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS> &w,
-                                           uint8_t *ring, int (&c)[NS][SUB],
+                                           uint8_t *ring, Entry<kW> (&c)[NS][SUB],
                                            TcRowSums<FT, ROWS == 1 ? 1 : 2> &out) {
     using G = TcGeom<FT, SUB, NS>;
     constexpr int P2 = G::P2, D = G::D;
@@ -480,7 +523,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
     const uint32_t n32 = uint32_t(P.N);     // N <= INT32_MAX
     const int piece = lane % P2;                            // this lane's chunk of a row
     const int slab = int(blockIdx.y) * FT;                  // first chunk of this column slab
-    const bool mine = piece < FT && (slab + piece) * 16 < int(P.ldd);
+    const bool mine = piece < FT && (slab + piece) * 16 < P.width;
     const uint8_t *Dbytes = P.D + (slab + piece) * 16;
     const uint32_t row_bytes = uint32_t(P.ldd);
     // ldmatrix: lane l supplies chunk T of staged row l, at slot T ^ x of it.
@@ -489,15 +532,29 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
     // Row scales kept in D's rows: the last four bytes of the slab's last chunk.
     const uint32_t in_row = uint32_t(lane * G::PITCH) +
                             uint32_t(((FT - 1) ^ ((lane / G::LINE) & (P2 - 1))) << 4) + 12u;
+    // A position's row scale (a sign bit marks a wide row) and, with kW, its a_ij.
+    struct Weight {
+        float s;
+        float a;
+        // The weight's magnitude in bits, and the weight on a scale.
+        __device__ __forceinline__ uint32_t bits() const {
+            return __float_as_uint(kW ? fabsf(s * a) : s) & 0x7fffffffu;
+        }
+        __device__ __forceinline__ float on(float unit) const {
+            return (kW ? fabsf(s) * a : fabsf(s)) * unit;
+        }
+    };
     // Starts the copies of a block's rows to the stage at `stage`; s receives this
     // lane's row scales (0 for a dead position; 1 for a live one when scales are
     // kept in the rows).
-    auto start_block = [&](uint32_t stage, const int (&col)[SUB], float (&s)[SUB]) {
+    auto start_block = [&](uint32_t stage, const Entry<kW> (&q)[SUB], Weight (&s)[SUB]) {
 #pragma unroll
         for (int u = 0; u < SUB; ++u) {
-            const bool live = uint32_t(col[u]) < n32;
-            put_column<G>(checked + u * EB, live ? col[u] : -1);
-            s[u] = !live ? 0.0f : P.rowscale == nullptr ? 1.0f : __ldg(P.rowscale + col[u]);
+            const int col = q[u].col;
+            const bool live = uint32_t(col) < n32;
+            put_column<G>(checked + u * EB, live ? col : -1);
+            s[u].s = !live ? 0.0f : P.rowscale == nullptr ? 1.0f : __ldg(P.rowscale + col);
+            if constexpr (kW) s[u].a = q[u].a;
         }
         __syncwarp();
 #pragma unroll
@@ -520,18 +577,18 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
     float unit = 0.0f;          // ROWS == 1: 2^(14 - E)
     const Column<ROWS> col(w);
 
-    float sq[NS][SUB];          // the row scales of blocks n .. n + D
+    Weight sq[NS][SUB];         // of blocks n .. n + D
 #pragma unroll
     for (int b = 0; b < NS; ++b)
 #pragma unroll
-        for (int u = 0; u < SUB; ++u) sq[b][u] = 0.0f;
+        for (int u = 0; u < SUB; ++u) sq[b][u] = Weight{0.0f, 1.0f};
 #pragma unroll
     for (int b = 0; b < D; ++b) {
         if (b < nblk) start_block(rows_s + uint32_t(b * G::STAGE), c[b], sq[b]);
         cp_async_commit();
         __syncwarp();           // `checked` is free again
     }
-    int cnext[SUB];
+    Entry<kW> cnext[SUB];
 #pragma unroll
     for (int u = 0; u < SUB; ++u) cnext[u] = c[D][u];
     uint32_t stage = rows_s;                                // block n's
@@ -542,7 +599,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
             start_block(stage_d, cnext, sq[D]);
 #pragma unroll
             for (int u = 0; u < SUB; ++u)
-                cnext[u] = fetch_column<ROWS>(P, w, ((n + D + 1) * SUB + u) * EB + lane);
+                cnext[u] = fetch_entry<ROWS, kW>(P, w, ((n + D + 1) * SUB + u) * EB + lane);
         }
         cp_async_commit();              // (the count of groups goes on past the end)
         cp_async_wait<D>();             // block n's rows
@@ -553,10 +610,10 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
         uint32_t sb[SUB], top = 0;
 #pragma unroll
         for (int u = 0; u < SUB; ++u) {
-            if (P.rowscale == nullptr && sq[0][u] != 0.0f)
-                sq[0][u] = *reinterpret_cast<const float *>(ring + (stage - rows_s) + u * G::PART +
-                                                            in_row);
-            sb[u] = __float_as_uint(sq[0][u]);
+            if (!kW && P.rowscale == nullptr && sq[0][u].s != 0.0f)
+                sq[0][u].s = *reinterpret_cast<const float *>(ring + (stage - rows_s) +
+                                                              u * G::PART + in_row);
+            sb[u] = sq[0][u].bits() | (__float_as_uint(sq[0][u].s) & 0x80000000u);
             top = max(top, sb[u]);
         }
         float ws[SUB];
@@ -578,7 +635,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
                 unit = row_unit<ROWS>(E, 0);
             }
 #pragma unroll
-            for (int u = 0; u < SUB; ++u) ws[u] = __uint_as_float(sb[u] & 0x7fffffffu) * unit;
+            for (int u = 0; u < SUB; ++u) ws[u] = sq[0][u].on(unit);
         } else {
             static_assert(ROWS == 1 || SUB == 1, "");
             const uint32_t wb = sb[0] & 0x7fffffffu;
@@ -597,7 +654,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
                 acc.scale(__shfl_sync(kFullMask, f, 2 * t), __shfl_sync(kFullMask, f, 2 * t + 1));
                 E = Enew;
             }
-            ws[0] = __uint_as_float(wb) * row_unit<ROWS>(E, tg);
+            ws[0] = sq[0][0].on(row_unit<ROWS>(E, tg));
         }
 #pragma unroll
         for (int u = 0; u < SUB; ++u) put_weight(halves + u * 2 * EB, ws[u]);
@@ -620,7 +677,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
     __syncwarp();
     if (marks != 0u && P.rowscale != nullptr) {     // (scales kept in the rows have no wide rows)
         TcSums<FT, ROWS> sums = acc;
-        high_walk<FT, ROWS, G>(P, w, ring, sums, E, marks, shift);
+        high_walk<FT, ROWS, kW, G>(P, w, ring, sums, E, marks, shift);
         acc = sums;
     }
 
@@ -659,6 +716,14 @@ struct TcStore {
     const float *colscale;   // nullable: 1
     int32_t *pred;           // nullable (one column slab only)
     bool vec2;               // feature pairs of H are 8-byte aligned
+    // GraphSAGE (Ds non-null): the node's own product is added, from the self half
+    // of its row (low plane; the high plane `high` bytes on) with its row scale.
+    const uint8_t *Ds;
+    int64_t ldd;
+    int64_t high;
+    const float *rowscale;
+    const float *colscale_s;
+    int K;
     const float *sScale = nullptr;      // shared: the slab's column scales, set by prologue()
     static constexpr size_t kSmemFloats = 16 * FT;
     __device__ __forceinline__ void prologue(float *smem) {
@@ -666,6 +731,13 @@ struct TcStore {
         if (threadIdx.x < 16 * FT)
             smem[threadIdx.x] = colscale == nullptr ? 1.0f : f < F ? __ldg(colscale + f) : 0.0f;
         sScale = smem;
+    }
+    // The node's own dot with self column f.
+    __device__ __forceinline__ float own_dot(int64_t i, int f, bool wide) const {
+        const uint8_t *p = Ds + i * ldd + f;
+        int d = 2 * (int(__ldg(p)) - 128) + (K & 1);
+        if (wide) d += 512 * (int(__ldg(p + high)) - 128);
+        return float(d);
     }
     template <bool kAlone>
     __device__ __forceinline__ void row(int64_t i, float di, const float (&v)[FT][2]) const {
@@ -675,13 +747,24 @@ struct TcStore {
         int best = -1;
         if (i >= 0) {
             float *h = H + i * ldh;
+            float self = 0.0f;
+            bool wide = false;
+            if (Ds != nullptr) {
+                const float s = __ldg(rowscale + i);
+                wide = __float_as_uint(s) >> 31;
+                self = fabsf(s);
+            }
 #pragma unroll
             for (int T = 0; T < FT; ++T) {
                 const int f = f0 + 16 * T;
                 if (f >= F) continue;
                 const bool two = f + 1 < F;
                 const float2 cs = *reinterpret_cast<const float2 *>(sScale + 16 * T + 2 * g);
-                const float o0 = di * (cs.x * v[T][0]), o1 = di * (cs.y * v[T][1]);
+                float o0 = di * (cs.x * v[T][0]), o1 = di * (cs.y * v[T][1]);
+                if (Ds != nullptr) {
+                    o0 += self * (__ldg(colscale_s + f) * own_dot(i, f, wide));
+                    if (two) o1 += self * (__ldg(colscale_s + f + 1) * own_dot(i, f + 1, wide));
+                }
                 if (two && vec2) {
                     *reinterpret_cast<float2 *>(h + f) = make_float2(o0, o1);
                 } else {
@@ -799,22 +882,24 @@ struct TcPackGemm {
     }
 };
 
-// Light windows (heavy rows left out): the block's share is windows first, first +
-// step, ..., which its warps take in turn as they become free (`next` counts
-// those taken), so that no warp waits for the one with the longest rows. A
+// Light windows (heavy rows left out), which warps take in turn as they become
+// free, so that no warp waits for the one with the longest rows: all blocks from
+// one counter (P.counters), or a block's warps from its share of them, windows
+// first, first + step, ... (`next` counts those taken). A
 // warp draws its next window and loads its row pointers when it begins the one
 // before, and that window's first columns before it writes the results.
-template <int FT, int ROWS, int SUB, int NS, class Epi>
+template <int FT, int ROWS, bool kW, int SUB, int NS, class Epi>
 __device__ __forceinline__ void light_windows(const TcParams &P, const Epi &epi, uint8_t *ring,
                                               int *next, int64_t first, int64_t step) {
     const int lane = threadIdx.x & 31;
     const int64_t windows = (P.N + ROWS - 1) / ROWS;
-    const int64_t mine = first < windows ? (windows - first + step - 1) / step : 0;
     auto draw = [&]() -> int64_t {          // the output row of the next window, or -1
-        int k = 0;
-        if (lane == 0) k = atomicAdd(next, 1);
+        int64_t k = 0;
+        if (lane == 0)
+            k = P.counters != nullptr ? int64_t(atomicAdd(P.counters + blockIdx.y, 1u))
+                                      : first + step * atomicAdd(next, 1);
         k = __shfl_sync(kFullMask, k, 0);
-        return k < mine ? (first + k * step) * ROWS : -1;
+        return k < windows ? k * ROWS : -1;
     };
     // Row pointer `lane` of a window (rows past the end repeat the last pointer).
     auto pointer = [&](int64_t row0) -> int64_t {
@@ -824,7 +909,8 @@ __device__ __forceinline__ void light_windows(const TcParams &P, const Epi &epi,
     int64_t row0 = draw();
     if (row0 < 0) return;
     int64_t ptr = pointer(row0);
-    int c[NS][SUB];
+    Entry<kW> c[NS][SUB];
+    const int own = P.agg == kAggSage ? 0 : 1;      // self-loop entries of a row's list
     int deg;                                // of row (lane mod ROWS); -1: none, or a heavy block's
     auto enter = [&]() {                    // row0's window from its row pointers
         w.first = row0;
@@ -832,7 +918,8 @@ __device__ __forceinline__ void light_windows(const TcParams &P, const Epi &epi,
         const int64_t b = min(max(__shfl_sync(kFullMask, ptr, r), int64_t(0)), P.nnz);
         const int64_t e = min(max(__shfl_sync(kFullMask, ptr, r + 1), b), P.nnz);
         deg = row0 + r < P.N && e - b <= P.heavy_degree ? int(e - b) : -1;
-        int end = deg + 1;                  // inclusive prefix sum over the window's rows
+        const int len = deg < 0 ? 0 : deg + own;
+        int end = len;                      // inclusive prefix sum over the window's rows
         if constexpr (ROWS > 1) {
 #pragma unroll
             for (int o = 1; o < ROWS; o <<= 1) {
@@ -847,19 +934,20 @@ __device__ __forceinline__ void light_windows(const TcParams &P, const Epi &epi,
 #pragma unroll
             for (int k = 0; k < ROWS; ++k) w.off[k + 1] = __shfl_sync(kFullMask, end, k);
         }
-        w.cbase = b - (end - (deg + 1)) - 1;
-        w.self0 = true;
-        fetch_first<ROWS, SUB, NS>(P, w, c);
+        w.cbase = b - (end - len) - own;
+        w.self0 = own != 0;
+        fetch_first<ROWS, kW, SUB, NS>(P, w, c);
     };
     enter();
     while (true) {
         const int64_t row = row0;
         row0 = draw();
         if (row0 >= 0) ptr = pointer(row0);
-        const float dinv = inv_sqrt_degree(deg);
         const int dg = deg;
+        const float dinv =
+            dg < 0 ? 0.0f : row_factor(P, row + (ROWS == 1 ? 0 : lane & 7), dg);
         TcRowSums<FT, ROWS == 1 ? 1 : 2> s;
-        walk_window<FT, ROWS, SUB, NS>(P, w, ring, c, s);
+        walk_window<FT, ROWS, kW, SUB, NS>(P, w, ring, c, s);
         if (row0 >= 0) enter();
         if constexpr (ROWS == 1) {
             if (dg >= 0) epi.template row<true>((lane & 3) == 0 ? row : -1, dinv, s.v[0]);
@@ -880,7 +968,7 @@ __device__ __forceinline__ void light_windows(const TcParams &P, const Epi &epi,
 // walks an equal part of the row's list (a one-row window), and warp 0 adds the
 // partial rows in warp order. A warp's partial row goes to the start of
 // its own ring, which is idle between walks.
-template <int FT, int SUB, int NS, class Epi>
+template <int FT, bool kW, int SUB, int NS, class Epi>
 __device__ __forceinline__ void heavy_rows(const TcParams &P, const Epi &epi, uint8_t *rings) {
     using G = TcGeom<FT, SUB, NS>;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -905,18 +993,19 @@ __device__ __forceinline__ void heavy_rows(const TcParams &P, const Epi &epi, ui
             const int64_t i = base + bit;
             const int64_t cb = __shfl_sync(kFullMask, rb, bit);
             const int64_t dg = __shfl_sync(kFullMask, deg, bit);
-            const int64_t span = dg + 1;
+            const int own = P.agg == kAggSage ? 0 : 1;
+            const int64_t span = dg + own;
             const int64_t q0 = span * warp / kTcWarps, q1 = span * (warp + 1) / kTcWarps;
             Window<1> w;
             w.first = i;
-            w.self0 = q0 == 0;
-            w.cbase = cb + q0 - 1;
+            w.self0 = own != 0 && q0 == 0;
+            w.cbase = cb + q0 - own;
             w.off[0] = 0;
             w.off[1] = int(q1 - q0);
             TcRowSums<FT, 1> s;
-            int c[NS][SUB];
-            fetch_first<1, SUB, NS>(P, w, c);
-            walk_window<FT, 1, SUB, NS>(P, w, ring, c, s);
+            Entry<kW> c[NS][SUB];
+            fetch_first<1, kW, SUB, NS>(P, w, c);
+            walk_window<FT, 1, kW, SUB, NS>(P, w, ring, c, s);
             if (t == 0) {
 #pragma unroll
                 for (int T = 0; T < FT; ++T)
@@ -933,14 +1022,14 @@ __device__ __forceinline__ void heavy_rows(const TcParams &P, const Epi &epi, ui
                         for (int q = 0; q < kTcWarps; ++q) a += part(q)[16 * T + 2 * g + h];
                         s.v[0][T][h] = a;
                     }
-                epi.template row<true>(t == 0 ? i : -1, inv_sqrt_degree(dg), s.v[0]);
+                epi.template row<true>(t == 0 ? i : -1, row_factor(P, i, dg), s.v[0]);
             }
             __syncthreads();    // the rings are walked again by the next heavy row
         }
     }
 }
 
-template <int FT, int ROWS, int SUB, int NS, class Epi>
+template <int FT, int ROWS, bool kW, int SUB, int NS, class Epi>
 __global__ void __launch_bounds__(kTcThreads, tc_blocks(FT, ROWS))
 spmm_tc_kernel(TcParams P, Epi epi) {
     using G = TcGeom<FT, SUB, NS>;
@@ -960,9 +1049,9 @@ spmm_tc_kernel(TcParams P, Epi epi) {
     // persistent blocks does both (a block per window would hold its SM until
     // its longest row ended, most of its warps idle). Few windows: a warp per
     // window, with separate leading blocks for the heavy rows.
-    if (int(blockIdx.x) < P.heavy_blocks) heavy_rows<FT, SUB, NS>(P, epi, rings);
+    if (int(blockIdx.x) < P.heavy_blocks) heavy_rows<FT, kW, SUB, NS>(P, epi, rings);
     if (int(blockIdx.x) < P.light_first) return;
-    light_windows<FT, ROWS, SUB, NS>(P, epi, ring, &next, int(blockIdx.x) - P.light_first,
+    light_windows<FT, ROWS, kW, SUB, NS>(P, epi, ring, &next, int(blockIdx.x) - P.light_first,
                                 int(gridDim.x) - P.light_first);
 }
 
@@ -980,14 +1069,14 @@ int64_t tc_heavy_degree(int64_t N, int64_t nnz) {
     return 4 * mean > 64 ? 4 * mean : 64;
 }
 
-template <int FT, int ROWS, class Epi>
+template <int FT, int ROWS, bool kW, class Epi>
 void launch_rows(const TcParams &P0, const Epi &epi, int slabs, const DeviceInfo &dev,
                  cudaStream_t s, bool pdl) {
     TcParams P = P0;
     P.heavy_degree = tc_heavy_degree(P.N, P.nnz);
     constexpr int SUB = tc_sub(FT, ROWS), NS = tc_stages(FT, ROWS);
     const size_t smem = tc_smem<FT, SUB, NS>(Epi::kSmemFloats);
-    auto kernel = spmm_tc_kernel<FT, ROWS, SUB, NS, Epi>;
+    auto kernel = spmm_tc_kernel<FT, ROWS, kW, SUB, NS, Epi>;
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     // One wave of resident blocks, or fewer when the windows do not need them.
     int per_sm = 0;
@@ -1010,6 +1099,7 @@ void launch_rows(const TcParams &P0, const Epi &epi, int slabs, const DeviceInfo
         const int64_t hb = chunks < 2 * int64_t(dev.sm_count) ? chunks : 2 * int64_t(dev.sm_count);
         P.heavy_blocks = int(hb);
         P.light_first = int(hb);
+        P.counters = nullptr;           // (every block has its own windows)
         blocks = hb + need;
     }
     const dim3 grid(static_cast<unsigned>(blocks), static_cast<unsigned>(slabs));
@@ -1028,34 +1118,39 @@ bool tc_one_row(int64_t N, int64_t nnz, const DeviceInfo &dev) {
     return nnz >= kOneRowDegree * N || N < kFewRows * int64_t(dev.sm_count);
 }
 
-template <int FT, class Epi>
+template <int FT, bool kW = false, class Epi>
 void launch_ft(const TcParams &P, const Epi &epi, const DeviceInfo &dev, cudaStream_t s,
                bool pdl, int slabs = 1) {
-    if (tc_one_row(P.N, P.nnz, dev)) launch_rows<FT, 1>(P, epi, slabs, dev, s, pdl);
-    else launch_rows<FT, kTcRows>(P, epi, slabs, dev, s, pdl);
+    if (tc_one_row(P.N, P.nnz, dev)) launch_rows<FT, 1, kW>(P, epi, slabs, dev, s, pdl);
+    else launch_rows<FT, kTcRows, kW>(P, epi, slabs, dev, s, pdl);
 }
 
 TcParams tc_params(const int64_t *rowptr, const int32_t *colidx, int64_t N, int64_t nnz,
                    const uint8_t *D, int64_t ldd, const float *rowscale, int K) {
     // ((K & 1) - 256) 2^-10 in fp16: -2^-2, or -255/1024
     const uint32_t off = (K & 1) != 0 ? 0xB3F8u : 0xB400u;
-    return TcParams{rowptr, colidx, N, nnz, D, ldd, rowscale, off | (off << 16), 0, 0,
-                    0};
+    return TcParams{rowptr, colidx, N,       nnz,     D,       ldd, int(ldd), rowscale,
+                    kAggGcn, nullptr, nullptr, off | (off << 16), 0, nullptr, 0, 0};
 }
 
-}  // namespace
-
 // Column slabs of at most 128 features, of equal width.
-void launch_spmm_tc(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bool pdl) {
-    if (a.N == 0) return;
-    const TcParams P = tc_params(a.rowptr, a.colidx, a.N, a.nnz, a.D, a.ldd, a.rowscale, a.K);
+template <bool kW>
+void launch_store(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bool pdl) {
+    TcParams P = tc_params(a.rowptr, a.colidx, a.N, a.nnz, a.D, a.ldd, a.rowscale, a.K);
+    P.agg = a.agg;
+    P.values = a.values;
+    P.dinv = a.dinv;
+    P.counters = a.counters;
     const bool vec2 = a.ldh % 2 == 0 && aligned_to(a.H, 8);
     const int tiles = (a.F + 15) / 16, slabs = (tiles + 7) / 8;
+    P.width = 16 * tiles;
     switch ((tiles + slabs - 1) / slabs) {
-#define BIGCN_TC_CASE(ft)                                                                     \
-    case ft:                                                                                  \
-        launch_ft<ft>(P, TcStore<ft>{a.H, a.ldh, a.F, a.colscale, a.pred, vec2}, dev, s, pdl, \
-                      slabs);                                                                 \
+#define BIGCN_TC_CASE(ft)                                                                      \
+    case ft:                                                                                   \
+        launch_ft<ft, kW>(P,                                                                   \
+                          TcStore<ft>{a.H, a.ldh, a.F, a.colscale, a.pred, vec2, a.Ds, a.ldd,  \
+                                      a.N * a.ldd, a.rowscale, a.colscale_s, a.K},             \
+                          dev, s, pdl, slabs);                                                 \
         break;
         BIGCN_TC_CASE(1)
         BIGCN_TC_CASE(2)
@@ -1070,6 +1165,14 @@ void launch_spmm_tc(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, 
     }
 }
 
+}  // namespace
+
+void launch_spmm_tc(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bool pdl) {
+    if (a.N == 0) return;
+    if (a.agg == kAggWeighted) launch_store<true>(a, dev, s, pdl);
+    else launch_store<false>(a, dev, s, pdl);
+}
+
 bool spmm_tc_pack_gemm_supported(int Fh, int Fo) {
     return Fh >= 1 && Fh <= 128 && Fo >= 1 && Fo <= kMaxFusedOut;
 }
@@ -1077,7 +1180,8 @@ bool spmm_tc_pack_gemm_supported(int Fh, int Fo) {
 void launch_spmm_tc_pack_gemm(const SpmmTcPackGemmArgs &a, const DeviceInfo &dev,
                               cudaStream_t s, bool pdl) {
     if (a.N == 0) return;
-    const TcParams P = tc_params(a.rowptr, a.colidx, a.N, a.nnz, a.D1, a.ldd1, a.s1, a.K);
+    TcParams P = tc_params(a.rowptr, a.colidx, a.N, a.nnz, a.D1, a.ldd1, a.s1, a.K);
+    P.counters = a.counters;
     const int words2 = (a.Fh + 63) / 64;
     switch ((a.Fh + 15) / 16) {
 #define BIGCN_TCPG_CASE(ft)                                                                 \

@@ -9,7 +9,8 @@
 //   bigcn_weighted_layer_forward
 //       pack_rows -> pack_weights -> the degree pass (which also forms the
 //       row scale s_j = alpha_j dinv_j) -> the XNOR product with s as its row
-//       scale (dots kept factored when K <= 32767) -> the aggregation, which
+//       scale (dots kept factored when K <= 32767, in byte planes for the
+//       tensor-core aggregation where they fit) -> the aggregation, which
 //       weights neighbour j by a_ij s_j and multiplies the sum by dinv_i.
 //
 // The degrees need a pass of their own: unlike 1 + row length, a weighted
@@ -109,6 +110,7 @@ constexpr int32_t kMaxDots16K = 32767;
 struct WeightedWorkspace {
     size_t a_bits, alpha, b_bits, beta, z, rowscale, bexp, bexp_bytes, dinv, s, total;
     bool compressed;
+    bool planes;             // laid out for byte planes (rows of ldz bytes)
     int64_t ldz;
 };
 
@@ -116,7 +118,9 @@ bool weighted_workspace(int64_t N, int32_t K, int32_t F, WeightedWorkspace *w) {
     if (N < 0 || K < 1 || F < 1) return false;
     const int64_t words = bigcn_words(K);
     w->compressed = K <= kMaxDots16K;
-    w->ldz = w->compressed ? (int64_t(F) + 7) / 8 * 8 : F;
+    w->planes = K <= kMaxPlanesK && F <= 256;
+    const int64_t pad = w->planes ? 16 : 8;
+    w->ldz = w->compressed ? (int64_t(F) + pad - 1) / pad * pad : F;
     if (N > kMaxElems / (words > w->ldz ? words : w->ldz)) return false;
     size_t off = 0;
     w->a_bits = off;   off = wround(off + size_t(N) * size_t(words) * 8);
@@ -250,18 +254,28 @@ extern "C" bigcn_status bigcn_weighted_layer_forward(
     // Factored rows carry dinv_j in their row scale (s_j = alpha_j dinv_j);
     // fp32 rows are the plain product and the aggregation reads dinv_j.
     launch_weighted_dinv(rowptr, values, N, nnz, alpha, dinv, w.compressed ? srow : nullptr, s);
+    const bool bytes = w.planes && planes_faster(N, nnz, F) &&
+                       xnor_gemm_bytes_supported(N, K, F, dev);
+    // (uint16 dots are padded to 8 columns even where the workspace has room for 16)
+    const int64_t ldz = bytes ? w.ldz : w.compressed ? (int64_t(F) + 7) / 8 * 8 : F;
     GemmArgs g{a_bits, w.compressed ? srow : alpha, N, b_bits, beta, F, K, words, nullptr,
-               w.ldz, nullptr, nullptr};
+               ldz, nullptr, nullptr};
     if (w.bexp_bytes > 0) g.b_e4m3 = reinterpret_cast<uint8_t *>(ws + w.bexp);
-    SpmmArgs a{rowptr, colidx, N, nnz, nullptr, w.ldz, F, H, ldh, false, false};
+    SpmmArgs a{rowptr, colidx, N, nnz, nullptr, ldz, F, H, ldh, false, false};
     a.agg = kAggWeighted;
     a.values = values;
     a.dinv = dinv;
-    if (w.compressed) {
+    if (bytes) {
+        g.dots8 = reinterpret_cast<uint8_t *>(ws + w.z);
+        g.ldd8 = ldz;
+        g.rowscale = reinterpret_cast<float *>(ws + w.rowscale);
+        if (N >= kTcCounters && xnor_gemm_counters(N, K, F, dev))
+            g.counters = reinterpret_cast<uint32_t *>(srow);     // (only the product reads s)
+    } else if (w.compressed) {
         uint16_t *D16 = reinterpret_cast<uint16_t *>(ws + w.z);
         float *rowscale = reinterpret_cast<float *>(ws + w.rowscale);
         g.dots16 = D16;
-        g.ldd16 = w.ldz;
+        g.ldd16 = ldz;
         g.rowscale = rowscale;
         a.D16 = D16;
         a.rowscale = rowscale;
@@ -272,6 +286,12 @@ extern "C" bigcn_status bigcn_weighted_layer_forward(
         a.Z = Z;
     }
     launch_xnor_gemm(g, dev, s);
-    launch_spmm_norm(a, dev, s);
+    if (bytes) {
+        SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, ldz, g.rowscale, F, K, H, ldh, beta,
+                     nullptr, kAggWeighted, nullptr, nullptr, values, dinv, g.counters};
+        launch_spmm_tc(t, dev, s);
+    } else {
+        launch_spmm_norm(a, dev, s);
+    }
     return launch_status();
 }

@@ -59,7 +59,8 @@ __device__ __forceinline__ void tc_epilogue_bytes(uint32_t tmem, int warp, int l
                                                   const float *__restrict__ alpha,
                                                   const int64_t *__restrict__ rowptr, int F,
                                                   float *__restrict__ rowscale,
-                                                  uint8_t *__restrict__ dots8, int64_t ldd8, int K) {
+                                                  uint8_t *__restrict__ dots8, int64_t ldd8, int K, int half,
+                                                  int valid) {
     constexpr int kSplit = kWarps / (4 * kHalves);     // warps sharing a row
     __shared__ uint8_t wide_s[kSplit][kUmmaM * kHalves];
     const int quad = warp & 3;
@@ -78,7 +79,7 @@ __device__ __forceinline__ void tc_epilogue_bytes(uint32_t tmem, int warp, int l
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
             const ByteDot d(__float2int_rn(__uint_as_float(acc[e])), K);
-            w |= d.wide() && c0 + e < cols;
+            w |= d.wide() && flag_column(n0 + c0 + e, half, valid);
             u[e / 4] |= (high ? d.hi() & 255u : d.lo()) << (8 * (e % 4));
         }
         if (row < N)
@@ -119,10 +120,11 @@ __device__ __forceinline__ void tc_epilogue(uint32_t tmem, int warp, int lane, i
                                             int32_t *__restrict__ dots,
                                             uint16_t *__restrict__ dots16, int64_t ldd16,
                                             float *__restrict__ rowscale,
-                                            uint8_t *__restrict__ dots8, int64_t ldd8, int K) {
+                                            uint8_t *__restrict__ dots8, int64_t ldd8, int K,
+                                            int half, int valid) {
     if (dots8 != nullptr) {     // byte planes (one column tile, or no wide dots)
         tc_epilogue_bytes<NT, kHalves, kWarps, kDeg>(tmem, warp, lane, m0, n0, N, alpha, rowptr, F,
-                                                     rowscale, dots8, ldd8, K);
+                                                     rowscale, dots8, ldd8, K, half, valid);
         return;
     }
     const bool vec_z = (ldz & 3) == 0 && (reinterpret_cast<uintptr_t>(Z) & 15) == 0;
@@ -206,7 +208,8 @@ xnor_gemm_tc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ al
                     int words, float *__restrict__ Z, int64_t ldz, int32_t *__restrict__ dots,
                     const int64_t *__restrict__ rowptr, uint16_t *__restrict__ dots16,
                     int64_t ldd16, float *__restrict__ rowscale, uint8_t *__restrict__ dots8,
-                    int64_t ldd8, const uint8_t *__restrict__ bexp) {
+                    int64_t ldd8, int half, int valid, uint32_t *counters,
+                    const uint8_t *__restrict__ bexp) {
     constexpr int kStageA = kUmmaM * kTcKBytes;
     constexpr int kStageB = NT * kTcKBytes;
     constexpr int kStage = kStageA + kStageB;
@@ -370,9 +373,10 @@ xnor_gemm_tc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ al
     if (ok)
         tc_epilogue<NT, 1, kTcThreads / 32, kDeg>(tmem, warp, lane, m0, n0, N, alpha, rowptr, beta, F,
                                                   Z, ldz, dots, dots16, ldd16, rowscale, dots8, ldd8,
-                                                  K);
+                                                  K, half, valid);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (counters != nullptr && blockIdx.x == 0 && tid < kTcCounters) counters[tid] = 0u;
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NT));
 }
@@ -412,7 +416,8 @@ xnor_gemm_tc_ws_kernel(const uint64_t *__restrict__ A, const float *__restrict__
                        float *__restrict__ Z, int64_t ldz, int32_t *__restrict__ dots,
                        const int64_t *__restrict__ rowptr, uint16_t *__restrict__ dots16,
                        int64_t ldd16, float *__restrict__ rowscale, uint8_t *__restrict__ dots8,
-                       int64_t ldd8, const uint8_t *__restrict__ bexp) {
+                       int64_t ldd8, int half, int valid, uint32_t *counters,
+                    const uint8_t *__restrict__ bexp) {
     constexpr int NT = kWsCols;
     constexpr int kStageA = kWsRows * kTcKBytes;        // two 128-row halves
     constexpr int kStageB = NT * kTcKBytes;
@@ -589,9 +594,11 @@ xnor_gemm_tc_ws_kernel(const uint64_t *__restrict__ A, const float *__restrict__
     if (!ok && tid == 0) atomicAdd(&g_tc_timeouts, 1u);
     if (ok && warp < kWsExpWarps)
         tc_epilogue<NT, 2, kWsExpWarps, kDeg>(tmem, warp, lane, m0, n0, N, alpha, rowptr, beta, F, Z,
-                                              ldz, dots, dots16, ldd16, rowscale, dots8, ldd8, K);
+                                              ldz, dots, dots16, ldd16, rowscale, dots8, ldd8, K, half,
+                                              valid);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (counters != nullptr && blockIdx.x == 0 && tid < kTcCounters) counters[tid] = 0u;
     if (warp == kMmaWarp)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(2 * NT));
@@ -652,7 +659,8 @@ void launch_nt2(const GemmArgs &g, cudaStream_t s, bool pdl) {
     }
     launch_kernel(kernel, grid, dim3(kTcThreads), smem, s, pdl || kBexp, dim3(1, 1, 1), g.A,
                   g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z, g.ldz, g.dots, g.rowptr,
-                  g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, static_cast<const uint8_t *>(g.b_e4m3));
+                  g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half > 0 ? g.half : INT32_MAX,
+                  g.half > 0 ? g.valid : g.F, g.counters, static_cast<const uint8_t *>(g.b_e4m3));
 }
 
 template <bool kDeg>
@@ -666,7 +674,8 @@ void launch_ws(const GemmArgs &g, cudaStream_t s, bool pdl) {
                   pdl, dim3(1, 1, 1), g.B, g.F, g.K, g.words, KB, g.b_e4m3);
     launch_kernel(kernel, grid, dim3(kWsThreads), smem, s, true, dim3(1, 1, 1), g.A, g.alpha, g.N,
                   g.beta, g.F, g.K, g.words, g.Z, g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16,
-                  g.rowscale, g.dots8, g.ldd8, static_cast<const uint8_t *>(g.b_e4m3));
+                  g.rowscale, g.dots8, g.ldd8, g.half > 0 ? g.half : INT32_MAX,
+                  g.half > 0 ? g.valid : g.F, g.counters, static_cast<const uint8_t *>(g.b_e4m3));
 }
 
 template <int NT, bool kDeg>

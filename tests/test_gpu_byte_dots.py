@@ -45,12 +45,12 @@ LAYERS = [
     (1100, 300, 64, 90.0, 0, 5),        # long rows
     (1100, 2047, 65, 90.0, 900, 5),     # split front, five tiles in eight chunks
     (1100, 2048, 128, 70.0, 0, 7),
-    (4000, 254, 256, 9.0, 0, 4),        # CUDA-core product in column tiles: never wide
+    (2000, 254, 256, 70.0, 0, 4),       # CUDA-core product in column tiles: never wide
     (2500, 3072, 64, 9.0, 0, 4),        # CUDA-core product, wide
     (152 * 128 + 77, 130, 33, 5.0, 0, 9),       # tcgen05 products
     (152 * 128 + 1, 1030, 128, 6.0, 500, 2),
-    (152 * 128 + 200, 600, 144, 6.0, 0, 9),     # two column slabs of five tiles (one short)
-    (152 * 128 + 77, 3072, 256, 5.0, 0, 50),    # warp-specialised product, two slabs
+    (152 * 128 + 200, 600, 144, 66.0, 0, 9),    # two column slabs of five tiles (one short)
+    (152 * 128 + 77, 3072, 256, 70.0, 0, 50),   # warp-specialised product, two slabs
     (152 * 128 + 77, 700, 256, 70.0, 0, 50),    # two slabs, one-row windows
 ]
 
@@ -98,3 +98,43 @@ def test_forward_with_wide_rows(cuda_device, N, K, Fh, Fo, deg):
     r2 = oracle.layer_forward(H1.cpu().numpy(), W2, c["rowptr"], c["colidx"])
     check_sum(out.cpu().numpy(), r2["H"], r2["absterm"], f"wide rows logits {N}x{K}x{Fo}", n)
     assert np.array_equal(pred.cpu().numpy(), out.cpu().numpy().argmax(1))
+
+
+# The other aggregators over the same planes: (N, K, F, mean degree, hub, planted every)
+AGGREGATORS = [
+    (700, 258, 5, 4.0, 90, 3),          # fronts, GraphSAGE's halves padded from 5 to 16
+    (3000, 511, 50, 6.0, 400, 2),       # eight-row windows, a heavy row
+    (1100, 300, 64, 90.0, 900, 5),      # one-row windows
+    (700, 200, 100, 4.0, 90, 3),        # weighted: the CUDA-core product in column tiles
+    (152 * 128 + 77, 1030, 100, 6.0, 0, 9),     # tcgen05 products (two halves: 224 columns)
+    (152 * 128 + 77, 600, 144, 70.0, 0, 9),     # two column slabs (GraphSAGE: uint16 dots)
+]
+
+
+@pytest.mark.parametrize("N,K,F,deg,hub,every", AGGREGATORS)
+@pytest.mark.parametrize("agg", ["mean", "sage", "weighted"])
+def test_aggregators_with_wide_rows(cuda_device, agg, N, K, F, deg, hub, every):
+    c = planted_case(N, K, F, deg, hub, every, seed=N + K + F)
+    rp, ci = c["rowptr"], c["colidx"]
+    d = {k: to_dev(v) for k, v in c.items() if v is not None}
+    H = torch.full((N, F), float("nan"), device=cuda_device)
+    rows = sampled(N, 600, K)
+    if agg == "weighted":
+        vals = inputs.edge_weights(rp, ci, K)
+        vals[::7] = 0.0
+        ws = torch.full((B.bigcn_weighted_layer_workspace_bytes(N, K, F),), 0xAB,
+                        dtype=torch.uint8, device=cuda_device)
+        B.bigcn_weighted_layer_forward(d["X"], None, None, d["W"], d["rowptr"], d["colidx"],
+                                       to_dev(vals), ws, H)
+        ref = oracle.layer_forward_weighted(c["X"], c["W"], rp, ci, vals, rows=rows)
+    else:
+        Wn = inputs.weights(K, F, seed=K + F) if agg == "sage" else None
+        ws = torch.full((B.bigcn_inductive_layer_workspace_bytes(agg, N, K, F),), 0xAB,
+                        dtype=torch.uint8, device=cuda_device)
+        B.bigcn_inductive_layer_forward(agg, d["X"], None, None, d["W"], d["rowptr"],
+                                        d["colidx"], ws, H, W_neigh=to_dev(Wn))
+        ref = oracle.layer_forward_inductive(c["X"], c["W"], rp, ci, agg, W_neigh=Wn, rows=rows)
+    torch.cuda.synchronize()
+    assert B.device_timeouts() == 0
+    check_sum(H.cpu().numpy()[rows], ref["H"], ref["absterm"],
+              f"{agg} layer with wide rows {N}x{K}x{F}", int(np.diff(rp)[rows].max()) + 2)
