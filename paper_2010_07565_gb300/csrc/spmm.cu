@@ -5,8 +5,8 @@
 // groups of L lanes; each group gathers a different neighbour's row of Z,
 // lane by lane in VEC-wide vectors (NV per lane), so rows narrower than a
 // warp still keep all 32 lanes busy, and U such gathers are issued before any
-// is consumed (U = 4, or 2 when each lane holds two vectors; twice that for
-// compressed rows spread over all 32 lanes). Neighbour indices (and, unless Z is pre-scaled, their
+// is consumed (U = 4; twice that for compressed rows of four dots a lane spread
+// over all 32 lanes). Neighbour indices (and, unless Z is pre-scaled, their
 // 1/sqrt(dhat_j)) are fetched 32 at a time, one per lane, then broadcast with
 // shuffles. The self-loop that A + I adds is entry 0 of every row's list.
 // Partial sums are combined across groups with xor shuffles and group 0
@@ -21,7 +21,17 @@
 // on many blocks), skip light rows, and give each heavy row to all 8 warps of
 // the block: warp w gathers the w-th eighth of the row's list, the eight
 // partial rows meet in shared memory and warp 0 adds them in warp order
-// (deterministic) before the same epilogue. Light warps skip heavy rows.
+// (deterministic) before the same epilogue. Light warps skip heavy rows; on
+// large graphs a block's warps take 64 rows in turn as they become free.
+//
+// What bounds it: rows in flight against L2's latency, and issue. Tests on every
+// gather (list end, column range, row end) and 64-bit row addresses cost 17
+// warp-instructions per entry and 64 features; full groups without them 4. On
+// 232,965 nodes of mean degree 492 (114.8 M rows of 512 bytes) 6180 -> 3440 us,
+// 17 TB/s of gathered rows; 169,343 nodes of mean degree 14, F = 256, 602 -> 298
+// us; 65,521 nodes of mean degree 16, F = 96, 81 -> 64 us; 2^20 nodes of mean
+// degree 16, 256 16-bit dots, 2010 -> 1663 us (rows of 537 MB of dots, 5.5 TB/s
+// from L2 and HBM).
 //
 // Rows of Z come in one of three forms (template S): fp32 rows weighted by
 // 1/sqrt(dhat_j) per neighbour (kDinv), fp32 rows that already carry it
@@ -91,6 +101,7 @@ struct SpmmParams {
     int64_t ldh;
     int heavy_blocks;        // leading blocks that take the heavy rows
     int64_t heavy_degree;    // rows with more neighbours are heavy
+    int pool;                // rows per light block
     bool vec_store;          // H rows start VEC-aligned: whole vectors may be stored
     const float *rowscale;   // kDots16: s_j
     const float *colscale;   // kDots16: beta_f
@@ -191,15 +202,27 @@ __device__ __forceinline__ RowSpan row_span(const int64_t *__restrict__ rowptr, 
 // Adds, into acc, the Z rows of entries [q0, q1) of row i's list (entry 0 is
 // the self-loop), weighted by 1/sqrt(dhat_j) (kDinv), 1 (kPre) or s_j (kDots16),
 // and for a weighted A (kAggWeighted) also by the entry's a_ij (1 for the
-// self-loop), with dhat_j read from p.dinv.
+// self-loop), with dhat_j read from p.dinv. Groups of P U valid entries take a
+// path without tests, each gather one multiply-add for its address (a lane
+// past the row's features reads its first ones and is never stored), whole
+// chunks of 32 unrolled; only a list's last group tests its entries.
 template <int VEC, int L, int NV, int U, int S, int AGG = kAggGcn>
 __device__ __forceinline__ void gather(const SpmmParams &p, int64_t i, int64_t b, int64_t q0,
                                        int64_t q1, int f0, float (&acc)[NV][VEC]) {
     using Src = RowSrc<VEC, S>;
     using V = typename Src::T;
     constexpr int P = 32 / L;
+    constexpr int kElem = S == kDots16 ? 2 : 4;
     const int lane = threadIdx.x & 31;
     const int g = lane / L, sl = lane % L;
+    const uint32_t ld_lo = uint32_t(uint64_t(p.ldz) * kElem);
+    const uint32_t ld_hi = uint32_t((uint64_t(p.ldz) * kElem) >> 32);
+    const char *zl[NV];         // this lane's vectors of row 0
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        const int f = f0 + (v * L + sl) * VEC;
+        zl[v] = static_cast<const char *>(p.Z) + int64_t(f < p.Fload ? f : 0) * kElem;
+    }
     for (int64_t base = q0; base < q1; base += 32) {
         int j = -1;
         float wj = 0.0f;
@@ -217,7 +240,34 @@ __device__ __forceinline__ void gather(const SpmmParams &p, int64_t i, int64_t b
             }
         }
         const int cnt = int(min(q1 - base, int64_t(32)));
-        for (int t0 = 0; t0 < cnt; t0 += P * U) {
+        // P U entries from t0 on, all of them valid.
+        auto whole = [&](int t0) {
+            V val[U][NV];
+            float w[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t jj = uint32_t(__shfl_sync(kFullMask, j, t0 + u * P + g));
+                w[u] = S == kPre ? 1.0f : __shfl_sync(kFullMask, wj, t0 + u * P + g);
+                const uint64_t off = uint64_t(jj) * ld_lo + (uint64_t(jj * ld_hi) << 32);
+#pragma unroll
+                for (int v = 0; v < NV; ++v)
+                    val[u][v] = __ldg(reinterpret_cast<const V *>(zl[v] + off));
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int v = 0; v < NV; ++v) Src::fma(acc[v], val[u][v], w[u]);
+        };
+        const unsigned valid = __ballot_sync(kFullMask, j >= 0);
+        int t0 = 0;
+        if (valid == kFullMask) {
+#pragma unroll
+            for (int t = 0; t < 32; t += P * U) whole(t);
+            continue;
+        }
+        if (valid == (1u << cnt) - 1u)
+            for (; t0 + P * U <= cnt; t0 += P * U) whole(t0);
+        for (; t0 < cnt; t0 += P * U) {
             V val[U][NV];
             float w[U];
 #pragma unroll
@@ -227,11 +277,11 @@ __device__ __forceinline__ void gather(const SpmmParams &p, int64_t i, int64_t b
                 w[u] = __shfl_sync(kFullMask, wj, src & 31);
                 const bool live = src < cnt && jj >= 0;
                 if (!live) w[u] = 0.0f;
-                const int64_t zrow = live ? jj : 0;
+                const uint64_t off = uint64_t(uint32_t(jj)) * ld_lo +
+                                     (uint64_t(uint32_t(jj) * ld_hi) << 32);
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
-                    const int f = f0 + (v * L + sl) * VEC;
-                    if (live && f < p.Fload) val[u][v] = Src::load(p.Z, zrow, p.ldz, f);
+                    if (live) val[u][v] = __ldg(reinterpret_cast<const V *>(zl[v] + off));
                     else val[u][v] = V{};
                 }
             }
@@ -357,21 +407,33 @@ argmax_rows_kernel(const float *__restrict__ H, int64_t N, int F, int64_t ldh,
     if (lane == 0) pred[i] = best;
 }
 
+// Light rows: the block's p.pool rows, which its warps take in turn as they
+// become free (`next` counts those taken): with a row per warp the block would
+// hold its place until its longest row ended.
 template <int VEC, int L, int NV, int U, int S, class Epi, int AGG = kAggGcn>
-__device__ __forceinline__ void light_rows(const SpmmParams &p, const Epi &epi, int f0) {
-    const int warp = threadIdx.x >> 5;
-    const int64_t i = int64_t(blockIdx.x - p.heavy_blocks) * kSpmmWarps + warp;
-    if (i >= p.N) return;
-    const RowSpan sp = row_span(p.rowptr, p.nnz, i, AGG, p.dinv);
-    if (p.heavy_blocks > 0 && sp.total - 1 > p.heavy_degree) return;   // a heavy block's row
-    float acc[NV][VEC];
+__device__ __forceinline__ void light_rows(const SpmmParams &p, const Epi &epi, int f0,
+                                           int *next) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t first = int64_t(blockIdx.x - p.heavy_blocks) * p.pool;
+    int k = warp;                           // the first rows go one to a warp
+    while (k < p.pool && first + k < p.N) {
+        const int64_t i = first + k;
+        int taken = 0;
+        if (p.pool > kSpmmWarps && lane == 0) taken = atomicAdd(next, 1);
+        const RowSpan sp = row_span(p.rowptr, p.nnz, i, AGG, p.dinv);
+        if (p.heavy_blocks == 0 || sp.total - 1 <= p.heavy_degree) {   // else a heavy block's row
+            float acc[NV][VEC];
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
+            for (int v = 0; v < NV; ++v)
 #pragma unroll
-        for (int c = 0; c < VEC; ++c) acc[v][c] = 0.0f;
-    gather<VEC, L, NV, U, S, AGG>(p, i, sp.b, sp.first, sp.total, f0, acc);
-    reduce_groups<VEC, L, NV>(acc);
-    epi(p, i, sp.dinv, f0, acc);
+                for (int c = 0; c < VEC; ++c) acc[v][c] = 0.0f;
+            gather<VEC, L, NV, U, S, AGG>(p, i, sp.b, sp.first, sp.total, f0, acc);
+            reduce_groups<VEC, L, NV>(acc);
+            epi(p, i, sp.dinv, f0, acc);
+        }
+        if (p.pool <= kSpmmWarps) return;
+        k = kSpmmWarps + __shfl_sync(kFullMask, taken, 0);
+    }
 }
 
 template <int VEC, int L, int NV, int U, int S, class Epi, int AGG = kAggGcn>
@@ -429,19 +491,30 @@ __device__ __forceinline__ void heavy_rows(const SpmmParams &p, const Epi &epi, 
     }
 }
 
+// Blocks per SM the registers are held to. Full groups carry no tests, so a warp
+// holds its rows in flight in few registers: 16-bit dots fit 48 a thread (2^20
+// rows of mean degree 16, F = 256: 1794 us at four blocks, 1663 at five); fp32
+// rows take 64, and two vectors a lane 80, with four rows of 1 KB in flight
+// (169,343 rows of mean degree 14, F = 256: 367 us with two at four blocks, 298
+// with four at three).
+constexpr int spmm_blocks(int NV, int S) { return S == kDots16 ? 5 : NV == 2 ? 3 : 4; }
+
 template <int VEC, int L, int NV, int U, int S, int AGG>
-__global__ void __launch_bounds__(kSpmmThreads, 4)
+__global__ void __launch_bounds__(kSpmmThreads, spmm_blocks(NV, S))
 spmm_norm_kernel(SpmmParams p) {
     constexpr int SLAB = L * NV * VEC;
     __shared__ float part[kSpmmWarps * SLAB];
+    __shared__ int next;
+    if (threadIdx.x == 0) next = 0;
     grid_dependency_wait();     // Z is the output of the previous kernel
+    __syncthreads();
     const int f0 = blockIdx.y * SLAB;
     using Epi = StoreRow<VEC, L, NV, S, AGG>;
     Epi epi;
     if (int(blockIdx.x) < p.heavy_blocks)
         heavy_rows<VEC, L, NV, U, S, Epi, AGG>(p, epi, f0, part);
     else
-        light_rows<VEC, L, NV, U, S, Epi, AGG>(p, epi, f0);
+        light_rows<VEC, L, NV, U, S, Epi, AGG>(p, epi, f0, &next);
 }
 
 // ---------------------------------------------------------------------------
@@ -556,6 +629,8 @@ spmm_pack_gemm_kernel(SpmmParams p, FusedLayer2 f, const uint64_t *__restrict__ 
     __shared__ uint64_t sW[kMaxFusedOut * 2];
     __shared__ float sBeta1[128];
     __shared__ float sBeta2[kMaxFusedOut];
+    __shared__ int next;
+    if (threadIdx.x == 0) next = 0;
     grid_dependency_wait();     // layer 1's Z' and the packed W2 come from earlier kernels
     for (int q = threadIdx.x; q < f.Fo * f.words2; q += kSpmmThreads) sW[q] = __ldg(wbits2 + q);
     for (int q = threadIdx.x; q < f.Fo; q += kSpmmThreads) sBeta2[q] = __ldg(beta2 + q);
@@ -569,7 +644,7 @@ spmm_pack_gemm_kernel(SpmmParams p, FusedLayer2 f, const uint64_t *__restrict__ 
     if (int(blockIdx.x) < p.heavy_blocks)
         heavy_rows<VEC, L, 1, U, S>(p, epi, 0, part);
     else
-        light_rows<VEC, L, 1, U, S>(p, epi, 0);
+        light_rows<VEC, L, 1, U, S>(p, epi, 0, &next);
 }
 
 // Leading blocks that look for heavy rows: up to two per SM, one per 32 rows.
@@ -577,6 +652,15 @@ int heavy_block_count(int64_t N, const DeviceInfo &dev) {
     const int64_t chunks = (N + 31) / 32;
     const int64_t cap = 2 * int64_t(dev.sm_count);
     return int(chunks < cap ? chunks : cap);
+}
+
+// Rows per light block: a pool of several per warp once that still leaves every
+// SM kPoolBlocks blocks to start (2^20 rows of 256 16-bit dots: 1807 us with a
+// row per warp, 1663 us with 64 per block).
+constexpr int kPoolRows = 64;
+constexpr int kPoolBlocks = 16;
+int pool_rows(int64_t N, const DeviceInfo &dev) {
+    return N >= int64_t(kPoolRows) * kPoolBlocks * dev.sm_count ? kPoolRows : kSpmmWarps;
 }
 
 // The heavy-row threshold for a walk of `per_iter` neighbours per round trip.
@@ -598,16 +682,16 @@ void launch_cfg(const SpmmArgs &a, const DeviceInfo &dev, int Fload, cudaStream_
     // where a warp holds only a few rows at a time (one row across all 32
     // lanes) it takes twice as many.
     constexpr int U = VEC == 8 ? (NV == 1 ? 4 : 2)
-                               : (S == kDots16 && L == 32 ? 2 : 1) * (NV == 1 ? 4 : 2);
+                               : (S == kDots16 && L == 32 && NV == 1 ? 2 : 1) * 4;
     constexpr int kStoreVec = VEC < 4 ? VEC : 4;    // 8-wide rows are stored as two float4
     const bool vec_store = a.ldh % kStoreVec == 0 && aligned_to(a.H, size_t(kStoreVec) * 4);
     const void *Z = S == kDots16 ? static_cast<const void *>(a.D16) : a.Z;
     const bool one_slab = a.F <= SLAB;
     SpmmParams p{a.rowptr, a.colidx, a.N, a.nnz, Z, a.ldz, Fload, a.F, a.H, a.ldh,
-                 heavy_block_count(a.N, dev), heavy_degree(a.N, a.nnz, (32 / L) * U), vec_store,
-                 a.rowscale, a.colscale, one_slab ? a.pred : nullptr, a.agg, a.Zs,
+                 heavy_block_count(a.N, dev), heavy_degree(a.N, a.nnz, (32 / L) * U),
+                 pool_rows(a.N, dev), vec_store, a.rowscale, a.colscale, one_slab ? a.pred : nullptr, a.agg, a.Zs,
                  a.colscale_s, a.ncols > 0 ? a.ncols : a.N, a.values, a.dinv};
-    dim3 grid(unsigned(p.heavy_blocks + (a.N + kSpmmWarps - 1) / kSpmmWarps),
+    dim3 grid(unsigned(p.heavy_blocks + (a.N + p.pool - 1) / p.pool),
               unsigned((a.F + SLAB - 1) / SLAB));
     launch_kernel(spmm_norm_kernel<VEC, L, NV, U, S, AGG>, grid, dim3(kSpmmThreads), 0, s, pdl,
                   dim3(1, 1, 1), p);
@@ -618,20 +702,16 @@ void launch_cfg(const SpmmArgs &a, const DeviceInfo &dev, int Fload, cudaStream_
 }
 
 // Lanes per neighbour L = the power of two >= the row's vector count (at
-// least 4, at most 32); NV = 2 vectors per lane once a row exceeds 32.
-// fp32 rows of Z larger than this in all are gathered in column slabs of at
-// most 16 vectors per lane group: the slabs (grid y) run mostly one after the
-// other, so each keeps only its share of Z in L2 (measured on 119 MB of
-// 128-wide rows: 7.17 -> 6.49 ms; 16-bit dots, at 8 per lane, lose by it).
-constexpr int64_t kSlabL2Bytes = int64_t(64) << 20;
-
+// least 4, at most 32); NV = 2 vectors per lane once a row exceeds 32. (Column
+// slabs that keep each share of a large Z in L2 paid while every gather was
+// tested; now the whole row in one walk is faster: 232,965 rows of mean degree
+// 492, 128 fp32 features, 3941 us in two slabs, 3509 us in one.)
 template <int VEC, int S, int AGG = kAggGcn>
 void launch_vec(const SpmmArgs &a, const DeviceInfo &dev, int Fload, cudaStream_t s, bool pdl) {
     const int nvec = Fload / VEC;
-    const int64_t zbytes = S == kDots16 ? 0 : a.N * int64_t(Fload) * 4;
     if (nvec <= 4) launch_cfg<VEC, 4, 1, S, AGG>(a, dev, Fload, s, pdl);
     else if (nvec <= 8) launch_cfg<VEC, 8, 1, S, AGG>(a, dev, Fload, s, pdl);
-    else if (nvec <= 16 || zbytes > kSlabL2Bytes) launch_cfg<VEC, 16, 1, S, AGG>(a, dev, Fload, s, pdl);
+    else if (nvec <= 16) launch_cfg<VEC, 16, 1, S, AGG>(a, dev, Fload, s, pdl);
     else if (nvec <= 32) launch_cfg<VEC, 32, 1, S, AGG>(a, dev, Fload, s, pdl);
     else launch_cfg<VEC, 32, 2, S, AGG>(a, dev, Fload, s, pdl);
 }
@@ -715,8 +795,8 @@ void launch_spmm_pack_gemm(const SpmmPackGemmArgs &a, const DeviceInfo &dev, cud
     const int U = c16 && VEC == 4 && L == 32 ? 8 : 4;
     const void *Z1 = c16 ? static_cast<const void *>(a.D1) : static_cast<const void *>(a.Z1);
     SpmmParams p{a.rowptr, a.colidx, a.N, a.nnz, Z1, c16 ? a.ldz1 : a.Fh, Fload, a.Fh, nullptr, 0,
-                 heavy_block_count(a.N, dev), heavy_degree(a.N, a.nnz, (32 / L) * U), false,
-                 a.s1, nullptr, nullptr};
+                 heavy_block_count(a.N, dev), heavy_degree(a.N, a.nnz, (32 / L) * U),
+                 kSpmmWarps, false, a.s1, nullptr, nullptr};
     p.ncols = a.N;
     FusedLayer2 f{a.H1, a.ldh, nullptr, nullptr, nullptr, a.Fo, (a.Fh + 63) / 64, a.Z2, a.ldz2};
     const dim3 grid(unsigned(p.heavy_blocks + (a.N + kSpmmWarps - 1) / kSpmmWarps));
