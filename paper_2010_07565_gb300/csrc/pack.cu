@@ -10,10 +10,9 @@
 // lane keeps a running sum of |y|. G warps (1, 2, 4 or 8, so that the grid
 // fills the GPU even when N is small) share a row, warp g taking chunks
 // g, g + G, ...; each warp issues eight chunks' loads (1 KB) before it
-// consumes any, and the grids are persistent (eight blocks per SM). The
-// whole-row kernel has no block barrier and stays at full occupancy, which
-// -- not a deeper unroll -- is what overlaps one warp's ballots with the
-// other warps' loads. The G partial |y| sums are added in a fixed order through
+// consumes any, and the grids are persistent. The whole-row kernel has no block
+// barrier; on many rows a warp packs four together (pack_group), which keeps more
+// loads in flight than full occupancy with one row each. The G partial |y| sums are added in a fixed order through
 // shared memory, so alpha does not depend on scheduling.
 //
 // pack_weights reads W (K x F) column-wise: thread (x, y) of a 32 x 8 block
@@ -39,22 +38,30 @@ constexpr int kPackWarps = kPackThreads / 32;
 constexpr int kPackBlocksPerSM = 8;   // resident blocks the persistent grids assume
 constexpr int kPackUnroll = 8;
 
-// Whole rows per warp: every warp walks rows on its own (persistent grid,
-// no block barrier), which keeps the kernel small enough for full occupancy.
-template <bool kAffine, bool kUpstream>
-__global__ void __launch_bounds__(kPackThreads, kPackBlocksPerSM)
+// Whole rows per warp, R at a time: every warp walks groups of rows on its own
+// (persistent grid, no block barrier).
+template <int R, int C, int kBlocks, bool kAffine, bool kUpstream>
+__global__ void __launch_bounds__(kPackThreads, kBlocks)
 pack_rows_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
                  const float *__restrict__ scale, const float *__restrict__ shift,
                  uint32_t *__restrict__ bits32, int64_t ld32, float *__restrict__ alpha) {
     if (kUpstream) grid_dependency_wait();      // X is the previous kernel's output
-    constexpr Affine kA = kAffine ? Affine::kGlobalLate : Affine::kNone;
+    constexpr Affine kA = kAffine ? Affine::kGlobal : Affine::kNone;
     const int lane = threadIdx.x & 31;
-    const int64_t nwarps = int64_t(gridDim.x) * kPackWarps;
-    for (int64_t row = int64_t(blockIdx.x) * kPackWarps + (threadIdx.x >> 5); row < N;
-         row += nwarps) {
-        const float l1 = pack_share<1, kPackUnroll, kA>(X + row * ldx, K, scale, shift, nullptr,
-                                                        bits32 + row * ld32, ld32, 0);
-        if (lane == 0) alpha[row] = l1 / float(K);
+    const int64_t step = int64_t(gridDim.x) * kPackWarps * R;
+    for (int64_t row = (int64_t(blockIdx.x) * kPackWarps + (threadIdx.x >> 5)) * R; row < N;
+         row += step) {
+        float l1[R];
+        const int rows = int(min(N - row, int64_t(R)));
+        pack_group<R, C, kA>(X + row * ldx, ldx, rows, K, scale, shift, bits32 + row * ld32, ld32,
+                             ld32, l1);
+        float mine = 0.0f;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float s = warp_sum(l1[r]);
+            if (lane == r) mine = s;
+        }
+        if (lane < rows) alpha[row + lane] = mine / float(K);
     }
     // Otherwise wait only now: finishing after the predecessor keeps the
     // chain's completion order for the kernels that follow.
@@ -150,6 +157,17 @@ pack_weights_kernel(WeightPack a, WeightPack b) {
     cluster.sync();   // peers keep their shared memory until block 0 has read it
 }
 
+// Rows a warp packs together once every warp has as many: four rows' chunks in
+// flight at once keep loads going where one row's end, its reduction and the next
+// row's first loads left gaps, and share the centring's loads (2^20 x 512: 438 ->
+// 332 us, 6.5 TB/s; 232,965 x 602: 149 -> 96; 100,003 x 300: 48 -> 28; 169,343 x
+// 128: 58 -> 21). Four chunks of each and four blocks per SM; long rows take eight
+// chunks and three blocks (2^20 x 4096: 3030 -> 2724 us, 6.3 TB/s; four chunks 2780;
+// on 602 features eight are slower, 105 us: the row's last batch is a test per chunk).
+constexpr int kManyR = 4;
+constexpr int kManyBlocks = 4;
+constexpr int kLongK = 2048;
+
 }  // namespace
 
 void launch_pack_rows(const float *X, int64_t N, int K, int64_t ldx, const float *scale,
@@ -162,9 +180,11 @@ void launch_pack_rows(const float *X, int64_t N, int K, int64_t ldx, const float
     const int64_t full_wave = int64_t(dev.sm_count) * 64;
     int G = 1;
     while (G < kPackWarps && N * G < full_wave && nchunks >= 2 * G * 8) G *= 2;
-    const int rows_per_block = kPackWarps / G;
+    const bool many = N >= int64_t(kManyR) * dev.sm_count * kManyBlocks * kPackWarps;
+    const int rows_per_block = G > 1 ? kPackWarps / G : many ? kPackWarps * kManyR : kPackWarps;
     const int64_t groups = (N + rows_per_block - 1) / rows_per_block;
-    const int64_t resident = int64_t(dev.sm_count) * kPackBlocksPerSM;
+    const int per_sm = G > 1 || !many ? kPackBlocksPerSM : K >= kLongK ? 3 : kManyBlocks;
+    const int64_t resident = int64_t(dev.sm_count) * per_sm;
     const dim3 grid(unsigned(groups < resident ? groups : resident)), block(kPackThreads), one(1, 1, 1);
     uint32_t *b32 = reinterpret_cast<uint32_t *>(bits);
     const int64_t ld32 = int64_t(words) * 2;
@@ -174,10 +194,19 @@ void launch_pack_rows(const float *X, int64_t N, int K, int64_t ldx, const float
             launch_kernel(kernel, grid, block, 0, stream, pdl, one, X, N, K, ldx, sc, sh, b32, ld32,
                           alpha);
         };
-        if (scale && x_upstream) run(pack_rows_kernel<true, true>, scale, shift);
-        else if (scale) run(pack_rows_kernel<true, false>, scale, shift);
-        else if (x_upstream) run(pack_rows_kernel<false, true>, no, no);
-        else run(pack_rows_kernel<false, false>, no, no);
+#define BIGCN_PACK_CASE(R, C, B)                                                          \
+    if (scale && x_upstream) run(pack_rows_kernel<R, C, B, true, true>, scale, shift);    \
+    else if (scale) run(pack_rows_kernel<R, C, B, true, false>, scale, shift);            \
+    else if (x_upstream) run(pack_rows_kernel<R, C, B, false, true>, no, no);             \
+    else run(pack_rows_kernel<R, C, B, false, false>, no, no);
+        if (many && K >= kLongK) {
+            BIGCN_PACK_CASE(kManyR, 8, 3)
+        } else if (many) {
+            BIGCN_PACK_CASE(kManyR, 4, kManyBlocks)
+        } else {
+            BIGCN_PACK_CASE(1, kPackUnroll, kPackBlocksPerSM)
+        }
+#undef BIGCN_PACK_CASE
     } else {
         auto run = [&](auto kernel, const float *sc, const float *sh) {
             launch_kernel(kernel, grid, block, 0, stream, pdl, one, X, N, K, ldx, sc, sh, b32, ld32,

@@ -106,4 +106,90 @@ __device__ __forceinline__ float pack_share(const float *__restrict__ x, int K,
     return warp_sum(l1);
 }
 
+// R rows of X (row stride ldx, `rows` of them real) packed by one warp together:
+// C chunks of each per batch, R C loads in flight, and the centring affine read
+// once for all of them. Lane r C + c keeps row r's ballot of chunk c, so that a
+// batch's half-words are one store. Row r's half-words go to out + r ldo, pad
+// half-words up to ld32 as zeros; l1[r] receives the lane's share of its |y| sum
+// (chunks in order, as pack_share's with G = 1).
+template <int R, int C, Affine kA>
+__device__ __forceinline__ void pack_group(const float *__restrict__ x, int64_t ldx, int rows,
+                                           int K, const float *__restrict__ scale,
+                                           const float *__restrict__ shift, uint32_t *out,
+                                           int64_t ldo, int64_t ld32, float (&l1)[R]) {
+    static_assert(R * C <= 32, "a lane per ballot");
+    static_assert(kA == Affine::kNone || kA == Affine::kGlobal, "");
+    const int lane = threadIdx.x & 31;
+    const int nchunks = (K + 31) >> 5, full = K >> 5;
+    const float *xl[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        xl[r] = x + int64_t(min(r, rows - 1)) * ldx + lane;
+        l1[r] = 0.0f;
+    }
+    const int mr = lane / C, mc = lane % C;      // the ballot this lane keeps
+    uint32_t *ol = out + int64_t(mr) * ldo + mc;
+    const bool mine = mr < R && mr < rows;
+    int c0 = 0;
+    for (; c0 + C <= full; c0 += C) {
+        float v[R][C], a[C], b[C];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) v[r][c] = __ldcs(xl[r] + 32 * c);
+        if (kA == Affine::kGlobal) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                a[c] = __ldg(scale + 32 * (c0 + c) + lane);
+                b[c] = __ldg(shift + 32 * (c0 + c) + lane);
+            }
+        }
+        uint32_t word = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                float y = v[r][c];
+                if (kA == Affine::kGlobal) y = __fmaf_rn(y, a[c], b[c]);
+                const unsigned m = __ballot_sync(kFullMask, y >= 0.0f);
+                if (lane == r * C + c) word = m;
+                l1[r] += fabsf(y);
+            }
+        if (mine) ol[c0] = word;
+#pragma unroll
+        for (int r = 0; r < R; ++r) xl[r] += 32 * C;
+    }
+    if (c0 < nchunks) {                          // the last, partial batch
+        float v[R][C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const bool in = (c0 + c) * 32 + lane < K;
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r][c] = in ? __ldcs(xl[r] + 32 * c) : 0.0f;
+        }
+        uint32_t word = 0;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int k = (c0 + c) * 32 + lane;
+            const bool in = k < K;
+            float a = 1.0f, b = 0.0f;
+            if (kA == Affine::kGlobal && in) {
+                a = __ldg(scale + k);
+                b = __ldg(shift + k);
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float y = v[r][c];
+                if (kA == Affine::kGlobal) y = __fmaf_rn(y, a, b);
+                const unsigned m = __ballot_sync(kFullMask, in && y >= 0.0f);
+                if (lane == r * C + c) word = m;
+                l1[r] += in ? fabsf(y) : 0.0f;
+            }
+        }
+        if (mine && c0 + mc < nchunks) ol[c0] = word;
+    }
+    for (int64_t h = nchunks; h < ld32; ++h)     // pad half-words (one, or a caller's extra words)
+        if (lane < rows) out[int64_t(lane) * ldo + h] = 0u;
+}
+
 }  // namespace bigcn

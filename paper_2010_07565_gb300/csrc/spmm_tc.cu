@@ -1109,13 +1109,17 @@ void launch_rows(const TcParams &P0, const Epi &epi, int slabs, const DeviceInfo
 // Rows per window: one when rows are long (a window's blocks then all belong to
 // one row; at a mean degree of 50 and 41 features 122 us against 113 us for eight
 // rows, at 120 and 100 features 301 against 366 us), or too few to give many
-// warps eight (1001 rows: 6.3 us against 7.8 us; 5000 rows: 11.0 against 10.0 us),
-// else eight (2^20 rows of mean degree 16, 64 features: 442 us against 894 us).
+// warps eight (1001 rows: 6.3 us against 7.8 us; 5000 rows of mean degree 6: 11.0
+// against 10.0 us; 10,000 of 30: 28.7 against 30.6 us), else eight (2^20 rows of
+// mean degree 16, 64 features: 442 us against 894 us).
 constexpr int64_t kOneRowDegree = 64;
 constexpr int64_t kFewRows = 16;        // per SM
+constexpr int64_t kFewLongRows = 128;   // per SM, of mean degree kFewDegree and more
+constexpr int64_t kFewDegree = 24;
 
 bool tc_one_row(int64_t N, int64_t nnz, const DeviceInfo &dev) {
-    return nnz >= kOneRowDegree * N || N < kFewRows * int64_t(dev.sm_count);
+    return nnz >= kOneRowDegree * N || N < kFewRows * int64_t(dev.sm_count) ||
+           (nnz >= kFewDegree * N && N < kFewLongRows * int64_t(dev.sm_count));
 }
 
 template <int FT, bool kW = false, class Epi>
