@@ -69,6 +69,17 @@ __device__ __forceinline__ void allow_dependent_launch() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// A word that the previous kernel of the chain wrote, read right after
+// grid_dependency_wait(). A read-only (__ldg) load is free of the wait for the
+// compiler, which may move it ahead of it when both are in straight line: the
+// product's first operand words then came from before the packing (seen as wrong
+// dots in one launch of ten). A volatile load stays behind the wait.
+__device__ __forceinline__ uint64_t load_upstream(const uint64_t *p) {
+    uint64_t v;
+    asm volatile("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // Launches `kernel` with optional programmatic serialization (pdl) and an
 // optional cluster shape; the launch error is left for launch_status().
 template <typename... KArgs, typename... Args>

@@ -104,7 +104,7 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
     grid_dependency_wait();
     if (blockIdx.x == 0 && tid < n_counters) counters[tid] = 0u;
     for (int q = tid; q < F * words; q += kFrontThreads)
-        Bs[slot(q / words) * pitch + (q % words)] = __ldg(wbits + q);
+        Bs[slot(q / words) * pitch + (q % words)] = load_upstream(wbits + q);
     __syncthreads();
 
     // Phase B: XNOR-popcount against every column.
@@ -321,7 +321,7 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int q = q0 + u * kSplitThreads;
-                    if (q < n) v[u] = __ldg(wbits + q);
+                    if (q < n) v[u] = load_upstream(wbits + q);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {

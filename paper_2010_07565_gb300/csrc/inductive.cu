@@ -150,6 +150,8 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
                                             beta + Fp, 0}
                                : WeightPack{nullptr, 1, 0, 0, nullptr, 0, nullptr, 0};
     launch_pack_weights2(wa, wb, s);
+    // Every kernel from here on may start while the one before it drains (each
+    // waits for it before it reads anything the call has written).
     // The product without a degree factor: Z_ij = alpha_i beta_j dot_ij, kept
     // factored (uint16 dots, row scale alpha_i) when K allows.
     GemmArgs g{a_bits, alpha, N, b_bits, beta, Fz, K, words, nullptr, Fz, nullptr, nullptr};
@@ -190,17 +192,17 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
         FrontArgs fr{X, N, K, ldx, scale, shift, b_bits, beta, Fz, words, nullptr, g.Z, g.ldz,
                      g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half, g.valid,
                      g.counters, kTcCounters};
-        launch_front(fr, dev, s);
+        launch_front(fr, dev, s, true);
     } else {
-        launch_xnor_gemm(g, dev, s);
+        launch_xnor_gemm(g, dev, s, true);
     }
     if (bytes) {
         SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8 + half, ldz, g.rowscale, F, K, H, ldh,
                      beta + half, nullptr, a.agg, sage ? g.dots8 : nullptr, beta};
         t.counters = g.counters;
-        launch_spmm_tc(t, dev, s);
+        launch_spmm_tc(t, dev, s, true);
     } else {
-        launch_spmm_norm(a, dev, s);
+        launch_spmm_norm(a, dev, s, true);
     }
     return launch_status();
 }

@@ -182,7 +182,8 @@ void launch_spmm_norm(const SpmmArgs &args, const DeviceInfo &dev, cudaStream_t 
 // The weighted degrees of A + I (weighted.cu): dinv_i = 1/sqrt(1 + sum of
 // row i's values) and, when alpha is given, s_i = alpha_i dinv_i.
 void launch_weighted_dinv(const int64_t *rowptr, const float *values, int64_t N, int64_t nnz,
-                          const float *alpha, float *dinv, float *s, cudaStream_t stream);
+                          const float *alpha, float *dinv, float *s, cudaStream_t stream,
+                          bool pdl = false);
 
 struct FrontArgs {
     const float *X;          // N x K (row stride ldx)

@@ -198,6 +198,10 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
         front_split_supported(N, K, F, dev) || (small && front_supported(N, K, F, dev));
     const bool bytes = w.planes && planes_faster(N, nnz, F) &&
                        (fused || xnor_gemm_bytes_supported(N, K, F, dev));
+    // Without events between them every kernel after the weights' packing may start
+    // while the one before it drains (each waits for it before it reads anything
+    // the call has written): 1001 nodes, K = 203, F = 19, 18.5 -> 18.0 us a call.
+    const bool pdl = n_events == 0;
     marks.mark();
     if (!fused) launch_pack_rows(X, N, K, ldx, scale, shift, a_bits, words, alpha, dev, s);
     marks.mark();
@@ -233,17 +237,17 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
                      g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8};
         fr.counters = g.counters;
         fr.n_counters = kTcCounters;
-        launch_front(fr, dev, s);
+        launch_front(fr, dev, s, pdl);
     } else {
-        launch_xnor_gemm(g, dev, s);
+        launch_xnor_gemm(g, dev, s, pdl);
     }
     marks.mark();
     if (bytes) {        // byte planes: the aggregation on the tensor cores
         SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, w.ldd8, g.rowscale, F, K, H, ldh, beta, nullptr};
         t.counters = g.counters;
-        launch_spmm_tc(t, dev, s);
+        launch_spmm_tc(t, dev, s, pdl);
     } else {
-        launch_spmm_norm(a, dev, s);
+        launch_spmm_norm(a, dev, s, pdl);
     }
     marks.mark();
     const bigcn_status ls = launch_status();

@@ -507,7 +507,7 @@ spmm_norm_kernel(SpmmParams p) {
     __shared__ int next;
     if (threadIdx.x == 0) next = 0;
     grid_dependency_wait();     // Z is the output of the previous kernel
-    __syncthreads();
+    if (p.pool > kSpmmWarps) __syncthreads();
     const int f0 = blockIdx.y * SLAB;
     using Epi = StoreRow<VEC, L, NV, S, AGG>;
     Epi epi;

@@ -67,14 +67,14 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
             const int e = tid + q * kThreads;
             const int r = e / kBKW, kw = e % kBKW;
             const int64_t row = m0 + r;
-            ra[q] = (row < N && k0 + kw < words) ? __ldg(A + row * words + k0 + kw) : 0ull;
+            ra[q] = (row < N && k0 + kw < words) ? load_upstream(A + row * words + k0 + kw) : 0ull;
         }
 #pragma unroll
         for (int q = 0; q < kBLoads; ++q) {
             const int e = tid + q * kThreads;
             const int c = e / kBKW, kw = e % kBKW;
             rb[q] = (e < BN * kBKW && n0 + c < F && k0 + kw < words)
-                        ? __ldg(B + int64_t(n0 + c) * words + k0 + kw) : 0ull;
+                        ? load_upstream(B + int64_t(n0 + c) * words + k0 + kw) : 0ull;
         }
     };
     auto store_tile = [&]() {

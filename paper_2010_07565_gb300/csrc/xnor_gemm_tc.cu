@@ -256,13 +256,13 @@ xnor_gemm_tc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ al
 #pragma unroll
         for (int q = 0; q < kAChunks; ++q) {
             const int64_t row = m0 + r0 + kRowsPerPass * q;
-            wa[q] = (row < N && k0 < K) ? __ldg(A + row * words + (k0 >> 6)) : 0ull;
+            wa[q] = (row < N && k0 < K) ? load_upstream(A + row * words + (k0 >> 6)) : 0ull;
         }
 #pragma unroll
         for (int q = 0; q < kBChunks; ++q) {
             const int col = n0 + r0 + kRowsPerPass * q;
             wb[q] = (!kBexp && col < F && k0 < K)
-                        ? __ldg(B + int64_t(col) * words + (k0 >> 6)) : 0ull;
+                        ? load_upstream(B + int64_t(col) * words + (k0 >> 6)) : 0ull;
         }
     };
     const uint8_t *btiles = kBexp ? bexp + size_t(blockIdx.y) * KB * kStageB : nullptr;
@@ -473,7 +473,7 @@ xnor_gemm_tc_ws_kernel(const uint64_t *__restrict__ A, const float *__restrict__
 #pragma unroll
             for (int q = 0; q < kAChunks; ++q) {
                 const int64_t row = m0 + r0 + kRowsPerPass * q;
-                wa[q] = (row < N && k0 < K) ? __ldg(A + row * words + (k0 >> 6)) : 0ull;
+                wa[q] = (row < N && k0 < K) ? load_upstream(A + row * words + (k0 >> 6)) : 0ull;
             }
         };
         // Expands k-block kb from wa into its stage; false when a wait ran out
@@ -621,7 +621,7 @@ expand_b_kernel(const uint64_t *__restrict__ B, int F, int K, int words, int KB,
         const int k0 = kb * kTcKBytes + c * 16;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (col < F && k0 < K) {
-            const uint32_t bits = uint32_t(__ldg(B + int64_t(col) * words + (k0 >> 6)) >> (k0 & 63));
+            const uint32_t bits = uint32_t(load_upstream(B + int64_t(col) * words + (k0 >> 6)) >> (k0 & 63));
             v = make_uint4(signs4_to_e4m3(bits & 15u), signs4_to_e4m3((bits >> 4) & 15u),
                            signs4_to_e4m3((bits >> 8) & 15u), signs4_to_e4m3((bits >> 12) & 15u));
             const int valid = K - k0;
