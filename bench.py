@@ -124,12 +124,14 @@ def tensor_core_aggregation(w):
 
 def z_rows(w):
     """Bytes per node of layer 1's and layer 2's factored products as the
-    forward keeps them (dot rows + row scale): fp16 dots in rows padded to 16
-    on the tensor-core path; else uint16 dots (rows padded to 8) or fp32 for
-    layer 1 and fp32 rows padded to 4 for layer 2."""
+    forward keeps them (dot rows + row scale): byte dots in rows padded to 16
+    on the tensor-core path (layer 2's row scale inside the padding where it
+    has room); else uint16 dots (rows padded to 8) or fp32 for layer 1 and fp32
+    rows padded to 4 for layer 2."""
     K, Fh, Fo = w.K, w.hidden, w.out
     if tensor_core_aggregation(w):
-        return 2.0 * ((Fh + 15) // 16 * 16) + 4.0, 2.0 * ((Fo + 15) // 16 * 16) + 4.0
+        Fo16 = (Fo + 15) // 16 * 16
+        return float((Fh + 15) // 16 * 16) + 4.0, Fo16 + (0.0 if Fo16 - Fo >= 4 else 4.0)
     z1 = 2.0 * ((Fh + 7) // 8 * 8) + 4.0 if K <= 32767 else 4.0 * Fh
     return z1, 4.0 * ((Fo + 3) // 4 * 4)
 
@@ -160,12 +162,12 @@ def kernel_work(w, nnz, name):
 
 def workload_bytes(w, nnz):
     """Bytes a 2-layer forward touches: the features, the CSR, both weight
-    matrices, both layers' factored products (16-bit dots and a row scale)
+    matrices, both layers' factored products (byte dots and a row scale)
     and the logits."""
     pad16 = lambda f: (f + 15) // 16 * 16
     return (4.0 * w.N * w.K + 8.0 * (w.N + 1) + 4.0 * nnz + 4.0 * w.K * w.hidden +
-            4.0 * w.hidden * w.out + w.N * (2.0 * pad16(w.hidden) + 4.0) +
-            w.N * (2.0 * pad16(w.out) + 4.0) + 4.0 * w.N * w.out)
+            4.0 * w.hidden * w.out + w.N * (1.0 * pad16(w.hidden) + 4.0) +
+            w.N * (1.0 * pad16(w.out) + 4.0) + 4.0 * w.N * w.out)
 
 
 def kernel_bitops(w, name):
@@ -186,9 +188,9 @@ KERNEL_FILES = {"pack_rows": "pack.cu", "pack_weights": "pack.cu", "xnor_gemm": 
 
 
 def sweep_tensor_core_aggregation(w):
-    """The one-layer entry points keep fp16 dots and aggregate on the tensor
-    cores for K <= 2048 and F <= 128 (csrc/layer.cu)."""
-    return w.K <= 2048 and w.hidden <= 128
+    """At the sweep's size the layer keeps byte dots and aggregates on the tensor
+    cores for K <= 3072 (csrc/layer.cu)."""
+    return w.K <= 3072
 
 
 def kernel_file(name, w=None):
@@ -259,10 +261,10 @@ def profile_file_traffic(fname, files):
 
 INDUCTIVE_SOURCES = {
     "gcn": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "layer.cu", "spmm_tc.cu"],
-    "mean": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm.cu"],
-    "sage": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm.cu"]}
+    "mean": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm_tc.cu"],
+    "sage": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm_tc.cu"]}
 BACKWARD_SOURCES = ["backward.cu", "pack.cu", "spmm.cu", "ablation.cu"]
-WEIGHTED_SOURCES = ["weighted.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm.cu"]
+WEIGHTED_SOURCES = ["weighted.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm_tc.cu"]
 
 
 class ClockSampler:
@@ -716,10 +718,10 @@ def run_sweep(args, rank, world, local_rank):
     hbm = float(peaks.get("hbm_gbs", FALLBACK_HBM_GBS))
     mean_us = [1e3 * statistics.fmean(t) for t in per_kernel]
     words = (K + 63) // 64
-    # The layer keeps Z factored when K <= 32767: fp16 dots in rows padded to
-    # 16 (K <= 2048, F <= 128) or uint16 dots in rows padded to 8, plus a row scale.
+    # The layer keeps Z factored when K <= 32767: byte dots in rows padded to
+    # 16 (K <= 3072) or uint16 dots in rows padded to 8, plus a row scale.
     if sweep_tensor_core_aggregation(w):
-        z_bytes = 2.0 * N * ((F + 15) // 16 * 16) + 4.0 * N
+        z_bytes = 1.0 * N * ((F + 15) // 16 * 16) + 4.0 * N
     elif K <= 32767:
         z_bytes = 2.0 * N * ((F + 7) // 8 * 8) + 4.0 * N
     else:
@@ -1040,8 +1042,10 @@ def run_inductive(args, rank, world, local_rank):
     peaks, peak_kind = load_peaks()
     hbm = float(peaks.get("hbm_gbs", FALLBACK_HBM_GBS))
     words = (K + 63) // 64
-    Fz = 2 * ((F + 7) // 8 * 8) if agg == "sage" else (F + 7) // 8 * 8
-    zrow = 2.0 * Fz + 4.0 if K <= 32767 else 4.0 * Fz
+    planes = K <= 3072 and F <= 128         # byte dots, else uint16
+    Fp = (F + 15) // 16 * 16 if planes else (F + 7) // 8 * 8
+    Fz = 2 * Fp if agg == "sage" else Fp
+    zrow = 1.0 * Fz + 4.0 if planes else 2.0 * Fz + 4.0 if K <= 32767 else 4.0 * Fz
     layer_bytes = (4.0 * N * K + 2 * 8.0 * N * words + 2.0 * N * zrow + 8.0 * (N + 1) +
                    4.0 * nnz + 4.0 * N * F)
     mean_ms = max_ms / args.steps
@@ -1128,8 +1132,9 @@ def run_weighted(args, rank, world, local_rank):
     peaks, peak_kind = load_peaks()
     hbm = float(peaks.get("hbm_gbs", FALLBACK_HBM_GBS))
     words = (K + 63) // 64
-    Fz = (F + 7) // 8 * 8
-    zrow = 2.0 * Fz + 4.0 if K <= 32767 else 4.0 * Fz
+    planes = K <= 3072 and F <= 128         # byte dots, else uint16
+    Fz = (F + 15) // 16 * 16 if planes else (F + 7) // 8 * 8
+    zrow = 1.0 * Fz + 4.0 if planes else 2.0 * Fz + 4.0 if K <= 32767 else 4.0 * Fz
     layer_bytes = (4.0 * N * K + 2 * 8.0 * N * words + 2.0 * N * zrow + 2 * 8.0 * (N + 1) +
                    4.0 * nnz + 2 * 4.0 * nnz + 4 * 4.0 * N + 4.0 * N * F)
     mean_ms = max_ms / args.steps
