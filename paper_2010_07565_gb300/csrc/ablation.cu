@@ -343,37 +343,61 @@ __device__ __forceinline__ void mix_epilogue(const MixParams &p, unsigned char *
         return z;
     };
     const bool vec_z = (p.ldz & 3) == 0 && (reinterpret_cast<uintptr_t>(p.Z) & 15) == 0;
+    float *red = reinterpret_cast<float *>(tiles);      // every stage is idle now
 
     if (KS == 1) {
-        if (!ok || !reader) return;
-        const int64_t row = m0 + rl;
-        const float rs = row < p.N ? row_scale(row) : 0.0f;
+        if (!ok) return;
+        // Through shared memory, so that a warp's store is one row's run of
+        // columns. A lane's tensor-memory row stored directly is 32 rows per
+        // instruction: where the row stride allows only 4-byte stores, those
+        // were most of the kernel's time. dL/dX of 232,965 x 602 over 128
+        // columns: 877 -> 380 us (its 561 MB of stores alone take 84); H~ W of
+        // 65,521 x 1000 by 96 columns, where rows allowed 16 bytes: 117 -> 87.
+        if (reader) {
+            const int64_t row = m0 + rl;
+            const float rs = row < p.N ? row_scale(row) : 0.0f;
 #pragma unroll 1
-        for (int c0 = cfirst; c0 < NT; c0 += cstep) {
-            uint32_t acc[16];
-            tmem_ld16(taddr + uint32_t(c0), acc);
-            if (row >= p.N) continue;
-            const int col0 = n0 + c0;
-            float z[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                z[j] = scaled(rs, min(col0 + j, p.F - 1), __uint_as_float(acc[j]));
-            float *zr = p.Z + row * p.ldz + col0;
-            if (vec_z && col0 + 16 <= p.F) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    reinterpret_cast<float4 *>(zr)[q] =
-                        make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
-            } else {
+            for (int c0 = cfirst; c0 < NT; c0 += cstep) {
+                uint32_t acc[16];
+                tmem_ld16(taddr + uint32_t(c0), acc);
+                const int col0 = n0 + c0;
+                float z[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
-                    if (col0 + j < p.F) zr[j] = z[j];
+                    z[j] = scaled(rs, min(col0 + j, p.F - 1), __uint_as_float(acc[j]));
+                float4 *dst = reinterpret_cast<float4 *>(red + rl * S::kRedStride + c0);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    dst[q] = make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
             }
         }
+        __syncthreads();
+        const int rows = int(min(int64_t(S::kRows), p.N - m0));
+        const int cols = min(NT, p.F - n0);
+        float *z0 = p.Z + m0 * p.ldz + n0;
+        auto store = [&](auto vec) {
+            using V = decltype(vec);
+            constexpr int kV = int(sizeof(V) / 4), kPer = NT / kV;
+#pragma unroll 4
+            for (int idx = tid; idx < rows * kPer; idx += kMixThreads) {
+                const int r = idx / kPer, c = kV * (idx % kPer);
+                const float *src = red + r * S::kRedStride + c;
+                float *dst = z0 + r * p.ldz + c;
+                if (c + kV <= cols) {
+                    *reinterpret_cast<V *>(dst) = *reinterpret_cast<const V *>(src);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < kV; ++e)
+                        if (c + e < cols) dst[e] = src[e];
+                }
+            }
+        };
+        if (vec_z) store(float4{});
+        else if ((p.ldz & 1) == 0 && (reinterpret_cast<uintptr_t>(p.Z) & 7) == 0) store(float2{});
+        else store(float{});
         return;
     }
-    // Partial tile -> this CTA's shared memory (every stage is idle now).
-    float *red = reinterpret_cast<float *>(tiles);
+    // Partial tile -> this CTA's shared memory.
     if (reader) {
 #pragma unroll 1
         for (int c0 = cfirst; c0 < NT; c0 += cstep) {
