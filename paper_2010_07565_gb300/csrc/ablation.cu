@@ -757,10 +757,11 @@ binary_real_tc_kernel(const MixParams p) {
 // contraction over nodes in k-blocks of 64, split over S CTAs (grid z) that
 // each write a fp32 partial; the partials are added in order afterwards.
 // A (K-major: a row per feature, 64 nodes along it) is built from the nodes'
-// packed words: a producer warp takes 32 consecutive features of one 8-node
-// chunk, so its eight word loads are broadcasts, and gathers bit k of each
-// node into a byte of signs. B holds alpha_i G_ij (rounded once) as three
-// bf16 parts, read coalesced across the columns. Warp roles and barriers are
+// packed words: a producer warp takes two groups of 32 features of one 8-node
+// chunk; its lanes load one 32-bit word each (8 nodes x 2 groups, and the 8
+// nodes' alphas), and a shuffle per node gives each lane bit k of that node.
+// B holds alpha_i G_ij (rounded once) as three bf16 parts, read coalesced
+// across the columns. Warp roles and barriers are
 // those of the ablation products.
 template <int NT>
 struct SignTShape {
@@ -819,49 +820,77 @@ sign_t_real_tc_kernel(const SignTParams p) {
                              (it > 0 || k > 0 || part > 0) ? 1u : 0u);
         });
     } else {
+        constexpr int kBTasks = NT / 64;
+        const int c = warp & 7, half = (warp >> 3) & 1;
+        // One k-block's inputs, in flight while the stage before is taken and this
+        // one is waited for; with the loads behind the wait, and sixteen 64-bit
+        // broadcasts a warp for the signs, the latency of 90 k-blocks in series
+        // was most of the time (232,965 nodes, 602 x 128: 514 -> 205 us; the three
+        // parts' products alone are 57 us of tensor time on 130 SMs). Lane l < 16
+        // holds half `half` of word m0 / 64 + (l >> 3) of node 8c + (l & 7),
+        // lane 16 + e that node's alpha; g the columns of G.
+        uint32_t small = 0u;
+        float g[kBTasks][8];
+        auto load = [&](int64_t kb) {
+            const int64_t i0 = kb * kMixK + 8 * c;
+            const int64_t i = i0 + (lane & 7);
+            small = 0u;
+            if (i < p.N) {
+                const int wi = m0 / 64 + (lane >> 3);
+                if (lane < 16) {
+                    if (wi < p.words)
+                        small = __ldg(reinterpret_cast<const uint32_t *>(p.bits + i * p.words + wi) +
+                                      half);
+                } else if (lane < 24) {
+                    small = __float_as_uint(__ldg(p.alpha + i));
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kBTasks; ++q) {
+                const int j = n0 + 32 * (half + 2 * q) + lane;
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    g[q][e] = (i0 + e < p.N && j < p.F) ? __ldg(p.G + (i0 + e) * p.ldg + j) : 0.0f;
+            }
+        };
+        if (kb0 < kb1) load(kb0);
 #pragma unroll 1
         for (int64_t kb = kb0; kb < kb1; ++kb) {
             const int it = int(kb - kb0);
             const int s = it % kStages;
-            if (it >= kStages &&
-                !wait_or_abort(smem_addr(&sy.empty[s]), uint32_t(it / kStages - 1) & 1u,
-                               &sy.abort)) {
+            // One answer for the warp: its lanes shuffle below.
+            const bool free_stage =
+                it < kStages || wait_or_abort(smem_addr(&sy.empty[s]),
+                                              uint32_t(it / kStages - 1) & 1u, &sy.abort);
+            if (!__all_sync(0xFFFFFFFFu, free_stage)) {
                 sy.abort = 1u;
                 break;
             }
             unsigned char *sa = tiles + s * S::kStage;
             unsigned char *sb = sa + S::kTileA;
-            const int64_t i0 = kb * kMixK;
-            // A: 4 x 8 (feature group, node chunk) tasks of 32 features x 8 nodes.
-            for (int t = warp; t < 32; t += kProducerWarps) {
-                const int c = t & 7, mh = t >> 3;
-                const int m = 32 * mh + lane, f = m0 + m;
-                const int wi = (m0 + 32 * mh) / 64;          // the same word for the warp
+            // A: feature groups half and half + 2 of the node chunk, a feature per lane.
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
                 uint32_t byte = 0;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int64_t i = i0 + 8 * c + e;
-                    const uint64_t w =
-                        (i < p.N && wi < p.words) ? __ldg(p.bits + i * p.words + wi) : 0ull;
-                    byte |= uint32_t((w >> (f & 63)) & 1ull) << e;
-                }
-                *reinterpret_cast<uint4 *>(sa + sw128_offset(m, c)) = signs8_to_bf16(byte);
+                for (int e = 0; e < 8; ++e)
+                    byte |= ((__shfl_sync(0xFFFFFFFFu, small, 8 * q + e) >> lane) & 1u) << e;
+                *reinterpret_cast<uint4 *>(sa + sw128_offset(32 * (half + 2 * q) + lane, c)) =
+                    signs8_to_bf16(byte);
             }
-            // B: (NT / 32) x 8 (column group, node chunk) tasks of 32 columns x 8 nodes.
-            for (int t = warp; t < (NT / 32) * 8; t += kProducerWarps) {
-                const int c = t & 7, jh = t >> 3;
-                const int r = 32 * jh + lane, j = n0 + r;
-                float v[8];
+            // B: column groups half, half + 2, ..., a column per lane.
+            float al[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int64_t i = i0 + 8 * c + e;
-                    v[e] = (i < p.N && j < p.F) ? __ldg(p.alpha + i) * __ldg(p.G + i * p.ldg + j)
-                                                : 0.0f;
-                }
+            for (int e = 0; e < 8; ++e)
+                al[e] = __uint_as_float(__shfl_sync(0xFFFFFFFFu, small, 16 + e));
+#pragma unroll
+            for (int q = 0; q < kBTasks; ++q) {
                 uint32_t h[4], mi[4], lo[4];
 #pragma unroll
-                for (int w = 0; w < 4; ++w) split3x2(v[2 * w], v[2 * w + 1], h[w], mi[w], lo[w]);
-                const uint32_t off = sw128_offset(r, c);
+                for (int w = 0; w < 4; ++w)
+                    split3x2(al[2 * w] * g[q][2 * w], al[2 * w + 1] * g[q][2 * w + 1], h[w], mi[w],
+                             lo[w]);
+                const uint32_t off = sw128_offset(32 * (half + 2 * q) + lane, c);
                 *reinterpret_cast<uint4 *>(sb + off) = make_uint4(h[0], h[1], h[2], h[3]);
                 *reinterpret_cast<uint4 *>(sb + S::kTileB + off) =
                     make_uint4(mi[0], mi[1], mi[2], mi[3]);
@@ -870,6 +899,7 @@ sign_t_real_tc_kernel(const SignTParams p) {
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive(smem_addr(&sy.full[s]));
+            if (kb + 1 < kb1) load(kb + 1);
         }
     }
     // The last MMA is done once `done` completes; then warps 0-15 move the

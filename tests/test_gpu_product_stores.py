@@ -1,5 +1,6 @@
 """GPU: the stores of the ablation products' unsplit tiles (one k-block, so no
-cluster split) at every store width.
+cluster split) at every store width, and the weight gradient's contraction over
+nodes at the edges of its tiles.
 """
 import numpy as np
 import pytest
@@ -55,4 +56,26 @@ def test_unsplit_tiles_store_their_rows(cuda_device, N, F, ldz, skip):
     check(Z.cpu().numpy(), ref, mag, f"H~ W {N}x{F} stride {ldz}", nterms=K)
     rows = buf[skip:].view(N, ldz)
     assert torch.all(buf[:skip] == -7.0) and torch.all(rows[:, F:] == -7.0)
+    assert B.device_timeouts() == 0
+
+
+# Nodes, features and columns at and one past their tiles of 64, 128 and 64 to 256.
+GRADIENTS = [(63, 64, 64), (65, 65, 65), (193, 129, 129), (128, 31, 257), (4097, 97, 128)]
+
+
+@pytest.mark.parametrize("N,K,F", GRADIENTS)
+def test_weight_gradient_at_tile_edges(cuda_device, N, K, F):
+    case = inputs.layer_case(N, K, F, seed=N + K, mean_degree=3.0, hub_degree=0)
+    dH = np.random.Generator(np.random.PCG64(F)).standard_normal((N, F)).astype(np.float32)
+    d = {k: to_dev(v) for k, v in case.items()}
+    ws = torch.empty(B.bigcn_layer_backward_workspace_bytes(N, K, F), dtype=torch.uint8,
+                     device=cuda_device)
+    dW = torch.full((K, F), float("nan"), device=cuda_device)
+    B.bigcn_layer_backward(d["X"], d["s"], d["t"], d["W"], d["rowptr"], d["colidx"], to_dev(dH),
+                           ws, dW)
+    torch.cuda.synchronize()
+    ref = oracle.layer_backward(case["X"], case["W"], case["rowptr"], case["colidx"],
+                                dH.astype(np.float64), case["s"], case["t"])
+    scale = np.broadcast_to(ref["Wg_abs"] * (1.0 + ref["beta"]), dW.shape)
+    check(dW.cpu().numpy().astype(np.float64), ref["dW"], scale, f"dW {N}x{K}x{F}", nterms=N + K)
     assert B.device_timeouts() == 0
