@@ -11,9 +11,10 @@
 // fills the GPU even when N is small) share a row, warp g taking chunks
 // g, g + G, ...; each warp issues eight chunks' loads (1 KB) before it
 // consumes any, and the grids are persistent. The whole-row kernel has no block
-// barrier; on many rows a warp packs four together (pack_group), which keeps more
-// loads in flight than full occupancy with one row each. The G partial |y| sums are added in a fixed order through
-// shared memory, so alpha does not depend on scheduling.
+// barrier; on many rows a warp packs two or four together (pack_group), which
+// keeps more loads in flight than full occupancy with one row each. The G
+// partial |y| sums are added in a fixed order through shared memory, so alpha
+// does not depend on scheduling.
 //
 // pack_weights reads W (K x F) column-wise: thread (x, y) of a 32 x 8 block
 // owns one column and builds whole 64-bit words from 64 coalesced row reads,
@@ -46,22 +47,29 @@ pack_rows_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
                  const float *__restrict__ scale, const float *__restrict__ shift,
                  uint32_t *__restrict__ bits32, int64_t ld32, float *__restrict__ alpha) {
     if (kUpstream) grid_dependency_wait();      // X is the previous kernel's output
-    constexpr Affine kA = kAffine ? Affine::kGlobal : Affine::kNone;
     const int lane = threadIdx.x & 31;
     const int64_t step = int64_t(gridDim.x) * kPackWarps * R;
     for (int64_t row = (int64_t(blockIdx.x) * kPackWarps + (threadIdx.x >> 5)) * R; row < N;
          row += step) {
-        float l1[R];
-        const int rows = int(min(N - row, int64_t(R)));
-        pack_group<R, C, kA>(X + row * ldx, ldx, rows, K, scale, shift, bits32 + row * ld32, ld32,
-                             ld32, l1);
-        float mine = 0.0f;
+        if constexpr (R == 1) {
+            constexpr Affine kLate = kAffine ? Affine::kGlobalLate : Affine::kNone;
+            const float l1 = pack_share<1, C, kLate>(X + row * ldx, K, scale, shift, nullptr,
+                                                     bits32 + row * ld32, ld32, 0);
+            if (lane == 0) alpha[row] = l1 / float(K);
+        } else {
+            constexpr Affine kA = kAffine ? Affine::kGlobal : Affine::kNone;
+            float l1[R];
+            const int rows = int(min(N - row, int64_t(R)));
+            pack_group<R, C, kA>(X + row * ldx, ldx, rows, K, scale, shift, bits32 + row * ld32,
+                                 ld32, ld32, l1);
+            float mine = 0.0f;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float s = warp_sum(l1[r]);
-            if (lane == r) mine = s;
+            for (int r = 0; r < R; ++r) {
+                const float s = warp_sum(l1[r]);
+                if (lane == r) mine = s;
+            }
+            if (lane < rows) alpha[row + lane] = mine / float(K);
         }
-        if (lane < rows) alpha[row + lane] = mine / float(K);
     }
     // Otherwise wait only now: finishing after the predecessor keeps the
     // chain's completion order for the kernels that follow.
@@ -167,6 +175,13 @@ pack_weights_kernel(WeightPack a, WeightPack b) {
 constexpr int kManyR = 4;
 constexpr int kManyBlocks = 4;
 constexpr int kLongK = 2048;
+// Fewer rows than that, but two for each of those warps: two rows together
+// (11,000 x 3000: 38.0 -> 32.2 us; 17,330 x 2354: 42.0 -> 33.3, where four leave a
+// second round of few warps, 36.9; 19,400 x 600: 18.4 -> 15.1; 12,000 x 128: 8.5
+// -> 7.9). Fewer still go one to a warp through pack_share, which spends a third
+// fewer instructions on one row than pack_group does (17,330 x 2354: 42.0 against
+// 56.0).
+constexpr int kPairR = 2;
 
 }  // namespace
 
@@ -181,9 +196,12 @@ void launch_pack_rows(const float *X, int64_t N, int K, int64_t ldx, const float
     int G = 1;
     while (G < kPackWarps && N * G < full_wave && nchunks >= 2 * G * 8) G *= 2;
     const bool many = N >= int64_t(kManyR) * dev.sm_count * kManyBlocks * kPackWarps;
-    const int rows_per_block = G > 1 ? kPackWarps / G : many ? kPackWarps * kManyR : kPackWarps;
+    const bool pairs =
+        G == 1 && !many && N >= int64_t(kPairR) * dev.sm_count * kManyBlocks * kPackWarps;
+    const int per_warp = many ? kManyR : pairs ? kPairR : 1;
+    const int rows_per_block = G > 1 ? kPackWarps / G : kPackWarps * per_warp;
     const int64_t groups = (N + rows_per_block - 1) / rows_per_block;
-    const int per_sm = G > 1 || !many ? kPackBlocksPerSM : K >= kLongK ? 3 : kManyBlocks;
+    const int per_sm = many && K >= kLongK ? 3 : many || pairs ? kManyBlocks : kPackBlocksPerSM;
     const int64_t resident = int64_t(dev.sm_count) * per_sm;
     const dim3 grid(unsigned(groups < resident ? groups : resident)), block(kPackThreads), one(1, 1, 1);
     uint32_t *b32 = reinterpret_cast<uint32_t *>(bits);
@@ -203,6 +221,8 @@ void launch_pack_rows(const float *X, int64_t N, int K, int64_t ldx, const float
             BIGCN_PACK_CASE(kManyR, 8, 3)
         } else if (many) {
             BIGCN_PACK_CASE(kManyR, 4, kManyBlocks)
+        } else if (pairs) {
+            BIGCN_PACK_CASE(kPairR, 8, kManyBlocks)
         } else {
             BIGCN_PACK_CASE(1, kPackUnroll, kPackBlocksPerSM)
         }
