@@ -265,7 +265,7 @@ __device__ __forceinline__ void gather(const SpmmParams &p, int64_t i, int64_t b
             for (int t = 0; t < 32; t += P * U) whole(t);
             continue;
         }
-        if (valid == (1u << cnt) - 1u)
+        if (valid == kFullMask >> (32 - cnt))      // (1 <= cnt <= 32)
             for (; t0 + P * U <= cnt; t0 += P * U) whole(t0);
         for (; t0 < cnt; t0 += P * U) {
             V val[U][NV];
