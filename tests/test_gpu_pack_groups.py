@@ -34,3 +34,18 @@ def test_rows_packed_together(cuda_device, together, extra, K, centred):
     assert not got[:, -1].any()
     # K fp32 roundings of a sum of non-negative terms, and the division's.
     assert np.allclose(alpha.cpu().numpy(), oracle.row_scale(Y), rtol=(K + 2) * 2.0 ** -24, atol=0)
+
+
+@pytest.mark.parametrize("together", [1, 2, 4])
+@pytest.mark.parametrize("K,words", [(64, 2), (33, 18), (65, 40), (300, 64)])
+def test_rows_longer_than_their_signs(cuda_device, together, K, words):
+    """Words past the signs are written as zeros however many a row has."""
+    N = together * PER_ROW * torch.cuda.get_device_properties(0).multi_processor_count + 3
+    X = np.random.default_rng(K).standard_normal((N, K)).astype(np.float32)
+    bits = torch.full((N, words), -1, dtype=torch.int64, device=cuda_device)
+    alpha = torch.full((N,), float("nan"), device=cuda_device)
+    B.bigcn_pack_rows(to_dev(X), None, None, bits, alpha)
+    got = bits.cpu().numpy().view(np.uint64)
+    n = (K + 63) // 64
+    assert np.array_equal(got[:, :n], np.asarray(oracle.pack(oracle.sign(X))).view(np.uint64))
+    assert not got[:, n:].any()
