@@ -347,7 +347,10 @@ struct TcSums {
 __device__ __forceinline__ void put_weight(uint16_t *halves, float ws) {
     const int lane = threadIdx.x & 31;
     const __half hi = __float2half_rn(ws);
-    const __half lo = __float2half_rn(ws - __half2float(hi));
+    const float h = __half2float(hi);
+    // (an infinite weight has no low part: Inf - Inf would make its row NaN in every
+    // column, where Inf times a dot is Inf of the dot's sign)
+    const __half lo = __float2half_rn(ws == h ? 0.0f : ws - h);
     const int at = ((lane >> 1) & 3) * 8 + (lane >> 3) * 2 + (lane & 1);
     halves[at] = __half_as_ushort(hi);
     halves[EB + at] = __half_as_ushort(lo);

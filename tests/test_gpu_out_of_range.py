@@ -34,19 +34,16 @@ def bad_graph(N, seed):
     return rp, ci, (ci >= 0) & (ci < N)
 
 
-def reference(rp, ci, good, Z, values=None):
+def reference(rp, ci, good, Z):
     """D^-1/2 (A + I) D^-1/2 Z without the bad entries, degrees with them; and the
     sums of the terms' magnitudes."""
     N = len(rp) - 1
     row = np.repeat(np.arange(N), np.diff(rp))
-    v = np.ones(len(ci)) if values is None else values.astype(np.float64)
-    deg = 1.0 + (np.diff(rp) if values is None
-                 else np.add.reduceat(np.append(v, 0.0), rp[:-1]) * (np.diff(rp) > 0))
-    d = 1.0 / np.sqrt(deg)
+    d = 1.0 / np.sqrt(1.0 + np.diff(rp))
     out = []
     for z in (Z * d[:, None], np.abs(Z) * d[:, None]):
         s = z.copy()
-        np.add.at(s, row[good], v[good, None] * z[ci[good]])
+        np.add.at(s, row[good], z[ci[good]])
         out.append(s * d[:, None])
     return out
 
