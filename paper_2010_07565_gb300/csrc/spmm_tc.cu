@@ -169,7 +169,7 @@ __device__ __forceinline__ uint32_t high_to_half2(uint32_t h) {
     return r;
 }
 
-// 2^e as a float for e in [-126, 127].
+// 2^e as a float for e in [-126, 127] (0 for -127).
 __device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) << 23); }
 
 // Unbiased exponent of a non-negative float's bits (-127 for zero and subnormals).
@@ -177,6 +177,17 @@ __device__ __forceinline__ int exponent_of(uint32_t bits) { return int(bits >> 2
 
 constexpr int kNoScale = -126;      // exponent of a row that has seen no weight yet
 constexpr int kDotShift = 10;       // the A operands are dots times 2^-10
+
+// A row whose largest weight has exponent E multiplies its weights by 2^unit_exponent(E)
+// (to just below 2^15, as far as a float's exponent goes: weights under 2^-113 stay
+// smaller), its sums by 2^back_exponent(E) in the end; a sum begun at E goes on at a
+// larger E2 times scale_change(E, E2) (0 where that is below fp32: the sum was made of
+// weights under 2^-126 of the new one).
+__device__ __forceinline__ int unit_exponent(int E) { return min(14 - E, 127); }
+__device__ __forceinline__ int back_exponent(int E) { return kDotShift - unit_exponent(E); }
+__device__ __forceinline__ float scale_change(int E, int E2) {
+    return exp2i(max(unit_exponent(E2) - unit_exponent(E), -127));
+}
 
 struct TcParams {
     const int64_t *rowptr;
@@ -413,11 +424,11 @@ __device__ __forceinline__ void fetch_first(const TcParams &P, const Window<ROWS
             c[b][u] = fetch_entry<ROWS, kW>(P, w, (b * SUB + u) * EB + lane);
 }
 
-// The row of a window (its scale's exponent E: see walk_window) as the weight 2^(14
-// - E) that its entries' scales are multiplied by; tg = the lane's row.
+// What the scales of a window's row are multiplied by (its exponent E: see
+// walk_window); tg = the lane's row.
 template <int ROWS>
 __device__ __forceinline__ float row_unit(int E, int tg) {
-    return exp2i(min(14 - (ROWS == 1 ? E : __shfl_sync(kFullMask, E, tg)), 127));
+    return exp2i(unit_exponent(ROWS == 1 ? E : __shfl_sync(kFullMask, E, tg)));
 }
 
 // Where lane (g, t) finds the positions of row g (its column of B) in an
@@ -630,7 +641,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
                 }
                 const int e = exponent_of(__reduce_max_sync(kFullMask, wb));
                 if (e > E) {            // keep the sums on the row's current scale
-                    const float f = exp2i(max(E - e, -126));
+                    const float f = scale_change(E, e);
                     acc.scale(f, f);
                     E = e;
                     bound = (uint32_t(E + 127) << 23) | 0x7fffffu;
@@ -653,7 +664,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
                     const int e = exponent_of(__reduce_max_sync(kFullMask, tg == r ? wb : 0u));
                     if ((lane & 7) == r) Enew = max(Enew, e);
                 }
-                const float f = exp2i(max(E - Enew, -126));
+                const float f = scale_change(E, Enew);
                 acc.scale(__shfl_sync(kFullMask, f, 2 * t), __shfl_sync(kFullMask, f, 2 * t + 1));
                 E = Enew;
             }
@@ -685,7 +696,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
     }
 
     if constexpr (ROWS == 1) {
-        const float back = exp2i(max(min(E - 14 + kDotShift, 127), -126));
+        const float back = exp2i(back_exponent(E));
 #pragma unroll
         for (int T = 0; T < FT; ++T) {
             out.v[0][T][0] = (acc.v[0][T][0] + acc.v[0][T][1]) * back;
@@ -695,7 +706,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int Er = __shfl_sync(kFullMask, E, 2 * t + r);
-            const float back = exp2i(max(min(Er - 14 + kDotShift, 127), -126));
+            const float back = exp2i(back_exponent(Er));
 #pragma unroll
             for (int T = 0; T < FT; ++T) {
                 constexpr int L = TcSums<FT, ROWS>::PARTS - 1;

@@ -93,3 +93,21 @@ def test_infinite_row_scale(cuda_device, agg, N, K, F, deg):
     assert np.array_equal(got[inf], ref[inf])
     ok = np.isfinite(ref)
     assert (np.abs(got[ok] - ref[ok]) <= 1e-5 * mag[ok] + 1e-30).all()
+
+
+@pytest.mark.parametrize("agg", AGGS)
+@pytest.mark.parametrize("N,K,F,deg", SHAPES)
+@pytest.mark.parametrize("powers", [[-35], [-36], [-33, -34, -35, -36, -37]])
+def test_tiny_row_scales(cuda_device, agg, N, K, F, deg, powers):
+    """Row scales so small that the weights' power-of-two scale ends at a float's largest
+    exponent (below 2^-113), alone and among larger ones that raise it."""
+    c, v, Wn = make(N, K, F, deg, agg, seed=N + F + len(powers))
+    p = np.asarray(powers)[np.arange(N) // 64 % len(powers)]
+    c["X"] = (c["X"] * 10.0 ** p[:, None]).astype(np.float32)
+    ref, mag = reference(c, agg, v, Wn)
+    got = run(c, agg, cuda_device, v, Wn)
+    # n additions, truncated (tensor cores) or rounded to 24 bits, and a few roundings of
+    # the scales; what lies below the normal range loses bits, 2^-149 at each step
+    n = np.diff(c["rowptr"]).max() + 8
+    bad = np.abs(got - ref) > n * (2.0 ** -23 * mag + 2.0 ** -149)
+    assert not bad.any(), (int(bad.sum()), got[bad][:4], ref[bad][:4])
