@@ -31,15 +31,20 @@
 // 2^-24, and one packed fma, u 2^-24 * 2^15 + ((K & 1) - 256) 2^-10, makes
 // them dot * 2^-10: every step exact, and no entry's value ever leaves fp16.
 // Rows marked wide add hi * 2^-1 (dot = 2 lo + (K & 1) + 512 hi) in a second
-// walk over the blocks that hold any, with the weights of the other entries
-// zero: as long as the first where every row is wide.
+// walk over the blocks that hold any (again_walk), with the weights of the other
+// entries zero: as long as the first where every row is wide.
 //
-// B carries the weights as two fp16 parts, hi = fp16(s' ) and lo = fp16(s' -
-// hi) with s' = s_j * 2^(14 - E) (an exact power-of-two scaling that puts the
-// row's largest weight just below 2^15), so the product keeps 22 bits of each
-// weight. E is the largest exponent among the weights seen so far for
+// B carries the weights as two fp16 parts, hi = fp16(s') and lo = fp16((s' - hi) 2^11)
+// with s' = s_j * 2^(14 - E) (an exact power-of-two scaling that puts the
+// row's largest weight just below 2^15), and lo's sums, kept apart, are multiplied by
+// 2^-11 in the end: together 23 bits or more of each weight down to 2^-24 of the
+// row's largest. E is the largest exponent among the weights seen so far for
 // that output row: when a later entry raises it, the row's accumulators are
-// multiplied by the exact power of two that keeps them consistent.
+// multiplied by the exact power of two that keeps them consistent. A window with
+// smaller weights than that (they decide the columns in which the large neighbours'
+// dots are zero) is walked again in bands of 2^24, each on a scale of its own
+// (again_walk): as good as fp32 multiply-adds at any ratio, at the cost of one more walk
+// per band.
 //
 // A warp takes a window of consecutive output rows whose lists (self entry
 // first, then the CSR neighbours) it walks as one stream of positions, 32 to a
@@ -175,18 +180,32 @@ __device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) 
 // Unbiased exponent of a non-negative float's bits (-127 for zero and subnormals).
 __device__ __forceinline__ int exponent_of(uint32_t bits) { return int(bits >> 23) - 127; }
 
-constexpr int kNoScale = -126;      // exponent of a row that has seen no weight yet
+constexpr int kNoScale = -127;      // exponent of a row that has seen no normal weight yet
 constexpr int kDotShift = 10;       // the A operands are dots times 2^-10
+constexpr int kLoShift = 11;        // lo parts are kept times 2^11, and so are their sums
+// Weights of a row from 2^kBandLow up (on its scale) are held to 2^-23 of themselves; a
+// row that has smaller ones takes them in bands, each 2^24 below the one before.
+constexpr int kBandLow = -10;
+constexpr int kBandStep = 24;
+// The first walk notes a weight's exponent where it lies this far below its row's: the
+// row's may then rise by as much again before what it did not note could need a band.
+constexpr int kLookBelow = 12;
 
-// A row whose largest weight has exponent E multiplies its weights by 2^unit_exponent(E)
-// (to just below 2^15, as far as a float's exponent goes: weights under 2^-113 stay
-// smaller), its sums by 2^back_exponent(E) in the end; a sum begun at E goes on at a
-// larger E2 times scale_change(E, E2) (0 where that is below fp32: the sum was made of
-// weights under 2^-126 of the new one).
+// A row whose largest weight has exponent E multiplies its weights by 2^u, u =
+// unit_exponent(E) (to just below 2^15, as far as a float's exponent goes: weights under
+// 2^-113 stay smaller), and its sums by 2^(kDotShift - u) in the end; a sum begun at E
+// goes on at a larger E2 times scale_change(E, E2) (0 where that is below fp32: the sum
+// was made of weights under 2^-126 of the new one).
 __device__ __forceinline__ int unit_exponent(int E) { return min(14 - E, 127); }
-__device__ __forceinline__ int back_exponent(int E) { return kDotShift - unit_exponent(E); }
 __device__ __forceinline__ float scale_change(int E, int E2) {
     return exp2i(max(unit_exponent(E2) - unit_exponent(E), -127));
+}
+// Unit exponent of band k of a row with unit exponent u, and the band of a weight of
+// exponent e: the first in which it reaches 2^kBandLow, or the last there is.
+__device__ __forceinline__ int band_unit(int u, int k) { return min(u + kBandStep * k, 127); }
+__device__ __forceinline__ int band_of(int e, int u) {
+    const int need = (kBandLow - e - u + kBandStep - 1) / kBandStep;
+    return e + u >= kBandLow ? 0 : min(need, (127 - u + kBandStep - 1) / kBandStep);
 }
 
 struct TcParams {
@@ -353,15 +372,16 @@ struct TcSums {
 };
 
 // A lane's weight on its row's scale as its two fp16 parts in shared memory (`halves`:
-// EB hi parts, then EB lo parts), entries 2t, 2t + 1, and those 8, 16 and 24 on,
+// EB hi parts, then EB lo parts times 2^kLoShift), entries 2t, 2t + 1, and those 8, 16 and 24 on,
 // next to one another, so that a lane's B fragments are one load.
 __device__ __forceinline__ void put_weight(uint16_t *halves, float ws) {
     const int lane = threadIdx.x & 31;
     const __half hi = __float2half_rn(ws);
-    const float h = __half2float(hi);
-    // (an infinite weight has no low part: Inf - Inf would make its row NaN in every
-    // column, where Inf times a dot is Inf of the dot's sign)
-    const __half lo = __float2half_rn(ws == h ? 0.0f : ws - h);
+    // (the limit, far below any difference, makes an infinite weight's low part finite:
+    // Inf - Inf would make its row NaN in every column, where Inf times a dot is Inf of
+    // the dot's sign)
+    const __half lo = __float2half_rn(
+        fmaxf((ws - __half2float(hi)) * float(1 << kLoShift), -32768.0f));
     const int at = ((lane >> 1) & 3) * 8 + (lane >> 3) * 2 + (lane & 1);
     halves[at] = __half_as_ushort(hi);
     halves[EB + at] = __half_as_ushort(lo);
@@ -424,13 +444,6 @@ __device__ __forceinline__ void fetch_first(const TcParams &P, const Window<ROWS
             c[b][u] = fetch_entry<ROWS, kW>(P, w, (b * SUB + u) * EB + lane);
 }
 
-// What the scales of a window's row are multiplied by (its exponent E: see
-// walk_window); tg = the lane's row.
-template <int ROWS>
-__device__ __forceinline__ float row_unit(int E, int tg) {
-    return exp2i(unit_exponent(ROWS == 1 ? E : __shfl_sync(kFullMask, E, tg)));
-}
-
 // Where lane (g, t) finds the positions of row g (its column of B) in an
 // eight-row window.
 template <int ROWS>
@@ -453,66 +466,137 @@ struct Column {
     }
 };
 
-// The second walk of a window that has wide rows: adds their high plane (weights
-// on the scales that the first walk ended with; other entries weigh nothing) for
-// the 32-position sub-blocks marked in `marks` (bit q: sub-blocks q << shift ..
-// ((q + 1) << shift) - 1). Two stages: the next sub-block's rows are copied
-// while one is multiplied. A function of its own, so that the first walk's
-// registers need not hold both.
-template <int FT, int ROWS, bool kW, class G>
-__device__ __noinline__ void high_walk(TcParams P, Window<ROWS> w, uint8_t *ring,
-                                       TcSums<FT, ROWS> &sums, int E, uint32_t marks, int shift) {
+// A window's sums as values, from band k of its rows' scales (unit exponents u: ROWS ==
+// 1 the row's, else lane r holds row r's); kAdd: added to `out`.
+template <bool kAdd, int FT, int ROWS>
+__device__ __forceinline__ void put_sums(const TcSums<FT, ROWS> &acc, int u, int k,
+                                         TcRowSums<FT, ROWS == 1 ? 1 : 2> &out) {
+    constexpr float kLo = 1.0f / float(1 << kLoShift);
+    constexpr int L = TcSums<FT, ROWS>::PARTS - 1;
+    const int t = threadIdx.x & 3;
+#pragma unroll
+    for (int r = 0; r < (ROWS == 1 ? 1 : 2); ++r) {
+        const int ur = ROWS == 1 ? u : __shfl_sync(kFullMask, u, 2 * t + r);
+        const float back = exp2i(kDotShift - band_unit(ur, k));
+        const int lo = ROWS == 1 ? 1 : r;       // columns 0 and 1, or one of each set
+#pragma unroll
+        for (int T = 0; T < FT; ++T)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float v =
+                    fmaf(acc.v[L][T][2 * h + lo], kLo, acc.v[0][T][2 * h + r]) * back;
+                out.v[r][T][h] = kAdd ? out.v[r][T][h] + v : v;
+            }
+    }
+}
+
+// What becomes of an eight-row window's results: kept for the caller.
+template <int FT>
+struct KeepSums {
+    TcRowSums<FT, 2> *sums;
+    __device__ __forceinline__ void operator()(const TcRowSums<FT, 2> &s) const { *sums = s; }
+};
+
+// What a window with wide rows or with weights far below their row's largest still
+// needs (rarely) after its first walk, which left `sums` and the exponents E. last == 0:
+// adds the wide rows' high plane in the 32-position sub-blocks marked in `marks` (bit q:
+// sub-blocks q << shift .. ((q + 1) << shift) - 1). last > 0: the whole window again, band
+// after band of its weights from `last` down to 0, the smallest first, each on its own
+// scale. The results go to emit().
+//
+// A pass walks the low plane, or the high plane for the wide rows; entries it does not
+// take weigh nothing and are not copied. Two stages: the next sub-block's rows are copied
+// while one is multiplied. A function of its own, which calls none and returns nothing:
+// the first walk's registers need not hold both, nor meet its results again (returning
+// the sums cost the walk of 128 features 3 % where no window came here).
+template <int FT, int ROWS, bool kW, class G, class Emit>
+__device__ __noinline__ void rest_of_window(TcParams P, Window<ROWS> w, uint8_t *ring,
+                                            TcSums<FT, ROWS> sums, int E, uint32_t marks,
+                                            int shift, int last, Emit emit) {
     const int lane = threadIdx.x & 31;
     const int piece = lane % G::P2, slab = int(blockIdx.y) * FT;
     const bool mine = piece < FT && (slab + piece) * 16 < P.width;
-    const uint8_t *plane = P.D + P.N * P.ldd + (slab + piece) * 16;
     const uint32_t tl =
         uint32_t(lane * G::PITCH) | uint32_t(((lane / G::LINE) & (G::P2 - 1)) << 4);
     int *checked = reinterpret_cast<int *>(ring + G::CHECKED);
     uint16_t *halves = reinterpret_cast<uint16_t *>(ring + G::HALVES);
     const Column<ROWS> col(w);
     const int nsub = (w.off[ROWS] + EB - 1) / EB;
-    TcSums<FT, ROWS> acc = sums;
-    // The first marked sub-block from b on (nsub: none).
+    const uint32_t offset = P.offset;
+    const int own_u = unit_exponent(E);
+    bool high = last == 0;
+    int band = last;
+    // The first sub-block of this pass from b on (nsub: none).
     auto next = [&](int b) {
-        while (b < nsub && !((marks >> (b >> shift)) & 1u)) ++b;
+        while (high && b < nsub && !((marks >> (b >> shift)) & 1u)) ++b;
         return b;
     };
-    auto start = [&](int b, int st) -> float {      // copies; the lane's scale if wide, else 0
+    // Starts a sub-block's copies; the lane's weight on its scale, 0 if not taken.
+    auto start = [&](int b, int st) -> float {
         Entry<kW> q;
         q.col = -1;
         if (b < nsub) q = fetch_entry<ROWS, kW>(P, w, b * EB + lane);
-        const float sj = uint32_t(q.col) < uint32_t(P.N) ? __ldg(P.rowscale + q.col) : 0.0f;
-        const bool wide = __float_as_uint(sj) >> 31;
-        const float s = wide ? fabsf(sj) * q.a : 0.0f;
+        float sj = 0.0f;
+        if (uint32_t(q.col) < uint32_t(P.N))
+            sj = P.rowscale != nullptr
+                     ? __ldg(P.rowscale + q.col)
+                     : *reinterpret_cast<const float *>(P.D + (int64_t(q.col) + 1) * P.ldd - 4);
+        const float s = kW ? fabsf(sj) * q.a : fabsf(sj);
+        const int u =
+            ROWS == 1 ? own_u : __shfl_sync(kFullMask, own_u, row_of<ROWS>(w, b * EB + lane));
+        const bool take = s != 0.0f && (!high || __float_as_uint(sj) >> 31) &&
+                          (last == 0 || band_of(exponent_of(__float_as_uint(fabsf(s))), u) == band);
         __syncwarp();
-        put_column<G>(checked, wide ? q.col : -1);
+        put_column<G>(checked, take ? q.col : -1);
         __syncwarp();
-        copy_plane<G>(smem_addr(ring) + uint32_t(st * G::PART), checked, plane, uint32_t(P.ldd), mine);
+        copy_plane<G>(smem_addr(ring) + uint32_t(st * G::PART), checked,
+                      P.D + (high ? P.N * P.ldd : 0) + (slab + piece) * 16, uint32_t(P.ldd), mine);
         cp_async_commit();
-        return s;
+        return take ? s * exp2i(band_unit(u, band)) : 0.0f;
     };
-    int b = next(0), st = 0;
-    float s = start(b, 0);
-    while (b < nsub) {
-        const int b2 = next(b + 1);
-        const float s2 = start(b2, st ^ 1);
-        cp_async_wait<1>();
-        put_weight(halves, s * row_unit<ROWS>(E, row_of<ROWS>(w, b * EB + lane)));
+    TcSums<FT, ROWS> acc = {};
+    if (last == 0) acc = sums;
+    TcRowSums<FT, ROWS == 1 ? 1 : 2> out = {};
+#pragma unroll 1
+    while (true) {
+        int b = next(0), st = 0;
+        float ws = start(b, 0);
+#pragma unroll 1
+        while (b < nsub) {
+            const int b2 = next(b + 1);
+            const float ws2 = start(b2, st ^ 1);
+            cp_async_wait<1>();
+            put_weight(halves, ws);
+            __syncwarp();
+            const uint32_t rows = smem_addr(ring) + uint32_t(st * G::PART) + tl;
+            if (high)
+                multiply<FT, ROWS>(acc, rows, halves, b * EB - col.lo, col.len,
+                                   [](uint32_t h) { return high_to_half2(h); });
+            else
+                multiply<FT, ROWS>(acc, rows, halves, b * EB - col.lo, col.len,
+                                   [&](uint32_t h) { return bytes_to_half2(h, offset); });
+            __syncwarp();
+            b = b2;
+            ws = ws2;
+            st ^= 1;
+        }
+        cp_async_wait<0>();
         __syncwarp();
-        multiply<FT, ROWS>(acc, smem_addr(ring) + uint32_t(st * G::PART) + tl, halves,
-                           b * EB - col.lo, col.len, [](uint32_t h) { return high_to_half2(h); });
-        __syncwarp();
-        b = b2;
-        s = s2;
-        st ^= 1;
+        if (!high && marks != 0u) {
+            high = true;
+            continue;
+        }
+        put_sums<true>(acc, own_u, band, out);
+        if (band == 0) break;
+        --band;
+        high = false;
+        acc = {};
     }
-    cp_async_wait<0>();
-    __syncwarp();
-    sums = acc;
+    emit(out);
 }
 
-// Walks a window's position stream and leaves its sums in `out`; c holds the
+// Walks a window's position stream and leaves its sums in `out`, or, when that takes
+// more than this walk, has them passed to emit() and returns false; c holds the
 // columns of its first blocks (fetch_first). The warp's ring `ring` (shared,
 // TcGeom<FT, SUB, NS>::WARP bytes) is free on entry and on exit.
 //
@@ -520,15 +604,15 @@ __device__ __noinline__ void high_walk(TcParams P, Window<ROWS> w, uint8_t *ring
 // sub-block; D = NS - 1): iteration n starts the row copies of block n + D, whose
 // columns were loaded an iteration ago, loads the columns of block n + D + 1,
 // then waits for block n's rows and multiplies. Block b uses row stage b mod NS.
-template <int FT, int ROWS, bool kW, int SUB, int NS>
-__device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS> &w,
+template <int FT, int ROWS, bool kW, int SUB, int NS, class Emit>
+__device__ __forceinline__ bool walk_window(const TcParams &P, const Window<ROWS> &w,
                                            uint8_t *ring, Entry<kW> (&c)[NS][SUB],
-                                           TcRowSums<FT, ROWS == 1 ? 1 : 2> &out) {
+                                           TcRowSums<FT, ROWS == 1 ? 1 : 2> &out,
+                                           const Emit &emit) {
     using G = TcGeom<FT, SUB, NS>;
     constexpr int P2 = G::P2, D = G::D;
     constexpr int BLOCK = SUB * EB;
     const int lane = threadIdx.x & 31;
-    const int t = lane & 3;
     const int total = w.off[ROWS];
     const int nblk = (total + BLOCK - 1) / BLOCK;
     const uint32_t rows_s = smem_addr(ring);
@@ -586,9 +670,17 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
     // Sub-blocks that hold wide rows, as high_walk takes them.
     uint32_t marks = 0;
     const int shift = max(0, 27 - __clz(max(nblk * SUB - 1, 0)));
-    int E = kNoScale;           // ROWS == 1: the row's; else of row (lane & 7)
-    uint32_t bound = 0;         // ROWS == 1: the largest scale (bits) that E covers
-    float unit = 0.0f;          // ROWS == 1: 2^(14 - E)
+    // The weights (bits) that a row's exponent E covers, up to 2^(E + 1): E is these bits'
+    // exponent (kNoScale: 0). ROWS == 1: the row's; else of row (lane & 7).
+    uint32_t bound = 0;
+    auto exponent = [](uint32_t bound_) { return int(bound_ >> 23) - 127; };
+    auto covers = [](int e) { return e > kNoScale ? (uint32_t(e + 127) << 23) | 0x7fffffu : 0u; };
+    // Weights from here down (bits; 0 aside) are noted: kLookBelow exponents below E.
+    auto look_from = [](uint32_t bound_) {
+        return uint32_t(max(int(bound_) - ((kLookBelow + 1) << 23), 0));
+    };
+    float unit = 0.0f;          // ROWS == 1: 2^unit_exponent(E)
+    int least = 127;            // no weight of the window but 0 has a smaller exponent
     const Column<ROWS> col(w);
 
     Weight sq[NS][SUB];         // of blocks n .. n + D
@@ -621,7 +713,7 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
 
         // This block's weights (0 for dead entries) on the scale of the row they
         // belong to; a sign bit marks a wide row.
-        uint32_t sb[SUB], top = 0;
+        uint32_t sb[SUB], top = 0, low = ~0u;
 #pragma unroll
         for (int u = 0; u < SUB; ++u) {
             if (!kW && P.rowscale == nullptr && sq[0][u].s != 0.0f)
@@ -629,46 +721,55 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
                                                               u * G::PART + in_row);
             sb[u] = sq[0][u].bits() | (__float_as_uint(sq[0][u].s) & 0x80000000u);
             top = max(top, sb[u]);
+            low = min(low, sb[u] - 1u);
         }
         float ws[SUB];
         if constexpr (ROWS == 1) {
-            if (__any_sync(kFullMask, top > bound)) {   // a wide row, or a larger weight
+            // a wide row, a larger weight, or a much smaller one
+            if (__any_sync(kFullMask, top > bound || low < look_from(bound))) {
                 uint32_t wb = 0;
 #pragma unroll
                 for (int u = 0; u < SUB; ++u) {
                     if (__any_sync(kFullMask, sb[u] >> 31)) marks |= 1u << ((n * SUB + u) >> shift);
-                    wb = max(wb, sb[u] & 0x7fffffffu);
+                    const uint32_t b = sb[u] & 0x7fffffffu;
+                    wb = max(wb, b);
+                    if (b != 0u) least = min(least, exponent_of(b));
                 }
-                const int e = exponent_of(__reduce_max_sync(kFullMask, wb));
+                const int E = exponent(bound), e = exponent_of(__reduce_max_sync(kFullMask, wb));
                 if (e > E) {            // keep the sums on the row's current scale
+                    if (E != kNoScale) least = min(least, E - kLookBelow);
                     const float f = scale_change(E, e);
                     acc.scale(f, f);
-                    E = e;
-                    bound = (uint32_t(E + 127) << 23) | 0x7fffffu;
+                    bound = covers(e);
                 }
-                unit = row_unit<ROWS>(E, 0);
+                unit = exp2i(unit_exponent(max(E, e)));
             }
 #pragma unroll
             for (int u = 0; u < SUB; ++u) ws[u] = sq[0][u].on(unit);
         } else {
             static_assert(ROWS == 1 || SUB == 1, "");
-            const uint32_t wb = sb[0] & 0x7fffffffu;
             const int tg = row_of<ROWS>(w, n * EB + lane);
-            const int Et = __shfl_sync(kFullMask, E, tg);
-            if (__any_sync(kFullMask, sb[0] > ((uint32_t(Et + 127) << 23) | 0x7fffffu))) {
+            uint32_t cover = __shfl_sync(kFullMask, bound, tg);
+            if (__any_sync(kFullMask, sb[0] > cover || low < look_from(cover))) {
+                const uint32_t wb = sb[0] & 0x7fffffffu;
                 if (__any_sync(kFullMask, sb[0] >> 31)) marks |= 1u << (n >> shift);
+                if (wb != 0u) least = min(least, exponent_of(wb));
                 const int tlo = row_of<ROWS>(w, n * EB);
                 const int thi = row_of<ROWS>(w, min(n * EB + EB, total) - 1);
+                const int E = exponent(bound);
                 int Enew = E;
                 for (int r = tlo; r <= thi; ++r) {
                     const int e = exponent_of(__reduce_max_sync(kFullMask, tg == r ? wb : 0u));
                     if ((lane & 7) == r) Enew = max(Enew, e);
                 }
+                if (Enew > E && E != kNoScale) least = min(least, E - kLookBelow);
                 const float f = scale_change(E, Enew);
+                const int t = lane & 3;
                 acc.scale(__shfl_sync(kFullMask, f, 2 * t), __shfl_sync(kFullMask, f, 2 * t + 1));
-                E = Enew;
+                bound = covers(Enew);
+                cover = __shfl_sync(kFullMask, bound, tg);
             }
-            ws[0] = sq[0][0].on(row_unit<ROWS>(E, tg));
+            ws[0] = sq[0][0].on(exp2i(unit_exponent(exponent(cover))));
         }
 #pragma unroll
         for (int u = 0; u < SUB; ++u) put_weight(halves + u * 2 * EB, ws[u]);
@@ -689,32 +790,25 @@ __device__ __forceinline__ void walk_window(const TcParams &P, const Window<ROWS
     }
     cp_async_wait<0>();         // the ring is idle before the next window
     __syncwarp();
-    if (marks != 0u && P.rowscale != nullptr) {     // (scales kept in the rows have no wide rows)
-        TcSums<FT, ROWS> sums = acc;
-        high_walk<FT, ROWS, kW, G>(P, w, ring, sums, E, marks, shift);
-        acc = sums;
-    }
-
-    if constexpr (ROWS == 1) {
-        const float back = exp2i(back_exponent(E));
-#pragma unroll
-        for (int T = 0; T < FT; ++T) {
-            out.v[0][T][0] = (acc.v[0][T][0] + acc.v[0][T][1]) * back;
-            out.v[0][T][1] = (acc.v[0][T][2] + acc.v[0][T][3]) * back;
-        }
-    } else {
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int Er = __shfl_sync(kFullMask, E, 2 * t + r);
-            const float back = exp2i(back_exponent(Er));
-#pragma unroll
-            for (int T = 0; T < FT; ++T) {
-                constexpr int L = TcSums<FT, ROWS>::PARTS - 1;
-                out.v[r][T][0] = (acc.v[0][T][r] + acc.v[L][T][r]) * back;
-                out.v[r][T][1] = (acc.v[0][T][2 + r] + acc.v[L][T][2 + r]) * back;
-            }
+    if (P.rowscale == nullptr) marks = 0u;      // (scales kept in the rows have no wide rows)
+    const int E = exponent(bound);
+    const int umin = ROWS == 1 ? unit_exponent(E) : __reduce_min_sync(kFullMask, unit_exponent(E));
+    const int last = band_of(__reduce_min_sync(kFullMask, least), umin);
+    if (last != 0 || (marks != 0u && P.rowscale != nullptr)) {
+        if (P.rowscale == nullptr) marks = 0u;
+        if constexpr (ROWS == 1) {
+            rest_of_window<FT, ROWS, kW, G>(P, w, ring, acc, E, marks, shift, last, emit);
+            return false;
+        } else {
+            TcRowSums<FT, 2> sums;
+            rest_of_window<FT, ROWS, kW, G>(P, w, ring, acc, E, marks, shift, last,
+                                            KeepSums<FT>{&sums});
+            out = sums;
+            return true;
         }
     }
+    put_sums<false>(acc, unit_exponent(E), 0, out);
+    return true;
 }
 
 // Epilogue of the plain aggregation: H_if = dinv_i * (c_f * sum_f) for f < F
@@ -896,6 +990,46 @@ struct TcPackGemm {
     }
 };
 
+// What becomes of a light window's sums: the epilogue, row by row (dg: the degree of row
+// (lane mod ROWS), -1 for none or a heavy block's; dinv: its factor).
+template <int FT, int ROWS, class Epi>
+struct LightRows {
+    Epi epi;
+    int64_t row;
+    int dg;
+    float dinv;
+    __device__ __forceinline__ void operator()(
+        const TcRowSums<FT, ROWS == 1 ? 1 : 2> &s) const {
+        const int lane = threadIdx.x & 31;
+        if constexpr (ROWS == 1) {
+            if (dg >= 0) epi.template row<true>((lane & 3) == 0 ? row : -1, dinv, s.v[0]);
+        } else {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int q = 2 * (lane & 3) + r;
+                const bool has = __shfl_sync(kFullMask, dg, q) >= 0;
+                const float di = __shfl_sync(kFullMask, dinv, q);
+                epi.template row<false>(has ? row + q : -1, di, s.v[r]);
+            }
+        }
+    }
+};
+
+// What becomes of a warp's part of a heavy row: a partial row in shared memory.
+template <int FT>
+struct HeavyPart {
+    float *part;
+    __device__ __forceinline__ void operator()(const TcRowSums<FT, 1> &s) const {
+        const int lane = threadIdx.x & 31;
+        if ((lane & 3) == 0) {
+#pragma unroll
+            for (int T = 0; T < FT; ++T)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) part[16 * T + 2 * (lane >> 2) + h] = s.v[0][T][h];
+        }
+    }
+};
+
 // Light windows (heavy rows left out), which warps take in turn as they become
 // free, so that no warp waits for the one with the longest rows: all blocks from
 // one counter (P.counters), or a block's warps from its share of them, windows
@@ -960,20 +1094,11 @@ __device__ __forceinline__ void light_windows(const TcParams &P, const Epi &epi,
         const int dg = deg;
         const float dinv =
             dg < 0 ? 0.0f : row_factor(P, row + (ROWS == 1 ? 0 : lane & 7), dg);
+        const LightRows<FT, ROWS, Epi> emit{epi, row, dg, dinv};
         TcRowSums<FT, ROWS == 1 ? 1 : 2> s;
-        walk_window<FT, ROWS, kW, SUB, NS>(P, w, ring, c, s);
+        const bool whole = walk_window<FT, ROWS, kW, SUB, NS>(P, w, ring, c, s, emit);
         if (row0 >= 0) enter();
-        if constexpr (ROWS == 1) {
-            if (dg >= 0) epi.template row<true>((lane & 3) == 0 ? row : -1, dinv, s.v[0]);
-        } else {
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int q = 2 * (lane & 3) + r;
-                const bool has = __shfl_sync(kFullMask, dg, q) >= 0;
-                const float di = __shfl_sync(kFullMask, dinv, q);
-                epi.template row<false>(has ? row + q : -1, di, s.v[r]);
-            }
-        }
+        if (whole) emit(s);
         if (row0 < 0) return;
     }
 }
@@ -1019,13 +1144,8 @@ __device__ __forceinline__ void heavy_rows(const TcParams &P, const Epi &epi, ui
             TcRowSums<FT, 1> s;
             Entry<kW> c[NS][SUB];
             fetch_first<1, kW, SUB, NS>(P, w, c);
-            walk_window<FT, 1, kW, SUB, NS>(P, w, ring, c, s);
-            if (t == 0) {
-#pragma unroll
-                for (int T = 0; T < FT; ++T)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) part(warp)[16 * T + 2 * g + h] = s.v[0][T][h];
-            }
+            const HeavyPart<FT> emit{part(warp)};
+            if (walk_window<FT, 1, kW, SUB, NS>(P, w, ring, c, s, emit)) emit(s);
             __syncthreads();
             if (warp == 0) {
 #pragma unroll

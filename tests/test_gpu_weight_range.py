@@ -111,3 +111,31 @@ def test_tiny_row_scales(cuda_device, agg, N, K, F, deg, powers):
     n = np.diff(c["rowptr"]).max() + 8
     bad = np.abs(got - ref) > n * (2.0 ** -23 * mag + 2.0 ** -149)
     assert not bad.any(), (int(bad.sum()), got[bad][:4], ref[bad][:4])
+
+
+# Weight ratios up to 10^(max - min) within a row
+@pytest.mark.parametrize("agg", AGGS)
+@pytest.mark.parametrize("N,K,F,deg", SHAPES + [(700, 600, 40, 80.0), (3000, 600, 128, 6.0)])
+@pytest.mark.parametrize("powers", [[0, -8], [0, -10], [0, -12, -24], [30, -36], [35, 0, -35]])
+def test_unlike_weights(cuda_device, agg, N, K, F, deg, powers):
+    """Where the dots of a row's large neighbours are zero, the small ones' sum is all
+    there is: each column is held to the magnitudes of its own terms."""
+    c, v, Wn = make(N, K, F, deg, agg, seed=N + F + len(powers))
+    g = np.random.default_rng(N)
+    if K > 256:         # some wide rows
+        r = np.arange(0, N, 5)
+        c["X"][r] = np.abs(c["X"][r]) * np.where(c["W"].T[r % F] >= 0, 1, -1)
+
+    def draw(n):                # few large ones
+        return 10.0 ** np.asarray(powers)[
+            np.where(g.random(n) < 0.03, 0, g.integers(1, len(powers), n))]
+
+    if agg == "weighted" and max(powers) - min(powers) < 39:     # the edges' own weights
+        v = (v * draw(len(v))).astype(np.float32)
+    else:
+        c["X"] = (c["X"] * draw(N)[:, None]).astype(np.float32)
+    ref, mag = reference(c, agg, v, Wn)
+    got = run(c, agg, cuda_device, v, Wn)
+    n = np.diff(c["rowptr"]).max() + 8
+    bad = np.abs(got - ref) > n * (2.0 ** -23 * mag + 2.0 ** -149)
+    assert not bad.any(), (int(bad.sum()), got[bad][:4], ref[bad][:4])
