@@ -555,7 +555,7 @@ bigcn_status bigcn_spmm_prescaled_rows(const int64_t *rowptr, const int32_t *col
                                        int64_t ldh, void *stream);
 
 /* Bytes of the device scratch array behind bigcn_layer_forward_static. */
-#define BIGCN_STATIC_SCRATCH_BYTES ((size_t)32 << 20)
+#define BIGCN_STATIC_SCRATCH_BYTES (((size_t)32 << 20) + 256) /* the last 256: control words */
 
 /*
  * bigcn_layer_forward without a caller-supplied workspace, for callers that
@@ -566,7 +566,7 @@ bigcn_status bigcn_spmm_prescaled_rows(const int64_t *rowptr, const int32_t *col
  * load. (The paper has no counterpart: this is an interface convenience.)
  *
  * The workspace is a file-scope __device__ array of BIGCN_STATIC_SCRATCH_BYTES
- * (32 MiB) inside this library. Every GPU on which the library's device code
+ * (32 MiB and 256 bytes) inside this library. Every GPU on which its device code
  * is loaded holds that array until the process exits. The call allocates
  * nothing: no cudaMalloc, no cudaFree, no allocating library routine.
  *

@@ -26,7 +26,7 @@ _lock = threading.Lock()
 BIGCN_OK = 0
 STATUS_NAMES = {0: "BIGCN_OK", 1: "BIGCN_ERR_INVALID_ARG", 2: "BIGCN_ERR_MISALIGNED",
                 3: "BIGCN_ERR_CUDA", 4: "BIGCN_ERR_UNSUPPORTED", 5: "BIGCN_ERR_SCRATCH_LIMIT"}
-STATIC_SCRATCH_BYTES = 32 << 20   # BIGCN_STATIC_SCRATCH_BYTES
+STATIC_SCRATCH_BYTES = (32 << 20) + 256   # BIGCN_STATIC_SCRATCH_BYTES
 
 _p = ctypes.c_void_p
 _i32 = ctypes.c_int32

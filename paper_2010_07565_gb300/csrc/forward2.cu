@@ -51,7 +51,7 @@ bool forward2_tc(int32_t K, int32_t Fh, int32_t Fo) {
 // bytes a compressed row saves).
 struct Forward2Workspace {
     size_t bits1, alpha1, wbits1, beta1, z1, s1, wbits2, beta2, z2, h1, bits2, alpha2, d2, s2,
-        total;
+        control, total;
     bool c16, tc;
 };
 
@@ -82,6 +82,7 @@ bool forward2_workspace(int64_t N, int32_t K, int32_t Fh, int32_t Fo, Forward2Wo
     w->alpha2 = take(size_t(N) * 4);
     w->d2 = take(w->tc ? size_t(N) * Fo16 : 0);      // (no wide dots: Fh <= 128)
     w->s2 = take(w->tc ? size_t(N) * 4 : 0);
+    w->control = take(kControlBytes);
     w->total = off;
     return true;
 }
@@ -169,13 +170,10 @@ extern "C" bigcn_status bigcn_forward_2layer(
     const int words1 = bigcn_words(K), words2 = bigcn_words(Fh);
     const int64_t Fh8 = (Fh + 7) / 8 * 8, Fo4 = (Fo + 3) / 4 * 4;
     const int64_t Fh16 = (Fh + 15) / 16 * 16, Fo16 = (Fo + 15) / 16 * 16;
-        const bool fused = spmm_pack_gemm_supported(Fh, Fo);
+    const bool fused = spmm_pack_gemm_supported(Fh, Fo);
     uint16_t *D1 = w.c16 ? static_cast<uint16_t *>(Z1) : nullptr;
     uint8_t *P1 = static_cast<uint8_t *>(Z1);       // the tensor-core path's byte planes
-    // Both aggregations' window counters, which the front sets to zero (alpha1 is
-    // not used by it).
-    uint32_t *counters =
-        w.tc && N >= 2 * kTcCounters ? reinterpret_cast<uint32_t *>(alpha1) : nullptr;
+    uint32_t *control = static_cast<uint32_t *>(at(w.control));
     float *Z1f = w.c16 ? nullptr : static_cast<float *>(Z1);
     cudaStream_t s = as_stream(stream);
     EventMarks marks(events, n_events, s);
@@ -185,7 +183,7 @@ extern "C" bigcn_status bigcn_forward_2layer(
     mark();
     WeightPack p1{W1, K, Fh, ldw1, wbits1, words1, beta1, 0};
     WeightPack p2{W2, Fh, Fo, ldw2, wbits2, words2, beta2, 0};
-    launch_pack_weights2(p1, p2, s);
+    launch_pack_weights2(p1, p2, control, s);
     mark();
     if (front_supported(N, K, Fh, dev)) {
         FrontArgs fr{X, N, K, ldx, scale, shift, wbits1, beta1, Fh, words1, rowptr, Z1f, Fh};
@@ -193,8 +191,6 @@ extern "C" bigcn_status bigcn_forward_2layer(
             fr.dots8 = P1;
             fr.ldd8 = Fh16;
             fr.rowscale = s1;
-            fr.counters = counters;
-            fr.n_counters = 2 * kTcCounters;
         } else if (w.c16) {
             fr.D16 = D1;
             fr.ldd16 = Fh8;
@@ -222,11 +218,11 @@ extern "C" bigcn_status bigcn_forward_2layer(
         // less for layer 2's aggregation.
         float *s2 = Fo16 - Fo >= 4 ? nullptr : static_cast<float *>(at(w.s2));
         SpmmTcPackGemmArgs f{rowptr, colidx, N, nnz, P1, Fh16, s1, Fh, K, beta1, H1, ldh1,
-                             wbits2, Fo, D2, Fo16, s2, counters};
+                             wbits2, Fo, D2, Fo16, s2, control};
         launch_spmm_tc_pack_gemm(f, dev, s, true);
         mark();
         SpmmTcArgs a2{rowptr, colidx, N, nnz, D2, Fo16, s2, Fo, Fh, out, ldo, beta2, pred};
-        if (counters != nullptr) a2.counters = counters + kTcCounters;
+        a2.counters = control + kTcCounters;
         launch_spmm_tc(a2, dev, s, true);
         mark();
         const bigcn_status ls = launch_status();

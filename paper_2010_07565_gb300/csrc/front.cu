@@ -55,8 +55,7 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
              const uint64_t *__restrict__ wbits, const float *__restrict__ beta, int F, int words,
              const int64_t *__restrict__ rowptr, float *__restrict__ Z, int64_t ldz,
              uint16_t *__restrict__ D16, int64_t ldd16, float *__restrict__ rowscale,
-             uint8_t *__restrict__ dots8, int64_t ldd8, int half, int valid, uint32_t *counters,
-             int n_counters) {
+             uint8_t *__restrict__ dots8, int64_t ldd8, int half, int valid) {
     constexpr int BM = 16 * RI;
     constexpr int kGroup = BM / kFrontWarps < 4 ? BM / kFrontWarps : 4;   // rows packed together
     // Thread cg owns V neighbouring columns (and the V that lie 64 further on),
@@ -102,7 +101,6 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
     // (phase A above only read the call's inputs), then stage them (coalesced,
     // once per block).
     grid_dependency_wait();
-    if (blockIdx.x == 0 && tid < n_counters) counters[tid] = 0u;
     for (int q = tid; q < F * words; q += kFrontThreads)
         Bs[slot(q / words) * pitch + (q % words)] = load_upstream(wbits + q);
     __syncthreads();
@@ -190,8 +188,7 @@ void launch_ri_cj(const FrontArgs &a, int BM, size_t smem, cudaStream_t s, bool 
     launch_kernel(front_kernel<RI, CJ>, dim3(grid), dim3(kFrontThreads), smem, s, pdl,
                   dim3(1, 1, 1), a.X, a.N, a.K, a.ldx, a.scale, a.shift, a.wbits, a.beta, a.F,
                   a.words, a.rowptr, a.Z, a.ldz, a.D16, a.ldd16, a.rowscale, a.dots8, a.ldd8,
-                  a.half > 0 ? a.half : INT32_MAX, a.half > 0 ? a.valid : a.F, a.counters,
-                  a.counters != nullptr ? a.n_counters : 0);
+                  a.half > 0 ? a.half : INT32_MAX, a.half > 0 ? a.valid : a.F);
 }
 
 template <int RI>
@@ -270,7 +267,7 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
                    int words, const int64_t *__restrict__ rowptr, float *__restrict__ Z,
                    int64_t ldz, uint16_t *__restrict__ D16, int64_t ldd16,
                    float *__restrict__ rowscale, int P, int pitch, uint8_t *__restrict__ dots8,
-                   int64_t ldd8, int half, int valid, uint32_t *counters, int n_counters) {
+                   int64_t ldd8, int half, int valid) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float part[kSplitWarps];
     __shared__ int wide_s[kSplitWarps];      // byte planes: row r of the group holds a wide dot
@@ -314,7 +311,6 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
         if (tid < R) wide_s[tid] = 0;
         if (!staged) {
             grid_dependency_wait();     // the packed weight columns come from the previous kernel
-            if (blockIdx.x == 0 && tid < n_counters) counters[tid] = 0u;
             const int n = F * words;
             for (int q0 = tid; q0 < n; q0 += 4 * kSplitThreads) {
                 uint64_t v[4];
@@ -416,8 +412,7 @@ void launch_split(const FrontArgs &a, const DeviceInfo &dev, cudaStream_t s, boo
     const size_t smem = split_smem(a.F, a.K, pitch, affine);
     void (*kernel)(const float *, int64_t, int, int64_t, const float *, const float *,
                    const uint64_t *, const float *, int, int, const int64_t *, float *, int64_t,
-                   uint16_t *, int64_t, float *, int, int, uint8_t *, int64_t, int, int,
-                   uint32_t *, int);
+                   uint16_t *, int64_t, float *, int, int, uint8_t *, int64_t, int, int);
     if (G == 2) kernel = affine ? front_split_kernel<2, true> : front_split_kernel<2, false>;
     else if (G == 4) kernel = affine ? front_split_kernel<4, true> : front_split_kernel<4, false>;
     else kernel = affine ? front_split_kernel<8, true> : front_split_kernel<8, false>;
@@ -433,7 +428,7 @@ void launch_split(const FrontArgs &a, const DeviceInfo &dev, cudaStream_t s, boo
                   dim3(kSplitThreads), smem, s, pdl, dim3(1, 1, 1), a.X, a.N, a.K, a.ldx, a.scale,
                   a.shift, a.wbits, a.beta, a.F, a.words, a.rowptr, a.Z, a.ldz, a.D16, a.ldd16,
                   a.rowscale, P, pitch, a.dots8, a.ldd8, a.half > 0 ? a.half : INT32_MAX,
-                  a.half > 0 ? a.valid : a.F, a.counters, a.counters != nullptr ? a.n_counters : 0);
+                  a.half > 0 ? a.valid : a.F);
 }
 
 }  // namespace

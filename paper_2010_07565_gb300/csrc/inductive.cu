@@ -34,10 +34,10 @@ constexpr size_t kIAlign = 256;
 size_t iround(size_t x) { return (x + kIAlign - 1) / kIAlign * kIAlign; }
 constexpr int32_t kMaxDots16K = 32767;
 
-// Workspace: A bits, alpha, B bits, beta, Z (factored or fp32), row scale.
+// Workspace: A bits, alpha, B bits, beta, Z (factored or fp32), row scale, control words.
 // Fz = product columns (F, or 2 Fp for GraphSAGE).
 struct InductiveWorkspace {
-    size_t a_bits, alpha, b_bits, beta, z, rowscale, total;
+    size_t a_bits, alpha, b_bits, beta, z, rowscale, control, total;
     int64_t Fp, Fz, ldz;
     bool compressed;
     bool planes;             // laid out for byte planes (rows of ldz bytes)
@@ -64,7 +64,8 @@ bool inductive_workspace(int32_t agg, int64_t N, int32_t K, int32_t F, Inductive
     w->z = off;      off = iround(off + size_t(N) * size_t(w->ldz) * (w->compressed ? 2 : 4));
     w->rowscale = off;
     if (w->compressed) off = iround(off + size_t(N) * 4);
-    w->total = off;
+    w->control = off;
+    w->total = off + kControlBytes;
     return true;
 }
 
@@ -149,7 +150,8 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
     const WeightPack wb = sage ? WeightPack{W_neigh, K, F, ldwn, b_bits + Fp * words, words,
                                             beta + Fp, 0}
                                : WeightPack{nullptr, 1, 0, 0, nullptr, 0, nullptr, 0};
-    launch_pack_weights2(wa, wb, s);
+    uint32_t *control = reinterpret_cast<uint32_t *>(ws + w.control);
+    launch_pack_weights2(wa, wb, control, s);
     // Every kernel from here on may start while the one before it drains (each
     // waits for it before it reads anything the call has written).
     // The product without a degree factor: Z_ij = alpha_i beta_j dot_ij, kept
@@ -166,8 +168,6 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
             g.half = int(Fp);
             g.valid = F;
         }
-        if (N >= kTcCounters && (fused || xnor_gemm_counters(N, K, Fz, dev)))
-            g.counters = reinterpret_cast<uint32_t *>(alpha);    // (only the product reads alpha)
     } else if (w.compressed) {
         uint16_t *D16 = reinterpret_cast<uint16_t *>(ws + w.z);
         float *rowscale = reinterpret_cast<float *>(ws + w.rowscale);
@@ -190,8 +190,7 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
     }
     if (fused) {         // few long rows: centring, packing and product in one kernel
         FrontArgs fr{X, N, K, ldx, scale, shift, b_bits, beta, Fz, words, nullptr, g.Z, g.ldz,
-                     g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half, g.valid,
-                     g.counters, kTcCounters};
+                     g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half, g.valid};
         launch_front(fr, dev, s, true);
     } else {
         launch_xnor_gemm(g, dev, s, true);
@@ -199,7 +198,7 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
     if (bytes) {
         SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8 + half, ldz, g.rowscale, F, K, H, ldh,
                      beta + half, nullptr, a.agg, sage ? g.dots8 : nullptr, beta};
-        t.counters = g.counters;
+        t.counters = control;
         launch_spmm_tc(t, dev, s, true);
     } else {
         launch_spmm_norm(a, dev, s, true);

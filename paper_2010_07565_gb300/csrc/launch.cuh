@@ -22,7 +22,8 @@ void launch_pack_rows(const float *X, int64_t N, int K, int64_t ldx, const float
 
 // Step 3: sign-pack weight columns, per-column scale (Eqs. 3-4).
 void launch_pack_weights(const float *Wt, int K, int F, int64_t ldw, uint64_t *bits,
-                         int words, float *beta, cudaStream_t stream);
+                         int words, float *beta, cudaStream_t stream,
+                         uint32_t *control = nullptr);
 
 // One weight matrix to pack: W (K x F, row stride ldw) -> bits (F x words), beta.
 struct WeightPack {
@@ -36,9 +37,18 @@ struct WeightPack {
     int tiles;               // set by the launcher
 };
 
-// Step 3 for two matrices in one launch (b.W == nullptr: a only).
+// Control words of a call: the window counters of up to two aggregations
+// (kTcCounters each: see SpmmTcArgs). They lie in the workspace, in a piece of their own
+// of kControlBytes, and the packing of the weights sets them to zero.
+constexpr int kTcCounters = 2;      // one per column slab
+constexpr int kControlWords = 2 * kTcCounters;
+constexpr size_t kControlBytes = 256;
+
+// Step 3 for two matrices in one launch (b.W == nullptr: a only); `control` (nullable):
+// the call's control words, set to zero.
 // The kernel lets its dependent launch at once (it is the first of a chain).
-void launch_pack_weights2(const WeightPack &a, const WeightPack &b, cudaStream_t stream);
+void launch_pack_weights2(const WeightPack &a, const WeightPack &b, uint32_t *control,
+                          cudaStream_t stream);
 
 struct GemmArgs {
     const uint64_t *A;       // N x words packed node rows
@@ -72,10 +82,6 @@ struct GemmArgs {
     // `valid` (0: all F; GraphSAGE's halves are padded with columns of no weight).
     int half = 0;
     int valid = 0;
-    // Nullable: the aggregation's window counters (kTcCounters words, which may be
-    // alpha[0 ..]), set to zero once alpha has been read. Left alone by a product
-    // that reads a row's alpha in several blocks: xnor_gemm_counters says.
-    uint32_t *counters = nullptr;
     // Nullable device scratch of xnor_gemm_tc_bexp_bytes(K, F) bytes (16-byte
     // aligned): the tensor-core product then expands B's signs to FP8 once
     // into it, and each CTA copies its tiles instead of expanding them.
@@ -117,11 +123,6 @@ inline bool planes_faster(int64_t N, int64_t nnz, int F) {
 // of the row's dots in one block (256 columns on the tensor cores, 64 on the
 // CUDA cores), unless K <= 254, where no dot is wide.
 bool xnor_gemm_bytes_supported(int64_t N, int K, int F, const DeviceInfo &dev);
-
-// Window counters of one aggregation on the tensor cores (one per column slab).
-constexpr int kTcCounters = 2;
-// Whether launch_xnor_gemm zeroes GemmArgs::counters for these sizes.
-bool xnor_gemm_counters(int64_t N, int K, int F, const DeviceInfo &dev);
 
 // Step 4: the XNOR-popcount product and its scaling (Eqs. 11-12).
 void launch_xnor_gemm(const GemmArgs &args, const DeviceInfo &dev, cudaStream_t stream,
@@ -209,8 +210,6 @@ struct FrontArgs {
     int64_t ldd8 = 0;
     int half = 0;
     int valid = 0;
-    uint32_t *counters = nullptr;    // nullable: kTcCounters words to set to zero
-    int n_counters = 0;
 };
 
 // Whether the fused pack + XNOR-GEMM kernel fits (F <= 128, packed tiles in

@@ -59,7 +59,7 @@ constexpr int32_t kMaxDots16K = 32767;
 // FP8 tiles of the weight signs for the tensor-core product (about F x K bytes
 // when K >= 128 and F >= 32).
 struct LayerWorkspace {
-    size_t a_bits, alpha, b_bits, beta, z, rowscale, bexp, bexp_bytes, total;
+    size_t a_bits, alpha, b_bits, beta, z, rowscale, bexp, bexp_bytes, control, total;
     bool compressed;
     bool planes;             // both byte planes fit the Z piece
     int64_t ldd;             // uint16 dots per compressed row
@@ -95,7 +95,8 @@ bool layer_workspace(int64_t N, int32_t K, int32_t F, LayerWorkspace *w) {
     w->bexp = off;
     w->bexp_bytes = xnor_gemm_tc_bexp_bytes(K, F);
     off = round_up(off + w->bexp_bytes);
-    w->total = off;
+    w->control = off;
+    w->total = off + kControlBytes;
     return true;
 }
 }  // namespace
@@ -205,7 +206,8 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     marks.mark();
     if (!fused) launch_pack_rows(X, N, K, ldx, scale, shift, a_bits, words, alpha, dev, s);
     marks.mark();
-    launch_pack_weights(Wt, K, F, ldw, b_bits, words, beta, s);
+    uint32_t *control = reinterpret_cast<uint32_t *>(ws + w.control);
+    launch_pack_weights(Wt, K, F, ldw, b_bits, words, beta, s, control);
     marks.mark();
     GemmArgs g{a_bits, alpha, N, b_bits, beta, F, K, words, Zs, F, nullptr, rowptr};
     if (w.bexp_bytes > 0) g.b_e4m3 = reinterpret_cast<uint8_t *>(ws + w.bexp);
@@ -215,10 +217,6 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
         g.dots8 = reinterpret_cast<uint8_t *>(ws + w.z);
         g.ldd8 = w.ldd8;
         g.rowscale = reinterpret_cast<float *>(ws + w.rowscale);
-        // The aggregation's window counters lie in alpha, which only the product
-        // reads (the front not at all).
-        if (N >= kTcCounters && (fused || xnor_gemm_counters(N, K, F, dev)))
-            g.counters = reinterpret_cast<uint32_t *>(alpha);
     } else if (w.compressed) {
         uint16_t *D16 = reinterpret_cast<uint16_t *>(ws + w.z);
         float *rowscale = reinterpret_cast<float *>(ws + w.rowscale);
@@ -235,8 +233,6 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     if (fused) {
         FrontArgs fr{X, N, K, ldx, scale, shift, b_bits, beta, F, words, rowptr, g.Z, g.ldz,
                      g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8};
-        fr.counters = g.counters;
-        fr.n_counters = kTcCounters;
         launch_front(fr, dev, s, pdl);
     } else {
         launch_xnor_gemm(g, dev, s, pdl);
@@ -244,7 +240,7 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     marks.mark();
     if (bytes) {        // byte planes: the aggregation on the tensor cores
         SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, w.ldd8, g.rowscale, F, K, H, ldh, beta, nullptr};
-        t.counters = g.counters;
+        t.counters = control;
         launch_spmm_tc(t, dev, s, pdl);
     } else {
         launch_spmm_norm(a, dev, s, pdl);

@@ -115,7 +115,7 @@ constexpr int kMaxCluster = 8;
 // Blocks with blockIdx.x < a.tiles pack matrix a, the rest matrix b (one
 // launch can pack both layers' weights); each block owns 32 columns.
 __global__ void __launch_bounds__(kWCols *kWRows, 2)
-pack_weights_kernel(WeightPack a, WeightPack b) {
+pack_weights_kernel(WeightPack a, WeightPack b, uint32_t *control) {
     __shared__ float partial[kWRows][kWCols];
     __shared__ float colsum[kWCols];
     allow_dependent_launch();   // what follows may start on the call's own inputs
@@ -129,6 +129,8 @@ pack_weights_kernel(WeightPack a, WeightPack b) {
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int j = tile * kWCols + tx;
     const int K = m.K;
+    if (control != nullptr && blockIdx.x == 0 && rank == 0 && ty == 0 && tx < kControlWords)
+        control[tx] = 0u;
 
     float l1 = 0.0f;
     if (j < m.F) {
@@ -252,7 +254,8 @@ void launch_pack_rows(const float *X, int64_t N, int K, int64_t ldx, const float
     }
 }
 
-void launch_pack_weights2(const WeightPack &a, const WeightPack &b, cudaStream_t stream) {
+void launch_pack_weights2(const WeightPack &a, const WeightPack &b, uint32_t *control,
+                          cudaStream_t stream) {
     // One block row per 8 words of the longer matrix, at most a cluster of 8.
     auto rows = [](const WeightPack &m) { return (m.words + kWRows - 1) / kWRows; };
     WeightPack A = a, B = b;
@@ -262,14 +265,14 @@ void launch_pack_weights2(const WeightPack &a, const WeightPack &b, cudaStream_t
     if (B.tiles > 0 && rows(B) > S) S = rows(B);
     if (S > kMaxCluster) S = kMaxCluster;
     launch_kernel(pack_weights_kernel, dim3(A.tiles + B.tiles, S, 1), dim3(kWCols, kWRows, 1), 0,
-                  stream, false, dim3(1, S, 1), A, B);
+                  stream, false, dim3(1, S, 1), A, B, control);
 }
 
 void launch_pack_weights(const float *Wt, int K, int F, int64_t ldw, uint64_t *bits,
-                         int words, float *beta, cudaStream_t stream) {
+                         int words, float *beta, cudaStream_t stream, uint32_t *control) {
     WeightPack a{Wt, K, F, ldw, bits, words, beta, 0};
     WeightPack none{nullptr, 1, 0, 0, nullptr, 0, nullptr, 0};
-    launch_pack_weights2(a, none, stream);
+    launch_pack_weights2(a, none, control, stream);
 }
 
 }  // namespace bigcn

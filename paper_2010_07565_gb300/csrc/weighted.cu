@@ -131,9 +131,9 @@ size_t wround(size_t x) { return (x + kWAlign - 1) / kWAlign * kWAlign; }
 constexpr int32_t kMaxDots16K = 32767;
 
 // Workspace: A bits, alpha, B bits, beta, Z (factored or fp32), row scale,
-// the tensor-core product's FP8 weight tiles, dinv, s.
+// the tensor-core product's FP8 weight tiles, dinv, s, control words.
 struct WeightedWorkspace {
-    size_t a_bits, alpha, b_bits, beta, z, rowscale, bexp, bexp_bytes, dinv, s, total;
+    size_t a_bits, alpha, b_bits, beta, z, rowscale, bexp, bexp_bytes, dinv, s, control, total;
     bool compressed;
     bool planes;             // laid out for byte planes (rows of ldz bytes)
     int64_t ldz;
@@ -159,7 +159,8 @@ bool weighted_workspace(int64_t N, int32_t K, int32_t F, WeightedWorkspace *w) {
     off = wround(off + w->bexp_bytes);
     w->dinv = off;     off = wround(off + size_t(N) * 4);
     w->s = off;        off = wround(off + size_t(N) * 4);
-    w->total = off;
+    w->control = off;
+    w->total = off + kControlBytes;
     return true;
 }
 
@@ -276,7 +277,8 @@ extern "C" bigcn_status bigcn_weighted_layer_forward(
     cudaStream_t s = as_stream(stream);
 
     launch_pack_rows(X, N, K, ldx, scale, shift, a_bits, words, alpha, dev, s);
-    launch_pack_weights(Wt, K, F, ldw, b_bits, words, beta, s);
+    uint32_t *control = reinterpret_cast<uint32_t *>(ws + w.control);
+    launch_pack_weights(Wt, K, F, ldw, b_bits, words, beta, s, control);
     // Every kernel after the weights' packing may start while the one before it
     // drains (each waits for it before it reads anything the call has written).
     // Factored rows carry dinv_j in their row scale (s_j = alpha_j dinv_j);
@@ -298,8 +300,6 @@ extern "C" bigcn_status bigcn_weighted_layer_forward(
         g.dots8 = reinterpret_cast<uint8_t *>(ws + w.z);
         g.ldd8 = ldz;
         g.rowscale = reinterpret_cast<float *>(ws + w.rowscale);
-        if (N >= kTcCounters && xnor_gemm_counters(N, K, F, dev))
-            g.counters = reinterpret_cast<uint32_t *>(srow);     // (only the product reads s)
     } else if (w.compressed) {
         uint16_t *D16 = reinterpret_cast<uint16_t *>(ws + w.z);
         float *rowscale = reinterpret_cast<float *>(ws + w.rowscale);
@@ -317,7 +317,7 @@ extern "C" bigcn_status bigcn_weighted_layer_forward(
     launch_xnor_gemm(g, dev, s, true);
     if (bytes) {
         SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, ldz, g.rowscale, F, K, H, ldh, beta,
-                     nullptr, kAggWeighted, nullptr, nullptr, values, dinv, g.counters};
+                     nullptr, kAggWeighted, nullptr, nullptr, values, dinv, control};
         launch_spmm_tc(t, dev, s, true);
     } else {
         launch_spmm_norm(a, dev, s, true);

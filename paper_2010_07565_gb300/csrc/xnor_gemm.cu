@@ -44,8 +44,7 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
                       int K, int words, float *__restrict__ Z, int64_t ldz,
                       int32_t *__restrict__ dots, const int64_t *__restrict__ rowptr,
                       uint16_t *__restrict__ dots16, int64_t ldd16, float *__restrict__ rowscale,
-                      uint8_t *__restrict__ dots8, int64_t ldd8, int half, int valid,
-                      uint32_t *counters) {
+                      uint8_t *__restrict__ dots8, int64_t ldd8, int half, int valid) {
     constexpr int BN = 16 * TN;
     constexpr int kALoads = kBM * kBKW / kThreads;                         // 4
     constexpr int kBLoads = (BN * kBKW + kThreads - 1) / kThreads;          // 1..2
@@ -189,12 +188,6 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
             if (dots != nullptr) dots[row * F + col] = d;
         }
     }
-    if constexpr (!kSplit) {
-        if (counters != nullptr && blockIdx.x == 0) {   // (one column tile: alpha has been read)
-            __syncthreads();
-            if (tid < kTcCounters) counters[tid] = 0u;
-        }
-    }
 }
 
 template <int TN, bool kDeg>
@@ -212,14 +205,14 @@ void launch_tn(const GemmArgs &g, const DeviceInfo &dev, cudaStream_t s, bool pd
     if (S == 1) {
         launch_kernel(xnor_gemm_popc_kernel<TN, kDeg, false>, dim3(gx, gy), dim3(kThreads), 0, s,
                       pdl, dim3(1, 1, 1), g.A, g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z,
-                      g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half > 0 ? g.half : INT32_MAX,
-                      g.half > 0 ? g.valid : g.F, g.counters);
+                      g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8,
+                      g.half > 0 ? g.half : INT32_MAX, g.half > 0 ? g.valid : g.F);
         return;
     }
     launch_kernel(xnor_gemm_popc_kernel<TN, kDeg, true>, dim3(gx, gy, S), dim3(kThreads), 0, s,
                   pdl, dim3(1, 1, S), g.A, g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z,
-                  g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half > 0 ? g.half : INT32_MAX,
-                      g.half > 0 ? g.valid : g.F, g.counters);
+                  g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8,
+                  g.half > 0 ? g.half : INT32_MAX, g.half > 0 ? g.valid : g.F);
 }
 
 template <bool kDeg>
@@ -230,12 +223,6 @@ void launch_deg(const GemmArgs &g, const DeviceInfo &dev, cudaStream_t s, bool p
 }
 
 }  // namespace
-
-bool xnor_gemm_counters(int64_t N, int K, int F, const DeviceInfo &dev) {
-    // One block reads the first rows' alpha: one column tile, k-steps not split.
-    if (xnor_gemm_tc_supported(N, K, F, dev)) return F <= 256;
-    return F <= 64 && (N + kBM - 1) / kBM >= dev.sm_count;
-}
 
 bool xnor_gemm_bytes_supported(int64_t N, int K, int F, const DeviceInfo &dev) {
     return K <= 32767 && F <= (xnor_gemm_tc_supported(N, K, F, dev) ? 256 : K <= 254 ? 256 : 64);

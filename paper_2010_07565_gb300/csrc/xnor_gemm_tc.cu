@@ -208,8 +208,7 @@ xnor_gemm_tc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ al
                     int words, float *__restrict__ Z, int64_t ldz, int32_t *__restrict__ dots,
                     const int64_t *__restrict__ rowptr, uint16_t *__restrict__ dots16,
                     int64_t ldd16, float *__restrict__ rowscale, uint8_t *__restrict__ dots8,
-                    int64_t ldd8, int half, int valid, uint32_t *counters,
-                    const uint8_t *__restrict__ bexp) {
+                    int64_t ldd8, int half, int valid, const uint8_t *__restrict__ bexp) {
     constexpr int kStageA = kUmmaM * kTcKBytes;
     constexpr int kStageB = NT * kTcKBytes;
     constexpr int kStage = kStageA + kStageB;
@@ -376,7 +375,6 @@ xnor_gemm_tc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ al
                                                   K, half, valid);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (counters != nullptr && blockIdx.x == 0 && tid < kTcCounters) counters[tid] = 0u;
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NT));
 }
@@ -416,8 +414,8 @@ xnor_gemm_tc_ws_kernel(const uint64_t *__restrict__ A, const float *__restrict__
                        float *__restrict__ Z, int64_t ldz, int32_t *__restrict__ dots,
                        const int64_t *__restrict__ rowptr, uint16_t *__restrict__ dots16,
                        int64_t ldd16, float *__restrict__ rowscale, uint8_t *__restrict__ dots8,
-                       int64_t ldd8, int half, int valid, uint32_t *counters,
-                    const uint8_t *__restrict__ bexp) {
+                       int64_t ldd8, int half, int valid,
+                       const uint8_t *__restrict__ bexp) {
     constexpr int NT = kWsCols;
     constexpr int kStageA = kWsRows * kTcKBytes;        // two 128-row halves
     constexpr int kStageB = NT * kTcKBytes;
@@ -598,7 +596,6 @@ xnor_gemm_tc_ws_kernel(const uint64_t *__restrict__ A, const float *__restrict__
                                               valid);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (counters != nullptr && blockIdx.x == 0 && tid < kTcCounters) counters[tid] = 0u;
     if (warp == kMmaWarp)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(2 * NT));
@@ -660,7 +657,7 @@ void launch_nt2(const GemmArgs &g, cudaStream_t s, bool pdl) {
     launch_kernel(kernel, grid, dim3(kTcThreads), smem, s, pdl || kBexp, dim3(1, 1, 1), g.A,
                   g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z, g.ldz, g.dots, g.rowptr,
                   g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half > 0 ? g.half : INT32_MAX,
-                  g.half > 0 ? g.valid : g.F, g.counters, static_cast<const uint8_t *>(g.b_e4m3));
+                  g.half > 0 ? g.valid : g.F, static_cast<const uint8_t *>(g.b_e4m3));
 }
 
 template <bool kDeg>
@@ -675,7 +672,7 @@ void launch_ws(const GemmArgs &g, cudaStream_t s, bool pdl) {
     launch_kernel(kernel, grid, dim3(kWsThreads), smem, s, true, dim3(1, 1, 1), g.A, g.alpha, g.N,
                   g.beta, g.F, g.K, g.words, g.Z, g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16,
                   g.rowscale, g.dots8, g.ldd8, g.half > 0 ? g.half : INT32_MAX,
-                  g.half > 0 ? g.valid : g.F, g.counters, static_cast<const uint8_t *>(g.b_e4m3));
+                  g.half > 0 ? g.valid : g.F, static_cast<const uint8_t *>(g.b_e4m3));
 }
 
 template <int NT, bool kDeg>

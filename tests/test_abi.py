@@ -154,3 +154,19 @@ def test_forward_2layer_aggregation_query(lib):
     assert B.bigcn_forward_2layer_aggregation(500, 64, 65) == 0
     with pytest.raises(B.BigcnError):
         B.bigcn_forward_2layer_aggregation(0, 64, 7)
+
+
+def test_static_scratch_takes_what_it_took(lib):
+    """The control words (256 bytes) came on top of both the workspace and the static
+    scratch: the sizes up to 32 MiB without them are taken, those above refused."""
+    f = lib.bigcn_layer_forward_static
+    X, W, rp, ci, H = None, P, P, P, P          # (X null: what is taken ends at the next check)
+    took = set()
+    for K, F in ((64, 64), (602, 64), (602, 100), (4096, 8)):
+        N = (32 << 20) // (lib.bigcn_layer_workspace_bytes(100000, K, F) // 100000 + 1)
+        for n in range(max(N - 1500, 1), N + 1500):
+            need = lib.bigcn_layer_workspace_bytes(n, K, F)
+            refused = f(X, n, K, K, None, None, W, F, F, rp, ci, n, H, F, None) == 5
+            assert refused == (need - 256 > 32 << 20), (n, K, F)
+            took.add(refused)
+    assert took == {False, True}
