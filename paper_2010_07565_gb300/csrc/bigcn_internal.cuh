@@ -150,20 +150,44 @@ __device__ __forceinline__ uint16_t encode_dot(int dot, bool valid) {
     return uint16_t(valid ? dot + 32768 : 32768);
 }
 
-// A dot in byte planes. A dot has the parity of K, so it is 2 v + (K & 1) with
-// |v| <= K / 2 <= 16383, and v = lo + 256 hi with lo in [-128, 127]. The low plane
-// holds lo + 128, the high plane hi + 128. For dots of about sqrt(K) (signs
-// that agree about half the time) v fits the low byte alone: only a row in
-// which some dot does not -- a wide row -- has its high plane written and read,
-// and the sign bit of its row scale (the scale itself is never negative) says
-// so. Half the bytes of a 16-bit dot, and nothing is rounded.
+// A dot in byte planes. A dot has the parity of K, so it is 2 v + (K & 1), and for dots
+// of about sqrt(K) (signs that agree about half the time) v + 128 fits a byte: a row's
+// bytes lie in the low plane. A row in which some dot does not -- a wide row -- is kept as
+// fp16 instead, feature f's half at byte f & ~1 of the row in the low plane (even f) or
+// the high plane (odd f), and the sign bit of its row scale (the scale itself is never
+// negative) says so. Half the bytes of a 16-bit dot, and nothing is rounded: a half holds
+// the dot times 2^-10, or, where K is odd and the dot may pass fp16's 11 bits, the dot
+// less 1 (then even, and below 4096 as K <= kMaxPlanesK).
 struct ByteDot {
     int b;                                          // v + 128
     __device__ __forceinline__ ByteDot(int dot, int K) : b(((dot - (K & 1)) >> 1) + 128) {}
     __device__ __forceinline__ bool wide() const { return unsigned(b) > 255u; }
-    __device__ __forceinline__ uint32_t lo() const { return uint32_t(b) & 255u; }
-    __device__ __forceinline__ uint32_t hi() const { return uint32_t((b >> 8) + 128); }
+    __device__ __forceinline__ uint32_t byte() const { return uint32_t(b) & 255u; }
 };
+__host__ __device__ constexpr int half_dot_bias(int K) { return K > 2048 ? (K & 1) : 0; }
+__device__ __forceinline__ uint32_t half_dot(int dot, int K) {
+    return __half_as_ushort(__float2half_rn(float(dot - half_dot_bias(K)) * (1.0f / 1024.0f)));
+}
+
+// Two bytes of such a row, each in a half-word (as fp16 subnormals u 2^-24), to two dots
+// times 2^-10: u 2^-24 2^15 + ((K & 1) - 256) 2^-10, exact; byte_dot_offset is the last
+// term, twice.
+__host__ __device__ constexpr uint32_t byte_dot_offset(int K) {
+    return (K & 1) != 0 ? 0xB3F8B3F8u : 0xB400B400u;    // -255/1024, -1/4
+}
+__device__ __forceinline__ uint32_t bytes_to_half2(uint32_t h, uint32_t offset) {
+    uint32_t r;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(h), "r"(0x78007800u), "r"(offset));
+    return r;
+}
+// Whether more than one row in `share` is wide (*wide_rows of N), by which two kernels
+// launched one after the other agree on who does the aggregation: a load behind the
+// dependency wait, as load_upstream.
+__device__ __forceinline__ bool many_wide(const uint32_t *wide_rows, int64_t N, int share) {
+    uint32_t n;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(n) : "l"(wide_rows) : "memory");
+    return int64_t(n) * share > N;
+}
 
 // Whether column c counts for a row's wide flag: of each half of `half` columns
 // the first `valid`.

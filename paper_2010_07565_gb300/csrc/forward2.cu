@@ -107,7 +107,8 @@ extern "C" int32_t bigcn_forward_2layer_launches(int64_t N, int32_t K, int32_t F
     if (N < 0 || K < 1 || Fh < 1 || Fo < 1) return -1;
     DeviceInfo dev;
     if (current_device(&dev) != BIGCN_OK) return -1;
-    return 1 + (front_supported(N, K, Fh, dev) ? 1 : 2) +
+    const bool second = forward2_tc(K, Fh, Fo) && spmm_tc_second_kernel(N, K, Fh);
+    return 1 + (front_supported(N, K, Fh, dev) ? 1 : 2) + (second ? 1 : 0) +
            (forward2_tc(K, Fh, Fo) || spmm_pack_gemm_supported(Fh, Fo) ? 1 : 3) + 1;
 }
 
@@ -189,6 +190,7 @@ extern "C" bigcn_status bigcn_forward_2layer(
         FrontArgs fr{X, N, K, ldx, scale, shift, wbits1, beta1, Fh, words1, rowptr, Z1f, Fh};
         if (w.tc) {
             fr.dots8 = P1;
+            fr.wide_rows = control + kWideRowsWord;
             fr.ldd8 = Fh16;
             fr.rowscale = s1;
         } else if (w.c16) {
@@ -218,7 +220,8 @@ extern "C" bigcn_status bigcn_forward_2layer(
         // less for layer 2's aggregation.
         float *s2 = Fo16 - Fo >= 4 ? nullptr : static_cast<float *>(at(w.s2));
         SpmmTcPackGemmArgs f{rowptr, colidx, N, nnz, P1, Fh16, s1, Fh, K, beta1, H1, ldh1,
-                             wbits2, Fo, D2, Fo16, s2, control};
+                             wbits2, Fo, D2, Fo16, s2, control,
+                             control + kWideRowsWord};
         launch_spmm_tc_pack_gemm(f, dev, s, true);
         mark();
         SpmmTcArgs a2{rowptr, colidx, N, nnz, D2, Fo16, s2, Fo, Fh, out, ldo, beta2, pred};

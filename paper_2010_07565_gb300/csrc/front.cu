@@ -55,7 +55,8 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
              const uint64_t *__restrict__ wbits, const float *__restrict__ beta, int F, int words,
              const int64_t *__restrict__ rowptr, float *__restrict__ Z, int64_t ldz,
              uint16_t *__restrict__ D16, int64_t ldd16, float *__restrict__ rowscale,
-             uint8_t *__restrict__ dots8, int64_t ldd8, int half, int valid) {
+             uint8_t *__restrict__ dots8, int64_t ldd8, int half, int valid,
+             uint32_t *__restrict__ wide_rows) {
     constexpr int BM = 16 * RI;
     constexpr int kGroup = BM / kFrontWarps < 4 ? BM / kFrontWarps : 4;   // rows packed together
     // Thread cg owns V neighbouring columns (and the V that lie 64 further on),
@@ -124,6 +125,7 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
             for (int j = 0; j < CJ; ++j) mism[i][j] += __popcll(a[i] ^ b[j]);
     }
 
+    unsigned wides = 0;                     // this thread's share of the wide rows
 #pragma unroll
     for (int i = 0; i < RI; ++i) {
         const int64_t row = m0 + rg + 16 * i;
@@ -140,26 +142,37 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
                              : sAlpha[rg + 16 * i] *
                                    inv_sqrt_degree(__ldg(rowptr + row + 1) - __ldg(rowptr + row));
         if (dots8 != nullptr) {             // byte planes + row scale, V columns per store
-            if (cg == 0) rowscale[row] = flag_scale(ai, wide);
+            if (cg == 0) {
+                rowscale[row] = flag_scale(ai, wide);
+                wides += wide;
+            }
 #pragma unroll
             for (int j0 = 0; j0 < CJ; j0 += V) {
                 const int col = column(cg, j0);
                 if (col >= ldd8) continue;
-                uint32_t lo = 0, hi = 0;
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    const ByteDot d(K - 2 * mism[i][j0 + e], K);
-                    lo |= d.lo() << (8 * e);
-                    hi |= (d.hi() & 255u) << (8 * e);
-                }
                 uint8_t *p = dots8 + row * ldd8 + col;
                 auto put = [&](uint8_t *q, uint32_t v) {
                     if (V == 4) *reinterpret_cast<uint32_t *>(q) = v;
                     else if (V == 2) *reinterpret_cast<uint16_t *>(q) = uint16_t(v);
                     else *q = uint8_t(v);
                 };
-                put(p, lo);
-                if (wide) put(p + N * ldd8, hi);
+                if (!wide) {
+                    uint32_t bytes = 0;
+#pragma unroll
+                    for (int e = 0; e < V; ++e)
+                        bytes |= ByteDot(K - 2 * mism[i][j0 + e], K).byte() << (8 * e);
+                    put(p, bytes);
+                } else if (V == 1) {        // a half, in the plane of its column's parity
+                    *reinterpret_cast<uint16_t *>(p - (col & 1) + (col & 1) * N * ldd8) =
+                        uint16_t(half_dot(K - 2 * mism[i][j0], K));
+                } else {                    // even columns' halves, odd columns' halves
+                    uint32_t h[2] = {0, 0};
+#pragma unroll
+                    for (int e = 0; e < V; ++e)
+                        h[e & 1] |= half_dot(K - 2 * mism[i][j0 + e], K) << (16 * (e / 2));
+                    put(p, h[0]);
+                    put(p + N * ldd8, h[1]);
+                }
             }
             continue;
         }
@@ -178,6 +191,10 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
             if (col < F) Z[row * ldz + col] = ai * (__ldg(beta + col) * float(K - 2 * mism[i][j]));
         }
     }
+    if (dots8 != nullptr) {
+        wides = __reduce_add_sync(kFullMask, wides);
+        if (lane == 0 && wides != 0u) atomicAdd(wide_rows, wides);
+    }
 }
 
 template <int RI, int CJ>
@@ -188,7 +205,7 @@ void launch_ri_cj(const FrontArgs &a, int BM, size_t smem, cudaStream_t s, bool 
     launch_kernel(front_kernel<RI, CJ>, dim3(grid), dim3(kFrontThreads), smem, s, pdl,
                   dim3(1, 1, 1), a.X, a.N, a.K, a.ldx, a.scale, a.shift, a.wbits, a.beta, a.F,
                   a.words, a.rowptr, a.Z, a.ldz, a.D16, a.ldd16, a.rowscale, a.dots8, a.ldd8,
-                  a.half > 0 ? a.half : INT32_MAX, a.half > 0 ? a.valid : a.F);
+                  a.half > 0 ? a.half : INT32_MAX, a.half > 0 ? a.valid : a.F, a.wide_rows);
 }
 
 template <int RI>
@@ -267,7 +284,7 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
                    int words, const int64_t *__restrict__ rowptr, float *__restrict__ Z,
                    int64_t ldz, uint16_t *__restrict__ D16, int64_t ldd16,
                    float *__restrict__ rowscale, int P, int pitch, uint8_t *__restrict__ dots8,
-                   int64_t ldd8, int half, int valid) {
+                   int64_t ldd8, int half, int valid, uint32_t *__restrict__ wide_rows) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float part[kSplitWarps];
     __shared__ int wide_s[kSplitWarps];      // byte planes: row r of the group holds a wide dot
@@ -366,7 +383,7 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
                 if (sub != 0 || c >= Fw) continue;
                 if (dots8 != nullptr) {
                     const ByteDot d(K - 2 * mism, K);
-                    dots8[row2 * ldd8 + c] = uint8_t(d.lo());
+                    dots8[row2 * ldd8 + c] = uint8_t(d.byte());
                     if (d.wide() && flag_column(c, half, valid)) wide_s[rr] = 1;
                 } else if (D16 != nullptr)
                     D16[row2 * ldd16 + c] = encode_dot(K - 2 * mism, c < F);
@@ -375,15 +392,19 @@ front_split_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
             }
         }
         __syncthreads();                     // As and part are rewritten by the next rows
-        if (dots8 != nullptr) {              // the row's flag is known: its scale and high plane
+        if (dots8 != nullptr) {     // the row's flag is known: its scale; a wide row over its bytes
             const bool wide = wide_s[rr] != 0;
-            if (row2 < N && tt == 0) rowscale[row2] = flag_scale(ai, wide);
+            if (row2 < N && tt == 0) {
+                rowscale[row2] = flag_scale(ai, wide);
+                if (wide) atomicAdd(wide_rows, 1u);
+            }
             if (row2 < N && wide && sub == 0)
                 for (int j = 0; j < passes; ++j) {
                     const int c = tt / P + j * cstep;
                     if (c < F)
-                        dots8[(N + row2) * ldd8 + c] =
-                            uint8_t(ByteDot(j == 0 ? mine[0] : mine[1], K).hi());
+                        *reinterpret_cast<uint16_t *>(dots8 + ((c & 1) * N + row2) * ldd8 +
+                                                      (c & ~1)) =
+                            uint16_t(half_dot(j == 0 ? mine[0] : mine[1], K));
                 }
             __syncthreads();                 // wide_s is cleared for the next rows
         }
@@ -412,7 +433,8 @@ void launch_split(const FrontArgs &a, const DeviceInfo &dev, cudaStream_t s, boo
     const size_t smem = split_smem(a.F, a.K, pitch, affine);
     void (*kernel)(const float *, int64_t, int, int64_t, const float *, const float *,
                    const uint64_t *, const float *, int, int, const int64_t *, float *, int64_t,
-                   uint16_t *, int64_t, float *, int, int, uint8_t *, int64_t, int, int);
+                   uint16_t *, int64_t, float *, int, int, uint8_t *, int64_t, int, int,
+                   uint32_t *);
     if (G == 2) kernel = affine ? front_split_kernel<2, true> : front_split_kernel<2, false>;
     else if (G == 4) kernel = affine ? front_split_kernel<4, true> : front_split_kernel<4, false>;
     else kernel = affine ? front_split_kernel<8, true> : front_split_kernel<8, false>;
@@ -428,7 +450,7 @@ void launch_split(const FrontArgs &a, const DeviceInfo &dev, cudaStream_t s, boo
                   dim3(kSplitThreads), smem, s, pdl, dim3(1, 1, 1), a.X, a.N, a.K, a.ldx, a.scale,
                   a.shift, a.wbits, a.beta, a.F, a.words, a.rowptr, a.Z, a.ldz, a.D16, a.ldd16,
                   a.rowscale, P, pitch, a.dots8, a.ldd8, a.half > 0 ? a.half : INT32_MAX,
-                  a.half > 0 ? a.valid : a.F);
+                  a.half > 0 ? a.valid : a.F, a.wide_rows);
 }
 
 }  // namespace

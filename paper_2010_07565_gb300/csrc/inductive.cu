@@ -162,6 +162,7 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
     const int64_t half = sage ? Fp : 0;
     if (bytes) {
         g.dots8 = reinterpret_cast<uint8_t *>(ws + w.z);
+        g.wide_rows = control + kWideRowsWord;
         g.ldd8 = ldz;
         g.rowscale = reinterpret_cast<float *>(ws + w.rowscale);
         if (sage) {
@@ -190,7 +191,8 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
     }
     if (fused) {         // few long rows: centring, packing and product in one kernel
         FrontArgs fr{X, N, K, ldx, scale, shift, b_bits, beta, Fz, words, nullptr, g.Z, g.ldz,
-                     g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half, g.valid};
+                     g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.wide_rows, g.half,
+                     g.valid};
         launch_front(fr, dev, s, true);
     } else {
         launch_xnor_gemm(g, dev, s, true);
@@ -199,6 +201,7 @@ extern "C" bigcn_status bigcn_inductive_layer_forward(
         SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8 + half, ldz, g.rowscale, F, K, H, ldh,
                      beta + half, nullptr, a.agg, sage ? g.dots8 : nullptr, beta};
         t.counters = control;
+        t.wide_rows = g.wide_rows;
         launch_spmm_tc(t, dev, s, true);
     } else {
         launch_spmm_norm(a, dev, s, true);

@@ -38,10 +38,12 @@ struct WeightPack {
 };
 
 // Control words of a call: the window counters of up to two aggregations
-// (kTcCounters each: see SpmmTcArgs). They lie in the workspace, in a piece of their own
-// of kControlBytes, and the packing of the weights sets them to zero.
+// (kTcCounters each: see SpmmTcArgs) and the count of the product's wide rows. They lie
+// in the workspace, in a piece of their own of kControlBytes, and the packing of the
+// weights sets them to zero.
 constexpr int kTcCounters = 2;      // one per column slab
-constexpr int kControlWords = 2 * kTcCounters;
+constexpr int kWideRowsWord = 2 * kTcCounters;
+constexpr int kControlWords = kWideRowsWord + 1;
 constexpr size_t kControlBytes = 256;
 
 // Step 3 for two matrices in one launch (b.W == nullptr: a only); `control` (nullable):
@@ -74,10 +76,12 @@ struct GemmArgs {
     // dots16): the low plane (N rows of ldd8 bytes, a multiple of 16 >= F) and,
     // N * ldd8 bytes on, the high plane, of which only the rows whose scale in
     // rowscale carries the wide flag are written (ByteDot, flag_scale); padding
-    // columns hold anything. The input of launch_spmm_tc. Needs
+    // columns hold anything finite. *wide_rows (a control word) receives the number of
+    // wide rows. The input of launch_spmm_tc. Needs
     // xnor_gemm_bytes_supported.
     uint8_t *dots8 = nullptr;
     int64_t ldd8 = 0;
+    uint32_t *wide_rows = nullptr;
     // Columns that make a row wide: of each half of `half` columns the first
     // `valid` (0: all F; GraphSAGE's halves are padded with columns of no weight).
     int half = 0;
@@ -208,6 +212,7 @@ struct FrontArgs {
     float *rowscale = nullptr;
     uint8_t *dots8 = nullptr;    // byte planes, as in GemmArgs
     int64_t ldd8 = 0;
+    uint32_t *wide_rows = nullptr;
     int half = 0;
     int valid = 0;
 };
@@ -288,9 +293,20 @@ struct SpmmTcArgs {
     // Nullable: kTcCounters words that an earlier kernel of the call has set to
     // zero, from which all blocks take their windows (else each block its share).
     uint32_t *counters = nullptr;
+    // The number of wide rows (nullptr: none is). Where many are, the kernel leaves the
+    // aggregation to a second one (spmm_tc_second_kernel).
+    const uint32_t *wide_rows = nullptr;
 };
 void launch_spmm_tc(const SpmmTcArgs &args, const DeviceInfo &dev, cudaStream_t stream,
                     bool pdl = false);
+
+// Wide rows cost the tensor-core walk a walk of their own; with many it loses to the CUDA
+// cores over 16-bit dots. The host cannot know, so from some size on a second kernel
+// (launch_spmm_halves) is always launched behind the first and ends at once unless many
+// rows are wide (about 1.5 us); then the first only turns the other rows into halves.
+// 232,965 nodes of mean degree 492, K = 602, F = 128, a layer: no wide row 1790 us, one in
+// 256 2560, one in 16 3580, all 9800; with the second kernel 2690 from one in 256 on.
+bool spmm_tc_second_kernel(int64_t N, int K, int F);
 
 // Layer 1's tensor-core aggregation fused with layer 2's binarization and
 // XNOR product (spmm_tc.cu): from layer 1's byte planes D1 (row scale s1,
@@ -316,10 +332,18 @@ struct SpmmTcPackGemmArgs {
     int64_t ldd2;
     float *s2;               // nullptr: the last four bytes of D2's rows (ldd2 - Fo >= 4)
     uint32_t *counters = nullptr;    // as in SpmmTcArgs
+    const uint32_t *wide_rows = nullptr;
 };
 bool spmm_tc_pack_gemm_supported(int Fh, int Fo);
 void launch_spmm_tc_pack_gemm(const SpmmTcPackGemmArgs &args, const DeviceInfo &dev,
                               cudaStream_t stream, bool pdl = false);
+
+// The second kernels, on the CUDA cores (spmm.cu): the same aggregations over rows that
+// are all halves (ByteDot) by then, if more than one in `share` was wide.
+void launch_spmm_halves(const SpmmTcArgs &args, int share, const DeviceInfo &dev,
+                        cudaStream_t stream, bool pdl);
+void launch_spmm_halves_pack_gemm(const SpmmTcPackGemmArgs &args, int share,
+                                  const DeviceInfo &dev, cudaStream_t stream, bool pdl);
 
 // Ablation products of step 4 (ablation.cu): one operand real, the other
 // binarized, on the tensor cores with the real operand as three bf16 parts.

@@ -215,6 +215,7 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     if (bytes) {
         g.Z = nullptr;
         g.dots8 = reinterpret_cast<uint8_t *>(ws + w.z);
+        g.wide_rows = control + kWideRowsWord;
         g.ldd8 = w.ldd8;
         g.rowscale = reinterpret_cast<float *>(ws + w.rowscale);
     } else if (w.compressed) {
@@ -232,7 +233,7 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     }
     if (fused) {
         FrontArgs fr{X, N, K, ldx, scale, shift, b_bits, beta, F, words, rowptr, g.Z, g.ldz,
-                     g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8};
+                     g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.wide_rows};
         launch_front(fr, dev, s, pdl);
     } else {
         launch_xnor_gemm(g, dev, s, pdl);
@@ -241,6 +242,7 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     if (bytes) {        // byte planes: the aggregation on the tensor cores
         SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, w.ldd8, g.rowscale, F, K, H, ldh, beta, nullptr};
         t.counters = control;
+        t.wide_rows = g.wide_rows;
         launch_spmm_tc(t, dev, s, pdl);
     } else {
         launch_spmm_norm(a, dev, s, pdl);

@@ -86,7 +86,7 @@ template <> struct Vec<4> {
     }
 };
 
-enum : int { kDinv = 0, kPre = 1, kDots16 = 2 };
+enum : int { kDinv = 0, kPre = 1, kDots16 = 2, kHalves = 3 };
 
 struct SpmmParams {
     const int64_t *rowptr;
@@ -115,6 +115,10 @@ struct SpmmParams {
     int64_t ncols = 0;       // rows of Z (column indices must lie below); N when 0
     const float *values = nullptr;   // kAggWeighted: a_ij per CSR entry
     const float *dinv = nullptr;     // kAggWeighted: 1/sqrt(dhat) per node
+    // kHalves: Z's low plane (ldz in bytes); the high plane is `high` bytes on.
+    int64_t high = 0;
+    const uint32_t *wide_rows = nullptr;
+    int share = 0;
 };
 
 // How a lane loads VEC consecutive entries of a row of Z and adds them,
@@ -122,8 +126,8 @@ struct SpmmParams {
 template <int VEC, int S>
 struct RowSrc {
     using T = typename Vec<VEC>::T;
-    static __device__ __forceinline__ T load(const void *Z, int64_t row, int64_t ldz, int f) {
-        return __ldg(reinterpret_cast<const T *>(static_cast<const float *>(Z) + row * ldz + f));
+    static __device__ __forceinline__ T load(const char *p, int64_t) {
+        return __ldg(reinterpret_cast<const T *>(p));
     }
     static __device__ __forceinline__ void fma(float *acc, const T &v, float w) {
         Vec<VEC>::fma(acc, v, w);
@@ -141,8 +145,8 @@ __device__ __forceinline__ float dot16_hi(uint32_t w) {
 template <>
 struct RowSrc<4, kDots16> {
     using T = uint2;
-    static __device__ __forceinline__ T load(const void *Z, int64_t row, int64_t ldz, int f) {
-        return __ldg(reinterpret_cast<const uint2 *>(static_cast<const uint16_t *>(Z) + row * ldz + f));
+    static __device__ __forceinline__ T load(const char *p, int64_t) {
+        return __ldg(reinterpret_cast<const uint2 *>(p));
     }
     static __device__ __forceinline__ void fma(float *acc, const T &v, float w) {
         acc[0] = fmaf(w, dot16_lo(v.x), acc[0]);
@@ -157,8 +161,8 @@ struct RowSrc<4, kDots16> {
 template <>
 struct RowSrc<8, kDots16> {
     using T = uint4;
-    static __device__ __forceinline__ T load(const void *Z, int64_t row, int64_t ldz, int f) {
-        return __ldg(reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(Z) + row * ldz + f));
+    static __device__ __forceinline__ T load(const char *p, int64_t) {
+        return __ldg(reinterpret_cast<const uint4 *>(p));
     }
     static __device__ __forceinline__ void fma(float *acc, const T &v, float w) {
         acc[0] = fmaf(w, dot16_lo(v.x), acc[0]);
@@ -169,6 +173,28 @@ struct RowSrc<8, kDots16> {
         acc[5] = fmaf(w, dot16_hi(v.z), acc[5]);
         acc[6] = fmaf(w, dot16_lo(v.w), acc[6]);
         acc[7] = fmaf(w, dot16_hi(v.w), acc[7]);
+    }
+};
+
+// Eight halves (dots times 2^-10): the even features' from the low plane, the odd ones'
+// from the high plane, `high` bytes on.
+template <>
+struct RowSrc<8, kHalves> {
+    using T = uint4;
+    static __device__ __forceinline__ T load(const char *p, int64_t high) {
+        const uint2 e = __ldg(reinterpret_cast<const uint2 *>(p));
+        const uint2 o = __ldg(reinterpret_cast<const uint2 *>(p + high));
+        return make_uint4(e.x, e.y, o.x, o.y);
+    }
+    static __device__ __forceinline__ void fma(float *acc, const T &v, float w) {
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {       // features 4 (q % 2) + q / 2, and 2 on
+            const float2 d = __half22float2(*reinterpret_cast<const __half2 *>(&u[q]));
+            float *a = acc + 4 * (q % 2) + q / 2;
+            a[0] = fmaf(w, d.x, a[0]);
+            a[2] = fmaf(w, d.y, a[2]);
+        }
     }
 };
 
@@ -212,7 +238,7 @@ __device__ __forceinline__ void gather(const SpmmParams &p, int64_t i, int64_t b
     using Src = RowSrc<VEC, S>;
     using V = typename Src::T;
     constexpr int P = 32 / L;
-    constexpr int kElem = S == kDots16 ? 2 : 4;
+    constexpr int kElem = S == kHalves ? 1 : S == kDots16 ? 2 : 4;
     const int lane = threadIdx.x & 31;
     const int g = lane / L, sl = lane % L;
     const uint32_t ld_lo = uint32_t(uint64_t(p.ldz) * kElem);
@@ -232,10 +258,11 @@ __device__ __forceinline__ void gather(const SpmmParams &p, int64_t i, int64_t b
             if (j < 0 || j >= p.ncols) j = -1;
             if (j >= 0) {
                 wj = S == kPre              ? 1.0f
-                     : S == kDots16         ? __ldg(p.rowscale + j)
+                     : S >= kDots16         ? __ldg(p.rowscale + j)
                      : AGG == kAggWeighted  ? __ldg(p.dinv + j)
                                             : inv_sqrt_degree(__ldg(p.rowptr + j + 1) -
                                                               __ldg(p.rowptr + j));
+                if (S == kHalves) wj = fabsf(wj) * 1024.0f;
                 if (AGG == kAggWeighted && q > 0) wj *= __ldg(p.values + b + q - 1);
             }
         }
@@ -251,7 +278,7 @@ __device__ __forceinline__ void gather(const SpmmParams &p, int64_t i, int64_t b
                 const uint64_t off = uint64_t(jj) * ld_lo + (uint64_t(jj * ld_hi) << 32);
 #pragma unroll
                 for (int v = 0; v < NV; ++v)
-                    val[u][v] = __ldg(reinterpret_cast<const V *>(zl[v] + off));
+                    val[u][v] = Src::load(zl[v] + off, p.high);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u)
@@ -281,7 +308,7 @@ __device__ __forceinline__ void gather(const SpmmParams &p, int64_t i, int64_t b
                                      (uint64_t(uint32_t(jj) * ld_hi) << 32);
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
-                    if (live) val[u][v] = __ldg(reinterpret_cast<const V *>(zl[v] + off));
+                    if (live) val[u][v] = Src::load(zl[v] + off, p.high);
                     else val[u][v] = V{};
                 }
             }
@@ -321,17 +348,22 @@ struct StoreRow {
             float o[VEC];
 #pragma unroll
             for (int c = 0; c < VEC; ++c) {
-                if (S == kDots16)
+                if (S >= kDots16)
                     o[c] = f + c < p.F ? dinv * (__ldg(p.colscale + f + c) * acc[v][c]) : 0.0f;
                 else
                     o[c] = acc[v][c] * dinv;
             }
             if constexpr (AGG == kAggSage) {   // GraphSAGE: the node's own (self-half) product
-                const float si = S == kDots16 ? __ldg(p.rowscale + i) : 0.0f;
+                const float si = S >= kDots16 ? fabsf(__ldg(p.rowscale + i)) : 0.0f;
 #pragma unroll
                 for (int c = 0; c < VEC; ++c) {
                     if (f + c >= p.F) continue;
-                    if (S == kDots16) {
+                    if (S == kHalves) {
+                        const char *d = static_cast<const char *>(p.Zs) + i * p.ldz +
+                                        (c & 1 ? p.high : 0) + f + (c & ~1);
+                        o[c] += si * (__ldg(p.colscale_s + f + c) *
+                                      (__half2float(*reinterpret_cast<const __half *>(d)) * 1024.0f));
+                    } else if (S == kDots16) {
                         const uint32_t d = __ldg(static_cast<const uint16_t *>(p.Zs) + i * p.ldz + f + c);
                         o[c] += si * (__ldg(p.colscale_s + f + c) * (float(d) - 32768.0f));
                     } else {
@@ -507,6 +539,7 @@ spmm_norm_kernel(SpmmParams p) {
     __shared__ int next;
     if (threadIdx.x == 0) next = 0;
     grid_dependency_wait();     // Z is the output of the previous kernel
+    if (S == kHalves && !many_wide(p.wide_rows, p.N, p.share)) return;
     if (p.pool > kSpmmWarps) __syncthreads();
     const int f0 = blockIdx.y * SLAB;
     using Epi = StoreRow<VEC, L, NV, S, AGG>;
@@ -563,6 +596,10 @@ struct FusedLayer2 {
     int words2;
     float *Z2;
     int64_t ldz2;
+    // kHalves: layer 2's byte dots and row scale instead (SpmmTcPackGemmArgs).
+    uint8_t *D2 = nullptr;
+    int64_t ldd2 = 0;
+    float *s2 = nullptr;
 };
 
 template <int VEC, int L, int S>
@@ -577,7 +614,7 @@ struct PackGemmRow {
         float h[VEC];
 #pragma unroll
         for (int c = 0; c < VEC; ++c) {
-            if (S == kDots16)
+            if (S >= kDots16)
                 h[c] = fb + c < Fh ? dinv * (f.sBeta1[fb + c] * acc[0][c]) : 0.0f;
             else
                 h[c] = acc[0][c] * dinv;
@@ -606,6 +643,16 @@ struct PackGemmRow {
         }
         l1 = warp_sum(l1);
         const float a = (l1 / float(Fh)) * dinv;
+        if constexpr (S == kHalves) {       // Eq. 11's dots as bytes (|dot| <= 128) and the scale
+            if (lane == 0) *(f.s2 != nullptr ? f.s2 + i
+                                             : reinterpret_cast<float *>(f.D2 + (i + 1) * f.ldd2 - 4)) = a;
+            for (int jo = lane; jo < f.Fo; jo += 32) {
+                int mism = __popcll(w0 ^ f.sW[jo * f.words2]);
+                if (f.words2 > 1) mism += __popcll(w1 ^ f.sW[jo * f.words2 + 1]);
+                f.D2[i * f.ldd2 + jo] = uint8_t(ByteDot(Fh - 2 * mism, Fh).byte());
+            }
+            return;
+        }
         // Layer 2, Eqs. 11-12, pre-scaled by this row's 1/sqrt(dhat_i).
         for (int jo = lane; jo < f.ldz2; jo += 32) {
             float z = 0.0f;
@@ -632,9 +679,11 @@ spmm_pack_gemm_kernel(SpmmParams p, FusedLayer2 f, const uint64_t *__restrict__ 
     __shared__ int next;
     if (threadIdx.x == 0) next = 0;
     grid_dependency_wait();     // layer 1's Z' and the packed W2 come from earlier kernels
+    if (S == kHalves && !many_wide(p.wide_rows, p.N, p.share)) return;
     for (int q = threadIdx.x; q < f.Fo * f.words2; q += kSpmmThreads) sW[q] = __ldg(wbits2 + q);
-    for (int q = threadIdx.x; q < f.Fo; q += kSpmmThreads) sBeta2[q] = __ldg(beta2 + q);
-    if (S == kDots16)
+    if (S != kHalves)
+        for (int q = threadIdx.x; q < f.Fo; q += kSpmmThreads) sBeta2[q] = __ldg(beta2 + q);
+    if (S >= kDots16)
         for (int q = threadIdx.x; q < p.F; q += kSpmmThreads) sBeta1[q] = __ldg(beta1 + q);
     __syncthreads();
     f.sW = sW;
@@ -819,6 +868,73 @@ void launch_spmm_pack_gemm(const SpmmPackGemmArgs &a, const DeviceInfo &dev, cud
         else if (L == 16) run(spmm_pack_gemm_kernel<4, 16, kPre>);
         else run(spmm_pack_gemm_kernel<4, 32, kPre>);
     }
+}
+
+namespace {
+
+// Rows per light block of a kernel that mostly ends at once: eight blocks per SM (232,965
+// nodes of mean degree 492, 128 features: 2595 us, and 9 us where it has nothing to do;
+// sixteen 2500 and 18; three, all resident, 2790 and 6).
+int halves_pool(int64_t N, const DeviceInfo &dev) {
+    const int64_t rows = (N + 8 * int64_t(dev.sm_count) - 1) / (8 * int64_t(dev.sm_count));
+    return int(rows > kPoolRows ? rows : kPoolRows);
+}
+
+// Eight features a lane, L = the power of two >= the row's vectors.
+template <int L, int AGG>
+void launch_halves(const SpmmTcArgs &a, int share, const DeviceInfo &dev, cudaStream_t s,
+                   bool pdl) {
+    constexpr int U = 4;
+    const bool vec_store = a.ldh % 4 == 0 && aligned_to(a.H, 16);
+    SpmmParams p{a.rowptr, a.colidx, a.N, a.nnz, a.D, a.ldd, (a.F + 7) / 8 * 8, a.F, a.H, a.ldh,
+                 heavy_block_count(a.N, dev), heavy_degree(a.N, a.nnz, (32 / L) * U),
+                 halves_pool(a.N, dev), vec_store, a.rowscale, a.colscale, nullptr, a.agg, a.Ds,
+                 a.colscale_s, a.N, a.values, a.dinv, a.N * a.ldd, a.wide_rows, share};
+    launch_kernel(spmm_norm_kernel<8, L, 1, U, kHalves, AGG>,
+                  dim3(unsigned(p.heavy_blocks + (a.N + p.pool - 1) / p.pool)), dim3(kSpmmThreads),
+                  0, s, pdl, dim3(1, 1, 1), p);
+}
+
+template <int AGG>
+void launch_halves_agg(const SpmmTcArgs &a, int share, const DeviceInfo &dev, cudaStream_t s,
+                       bool pdl) {
+    if (a.F <= 32) launch_halves<4, AGG>(a, share, dev, s, pdl);
+    else if (a.F <= 64) launch_halves<8, AGG>(a, share, dev, s, pdl);
+    else if (a.F <= 128) launch_halves<16, AGG>(a, share, dev, s, pdl);
+    else launch_halves<32, AGG>(a, share, dev, s, pdl);
+}
+
+}  // namespace
+
+void launch_spmm_halves(const SpmmTcArgs &a, int share, const DeviceInfo &dev, cudaStream_t s,
+                        bool pdl) {
+    if (a.agg == kAggWeighted) launch_halves_agg<kAggWeighted>(a, share, dev, s, pdl);
+    else if (a.agg == kAggSage) launch_halves_agg<kAggSage>(a, share, dev, s, pdl);
+    else if (a.agg == kAggMean) launch_halves_agg<kAggMean>(a, share, dev, s, pdl);
+    else launch_halves_agg<kAggGcn>(a, share, dev, s, pdl);
+}
+
+void launch_spmm_halves_pack_gemm(const SpmmTcPackGemmArgs &a, int share, const DeviceInfo &dev,
+                                  cudaStream_t s, bool pdl) {
+    const int L = a.Fh <= 32 ? 4 : a.Fh <= 64 ? 8 : 16;
+    SpmmParams p{a.rowptr, a.colidx, a.N, a.nnz, a.D1, a.ldd1, (a.Fh + 7) / 8 * 8, a.Fh, nullptr, 0,
+                 heavy_block_count(a.N, dev), heavy_degree(a.N, a.nnz, (32 / L) * 4),
+                 halves_pool(a.N, dev), false, a.s1, nullptr, nullptr};
+    p.ncols = a.N;
+    p.high = a.N * a.ldd1;
+    p.wide_rows = a.wide_rows;
+    p.share = share;
+    FusedLayer2 f{a.H1, a.ldh1, nullptr, nullptr, nullptr, a.Fo, (a.Fh + 63) / 64, nullptr, 0,
+                  a.D2, a.ldd2, a.s2};
+    const dim3 grid(unsigned(p.heavy_blocks + (a.N + p.pool - 1) / p.pool));
+    const float *none = nullptr;
+    auto run = [&](auto kernel) {
+        launch_kernel(kernel, grid, dim3(kSpmmThreads), 0, s, pdl, dim3(1, 1, 1), p, f, a.wbits2,
+                      a.beta1, none);
+    };
+    if (L == 4) run(spmm_pack_gemm_kernel<8, 4, kHalves>);
+    else if (L == 8) run(spmm_pack_gemm_kernel<8, 8, kHalves>);
+    else run(spmm_pack_gemm_kernel<8, 16, kHalves>);
 }
 
 }  // namespace bigcn

@@ -5,7 +5,7 @@
 //
 // with s_j = alpha_j / sqrt(dhat_j) the row scale and c_f = beta_f the column
 // scale of Eqs. 11-12. The dots come in byte planes (ByteDot): one byte per
-// dot, rows of 16 * FT features, and a second byte for the rows marked wide.
+// dot, rows of 16 * FT features; the rows marked wide in fp16, over both planes.
 //
 // Why tensor cores: the aggregation reads one row of dots per CSR entry. Done
 // on CUDA cores, every gathered dot costs a decode and an FMA, and the kernel
@@ -27,12 +27,15 @@
 // A staged row is read with ldmatrix.trans as pairs of neighbouring features:
 // a lane's register then holds features 2g and 2g + 1 of two entries, which a
 // byte permute turns into two A registers (even features in matrix rows 0-7,
-// odd ones in rows 8-15). The bytes u = lo + 128 enter as fp16 subnormals u
+// odd ones in rows 8-15). The bytes u = v + 128 enter as fp16 subnormals u
 // 2^-24, and one packed fma, u 2^-24 * 2^15 + ((K & 1) - 256) 2^-10, makes
 // them dot * 2^-10: every step exact, and no entry's value ever leaves fp16.
-// Rows marked wide add hi * 2^-1 (dot = 2 lo + (K & 1) + 512 hi) in a second
-// walk over the blocks that hold any (again_walk), with the weights of the other
-// entries zero: as long as the first where every row is wide.
+// Rows marked wide weigh nothing in this walk and are added afterwards
+// (rest_of_window), the few of a window 16 together, their halves as they are. That is a
+// gather of twice the bytes and a pass over the window's index list more: where many rows
+// are wide, a second kernel on the CUDA cores takes the whole aggregation over
+// (spmm_tc_second_kernel). 232,965 nodes of mean degree 492, K = 602, F = 128, a layer: no
+// wide row 1790 us, one in 1024 2150, one in 256 2560, more 2595 (16-bit dots: 2990).
 //
 // B carries the weights as two fp16 parts, hi = fp16(s') and lo = fp16((s' - hi) 2^11)
 // with s' = s_j * 2^(14 - E) (an exact power-of-two scaling that puts the
@@ -43,7 +46,7 @@
 // multiplied by the exact power of two that keeps them consistent. A window with
 // smaller weights than that (they decide the columns in which the large neighbours'
 // dots are zero) is walked again in bands of 2^24, each on a scale of its own
-// (again_walk): as good as fp32 multiply-adds at any ratio, at the cost of one more walk
+// (rest_of_window): as good as fp32 multiply-adds at any ratio, at the cost of one more walk
 // per band.
 //
 // A warp takes a window of consecutive output rows whose lists (self entry
@@ -111,6 +114,7 @@ struct TcGeom {
     static constexpr int PART = EB * PITCH;        // one sub-block
     static constexpr int STAGE = SUB * PART;       // one block
     static constexpr int NS = NSTAGES;             // row ring depth (blocks)
+    static constexpr int PARTS = SUB * NS;         // sub-blocks in the ring
     static constexpr int D = NS - 1;               // blocks of rows copied ahead
     // One warp's ring: NS row stages (each starting on a 128-byte line), then the
     // checked columns of the block being copied and the weights of the block
@@ -148,6 +152,13 @@ __device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
                  : "memory");
 }
 
+__device__ __forceinline__ void ldsm_x2_trans(uint32_t addr, uint32_t (&r)[2]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+                 : "=r"(r[0]), "=r"(r[1])
+                 : "r"(addr)
+                 : "memory");
+}
+
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                           uint32_t b1) {
     asm volatile(
@@ -155,23 +166,6 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
         "{%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// Two low bytes (as fp16 subnormals u 2^-24) to two dots times 2^-10.
-__device__ __forceinline__ uint32_t bytes_to_half2(uint32_t h, uint32_t offset) {
-    uint32_t r;
-    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(h), "r"(0x78007800u), "r"(offset));
-    return r;
-}
-// Two high bytes (hi + 128, the same way) to hi * 2^-1.
-__device__ __forceinline__ uint32_t high_to_half2(uint32_t h) {
-    uint32_t r;     // (u 2^-24 2^15 - 2^-2) 2^8 = (u - 128) 2^-1
-    asm("{\n.reg .b32 t;\n"
-        "fma.rn.f16x2 t, %1, %2, %3;\n"
-        "mul.rn.f16x2 %0, t, %4;\n}"
-        : "=r"(r)
-        : "r"(h), "r"(0x78007800u), "r"(0xB400B400u), "r"(0x5C005C00u));
-    return r;
 }
 
 // 2^e as a float for e in [-126, 127] (0 for -127).
@@ -221,6 +215,7 @@ struct TcParams {
     const float *values;     // kAggWeighted: a_ij per CSR entry
     const float *dinv;       // kAggWeighted: 1/sqrt(dhat) per node
     uint32_t offset;         // ((K & 1) - 256) 2^-10, twice, in fp16
+    uint32_t half_bias;      // what a wide row's halves lack, 2^-10 half_dot_bias(K), in fp16, twice
     int64_t heavy_degree;    // rows with more neighbours are walked by whole blocks
     uint32_t *counters;      // nullable: windows taken so far by all blocks, per column slab
     int heavy_blocks;        // blocks [0, heavy_blocks) walk the heavy rows
@@ -323,10 +318,12 @@ __device__ __forceinline__ void put_column(int *checked, int j) {
 // Copy k of a lane moves chunk `piece` of staged row r0 + k STEP to its slot,
 // which for P2 = 8 alternates between two (4 rows on, bit 2 of the row flips),
 // else is the same for every k. `plane` points at chunk `piece` of row 0; `mine`:
-// the lane's chunk exists.
-template <class G>
+// the lane's chunk exists. kBoth: staged rows 16 to 31 come from the high plane, `high`
+// bytes on (16 positions' rows, low and high).
+template <class G, bool kBoth = false>
 __device__ __forceinline__ void copy_plane(uint32_t stage, const int *checked,
-                                           const uint8_t *plane, uint32_t row_bytes, bool mine) {
+                                           const uint8_t *plane, uint32_t row_bytes, bool mine,
+                                           int64_t high = 0) {
     constexpr int P2 = G::P2;
     const int lane = threadIdx.x & 31;
     const int r0 = lane / P2, piece = lane % P2;
@@ -351,7 +348,9 @@ __device__ __forceinline__ void copy_plane(uint32_t stage, const int *checked,
 #pragma unroll
         for (int k = 0; k < P2; ++k)
             cp_async16((base ^ (P2 == 8 && (k & 1) ? 64u : 0u)) + uint32_t(k * G::STEP * G::PITCH),
-                       plane + uint64_t(uint32_t(jj[k])) * row_bytes, jj[k]);
+                       plane + uint64_t(uint32_t(jj[k])) * row_bytes +
+                           (kBoth && r0 + k * G::STEP >= 16 ? high : 0),
+                       jj[k]);
 }
 
 // A window's sums in the MMA's accumulator layout: ROWS == 1 hi and lo in columns
@@ -374,6 +373,8 @@ struct TcSums {
 // A lane's weight on its row's scale as its two fp16 parts in shared memory (`halves`:
 // EB hi parts, then EB lo parts times 2^kLoShift), entries 2t, 2t + 1, and those 8, 16 and 24 on,
 // next to one another, so that a lane's B fragments are one load.
+// kBoth: 16 positions (lanes 0 to 15), hi parts and then lo parts.
+template <bool kBoth = false>
 __device__ __forceinline__ void put_weight(uint16_t *halves, float ws) {
     const int lane = threadIdx.x & 31;
     const __half hi = __float2half_rn(ws);
@@ -382,9 +383,12 @@ __device__ __forceinline__ void put_weight(uint16_t *halves, float ws) {
     // the dot's sign)
     const __half lo = __float2half_rn(
         fmaxf((ws - __half2float(hi)) * float(1 << kLoShift), -32768.0f));
-    const int at = ((lane >> 1) & 3) * 8 + (lane >> 3) * 2 + (lane & 1);
-    halves[at] = __half_as_ushort(hi);
-    halves[EB + at] = __half_as_ushort(lo);
+    constexpr int kN = kBoth ? EB / 2 : EB;
+    const int at = ((lane >> 1) & 3) * (kN / 4) + (lane >> 3) * 2 + (lane & 1);
+    if (!kBoth || lane < kN) {
+        halves[at] = __half_as_ushort(hi);
+        halves[kN + at] = __half_as_ushort(lo);
+    }
 }
 
 // One pass over a staged sub-block (shared address `rows` = the sub-block + this
@@ -428,6 +432,80 @@ __device__ __forceinline__ void multiply(TcSums<FT, ROWS> &acc, uint32_t rows,
                                    convert(__byte_perm(x[2 * kk + 1], 0u, 0x4341))};
             mma_16816(acc.v[0][T], a, b0[kk], b1[kk]);
             if constexpr (ROWS > 1) mma_16816(acc.v[1][T], a, c0[kk], c1[kk]);
+        }
+    }
+}
+
+// Bits of entries 2t, 2t + 1 (.x) and 8 + 2t, 9 + 2t (.y) as masks of fp16 pairs.
+__device__ __forceinline__ uint2 pair_masks(uint32_t bits) {
+    const int t = threadIdx.x & 3;
+    auto two = [](uint32_t b) {
+        return (b & 1u ? 0xffffu : 0u) | (b & 2u ? 0xffff0000u : 0u);
+    };
+    return make_uint2(two(bits >> (2 * t)), two(bits >> (8 + 2 * t)));
+}
+
+// One pass over 16 positions whose rows are staged low plane and high plane (shared
+// address `part`), some of them wide (bits of `wide`; `narrow`: of the others that weigh
+// anything), weights in `halves` (put_weight<true>). Wide rows' halves go into the MMA as
+// they are (staged rows 0 to 15 hold the even features, 16 to 31 the odd ones), the other
+// entries' masked out (what was staged for them may be any bits); bytes as in multiply().
+// ROWS > 1: the entries that belong to the lane's column g are the bits of `column`. The
+// sums stay in local memory (loops over T that are not unrolled): see rest_of_window.
+template <int FT, int ROWS, class G>
+__device__ __forceinline__ void multiply_both(const TcParams &P, TcSums<FT, ROWS> &acc,
+                                              uint32_t part, const uint16_t *halves,
+                                              uint32_t wide, uint32_t narrow, uint32_t column) {
+    constexpr int kN = EB / 2, P2 = G::P2;
+    const int lane = threadIdx.x & 31;
+    const int g = lane >> 2, t = lane & 3;
+    // ldmatrix: lane l's address is chunk T of staged row q, at slot T ^ swizzle.
+    auto staged = [&](int q) {
+        return part + (uint32_t(q * G::PITCH) | uint32_t(((q / G::LINE) & (P2 - 1)) << 4));
+    };
+    uint2 b = make_uint2(0u, 0u), c = b;
+    if constexpr (ROWS == 1) {
+        if (g < 2) b = *reinterpret_cast<const uint2 *>(halves + g * kN + t * 4);
+    } else {
+        const uint2 m = pair_masks(column);
+        b = *reinterpret_cast<const uint2 *>(halves + t * 4);
+        c = *reinterpret_cast<const uint2 *>(halves + kN + t * 4);
+        b = make_uint2(b.x & m.x, b.y & m.y);
+        c = make_uint2(c.x & m.x, c.y & m.y);
+    }
+    const uint2 m = pair_masks(wide);
+    if (wide != 0u) {
+        // entries 0-7 low, 0-7 high, 8-15 low, 8-15 high
+        const uint32_t rows = staged((lane & 7) | (lane & 8) << 1 | (lane & 16) >> 1);
+        const uint32_t bias = P.half_bias;
+#pragma unroll 1
+        for (int T = 0; T < FT; ++T) {
+            uint32_t x[4];
+            ldsm_x4_trans(rows ^ uint32_t(T << 4), x);
+            const uint32_t a[4] = {x[0] & m.x, x[1] & m.x, x[2] & m.y, x[3] & m.y};
+            const uint32_t one[4] = {bias, bias, bias, bias};       // + 1 per dot: see half_dot
+            mma_16816(acc.v[0][T], a, b.x & m.x, b.y & m.y);
+            if (bias != 0u) mma_16816(acc.v[0][T], one, b.x & m.x, b.y & m.y);
+            if constexpr (ROWS > 1) {
+                mma_16816(acc.v[1][T], a, c.x & m.x, c.y & m.y);
+                if (bias != 0u) mma_16816(acc.v[1][T], one, c.x & m.x, c.y & m.y);
+            }
+        }
+    }
+    if (narrow != 0u) {
+        // entries 0-7 and 8-15 of chunk T (lanes 0 to 15 give the addresses)
+        const uint32_t rows = staged(lane & 15);
+        const uint32_t offset = P.offset;
+#pragma unroll 1
+        for (int T = 0; T < FT; ++T) {
+            uint32_t x[2];
+            ldsm_x2_trans(rows ^ uint32_t(T << 4), x);
+            const uint32_t a[4] = {bytes_to_half2(__byte_perm(x[0], 0u, 0x4240), offset),
+                                   bytes_to_half2(__byte_perm(x[0], 0u, 0x4341), offset),
+                                   bytes_to_half2(__byte_perm(x[1], 0u, 0x4240), offset),
+                                   bytes_to_half2(__byte_perm(x[1], 0u, 0x4341), offset)};
+            mma_16816(acc.v[0][T], a, b.x & ~m.x, b.y & ~m.y);
+            if constexpr (ROWS > 1) mma_16816(acc.v[1][T], a, c.x & ~m.x, c.y & ~m.y);
         }
     }
 }
@@ -479,7 +557,7 @@ __device__ __forceinline__ void put_sums(const TcSums<FT, ROWS> &acc, int u, int
         const int ur = ROWS == 1 ? u : __shfl_sync(kFullMask, u, 2 * t + r);
         const float back = exp2i(kDotShift - band_unit(ur, k));
         const int lo = ROWS == 1 ? 1 : r;       // columns 0 and 1, or one of each set
-#pragma unroll
+#pragma unroll (kAdd ? 1 : FT)
         for (int T = 0; T < FT; ++T)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -499,98 +577,170 @@ struct KeepSums {
 
 // What a window with wide rows or with weights far below their row's largest still
 // needs (rarely) after its first walk, which left `sums` and the exponents E. last == 0:
-// adds the wide rows' high plane in the 32-position sub-blocks marked in `marks` (bit q:
+// adds the wide rows of the 32-position sub-blocks marked in `marks` (bit q:
 // sub-blocks q << shift .. ((q + 1) << shift) - 1). last > 0: the whole window again, band
 // after band of its weights from `last` down to 0, the smallest first, each on its own
 // scale. The results go to emit().
 //
-// A pass walks the low plane, or the high plane for the wide rows; entries it does not
-// take weigh nothing and are not copied. Two stages: the next sub-block's rows are copied
-// while one is multiplied. A function of its own, which calls none and returns nothing:
-// the first walk's registers need not hold both, nor meet its results again (returning
-// the sums cost the walk of 128 features 3 % where no window came here).
+// A pass looks at every position, collects the entries it takes, a lane each, and walks
+// them 16 together, as they come (a block of 32 positions that holds one wide row costs
+// the index and scale of 32 and the row of one): copies of one 16 are in flight while
+// the 16 before are multiplied. A function of its own, which calls none, keeps its sums
+// in local memory and (one-row windows) returns nothing: the first walk's registers need
+// not hold both, nor meet its results again (GraphSAGE's walk of 128 features, where no
+// window came here: 1880 us with the sums returned, 2190 with them in registers here).
 template <int FT, int ROWS, bool kW, class G, class Emit>
 __device__ __noinline__ void rest_of_window(TcParams P, Window<ROWS> w, uint8_t *ring,
                                             TcSums<FT, ROWS> sums, int E, uint32_t marks,
                                             int shift, int last, Emit emit) {
+    static_assert(G::PARTS >= 2, "one part is copied while one is multiplied");
     const int lane = threadIdx.x & 31;
     const int piece = lane % G::P2, slab = int(blockIdx.y) * FT;
     const bool mine = piece < FT && (slab + piece) * 16 < P.width;
-    const uint32_t tl =
-        uint32_t(lane * G::PITCH) | uint32_t(((lane / G::LINE) & (G::P2 - 1)) << 4);
+    const uint8_t *plane = P.D + (slab + piece) * 16;
+    const int64_t high = P.N * P.ldd;
+    const uint32_t ring_s = smem_addr(ring);
     int *checked = reinterpret_cast<int *>(ring + G::CHECKED);
     uint16_t *halves = reinterpret_cast<uint16_t *>(ring + G::HALVES);
-    const Column<ROWS> col(w);
+    float *floats = reinterpret_cast<float *>(ring + G::HALVES);
     const int nsub = (w.off[ROWS] + EB - 1) / EB;
-    const uint32_t offset = P.offset;
     const int own_u = unit_exponent(E);
-    bool high = last == 0;
     int band = last;
-    // The first sub-block of this pass from b on (nsub: none).
+    TcRowSums<FT, ROWS == 1 ? 1 : 2> out = {};
+    auto clear = [&]() {
+#pragma unroll 1
+        for (int T = 0; T < FT; ++T)
+#pragma unroll
+            for (int q = 0; q < 4 * TcSums<FT, ROWS>::PARTS; ++q) sums.v[q / 4][T][q % 4] = 0.0f;
+    };
+    if (last != 0) clear();
+
+    // Collected entries, lane q the q-th: column, weight, row (bits 0-2) and wide (bit 3).
+    int count = 0, pcol = 0, pinfo = 0;
+    float ps = 0.0f;
+    // The 16 in flight: part, weight (on its scale) and row of lane q's, and which are
+    // wide or narrow.
+    int in_flight = -1, frow = 0;
+    float fweight = 0.0f;
+    uint32_t fwide = 0, fnarrow = 0;
+    auto multiply_in_flight = [&]() {
+        put_weight<true>(halves, fweight);
+        uint32_t column = 0;
+        if constexpr (ROWS > 1)
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                const uint32_t b = __ballot_sync(kFullMask, frow == r);
+                if (lane >> 2 == r) column = b;
+            }
+        __syncwarp();
+        multiply_both<FT, ROWS, G>(P, sums, ring_s + uint32_t(in_flight * G::PART), halves, fwide,
+                                   fnarrow, column);
+        __syncwarp();
+    };
+    // Starts the copies of the first 16 collected entries and multiplies the 16 before.
+    auto flush = [&]() {
+        const int e = lane & 15;
+        const int col = __shfl_sync(kFullMask, pcol, e), info = __shfl_sync(kFullMask, pinfo, e);
+        const float s = __shfl_sync(kFullMask, ps, e);
+        const bool live = e < count, wide = live && (info & 8);
+        const int part = in_flight == 0 ? 1 : 0;
+        __syncwarp();
+        put_column<G>(checked, live && (lane < 16 || wide) ? col : -1);
+        __syncwarp();
+        copy_plane<G, true>(ring_s + uint32_t(part * G::PART), checked, plane, uint32_t(P.ldd), mine,
+                            high);
+        cp_async_commit();
+        if (in_flight >= 0) {
+            cp_async_wait<1>();
+            __syncwarp();
+            multiply_in_flight();
+        }
+        in_flight = part;
+        frow = info & 7;
+        const int u = ROWS == 1 ? own_u : __shfl_sync(kFullMask, own_u, frow);
+        fweight = live ? s * exp2i(band_unit(u, band)) : 0.0f;
+        fwide = __ballot_sync(kFullMask, wide) & 0xffffu;
+        fnarrow = __ballot_sync(kFullMask, live && !wide) & 0xffffu;
+        count = max(count - 16, 0);
+        pcol = __shfl_sync(kFullMask, pcol, e + 16);
+        pinfo = __shfl_sync(kFullMask, pinfo, e + 16);
+        ps = __shfl_sync(kFullMask, ps, e + 16);
+    };
+    // The first sub-block of this pass from b on (nsub: none), its entries and their scales.
     auto next = [&](int b) {
-        while (high && b < nsub && !((marks >> (b >> shift)) & 1u)) ++b;
+        while (last == 0 && b < nsub && !((marks >> (b >> shift)) & 1u)) ++b;
         return b;
     };
-    // Starts a sub-block's copies; the lane's weight on its scale, 0 if not taken.
-    auto start = [&](int b, int st) -> float {
+    auto entry = [&](int b) {
         Entry<kW> q;
         q.col = -1;
         if (b < nsub) q = fetch_entry<ROWS, kW>(P, w, b * EB + lane);
-        float sj = 0.0f;
-        if (uint32_t(q.col) < uint32_t(P.N))
-            sj = P.rowscale != nullptr
-                     ? __ldg(P.rowscale + q.col)
-                     : *reinterpret_cast<const float *>(P.D + (int64_t(q.col) + 1) * P.ldd - 4);
-        const float s = kW ? fabsf(sj) * q.a : fabsf(sj);
-        const int u =
-            ROWS == 1 ? own_u : __shfl_sync(kFullMask, own_u, row_of<ROWS>(w, b * EB + lane));
-        const bool take = s != 0.0f && (!high || __float_as_uint(sj) >> 31) &&
-                          (last == 0 || band_of(exponent_of(__float_as_uint(fabsf(s))), u) == band);
-        __syncwarp();
-        put_column<G>(checked, take ? q.col : -1);
-        __syncwarp();
-        copy_plane<G>(smem_addr(ring) + uint32_t(st * G::PART), checked,
-                      P.D + (high ? P.N * P.ldd : 0) + (slab + piece) * 16, uint32_t(P.ldd), mine);
-        cp_async_commit();
-        return take ? s * exp2i(band_unit(u, band)) : 0.0f;
+        return q;
     };
-    TcSums<FT, ROWS> acc = {};
-    if (last == 0) acc = sums;
-    TcRowSums<FT, ROWS == 1 ? 1 : 2> out = {};
+    auto scale_of = [&](const Entry<kW> &q) {
+        if (uint32_t(q.col) >= uint32_t(P.N)) return 0.0f;
+        return P.rowscale != nullptr
+                   ? __ldg(P.rowscale + q.col)
+                   : *reinterpret_cast<const float *>(P.D + (int64_t(q.col) + 1) * P.ldd - 4);
+    };
 #pragma unroll 1
     while (true) {
-        int b = next(0), st = 0;
-        float ws = start(b, 0);
+        int b0 = next(0), b1 = next(b0 + 1);
+        Entry<kW> q0 = entry(b0), q1 = entry(b1);
+        float s0 = scale_of(q0);
 #pragma unroll 1
-        while (b < nsub) {
-            const int b2 = next(b + 1);
-            const float ws2 = start(b2, st ^ 1);
-            cp_async_wait<1>();
-            put_weight(halves, ws);
-            __syncwarp();
-            const uint32_t rows = smem_addr(ring) + uint32_t(st * G::PART) + tl;
-            if (high)
-                multiply<FT, ROWS>(acc, rows, halves, b * EB - col.lo, col.len,
-                                   [](uint32_t h) { return high_to_half2(h); });
-            else
-                multiply<FT, ROWS>(acc, rows, halves, b * EB - col.lo, col.len,
-                                   [&](uint32_t h) { return bytes_to_half2(h, offset); });
-            __syncwarp();
-            b = b2;
-            ws = ws2;
-            st ^= 1;
+        while (true) {                              // (past the end: what is left collected)
+            const bool end = b0 >= nsub;
+            const int b2 = next(b1 + 1);
+            const float s1 = scale_of(q1);
+            const Entry<kW> q2 = entry(b2);
+            const int r = ROWS == 1 ? 0 : row_of<ROWS>(w, b0 * EB + lane);
+            const float s = kW ? fabsf(s0) * q0.a : fabsf(s0);
+            const bool wide = __float_as_uint(s0) >> 31;
+            const int u = ROWS == 1 ? own_u : __shfl_sync(kFullMask, own_u, r);
+            const bool take =
+                s0 != 0.0f && s != 0.0f &&          // (s0 is 0 where there is no entry)
+                (last == 0 ? wide : band_of(exponent_of(__float_as_uint(fabsf(s))), u) == band);
+            const unsigned taken = __ballot_sync(kFullMask, take);
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {           // 16 positions more: at most 31 collected
+                const unsigned m = (taken >> (16 * h)) & 0xffffu;
+                if (m == 0u && !end) continue;
+                const bool from = take && lane >> 4 == h;
+                const int to = count + __popc(m & ((1u << (lane & 15)) - 1u));
+                const bool here = lane >= count && lane < count + __popc(m);
+                if (from) {
+                    checked[to] = q0.col;
+                    floats[to] = s;
+                }
+                __syncwarp();
+                if (here) {
+                    pcol = checked[lane];
+                    ps = floats[lane];
+                }
+                __syncwarp();
+                if (from) checked[to] = r | (wide ? 8 : 0);
+                __syncwarp();
+                if (here) pinfo = checked[lane];
+                __syncwarp();
+                count += __popc(m);
+                if (count >= 16 || (end && count > 0)) flush();
+            }
+            if (end) break;
+            b0 = b1;
+            b1 = b2;
+            q0 = q1;
+            q1 = q2;
+            s0 = s1;
         }
         cp_async_wait<0>();
         __syncwarp();
-        if (!high && marks != 0u) {
-            high = true;
-            continue;
-        }
-        put_sums<true>(acc, own_u, band, out);
+        if (in_flight >= 0) multiply_in_flight();
+        in_flight = -1;
+        put_sums<true>(sums, own_u, band, out);
         if (band == 0) break;
         --band;
-        high = false;
-        acc = {};
+        clear();
     }
     emit(out);
 }
@@ -639,7 +789,9 @@ __device__ __forceinline__ bool walk_window(const TcParams &P, const Window<ROWS
             return __float_as_uint(kW ? fabsf(s * a) : s) & 0x7fffffffu;
         }
         __device__ __forceinline__ float on(float unit) const {
-            return (kW ? fabsf(s) * a : fabsf(s)) * unit;
+            float v;        // (a wide row's scale is negative: 0 in this walk; NaN stays)
+            asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(v) : "f"(s));
+            return (kW ? v * a : v) * unit;
         }
     };
     // Starts the copies of a block's rows to the stage at `stage`; s receives this
@@ -667,7 +819,7 @@ __device__ __forceinline__ bool walk_window(const TcParams &P, const Window<ROWS
         for (int T = 0; T < FT; ++T)
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc.v[p][T][q] = 0.0f;
-    // Sub-blocks that hold wide rows, as high_walk takes them.
+    // Sub-blocks that hold wide rows, as rest_of_window takes them.
     uint32_t marks = 0;
     const int shift = max(0, 27 - __clz(max(nblk * SUB - 1, 0)));
     // The weights (bits) that a row's exponent E covers, up to 2^(E + 1): E is these bits'
@@ -825,7 +977,8 @@ struct TcStore {
     int32_t *pred;           // nullable (one column slab only)
     bool vec2;               // feature pairs of H are 8-byte aligned
     // GraphSAGE (Ds non-null): the node's own product is added, from the self half
-    // of its row (low plane; the high plane `high` bytes on) with its row scale.
+    // of its row (its bytes, or its halves in the two planes, the high one `high` bytes on)
+    // with its row scale.
     const uint8_t *Ds;
     int64_t ldd;
     int64_t high;
@@ -842,10 +995,10 @@ struct TcStore {
     }
     // The node's own dot with self column f.
     __device__ __forceinline__ float own_dot(int64_t i, int f, bool wide) const {
-        const uint8_t *p = Ds + i * ldd + f;
-        int d = 2 * (int(__ldg(p)) - 128) + (K & 1);
-        if (wide) d += 512 * (int(__ldg(p + high)) - 128);
-        return float(d);
+        const uint8_t *p = Ds + i * ldd;
+        if (!wide) return float(2 * (int(__ldg(p + f)) - 128) + (K & 1));
+        const uint16_t h = *reinterpret_cast<const uint16_t *>(p + (f & 1 ? high : 0) + (f & ~1));
+        return fmaf(__half2float(__ushort_as_half(h)), 1024.0f, float(half_dot_bias(K)));
     }
     template <bool kAlone>
     __device__ __forceinline__ void row(int64_t i, float di, const float (&v)[FT][2]) const {
@@ -985,7 +1138,7 @@ struct TcPackGemm {
         for (int o = kAlone ? lane : g; o < Fo; o += kAlone ? 32 : 8) {
             int mism = __popcll(w0 ^ sW2[o * words2]);
             if (words2 > 1) mism += __popcll(w1 ^ sW2[o * words2 + 1]);
-            d[o] = uint8_t(ByteDot(Fh - 2 * mism, Fh).lo());
+            d[o] = uint8_t(ByteDot(Fh - 2 * mism, Fh).byte());
         }
     }
 };
@@ -1163,9 +1316,45 @@ __device__ __forceinline__ void heavy_rows(const TcParams &P, const Epi &epi, ui
     }
 }
 
+// The second kernel that takes over where more than one row in `share` is wide (wide_rows
+// nullptr: there is none), and the rows that are then made ready for it: `planes` from
+// their first byte (TcParams::D may be their other half). Not part of TcParams, which
+// rest_of_window takes along (there, 1790 -> 1930 us for GraphSAGE's walk).
+struct SecondKernel {
+    const uint32_t *wide_rows;
+    int share;
+    uint8_t *planes;
+};
+
+// Turns the rows that are not wide into halves too, in place, a chunk of 16 features a
+// thread (the even features' halves over its bytes, the odd ones' in the high plane).
+__device__ __forceinline__ void rows_to_halves(uint8_t *planes, int64_t ldd, int64_t N,
+                                               const float *rowscale, uint32_t offset) {
+    const int64_t chunks = ldd / 16, total = N * chunks;
+    for (int64_t q = int64_t(blockIdx.x) * kTcThreads + threadIdx.x; q < total;
+         q += int64_t(gridDim.x) * kTcThreads) {
+        if (__float_as_uint(__ldg(rowscale + q / chunks)) >> 31) continue;
+        uint4 *low = reinterpret_cast<uint4 *>(planes) + q;
+        const uint4 v = *low;
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        uint32_t e[4], o[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            e[k] = bytes_to_half2(__byte_perm(w[k], 0u, 0x4240), offset);
+            o[k] = bytes_to_half2(__byte_perm(w[k], 0u, 0x4341), offset);
+        }
+        *low = make_uint4(e[0], e[1], e[2], e[3]);
+        low[total] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+}
+__device__ __noinline__ void rows_to_halves_call(uint8_t *planes, int64_t ldd, int64_t N,
+                                                 const float *rowscale, uint32_t offset) {
+    rows_to_halves(planes, ldd, N, rowscale, offset);
+}
+
 template <int FT, int ROWS, bool kW, int SUB, int NS, class Epi>
 __global__ void __launch_bounds__(kTcThreads, tc_blocks(FT, ROWS))
-spmm_tc_kernel(TcParams P, Epi epi) {
+spmm_tc_kernel(TcParams P, Epi epi, SecondKernel second) {
     using G = TcGeom<FT, SUB, NS>;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int next;        // windows of the block's share that its warps have taken
@@ -1174,6 +1363,14 @@ spmm_tc_kernel(TcParams P, Epi epi) {
     uint8_t *rings = smem + ((128u - (smem_addr(smem) & 127u)) & 127u);
     float *extra = reinterpret_cast<float *>(rings + kTcWarps * G::WARP);
     grid_dependency_wait();     // the dots and row scales come from the previous kernel
+    if (second.wide_rows != nullptr && many_wide(second.wide_rows, P.N, second.share)) {
+        if (blockIdx.y != 0) return;
+        // (called or inlined, by which the walk below it comes out faster: 128 features in
+        // one-row windows 1765 us called, 1817 inlined; 64 in eight-row windows 503, 464)
+        if (ROWS == 1) rows_to_halves_call(second.planes, P.ldd, P.N, P.rowscale, P.offset);
+        else rows_to_halves(second.planes, P.ldd, P.N, P.rowscale, P.offset);
+        return;
+    }
     epi.prologue(extra);
     __syncthreads();
     const int warp = threadIdx.x >> 5;
@@ -1204,8 +1401,8 @@ int64_t tc_heavy_degree(int64_t N, int64_t nnz) {
 }
 
 template <int FT, int ROWS, bool kW, class Epi>
-void launch_rows(const TcParams &P0, const Epi &epi, int slabs, const DeviceInfo &dev,
-                 cudaStream_t s, bool pdl) {
+void launch_rows(const TcParams &P0, const Epi &epi, const SecondKernel &second, int slabs,
+                 const DeviceInfo &dev, cudaStream_t s, bool pdl) {
     TcParams P = P0;
     P.heavy_degree = tc_heavy_degree(P.N, P.nnz);
     constexpr int SUB = tc_sub(FT, ROWS), NS = tc_stages(FT, ROWS);
@@ -1237,7 +1434,7 @@ void launch_rows(const TcParams &P0, const Epi &epi, int slabs, const DeviceInfo
         blocks = hb + need;
     }
     const dim3 grid(static_cast<unsigned>(blocks), static_cast<unsigned>(slabs));
-    launch_kernel(kernel, grid, dim3(kTcThreads), smem, s, pdl, dim3(1, 1, 1), P, epi);
+    launch_kernel(kernel, grid, dim3(kTcThreads), smem, s, pdl, dim3(1, 1, 1), P, epi, second);
 }
 
 // Rows per window: one when rows are long (a window's blocks then all belong to
@@ -1257,18 +1454,28 @@ bool tc_one_row(int64_t N, int64_t nnz, const DeviceInfo &dev) {
 }
 
 template <int FT, bool kW = false, class Epi>
-void launch_ft(const TcParams &P, const Epi &epi, const DeviceInfo &dev, cudaStream_t s,
-               bool pdl, int slabs = 1) {
-    if (tc_one_row(P.N, P.nnz, dev)) launch_rows<FT, 1, kW>(P, epi, slabs, dev, s, pdl);
-    else launch_rows<FT, kTcRows, kW>(P, epi, slabs, dev, s, pdl);
+void launch_ft(const TcParams &P, const Epi &epi, const SecondKernel &second,
+               const DeviceInfo &dev, cudaStream_t s, bool pdl, int slabs = 1) {
+    if (tc_one_row(P.N, P.nnz, dev)) launch_rows<FT, 1, kW>(P, epi, second, slabs, dev, s, pdl);
+    else launch_rows<FT, kTcRows, kW>(P, epi, second, slabs, dev, s, pdl);
 }
 
 TcParams tc_params(const int64_t *rowptr, const int32_t *colidx, int64_t N, int64_t nnz,
                    const uint8_t *D, int64_t ldd, const float *rowscale, int K) {
-    // ((K & 1) - 256) 2^-10 in fp16: -2^-2, or -255/1024
-    const uint32_t off = (K & 1) != 0 ? 0xB3F8u : 0xB400u;
-    return TcParams{rowptr, colidx, N,       nnz,     D,       ldd, int(ldd), rowscale,
-                    kAggGcn, nullptr, nullptr, off | (off << 16), 0, nullptr, 0, 0};
+    // 2^-10 in fp16, as often as a wide row's halves lack 1
+    const uint32_t bias = half_dot_bias(K) != 0 ? 0x1400u : 0u;
+    return TcParams{rowptr, colidx, N, nnz, D, ldd, int(ldd), rowscale, kAggGcn, nullptr, nullptr,
+                    byte_dot_offset(K), bias | (bias << 16), 0, nullptr, 0, 0};
+}
+
+// One wide row in how many is many, for the second kernel to take over: where it still
+// beats this one's walk and the wide rows' own by what they cost there. One-row windows
+// (232,965 nodes of mean degree 492, F = 128: 2690 us against 1790 without wide rows, and
+// 2560 with one in 256); eight-row windows, whose wide rows cost most, over 16-bit dots
+// that stay in L2 (100,003 nodes of mean degree 50, F = 100: 270 against 235, 324 with one
+// in 1024) or do not (2^20 of 16, F = 64: 1270 against 950, 1330 with one in 64).
+int many_wide_share(int64_t N, int64_t nnz, int F, const DeviceInfo &dev) {
+    return tc_one_row(N, nnz, dev) ? 256 : N * int64_t(F) * 2 <= (int64_t(96) << 20) ? 4096 : 128;
 }
 
 // Column slabs of at most 128 features, of equal width.
@@ -1279,6 +1486,9 @@ void launch_store(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bo
     P.values = a.values;
     P.dinv = a.dinv;
     P.counters = a.counters;
+    const SecondKernel second{spmm_tc_second_kernel(a.N, a.K, a.F) ? a.wide_rows : nullptr,
+                              many_wide_share(a.N, a.nnz, a.F, dev),
+                              const_cast<uint8_t *>(a.Ds != nullptr ? a.Ds : a.D)};
     const bool vec2 = a.ldh % 2 == 0 && aligned_to(a.H, 8);
     const int tiles = (a.F + 15) / 16, slabs = (tiles + 7) / 8;
     P.width = 16 * tiles;
@@ -1288,7 +1498,7 @@ void launch_store(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bo
         launch_ft<ft, kW>(P,                                                                   \
                           TcStore<ft>{a.H, a.ldh, a.F, a.colscale, a.pred, vec2, a.Ds, a.ldd,  \
                                       a.N * a.ldd, a.rowscale, a.colscale_s, a.K},             \
-                          dev, s, pdl, slabs);                                                 \
+                          second, dev, s, pdl, slabs);                                         \
         break;
         BIGCN_TC_CASE(1)
         BIGCN_TC_CASE(2)
@@ -1301,9 +1511,15 @@ void launch_store(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bo
 #undef BIGCN_TC_CASE
         default: break;
     }
+    if (second.wide_rows != nullptr) launch_spmm_halves(a, second.share, dev, s, pdl);
 }
 
 }  // namespace
+
+bool spmm_tc_second_kernel(int64_t N, int K, int F) {
+    // (halves that lack a bias are rare enough to be left to the tensor cores)
+    return half_dot_bias(K) == 0 && N * int64_t(F) >= (int64_t(4) << 20);
+}
 
 void launch_spmm_tc(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bool pdl) {
     if (a.N == 0) return;
@@ -1320,13 +1536,16 @@ void launch_spmm_tc_pack_gemm(const SpmmTcPackGemmArgs &a, const DeviceInfo &dev
     if (a.N == 0) return;
     TcParams P = tc_params(a.rowptr, a.colidx, a.N, a.nnz, a.D1, a.ldd1, a.s1, a.K);
     P.counters = a.counters;
+    const SecondKernel second{spmm_tc_second_kernel(a.N, a.K, a.Fh) ? a.wide_rows : nullptr,
+                              many_wide_share(a.N, a.nnz, a.Fh, dev),
+                              const_cast<uint8_t *>(a.D1)};
     const int words2 = (a.Fh + 63) / 64;
     switch ((a.Fh + 15) / 16) {
 #define BIGCN_TCPG_CASE(ft)                                                                 \
     case ft: {                                                                              \
         TcPackGemm<ft> e{a.H1, a.ldh1, a.Fh, a.beta1, a.wbits2, a.Fo, words2, a.D2, a.ldd2, \
                          a.s2};                                                             \
-        launch_ft<ft>(P, e, dev, s, pdl);                                                   \
+        launch_ft<ft>(P, e, second, dev, s, pdl);                                           \
         break;                                                                              \
     }
         BIGCN_TCPG_CASE(1)
@@ -1340,6 +1559,7 @@ void launch_spmm_tc_pack_gemm(const SpmmTcPackGemmArgs &a, const DeviceInfo &dev
 #undef BIGCN_TCPG_CASE
         default: break;
     }
+    if (second.wide_rows != nullptr) launch_spmm_halves_pack_gemm(a, second.share, dev, s, pdl);
 }
 
 }  // namespace bigcn

@@ -298,6 +298,7 @@ extern "C" bigcn_status bigcn_weighted_layer_forward(
     a.dinv = dinv;
     if (bytes) {
         g.dots8 = reinterpret_cast<uint8_t *>(ws + w.z);
+        g.wide_rows = control + kWideRowsWord;
         g.ldd8 = ldz;
         g.rowscale = reinterpret_cast<float *>(ws + w.rowscale);
     } else if (w.compressed) {
@@ -317,7 +318,8 @@ extern "C" bigcn_status bigcn_weighted_layer_forward(
     launch_xnor_gemm(g, dev, s, true);
     if (bytes) {
         SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, ldz, g.rowscale, F, K, H, ldh, beta,
-                     nullptr, kAggWeighted, nullptr, nullptr, values, dinv, control};
+                     nullptr, kAggWeighted, nullptr, nullptr, values, dinv, control,
+                     g.wide_rows};
         launch_spmm_tc(t, dev, s, true);
     } else {
         launch_spmm_norm(a, dev, s, true);

@@ -44,7 +44,8 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
                       int K, int words, float *__restrict__ Z, int64_t ldz,
                       int32_t *__restrict__ dots, const int64_t *__restrict__ rowptr,
                       uint16_t *__restrict__ dots16, int64_t ldd16, float *__restrict__ rowscale,
-                      uint8_t *__restrict__ dots8, int64_t ldd8, int half, int valid) {
+                      uint8_t *__restrict__ dots8, int64_t ldd8, int half, int valid,
+                      uint32_t *__restrict__ wide_rows) {
     constexpr int BN = 16 * TN;
     constexpr int kALoads = kBM * kBKW / kThreads;                         // 4
     constexpr int kBLoads = (BN * kBKW + kThreads - 1) / kThreads;          // 1..2
@@ -137,6 +138,7 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
         cluster.sync();   // peers keep their counts until every block has read them
     }
 
+    unsigned wides = 0;                     // this thread's share of the wide rows
 #pragma unroll
     for (int i = 0; i < kTM; ++i) {
         if (kSplit && i % S != rank) continue;
@@ -153,15 +155,18 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
                 float s = __ldg(alpha + row);
                 if (kDegreeScale) s *= inv_sqrt_degree(__ldg(rowptr + row + 1) - __ldg(rowptr + row));
                 rowscale[row] = flag_scale(s, wide);
+                wides += wide;
             }
-            uint8_t *lo = dots8 + row * ldd8 + n0 + tx;
 #pragma unroll
-            for (int j = 0; j < TN; ++j)
-                if (n0 + tx + 16 * j < F) {
-                    const ByteDot d(K - 2 * mism[i][j], K);
-                    lo[16 * j] = uint8_t(d.lo());
-                    if (wide) lo[N * ldd8 + 16 * j] = uint8_t(d.hi());
-                }
+            for (int j = 0; j < TN; ++j) {
+                const int col = n0 + tx + 16 * j, dot = K - 2 * mism[i][j];
+                if (col >= F) continue;
+                if (wide)
+                    *reinterpret_cast<uint16_t *>(dots8 + ((col & 1) * N + row) * ldd8 +
+                                                  (col & ~1)) = uint16_t(half_dot(dot, K));
+                else
+                    dots8[row * ldd8 + col] = uint8_t(ByteDot(dot, K).byte());
+            }
             continue;
         }
         if (row >= N) continue;
@@ -188,6 +193,10 @@ xnor_gemm_popc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ 
             if (dots != nullptr) dots[row * F + col] = d;
         }
     }
+    if (dots8 != nullptr) {
+        wides = __reduce_add_sync(kFullMask, wides);
+        if ((tid & 31) == 0 && wides != 0u) atomicAdd(wide_rows, wides);
+    }
 }
 
 template <int TN, bool kDeg>
@@ -206,13 +215,13 @@ void launch_tn(const GemmArgs &g, const DeviceInfo &dev, cudaStream_t s, bool pd
         launch_kernel(xnor_gemm_popc_kernel<TN, kDeg, false>, dim3(gx, gy), dim3(kThreads), 0, s,
                       pdl, dim3(1, 1, 1), g.A, g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z,
                       g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8,
-                      g.half > 0 ? g.half : INT32_MAX, g.half > 0 ? g.valid : g.F);
+                      g.half > 0 ? g.half : INT32_MAX, g.half > 0 ? g.valid : g.F, g.wide_rows);
         return;
     }
     launch_kernel(xnor_gemm_popc_kernel<TN, kDeg, true>, dim3(gx, gy, S), dim3(kThreads), 0, s,
                   pdl, dim3(1, 1, S), g.A, g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z,
                   g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8,
-                  g.half > 0 ? g.half : INT32_MAX, g.half > 0 ? g.valid : g.F);
+                  g.half > 0 ? g.half : INT32_MAX, g.half > 0 ? g.valid : g.F, g.wide_rows);
 }
 
 template <bool kDeg>

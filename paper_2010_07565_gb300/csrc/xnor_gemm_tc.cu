@@ -52,15 +52,16 @@ constexpr int kTcStages = 2;
 // below): each thread writes its row's low bytes, 16 columns to a 16-byte
 // store, and notes whether any of its dots is wide; the warps sharing a row
 // meet in shared memory, and only a warp that holds a wide row reads tensor
-// memory again to write that row's high plane.
+// memory again to write that row's halves over its bytes and in the high plane.
 template <int NT, int kHalves, int kWarps, bool kDeg>
 __device__ __forceinline__ void tc_epilogue_bytes(uint32_t tmem, int warp, int lane, int64_t m0,
                                                   int n0, int64_t N,
                                                   const float *__restrict__ alpha,
                                                   const int64_t *__restrict__ rowptr, int F,
                                                   float *__restrict__ rowscale,
-                                                  uint8_t *__restrict__ dots8, int64_t ldd8, int K, int half,
-                                                  int valid) {
+                                                  uint8_t *__restrict__ dots8, int64_t ldd8,
+                                                  int K, int half, int valid,
+                                                  uint32_t *__restrict__ wide_rows) {
     constexpr int kSplit = kWarps / (4 * kHalves);     // warps sharing a row
     __shared__ uint8_t wide_s[kSplit][kUmmaM * kHalves];
     const int quad = warp & 3;
@@ -71,25 +72,19 @@ __device__ __forceinline__ void tc_epilogue_bytes(uint32_t tmem, int warp, int l
     const uint32_t taddr = tmem + (uint32_t(32 * quad) << 16) + uint32_t(hsel * NT);
     const int cols = min(F - n0, NT);                  // columns of this tile
     uint8_t *dr = dots8 + row * ldd8 + n0;
-    auto slice = [&](int c0, bool high) -> bool {      // 16 columns: store, any wide?
-        uint32_t acc[16];
+    bool wide = false;
+#pragma unroll 1
+    for (int c0 = 16 * cs; c0 < cols; c0 += 16 * kSplit) {
+        uint32_t acc[16], u[4] = {0u, 0u, 0u, 0u};
         tmem_ld16(taddr + uint32_t(c0), acc);
-        bool w = false;
-        uint32_t u[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
             const ByteDot d(__float2int_rn(__uint_as_float(acc[e])), K);
-            w |= d.wide() && flag_column(n0 + c0 + e, half, valid);
-            u[e / 4] |= (high ? d.hi() & 255u : d.lo()) << (8 * (e % 4));
+            wide |= d.wide() && flag_column(n0 + c0 + e, half, valid);
+            u[e / 4] |= d.byte() << (8 * (e % 4));
         }
-        if (row < N)
-            *reinterpret_cast<uint4 *>(dr + (high ? N * ldd8 : 0) + c0) =
-                make_uint4(u[0], u[1], u[2], u[3]);
-        return w;
-    };
-    bool wide = false;
-#pragma unroll 1
-    for (int c0 = 16 * cs; c0 < cols; c0 += 16 * kSplit) wide |= slice(c0, false);
+        if (row < N) *reinterpret_cast<uint4 *>(dr + c0) = make_uint4(u[0], u[1], u[2], u[3]);
+    }
     wide_s[cs][r] = uint8_t(wide && row < N);
     asm volatile("bar.sync 1, %0;" ::"n"(32 * kWarps) : "memory");     // the epilogue's warps
     wide = false;
@@ -100,9 +95,23 @@ __device__ __forceinline__ void tc_epilogue_bytes(uint32_t tmem, int warp, int l
         if (kDeg) ai *= inv_sqrt_degree(__ldg(rowptr + row + 1) - __ldg(rowptr + row));
         rowscale[row] = flag_scale(ai, wide);
     }
-    if (__any_sync(kFullMask, wide))
+    const unsigned wides = __ballot_sync(kFullMask, wide);
+    if (wides == 0u) return;
+    if (n0 == 0 && cs == 0 && lane == 0) atomicAdd(wide_rows, unsigned(__popc(wides)));
 #pragma unroll 1
-        for (int c0 = 16 * cs; c0 < cols; c0 += 16 * kSplit) slice(c0, true);
+    for (int c0 = 16 * cs; c0 < cols; c0 += 16 * kSplit) {
+        uint32_t acc[16], u[2][4] = {};         // halves of the even and of the odd columns
+        tmem_ld16(taddr + uint32_t(c0), acc);
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+            u[e & 1][e / 4] |= half_dot(__float2int_rn(__uint_as_float(acc[e])), K)
+                               << (16 * (e / 2 % 2));
+        if (wide)
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+                *reinterpret_cast<uint4 *>(dr + p * N * ldd8 + c0) =
+                    make_uint4(u[p][0], u[p][1], u[p][2], u[p][3]);
+    }
 }
 
 // Epilogue of a product tile by kWarps warps: warp w reads tensor-memory lanes
@@ -121,10 +130,12 @@ __device__ __forceinline__ void tc_epilogue(uint32_t tmem, int warp, int lane, i
                                             uint16_t *__restrict__ dots16, int64_t ldd16,
                                             float *__restrict__ rowscale,
                                             uint8_t *__restrict__ dots8, int64_t ldd8, int K,
-                                            int half, int valid) {
+                                            int half, int valid,
+                                            uint32_t *__restrict__ wide_rows) {
     if (dots8 != nullptr) {     // byte planes (one column tile, or no wide dots)
         tc_epilogue_bytes<NT, kHalves, kWarps, kDeg>(tmem, warp, lane, m0, n0, N, alpha, rowptr, F,
-                                                     rowscale, dots8, ldd8, K, half, valid);
+                                                     rowscale, dots8, ldd8, K, half, valid,
+                                                     wide_rows);
         return;
     }
     const bool vec_z = (ldz & 3) == 0 && (reinterpret_cast<uintptr_t>(Z) & 15) == 0;
@@ -208,7 +219,8 @@ xnor_gemm_tc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ al
                     int words, float *__restrict__ Z, int64_t ldz, int32_t *__restrict__ dots,
                     const int64_t *__restrict__ rowptr, uint16_t *__restrict__ dots16,
                     int64_t ldd16, float *__restrict__ rowscale, uint8_t *__restrict__ dots8,
-                    int64_t ldd8, int half, int valid, const uint8_t *__restrict__ bexp) {
+                    int64_t ldd8, int half, int valid, uint32_t *__restrict__ wide_rows,
+                    const uint8_t *__restrict__ bexp) {
     constexpr int kStageA = kUmmaM * kTcKBytes;
     constexpr int kStageB = NT * kTcKBytes;
     constexpr int kStage = kStageA + kStageB;
@@ -372,7 +384,7 @@ xnor_gemm_tc_kernel(const uint64_t *__restrict__ A, const float *__restrict__ al
     if (ok)
         tc_epilogue<NT, 1, kTcThreads / 32, kDeg>(tmem, warp, lane, m0, n0, N, alpha, rowptr, beta, F,
                                                   Z, ldz, dots, dots16, ldd16, rowscale, dots8, ldd8,
-                                                  K, half, valid);
+                                                  K, half, valid, wide_rows);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
@@ -415,7 +427,7 @@ xnor_gemm_tc_ws_kernel(const uint64_t *__restrict__ A, const float *__restrict__
                        const int64_t *__restrict__ rowptr, uint16_t *__restrict__ dots16,
                        int64_t ldd16, float *__restrict__ rowscale, uint8_t *__restrict__ dots8,
                        int64_t ldd8, int half, int valid,
-                       const uint8_t *__restrict__ bexp) {
+                       uint32_t *__restrict__ wide_rows, const uint8_t *__restrict__ bexp) {
     constexpr int NT = kWsCols;
     constexpr int kStageA = kWsRows * kTcKBytes;        // two 128-row halves
     constexpr int kStageB = NT * kTcKBytes;
@@ -593,7 +605,7 @@ xnor_gemm_tc_ws_kernel(const uint64_t *__restrict__ A, const float *__restrict__
     if (ok && warp < kWsExpWarps)
         tc_epilogue<NT, 2, kWsExpWarps, kDeg>(tmem, warp, lane, m0, n0, N, alpha, rowptr, beta, F, Z,
                                               ldz, dots, dots16, ldd16, rowscale, dots8, ldd8, K, half,
-                                              valid);
+                                              valid, wide_rows);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == kMmaWarp)
@@ -657,7 +669,8 @@ void launch_nt2(const GemmArgs &g, cudaStream_t s, bool pdl) {
     launch_kernel(kernel, grid, dim3(kTcThreads), smem, s, pdl || kBexp, dim3(1, 1, 1), g.A,
                   g.alpha, g.N, g.B, g.beta, g.F, g.K, g.words, g.Z, g.ldz, g.dots, g.rowptr,
                   g.dots16, g.ldd16, g.rowscale, g.dots8, g.ldd8, g.half > 0 ? g.half : INT32_MAX,
-                  g.half > 0 ? g.valid : g.F, static_cast<const uint8_t *>(g.b_e4m3));
+                  g.half > 0 ? g.valid : g.F, g.wide_rows,
+                  static_cast<const uint8_t *>(g.b_e4m3));
 }
 
 template <bool kDeg>
@@ -672,7 +685,8 @@ void launch_ws(const GemmArgs &g, cudaStream_t s, bool pdl) {
     launch_kernel(kernel, grid, dim3(kWsThreads), smem, s, true, dim3(1, 1, 1), g.A, g.alpha, g.N,
                   g.beta, g.F, g.K, g.words, g.Z, g.ldz, g.dots, g.rowptr, g.dots16, g.ldd16,
                   g.rowscale, g.dots8, g.ldd8, g.half > 0 ? g.half : INT32_MAX,
-                  g.half > 0 ? g.valid : g.F, static_cast<const uint8_t *>(g.b_e4m3));
+                  g.half > 0 ? g.valid : g.F, g.wide_rows,
+                  static_cast<const uint8_t *>(g.b_e4m3));
 }
 
 template <int NT, bool kDeg>

@@ -1,0 +1,95 @@
+"""Calls large enough that a second kernel stands by for data with many wide rows (byte
+dots: see test_gpu_byte_dots.py), on both sides of the share from which it takes over: every
+row wide, some, few (left to the tensor-core walk's own pass), none. And wide rows whose
+halves lack one of the dot (odd K above 2048)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_helpers import check_sum, to_dev
+from paper_2010_07565_gb300 import binding as B
+from paper_2010_07565_gb300 import inputs
+from test_gpu_byte_dots import planted_case, sampled
+
+pytestmark = pytest.mark.gpu
+
+
+def layer(dev, agg, c, seed):
+    N, K = c["X"].shape
+    F = c["W"].shape[1]
+    rp, ci = c["rowptr"], c["colidx"]
+    d = {k: to_dev(v) for k, v in c.items() if v is not None}
+    H = torch.full((N, F), float("nan"), device=dev)
+    rows = sampled(N, 500, seed)
+    ws = lambda n: torch.full((n,), 0xAB, dtype=torch.uint8, device=dev)
+    if agg == "weighted":
+        v = inputs.edge_weights(rp, ci, seed)
+        B.bigcn_weighted_layer_forward(d["X"], None, None, d["W"], d["rowptr"], d["colidx"],
+                                       to_dev(v), ws(B.bigcn_weighted_layer_workspace_bytes(N, K, F)),
+                                       H)
+        ref = oracle.layer_forward_weighted(c["X"], c["W"], rp, ci, v, rows=rows)
+    elif agg == "gcn":
+        B.bigcn_layer_forward(d["X"], None, None, d["W"], d["rowptr"], d["colidx"],
+                              ws(B.bigcn_layer_workspace_bytes(N, K, F)), H)
+        ref = oracle.layer_forward(c["X"], c["W"], rp, ci, rows=rows)
+    else:
+        Wn = inputs.weights(K, F, seed=seed) if agg == "sage" else None
+        B.bigcn_inductive_layer_forward(agg, d["X"], None, None, d["W"], d["rowptr"], d["colidx"],
+                                        ws(B.bigcn_inductive_layer_workspace_bytes(agg, N, K, F)),
+                                        H, W_neigh=to_dev(Wn))
+        ref = oracle.layer_forward_inductive(c["X"], c["W"], rp, ci, agg, W_neigh=Wn, rows=rows)
+    torch.cuda.synchronize()
+    assert B.device_timeouts() == 0
+    check_sum(H.cpu().numpy()[rows], ref["H"], ref["absterm"],
+              f"{agg} layer, wide rows {N}x{K}x{F}", int(np.diff(rp)[rows].max()) + 2)
+
+
+# (N, K, F, mean degree, hub): N F of 4 million and more; eight-row windows, one-row windows,
+# two column slabs, few features
+SIZES = [(66003, 300, 64, 6.0, 400), (33001, 511, 127, 70.0, 3000), (30011, 600, 144, 70.0, 0),
+         (281003, 260, 15, 3.0, 90)]
+
+
+@pytest.mark.parametrize("agg", ["gcn", "mean", "sage", "weighted"])
+@pytest.mark.parametrize("every", [1, 3, 100, 20000])
+@pytest.mark.parametrize("N,K,F,deg,hub", SIZES)
+def test_layer(cuda_device, agg, N, K, F, deg, hub, every):
+    if agg == "sage" and F > 128:
+        F = 128
+    layer(cuda_device, agg, planted_case(N, K, F, deg, hub, every, seed=N + K + every), K + every)
+
+
+@pytest.mark.parametrize("agg", ["gcn", "mean", "sage", "weighted"])
+@pytest.mark.parametrize("N,K,F,deg", [(1500, 2049, 64, 80.0), (2500, 2305, 48, 6.0),
+                                       (2500, 3071, 64, 6.0), (152 * 128 + 5, 2051, 64, 6.0)])
+@pytest.mark.parametrize("every", [1, 7])
+def test_odd_dots_beyond_fp16(cuda_device, agg, N, K, F, deg, every):
+    layer(cuda_device, agg, planted_case(N, K, F, deg, 300, every, seed=N + K + every), K + every)
+
+
+@pytest.mark.parametrize("N,K,Fh,Fo,deg,every", [
+    (66003, 300, 64, 7, 6.0, 2), (66003, 300, 64, 16, 6.0, 100), (33001, 602, 127, 41, 70.0, 3),
+    (33001, 602, 128, 64, 70.0, 1), (270001, 260, 16, 3, 3.0, 5), (66003, 300, 64, 7, 6.0, 30000)])
+def test_forward(cuda_device, N, K, Fh, Fo, deg, every):
+    c = planted_case(N, K, Fh, deg, 900, every, seed=N + K + Fo)
+    W2 = inputs.weights(Fh, Fo, seed=N + 1)
+    d = {k: to_dev(v) for k, v in c.items() if v is not None}
+    ws = torch.full((B.bigcn_forward_2layer_workspace_bytes(N, K, Fh, Fo),), 0xAB,
+                    dtype=torch.uint8, device=cuda_device)
+    out = torch.full((N, Fo), float("nan"), device=cuda_device)
+    pred = torch.full((N,), -1, dtype=torch.int32, device=cuda_device)
+    for H1 in (None, torch.full((N, Fh), float("nan"), device=cuda_device)):
+        B.bigcn_forward_2layer(d["X"], None, None, d["W"], to_dev(W2), d["rowptr"], d["colidx"],
+                               ws, out, H1=H1, pred=pred)
+        if H1 is None:
+            first = out.clone()
+    assert torch.equal(first, out)
+    rows = sampled(N, 400, K)
+    r1 = oracle.layer_forward(c["X"], c["W"], c["rowptr"], c["colidx"], rows=rows)
+    n = int(np.diff(c["rowptr"]).max()) + 1
+    check_sum(H1.cpu().numpy()[rows], r1["H"], r1["absterm"], f"many wide rows H1 {N}x{K}x{Fh}", n)
+    # Layer 2 on the GPU's own H1 (signs of values within rounding of zero may differ).
+    r2 = oracle.layer_forward(H1.cpu().numpy(), W2, c["rowptr"], c["colidx"], rows=rows)
+    check_sum(out.cpu().numpy()[rows], r2["H"], r2["absterm"], f"many wide rows logits {N}x{Fo}", n)
+    assert np.array_equal(pred.cpu().numpy(), out.cpu().numpy().argmax(1))
