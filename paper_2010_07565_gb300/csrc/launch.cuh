@@ -185,10 +185,11 @@ struct SpmmArgs {
 void launch_spmm_norm(const SpmmArgs &args, const DeviceInfo &dev, cudaStream_t stream,
                       bool pdl = false);
 // The weighted degrees of A + I (weighted.cu): dinv_i = 1/sqrt(1 + sum of
-// row i's values) and, when alpha is given, s_i = alpha_i dinv_i.
+// row i's values) and, when alpha is given, s_i = alpha_i dinv_i. *spread_rows (nullable)
+// is raised by the number of rows whose weights lie 2^21 and more apart.
 void launch_weighted_dinv(const int64_t *rowptr, const float *values, int64_t N, int64_t nnz,
-                          const float *alpha, float *dinv, float *s, cudaStream_t stream,
-                          bool pdl = false);
+                          const float *alpha, float *dinv, float *s, uint32_t *spread_rows,
+                          cudaStream_t stream, bool pdl = false);
 
 struct FrontArgs {
     const float *X;          // N x K (row stride ldx)
@@ -293,8 +294,9 @@ struct SpmmTcArgs {
     // Nullable: kTcCounters words that an earlier kernel of the call has set to
     // zero, from which all blocks take their windows (else each block its share).
     uint32_t *counters = nullptr;
-    // The number of wide rows (nullptr: none is). Where many are, the kernel leaves the
-    // aggregation to a second one (spmm_tc_second_kernel).
+    // The number of wide rows (nullptr: none is), for a weighted A that of rows with weights
+    // very unlike one another added: both cost the kernel further passes. Where there are
+    // many it leaves the aggregation to a second one (spmm_tc_second_kernel).
     const uint32_t *wide_rows = nullptr;
 };
 void launch_spmm_tc(const SpmmTcArgs &args, const DeviceInfo &dev, cudaStream_t stream,
@@ -305,8 +307,10 @@ void launch_spmm_tc(const SpmmTcArgs &args, const DeviceInfo &dev, cudaStream_t 
 // (launch_spmm_halves) is always launched behind the first and ends at once unless many
 // rows are wide (about 1.5 us); then the first only turns the other rows into halves.
 // 232,965 nodes of mean degree 492, K = 602, F = 128, a layer: no wide row 1790 us, one in
-// 256 2560, one in 16 3580, all 9800; with the second kernel 2690 from one in 256 on.
-bool spmm_tc_second_kernel(int64_t N, int K, int F);
+// 256 2560, one in 16 3580, all 9800; with the second kernel 2600 from one in 256 on.
+// Weights of 1e-8 to 1 on 100,003 nodes of mean degree 50, F = 100: 644 without, 264 with it.
+// nnz: 0 where it shall not count (a launch count that does not know it).
+bool spmm_tc_second_kernel(int64_t N, int64_t nnz, int K, int F);
 
 // Layer 1's tensor-core aggregation fused with layer 2's binarization and
 // XNOR product (spmm_tc.cu): from layer 1's byte planes D1 (row scale s1,

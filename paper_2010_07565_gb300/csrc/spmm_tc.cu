@@ -1359,6 +1359,8 @@ spmm_tc_kernel(TcParams P, Epi epi, SecondKernel second) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int next;        // windows of the block's share that its warps have taken
     if (threadIdx.x == 0) next = 0;
+    // (the second kernel waits for this one's end; its launch need not)
+    if (second.wide_rows != nullptr) allow_dependent_launch();
     // The rings start on a 128-byte line (the ldmatrix addressing relies on it).
     uint8_t *rings = smem + ((128u - (smem_addr(smem) & 127u)) & 127u);
     float *extra = reinterpret_cast<float *>(rings + kTcWarps * G::WARP);
@@ -1486,7 +1488,7 @@ void launch_store(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bo
     P.values = a.values;
     P.dinv = a.dinv;
     P.counters = a.counters;
-    const SecondKernel second{spmm_tc_second_kernel(a.N, a.K, a.F) ? a.wide_rows : nullptr,
+    const SecondKernel second{spmm_tc_second_kernel(a.N, a.nnz, a.K, a.F) ? a.wide_rows : nullptr,
                               many_wide_share(a.N, a.nnz, a.F, dev),
                               const_cast<uint8_t *>(a.Ds != nullptr ? a.Ds : a.D)};
     const bool vec2 = a.ldh % 2 == 0 && aligned_to(a.H, 8);
@@ -1516,9 +1518,10 @@ void launch_store(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bo
 
 }  // namespace
 
-bool spmm_tc_second_kernel(int64_t N, int K, int F) {
+bool spmm_tc_second_kernel(int64_t N, int64_t nnz, int K, int F) {
     // (halves that lack a bias are rare enough to be left to the tensor cores)
-    return half_dot_bias(K) == 0 && N * int64_t(F) >= (int64_t(4) << 20);
+    return half_dot_bias(K) == 0 && (N * int64_t(F) >= (int64_t(4) << 20) ||
+                                     double(nnz) * F >= double(int64_t(128) << 20));
 }
 
 void launch_spmm_tc(const SpmmTcArgs &a, const DeviceInfo &dev, cudaStream_t s, bool pdl) {
@@ -1536,7 +1539,7 @@ void launch_spmm_tc_pack_gemm(const SpmmTcPackGemmArgs &a, const DeviceInfo &dev
     if (a.N == 0) return;
     TcParams P = tc_params(a.rowptr, a.colidx, a.N, a.nnz, a.D1, a.ldd1, a.s1, a.K);
     P.counters = a.counters;
-    const SecondKernel second{spmm_tc_second_kernel(a.N, a.K, a.Fh) ? a.wide_rows : nullptr,
+    const SecondKernel second{spmm_tc_second_kernel(a.N, 0, a.K, a.Fh) ? a.wide_rows : nullptr,
                               many_wide_share(a.N, a.nnz, a.Fh, dev),
                               const_cast<uint8_t *>(a.D1)};
     const int words2 = (a.Fh + 63) / 64;

@@ -40,9 +40,25 @@ struct Compensated {
     __device__ __forceinline__ float value() const { return sum - lost; }
 };
 
+// The smallest (bits, less 1) and the largest (bits) of weights other than 0, the
+// self-loop's 1 among them.
+struct Spread {
+    uint32_t low = 0x3F800000u - 1u, high = 0x3F800000u;
+    __device__ __forceinline__ void add(float v) {
+        const uint32_t b = __float_as_uint(v) & 0x7fffffffu;
+        low = min(low, b - 1u);
+        high = max(high, b);
+    }
+    // So far apart (2^21 and more) that the tensor-core aggregation would take the row in
+    // several passes, the row scales' own spread added.
+    __device__ __forceinline__ bool far_apart() const {
+        return int(high >> 23) - int((low + 1u) >> 23) > 20;
+    }
+};
+
 // Sum of values[q] for q = q0, q0 + stride, ... below q1, four loads in flight.
 __device__ __forceinline__ float strided_sum(const float *__restrict__ values, int64_t q0,
-                                             int64_t q1, int stride) {
+                                             int64_t q1, int stride, Spread &spread) {
     Compensated c;
     for (int64_t q = q0; q < q1; q += 4 * int64_t(stride)) {
         float v[4];
@@ -52,7 +68,10 @@ __device__ __forceinline__ float strided_sum(const float *__restrict__ values, i
             v[k] = qk < q1 ? __ldg(values + qk) : 0.0f;
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) c.add(v[k]);
+        for (int k = 0; k < 4; ++k) {
+            c.add(v[k]);
+            spread.add(v[k]);
+        }
     }
     return c.value();
 }
@@ -71,8 +90,10 @@ constexpr int64_t kDegShort = 256;
 __global__ void __launch_bounds__(kDegThreads)
 weighted_dinv_kernel(const int64_t *__restrict__ rowptr, const float *__restrict__ values,
                      int64_t N, int64_t nnz, const float *__restrict__ alpha,
-                     float *__restrict__ dinv, float *__restrict__ s) {
+                     float *__restrict__ dinv, float *__restrict__ s,
+                     uint32_t *__restrict__ spread_rows) {
     __shared__ float part[kDegWarps];
+    __shared__ uint32_t part_low[kDegWarps], part_high[kDegWarps];
     constexpr int kBlockRows = kDegWarps * kDegRows;
     static_assert(kBlockRows == 32, "a lane per row of the block");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -88,11 +109,17 @@ weighted_dinv_kernel(const int64_t *__restrict__ rowptr, const float *__restrict
     const int own = lane / kDegLanes, sub = lane % kDegLanes;
     const int row = warp * kDegRows + own;          // this lane group's row
     const int64_t rb = __shfl_sync(kFullMask, b, row), re = __shfl_sync(kFullMask, e, row);
-    float v = re - rb <= kDegShort ? strided_sum(values, rb + sub, re, kDegLanes) : 0.0f;
+    Spread sp;
+    float v = re - rb <= kDegShort ? strided_sum(values, rb + sub, re, kDegLanes, sp) : 0.0f;
 #pragma unroll
-    for (int o = 1; o < kDegLanes; o <<= 1) v += __shfl_xor_sync(kFullMask, v, o);
+    for (int o = 1; o < kDegLanes; o <<= 1) {
+        v += __shfl_xor_sync(kFullMask, v, o);
+        sp.low = min(sp.low, __shfl_xor_sync(kFullMask, sp.low, o));
+        sp.high = max(sp.high, __shfl_xor_sync(kFullMask, sp.high, o));
+    }
     v = __shfl_sync(kFullMask, v, (lane % kDegRows) * kDegLanes);
     if (lane / kDegRows == warp) total = v;
+    unsigned far = __popc(__ballot_sync(kFullMask, sub == 0 && sp.far_apart()));  // rows of the warp
     // The warp's longer rows, and the block's heaviest.
     unsigned longer = __ballot_sync(kFullMask, e - b > kDegShort && e - b <= kDegHeavy) &
                       (((1u << kDegRows) - 1u) << (warp * kDegRows));
@@ -100,17 +127,35 @@ weighted_dinv_kernel(const int64_t *__restrict__ rowptr, const float *__restrict
         const int r = __ffs(longer) - 1;
         longer &= longer - 1u;
         const int64_t lb = __shfl_sync(kFullMask, b, r), le = __shfl_sync(kFullMask, e, r);
-        const float t = warp_sum(strided_sum(values, lb + lane, le, 32));
+        Spread ls;
+        const float t = warp_sum(strided_sum(values, lb + lane, le, 32, ls));
         if (lane == r) total = t;
+        ls.low = __reduce_min_sync(kFullMask, ls.low);
+        ls.high = __reduce_max_sync(kFullMask, ls.high);
+        far += ls.far_apart();
     }
     unsigned heavy = __ballot_sync(kFullMask, e - b > kDegHeavy);
     while (heavy != 0u) {
         const int r = __ffs(heavy) - 1;
         heavy &= heavy - 1u;
         const int64_t lb = __shfl_sync(kFullMask, b, r), le = __shfl_sync(kFullMask, e, r);
-        const float t = warp_sum(strided_sum(values, lb + threadIdx.x, le, kDegThreads));
-        if (lane == 0) part[warp] = t;
+        Spread ls;
+        const float t = warp_sum(strided_sum(values, lb + threadIdx.x, le, kDegThreads, ls));
+        ls.low = __reduce_min_sync(kFullMask, ls.low);
+        ls.high = __reduce_max_sync(kFullMask, ls.high);
+        if (lane == 0) {
+            part[warp] = t;
+            part_low[warp] = ls.low;
+            part_high[warp] = ls.high;
+        }
         __syncthreads();
+        if (warp == 0) {
+            for (int w = 1; w < kDegWarps; ++w) {
+                ls.low = min(ls.low, part_low[w]);
+                ls.high = max(ls.high, part_high[w]);
+            }
+            far += ls.far_apart();
+        }
         if (lane == r) {
             total = 0.0f;
             for (int w = 0; w < kDegWarps; ++w) total += part[w];
@@ -118,6 +163,7 @@ weighted_dinv_kernel(const int64_t *__restrict__ rowptr, const float *__restrict
         __syncthreads();    // part[] is rewritten by the next heavy row
     }
     grid_dependency_wait();     // alpha is the row packing's output
+    if (spread_rows != nullptr && lane == 0 && far != 0u) atomicAdd(spread_rows, far);
     const int64_t i = i0 + lane;
     if (lane / kDegRows == warp && i < N) {
         const float r = 1.0f / sqrtf(1.0f + total);
@@ -168,12 +214,13 @@ bool weighted_workspace(int64_t N, int32_t K, int32_t F, WeightedWorkspace *w) {
 
 namespace bigcn {
 void launch_weighted_dinv(const int64_t *rowptr, const float *values, int64_t N, int64_t nnz,
-                          const float *alpha, float *dinv, float *s, cudaStream_t stream, bool pdl) {
+                          const float *alpha, float *dinv, float *s, uint32_t *spread_rows,
+                          cudaStream_t stream, bool pdl) {
     if (N == 0) return;
     const int64_t rows = int64_t(kDegWarps) * kDegRows;
     const dim3 grid(unsigned((N + rows - 1) / rows));
     launch_kernel(weighted_dinv_kernel, grid, dim3(kDegThreads), 0, stream, pdl, dim3(1, 1, 1),
-                  rowptr, values, N, nnz, alpha, dinv, s);
+                  rowptr, values, N, nnz, alpha, dinv, s, spread_rows);
 }
 }  // namespace bigcn
 
@@ -190,7 +237,7 @@ extern "C" bigcn_status bigcn_weighted_dinv(const int64_t *rowptr, const float *
     DeviceInfo dev;
     const bigcn_status st = current_device(&dev);
     if (st != BIGCN_OK) return st;
-    launch_weighted_dinv(rowptr, values, N, nnz, nullptr, dinv, nullptr, as_stream(stream));
+    launch_weighted_dinv(rowptr, values, N, nnz, nullptr, dinv, nullptr, nullptr, as_stream(stream));
     return launch_status();
 }
 
@@ -283,8 +330,9 @@ extern "C" bigcn_status bigcn_weighted_layer_forward(
     // drains (each waits for it before it reads anything the call has written).
     // Factored rows carry dinv_j in their row scale (s_j = alpha_j dinv_j);
     // fp32 rows are the plain product and the aggregation reads dinv_j.
-    launch_weighted_dinv(rowptr, values, N, nnz, alpha, dinv, w.compressed ? srow : nullptr, s,
-                         true);
+    // (rows of very unlike weights count as wide rows do: see SpmmTcArgs)
+    launch_weighted_dinv(rowptr, values, N, nnz, alpha, dinv, w.compressed ? srow : nullptr,
+                         control + kWideRowsWord, s, true);
     const bool bytes = w.planes && planes_faster(N, nnz, F) &&
                        xnor_gemm_bytes_supported(N, K, F, dev);
     // (uint16 dots are padded to 8 columns even where the workspace has room for 16)

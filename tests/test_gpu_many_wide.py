@@ -93,3 +93,34 @@ def test_forward(cuda_device, N, K, Fh, Fo, deg, every):
     r2 = oracle.layer_forward(H1.cpu().numpy(), W2, c["rowptr"], c["colidx"], rows=rows)
     check_sum(out.cpu().numpy()[rows], r2["H"], r2["absterm"], f"many wide rows logits {N}x{Fo}", n)
     assert np.array_equal(pred.cpu().numpy(), out.cpu().numpy().argmax(1))
+
+
+@pytest.mark.parametrize("N,F,deg,hub", [(66003, 64, 6.0, 400), (33001, 127, 70.0, 5000)])
+@pytest.mark.parametrize("every", [1, 50, 40000])
+def test_unlike_weights(cuda_device, N, F, deg, hub, every):
+    """Rows of weights up to 1e20 apart: all (left to the second kernel), some, few; each
+    column held to the magnitudes of its own terms."""
+    K = 200
+    c = inputs.layer_case(N, K, F, seed=N, mean_degree=deg, hub_degree=hub, centred=False)
+    rp, ci = c["rowptr"], c["colidx"]
+    v = inputs.edge_weights(rp, ci, 3)
+    row = np.repeat(np.arange(N), np.diff(rp))
+    g = np.random.default_rng(N)
+    v = np.where(row % every == 0, v * 10.0 ** g.integers(-10, 11, len(v)), v).astype(np.float32)
+    d = {k: to_dev(x) for k, x in c.items() if x is not None}
+    H = torch.full((N, F), float("nan"), device=cuda_device)
+    ws = torch.full((B.bigcn_weighted_layer_workspace_bytes(N, K, F),), 0xAB, dtype=torch.uint8,
+                    device=cuda_device)
+    B.bigcn_weighted_layer_forward(d["X"], None, None, d["W"], d["rowptr"], d["colidx"], to_dev(v),
+                                   ws, H)
+    # fp64 on the GPU, over the exact dots
+    S = torch.where(d["X"] >= 0, 1.0, -1.0).double()
+    Z = (S @ torch.where(d["W"] >= 0, 1.0, -1.0).double()) * d["X"].double().abs().mean(
+        1, keepdim=True) * d["W"].double().abs().mean(0)
+    A = torch.sparse_csr_tensor(d["rowptr"], d["colidx"].long(), to_dev(v).double(), (N, N))
+    dinv = 1.0 / torch.sqrt(1.0 + A @ torch.ones((N, 1), dtype=torch.float64, device=cuda_device))
+    ref = dinv * (Z * dinv + A @ (Z * dinv))
+    mag = dinv * (Z.abs() * dinv + A @ (Z.abs() * dinv))
+    n = int(np.diff(rp).max()) + 8
+    bad = (H.double() - ref).abs() > n * (2.0 ** -23 * mag + 2.0 ** -149)
+    assert not bool(bad.any()), int(bad.sum())
