@@ -45,9 +45,10 @@ def layer(dev, agg, c, seed):
               f"{agg} layer, wide rows {N}x{K}x{F}", int(np.diff(rp)[rows].max()) + 2)
 
 
-# (N, K, F, mean degree, hub): N F of 4 million and more; eight-row windows, one-row windows,
-# two column slabs, few features
-SIZES = [(66003, 300, 64, 6.0, 400), (33001, 511, 127, 70.0, 3000), (30011, 600, 144, 70.0, 0),
+# (N, K, F, mean degree, hub): N F of 4 million and more; eight-row windows taken from one
+# counter by persistent blocks that also walk the heavy rows, one-row windows, two column
+# slabs, few features
+SIZES = [(110011, 300, 47, 12.0, 900), (33001, 511, 127, 70.0, 3000), (30011, 600, 144, 70.0, 0),
          (281003, 260, 15, 3.0, 90)]
 
 

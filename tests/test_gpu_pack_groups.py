@@ -49,3 +49,24 @@ def test_rows_longer_than_their_signs(cuda_device, together, K, words):
     n = (K + 63) // 64
     assert np.array_equal(got[:, :n], np.asarray(oracle.pack(oracle.sign(X))).view(np.uint64))
     assert not got[:, n:].any()
+
+
+@pytest.mark.parametrize("K", [2048, 2049, 2354])
+@pytest.mark.parametrize("centred", [False, True])
+@pytest.mark.parametrize("extra", [-1, 0, 3])
+def test_long_rows_packed_four_together(cuda_device, K, centred, extra):
+    """From 2048 features eight chunks of each row at a time, with a last, partial batch."""
+    N = 4 * PER_ROW * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    gen = torch.Generator(device=cuda_device)
+    gen.manual_seed(K)
+    X = torch.randn((N, K), generator=gen, device=cuda_device)
+    s = 0.5 + torch.rand(K, generator=gen, device=cuda_device) if centred else None
+    t = torch.randn(K, generator=gen, device=cuda_device) if centred else None
+    bits, alpha = B.pack_rows(X, s, t)
+    rows = np.unique(np.concatenate([np.arange(9), np.arange(N - 9, N), np.arange(0, N, 97)]))
+    cpu = lambda a: None if a is None else a.cpu().numpy()
+    Y = oracle.centre(X[rows].cpu().numpy(), cpu(s), cpu(t)) if centred else X[rows].cpu().numpy()
+    assert np.array_equal(bits.cpu().numpy().view(np.uint64)[rows],
+                          np.asarray(oracle.pack(oracle.sign(Y))).view(np.uint64))
+    assert np.allclose(alpha.cpu().numpy()[rows], oracle.row_scale(Y), rtol=(K + 2) * 2.0 ** -24,
+                       atol=0)
