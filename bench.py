@@ -188,9 +188,11 @@ KERNEL_FILES = {"pack_rows": "pack.cu", "pack_weights": "pack.cu", "xnor_gemm": 
 
 
 def sweep_tensor_core_aggregation(w):
-    """At the sweep's size the layer keeps byte dots and aggregates on the tensor
-    cores for K <= 3072 (csrc/layer.cu)."""
-    return w.K <= 3072
+    """Whether a sweep point's layer keeps byte dots and aggregates on the tensor cores: the
+    rule of csrc/layer.cu for 2^20 rows of the tensor-core product."""
+    K, F = w.K, w.hidden
+    unpadded = (F + 15) // 16 * 16 == (F + 7) // 8 * 8
+    return K <= 3072 and F <= 256 and (K <= 2048 and F <= 128 or unpadded)
 
 
 def kernel_file(name, w=None):

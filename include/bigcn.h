@@ -189,11 +189,17 @@ size_t bigcn_layer_workspace_bytes(int64_t N, int32_t K, int32_t F);
  * calls above within fp32 rounding; it runs the kernels of bigcn_pack_rows,
  * bigcn_pack_weights, bigcn_xnor_gemm_degscaled and bigcn_spmm_prescaled on
  * `stream`, except that when K <= 32767 the product keeps Z' factored in the
- * workspace -- the integer dots (in byte planes where K <= 3072, else as uint16
- * with a bias of 32768) and each row's alpha_i / sqrt(dhat_i) -- and the
+ * workspace -- the integer dots and each row's alpha_i / sqrt(dhat_i) -- and the
  * aggregation applies the row factor per neighbour and beta_j per column,
- * gathering a quarter or half of the bytes. No
- * activation follows (Sec. 4.1.2).
+ * gathering a quarter or half of the bytes. Where K <= 3072, F <= 256 and
+ * (F <= 128 and K <= 2048, or F mod 16 is 0 or above 8) the dots are kept a
+ * byte each (rows with a dot beyond a byte in fp16) and the aggregation runs on
+ * the tensor cores, unless rows of more than 128 dots are short and stay in L2
+ * as 16-bit dots (nnz < 64 N and N F <= 96 Mi) or a row's dots are spread over
+ * several blocks of the product (F > 64 with few rows); else they are uint16
+ * with a bias of 32768. In large calls (N F >= 4 Mi or nnz F >= 128 Mi) a second
+ * aggregation kernel stands by, which takes over where many rows are beyond a
+ * byte. No activation follows (Sec. 4.1.2).
  *
  * X N x K (ldx), Wt K x F (ldw), CSR as in bigcn_spmm_norm, H N x F (ldh).
  * workspace  device memory of at least bigcn_layer_workspace_bytes(N, K, F)
@@ -246,14 +252,14 @@ bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int32_t K, int
  * (Fh <= 128 and the packed tiles fit); and when Fh is a multiple of 4 and at
  * most 128 and Fo <= 64, layer 1's aggregation kernel also binarizes H1 and
  * computes layer 2's XNOR product while the row is in registers, so H1 never
- * goes through memory. When K <= 32767, layer 1's Z' stays factored in the
- * workspace (integer dots as biased uint16 and a row scale, as in
- * bigcn_layer_forward), so its aggregation gathers half-size rows. When
- * K <= 2048, Fh <= 128 and Fo <= 64, both products
+ * goes through memory. When K <= 2048, Fh <= 128 and Fo <= 64, both products
  * stay factored as byte dots and a row scale and both aggregations run on the
  * tensor cores (bigcn_forward_2layer_aggregation); layer 1's aggregation then
- * binarizes H1 and computes layer 2's dots for any Fh <= 128. The call
- * launches 4 to 7 kernels (bigcn_forward_2layer_launches).
+ * binarizes H1 and computes layer 2's dots for any Fh <= 128 (with a second
+ * kernel standing by in large calls, as in bigcn_layer_forward). Else, when
+ * K <= 32767, layer 1's Z' stays factored in the workspace as uint16 dots with a
+ * bias of 32768 and a row scale, so its aggregation gathers half-size rows. The
+ * call launches 4 to 7 kernels (bigcn_forward_2layer_launches).
  *
  * X N x K (ldx), W1 K x Fh (ldw1), W2 Fh x Fo (ldw2), CSR as in
  * bigcn_spmm_norm, out N x Fo (ldo).
@@ -272,7 +278,8 @@ bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int32_t K, int
 size_t bigcn_forward_2layer_workspace_bytes(int64_t N, int32_t K, int32_t Fh, int32_t Fo);
 
 /* Kernel launches bigcn_forward_2layer makes for these sizes on the current
- * device (4 to 7), or -1 on invalid sizes or a device error. */
+ * device (4 to 7; a stand-by kernel counts, and is timed, with the aggregation it
+ * stands by for), or -1 on invalid sizes or a device error. */
 int32_t bigcn_forward_2layer_launches(int64_t N, int32_t K, int32_t Fh, int32_t Fo);
 
 /* Which aggregation bigcn_forward_2layer runs for these widths: 1 = both on
@@ -490,8 +497,10 @@ size_t bigcn_weighted_layer_workspace_bytes(int64_t N, int32_t K, int32_t F);
  * zeta as in bigcn_layer_forward. Runs the kernels of bigcn_pack_rows,
  * bigcn_pack_weights, bigcn_weighted_dinv (which also forms each row's scale
  * s_j = alpha_j dinv_j), bigcn_xnor_gemm with s as its row scale (kept
- * factored, uint16 dots and s_j, when K <= 32767) and the weighted
- * aggregation. Arguments and errors are those of bigcn_layer_forward plus
+ * factored, dots and s_j, when K <= 32767: a byte per dot as in
+ * bigcn_layer_forward where K <= 3072 and F <= 256, on the same conditions but the
+ * one on F mod 16, else uint16) and the weighted aggregation; the stand-by kernel
+ * also takes over where many rows hold weights 2^21 and more apart. Arguments and errors are those of bigcn_layer_forward plus
  * `values` (nnz fp32, not overlapping the workspace or H); the workspace is
  * bigcn_weighted_layer_workspace_bytes(N, K, F) bytes, 256-byte aligned. The
  * tensor-core product's bounded waits behave as in bigcn_layer_forward.

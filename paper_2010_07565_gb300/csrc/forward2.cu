@@ -107,8 +107,8 @@ extern "C" int32_t bigcn_forward_2layer_launches(int64_t N, int32_t K, int32_t F
     if (N < 0 || K < 1 || Fh < 1 || Fo < 1) return -1;
     DeviceInfo dev;
     if (current_device(&dev) != BIGCN_OK) return -1;
-    const bool second = forward2_tc(K, Fh, Fo) && spmm_tc_second_kernel(N, 0, K, Fh);
-    return 1 + (front_supported(N, K, Fh, dev) ? 1 : 2) + (second ? 1 : 0) +
+    // (the aggregation's stand-by kernel counts, and is timed, with it)
+    return 1 + (front_supported(N, K, Fh, dev) ? 1 : 2) +
            (forward2_tc(K, Fh, Fo) || spmm_pack_gemm_supported(Fh, Fo) ? 1 : 3) + 1;
 }
 

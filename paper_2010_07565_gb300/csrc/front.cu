@@ -6,11 +6,12 @@
 //   Z'[i,j] = (alpha_i / sqrt(dhat_i)) * (beta_j * (K - 2 popc(a_i ^ b_j)))
 //
 // Each block owns BM = 16 * RI rows. Phase A: its 8 warps stream the rows of
-// X (one warp per row at a time, 8 chunks of 32 features in flight), and
-// every chunk's ballot lands directly in shared memory as a 32-bit half-word
-// of the packed row (up to four rows a warp packed together, pack_group: 232,965
-// x 602, F = 128, 230 -> 184 us with registers for four blocks per SM, 206 us with
-// three); the packed rows never go to global memory. Phase B: thread (cg, rg) counts mismatches for rows rg + 16 i and columns cg + 16 j
+// X (a warp packs two or four neighbouring rows together, four chunks of 32
+// features of each in flight, pack_group: 232,965 x 602, F = 128, 230 -> 184 us with
+// registers for four blocks per SM, 206 us with three), and every chunk's ballot
+// lands in shared memory as a 32-bit half-word of the packed row; the packed rows
+// never go to global memory. Phase B: thread (cg, rg) counts mismatches for rows
+// rg + 16 i and its CJ columns
 // against the packed weight columns, which the block loads once into shared
 // memory (odd row pitch: conflict-free). Several blocks per SM overlap one
 // block's HBM-bound phase A with another's POPC-bound phase B.
@@ -74,7 +75,7 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t m0 = int64_t(blockIdx.x) * BM;
 
-    // Phase A: centre + sign + pack + |y| sums, rows warp, warp + 8, ...
+    // Phase A: centre + sign + pack + |y| sums, kGroup neighbouring rows to a warp
     const int nhalf = 2 * words;
     for (int r0 = warp * kGroup; r0 < BM; r0 += kFrontWarps * kGroup) {
         uint32_t *a32 = reinterpret_cast<uint32_t *>(As + size_t(r0) * pitch);
@@ -133,7 +134,8 @@ front_kernel(const float *__restrict__ X, int64_t N, int K, int64_t ldx,
         if (dots8 != nullptr) {             // the row's 16 lanes agree on its flag
 #pragma unroll
             for (int j = 0; j < CJ; ++j)
-                if (flag_column(column(cg, j), half, valid)) wide |= ByteDot(K - 2 * mism[i][j], K).wide();
+                if (flag_column(column(cg, j), half, valid))
+                    wide |= ByteDot(K - 2 * mism[i][j], K).wide();
             wide = (__ballot_sync(kFullMask, wide) >> (tid & 16) & 0xffffu) != 0u;
         }
         if (row >= N) continue;

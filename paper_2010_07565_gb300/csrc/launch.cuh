@@ -309,7 +309,6 @@ void launch_spmm_tc(const SpmmTcArgs &args, const DeviceInfo &dev, cudaStream_t 
 // 232,965 nodes of mean degree 492, K = 602, F = 128, a layer: no wide row 1790 us, one in
 // 256 2560, one in 16 3580, all 9800; with the second kernel 2600 from one in 256 on.
 // Weights of 1e-8 to 1 on 100,003 nodes of mean degree 50, F = 100: 644 without, 264 with it.
-// nnz: 0 where it shall not count (a launch count that does not know it).
 bool spmm_tc_second_kernel(int64_t N, int64_t nnz, int K, int F);
 
 // Layer 1's tensor-core aggregation fused with layer 2's binarization and

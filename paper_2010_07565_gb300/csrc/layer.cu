@@ -48,7 +48,6 @@ void query_device(int dev) {
 constexpr size_t kAlign = 256;
 size_t round_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
-// Workspace carve-up of the fused layer; every piece 256-byte aligned.
 // Largest K whose dots (|dot| <= K) the compressed uint16 form holds.
 constexpr int32_t kMaxDots16K = 32767;
 
@@ -57,7 +56,7 @@ constexpr int32_t kMaxDots16K = 32767;
 // the aggregation can load eight dots at a time) or two byte planes (N x
 // round_up(F, 16) each), and a row scale (N); then the
 // FP8 tiles of the weight signs for the tensor-core product (about F x K bytes
-// when K >= 128 and F >= 32).
+// when K >= 128 and F >= 32) and the control words.
 struct LayerWorkspace {
     size_t a_bits, alpha, b_bits, beta, z, rowscale, bexp, bexp_bytes, control, total;
     bool compressed;
@@ -240,7 +239,8 @@ extern "C" bigcn_status bigcn_layer_forward_timed(const float *X, int64_t N, int
     }
     marks.mark();
     if (bytes) {        // byte planes: the aggregation on the tensor cores
-        SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, w.ldd8, g.rowscale, F, K, H, ldh, beta, nullptr};
+        SpmmTcArgs t{rowptr, colidx, N, nnz, g.dots8, w.ldd8, g.rowscale, F, K, H, ldh, beta,
+                     nullptr};
         t.counters = control;
         t.wide_rows = g.wide_rows;
         launch_spmm_tc(t, dev, s, pdl);

@@ -16,7 +16,8 @@
 // critical path of the whole launch: a warp walks its row U * 32 / L
 // neighbours per round trip. A row is heavy when it has more than
 // max(32, 4 * that width, 4 * the mean degree) neighbours, i.e. when its walk
-// would take several times longer than a typical row's. The first `heavy_blocks` blocks of every launch therefore scan the
+// would take several times longer than a typical row's. The first `heavy_blocks`
+// blocks of every launch therefore scan the
 // row pointers in chunks of 32 rows (so that the hubs of a small graph land
 // on many blocks), skip light rows, and give each heavy row to all 8 warps of
 // the block: warp w gathers the w-th eighth of the row's list, the eight
@@ -190,7 +191,9 @@ struct RowSrc<8, kHalves> {
         const uint32_t u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {       // features 4 (q % 2) + q / 2, and 2 on
-            const float2 d = __half22float2(*reinterpret_cast<const __half2 *>(&u[q]));
+            // (as whole dots, exact in fp16 too: the weights keep their full range)
+            const float2 d = __half22float2(__hmul2(*reinterpret_cast<const __half2 *>(&u[q]),
+                                                    __float2half2_rn(1024.0f)));
             float *a = acc + 4 * (q % 2) + q / 2;
             a[0] = fmaf(w, d.x, a[0]);
             a[2] = fmaf(w, d.y, a[2]);
@@ -262,7 +265,7 @@ __device__ __forceinline__ void gather(const SpmmParams &p, int64_t i, int64_t b
                      : AGG == kAggWeighted  ? __ldg(p.dinv + j)
                                             : inv_sqrt_degree(__ldg(p.rowptr + j + 1) -
                                                               __ldg(p.rowptr + j));
-                if (S == kHalves) wj = fabsf(wj) * 1024.0f;
+                if (S == kHalves) wj = fabsf(wj);
                 if (AGG == kAggWeighted && q > 0) wj *= __ldg(p.values + b + q - 1);
             }
         }
@@ -364,7 +367,8 @@ struct StoreRow {
                         o[c] += si * (__ldg(p.colscale_s + f + c) *
                                       (__half2float(*reinterpret_cast<const __half *>(d)) * 1024.0f));
                     } else if (S == kDots16) {
-                        const uint32_t d = __ldg(static_cast<const uint16_t *>(p.Zs) + i * p.ldz + f + c);
+                        const uint32_t d =
+                            __ldg(static_cast<const uint16_t *>(p.Zs) + i * p.ldz + f + c);
                         o[c] += si * (__ldg(p.colscale_s + f + c) * (float(d) - 32768.0f));
                     } else {
                         o[c] += __ldg(static_cast<const float *>(p.Zs) + i * p.ldz + f + c);
@@ -644,8 +648,9 @@ struct PackGemmRow {
         l1 = warp_sum(l1);
         const float a = (l1 / float(Fh)) * dinv;
         if constexpr (S == kHalves) {       // Eq. 11's dots as bytes (|dot| <= 128) and the scale
-            if (lane == 0) *(f.s2 != nullptr ? f.s2 + i
-                                             : reinterpret_cast<float *>(f.D2 + (i + 1) * f.ldd2 - 4)) = a;
+            float *s2 = f.s2 != nullptr ? f.s2 + i
+                                        : reinterpret_cast<float *>(f.D2 + (i + 1) * f.ldd2 - 4);
+            if (lane == 0) *s2 = a;
             for (int jo = lane; jo < f.Fo; jo += 32) {
                 int mism = __popcll(w0 ^ f.sW[jo * f.words2]);
                 if (f.words2 > 1) mism += __popcll(w1 ^ f.sW[jo * f.words2 + 1]);
@@ -738,8 +743,9 @@ void launch_cfg(const SpmmArgs &a, const DeviceInfo &dev, int Fload, cudaStream_
     const bool one_slab = a.F <= SLAB;
     SpmmParams p{a.rowptr, a.colidx, a.N, a.nnz, Z, a.ldz, Fload, a.F, a.H, a.ldh,
                  heavy_block_count(a.N, dev), heavy_degree(a.N, a.nnz, (32 / L) * U),
-                 pool_rows(a.N, dev), vec_store, a.rowscale, a.colscale, one_slab ? a.pred : nullptr, a.agg, a.Zs,
-                 a.colscale_s, a.ncols > 0 ? a.ncols : a.N, a.values, a.dinv};
+                 pool_rows(a.N, dev), vec_store, a.rowscale, a.colscale,
+                 one_slab ? a.pred : nullptr, a.agg, a.Zs, a.colscale_s,
+                 a.ncols > 0 ? a.ncols : a.N, a.values, a.dinv};
     dim3 grid(unsigned(p.heavy_blocks + (a.N + p.pool - 1) / p.pool),
               unsigned((a.F + SLAB - 1) / SLAB));
     launch_kernel(spmm_norm_kernel<VEC, L, NV, U, S, AGG>, grid, dim3(kSpmmThreads), 0, s, pdl,

@@ -1539,7 +1539,7 @@ void launch_spmm_tc_pack_gemm(const SpmmTcPackGemmArgs &a, const DeviceInfo &dev
     if (a.N == 0) return;
     TcParams P = tc_params(a.rowptr, a.colidx, a.N, a.nnz, a.D1, a.ldd1, a.s1, a.K);
     P.counters = a.counters;
-    const SecondKernel second{spmm_tc_second_kernel(a.N, 0, a.K, a.Fh) ? a.wide_rows : nullptr,
+    const SecondKernel second{spmm_tc_second_kernel(a.N, a.nnz, a.K, a.Fh) ? a.wide_rows : nullptr,
                               many_wide_share(a.N, a.nnz, a.Fh, dev),
                               const_cast<uint8_t *>(a.D1)};
     const int words2 = (a.Fh + 63) / 64;

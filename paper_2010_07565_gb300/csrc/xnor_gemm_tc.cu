@@ -630,7 +630,8 @@ expand_b_kernel(const uint64_t *__restrict__ B, int F, int K, int words, int KB,
         const int k0 = kb * kTcKBytes + c * 16;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (col < F && k0 < K) {
-            const uint32_t bits = uint32_t(load_upstream(B + int64_t(col) * words + (k0 >> 6)) >> (k0 & 63));
+            const uint64_t word = load_upstream(B + int64_t(col) * words + (k0 >> 6));
+            const uint32_t bits = uint32_t(word >> (k0 & 63));
             v = make_uint4(signs4_to_e4m3(bits & 15u), signs4_to_e4m3((bits >> 4) & 15u),
                            signs4_to_e4m3((bits >> 8) & 15u), signs4_to_e4m3((bits >> 12) & 15u));
             const int valid = K - k0;

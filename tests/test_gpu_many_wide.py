@@ -125,3 +125,25 @@ def test_unlike_weights(cuda_device, N, F, deg, hub, every):
     n = int(np.diff(rp).max()) + 8
     bad = (H.double() - ref).abs() > n * (2.0 ** -23 * mag + 2.0 ** -149)
     assert not bool(bad.any()), int(bad.sum())
+
+
+@pytest.mark.parametrize("power", [-37, 36])
+def test_row_scales_at_the_ends_of_fp32(cuda_device, power):
+    """The second kernel's weights are the row scales themselves."""
+    N, K, F = 66003, 300, 64
+    c = planted_case(N, K, F, 6.0, 400, 3, seed=5)
+    c["X"] = (c["X"] * 10.0 ** power).astype(np.float32)
+    if power > 0:               # (|y| sums of 300 terms and sums of dots stay finite)
+        c["X"] *= 0.1
+        c["W"] *= np.float32(1e-3)
+    d = {k: to_dev(x) for k, x in c.items() if x is not None}
+    H = torch.full((N, F), float("nan"), device=cuda_device)
+    ws = torch.full((B.bigcn_layer_workspace_bytes(N, K, F),), 0xAB, dtype=torch.uint8,
+                    device=cuda_device)
+    B.bigcn_layer_forward(d["X"], None, None, d["W"], d["rowptr"], d["colidx"], ws, H)
+    rows = sampled(N, 500, K)
+    ref = oracle.layer_forward(c["X"], c["W"], c["rowptr"], c["colidx"], rows=rows)
+    n = int(np.diff(c["rowptr"]).max()) + 8
+    err = np.abs(H.cpu().numpy()[rows].astype(np.float64) - ref["H"])
+    # (the oracle sums the row scale in fp64; products below the normal range lose bits)
+    assert (err <= (n + K) * (2.0 ** -23 * ref["absterm"] + 2.0 ** -149)).all()
