@@ -195,6 +195,12 @@ def sweep_tensor_core_aggregation(w):
     return K <= 3072 and F <= 256 and (K <= 2048 and F <= 128 or unpadded)
 
 
+def standby_launches(N, nnz, K, F):
+    """1 where a second aggregation kernel stands by for wide rows (csrc/spmm_tc.cu's rule,
+    for a product in byte dots); it is timed with the aggregation."""
+    return int((K <= 2048 or K % 2 == 0) and (N * F >= 4 << 20 or nnz * F >= 128 << 20))
+
+
 def kernel_file(name, w=None):
     if w is not None and name in ("L1.spmm+L2.pack_rows+L2.xnor_gemm", "L2.spmm") and \
             tensor_core_aggregation(w):
@@ -262,11 +268,13 @@ def profile_file_traffic(fname, files):
 
 
 INDUCTIVE_SOURCES = {
-    "gcn": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "layer.cu", "spmm_tc.cu"],
-    "mean": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm_tc.cu"],
-    "sage": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm_tc.cu"]}
+    "gcn": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "layer.cu", "spmm_tc.cu",
+            "spmm.cu"],
+    "mean": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm_tc.cu", "spmm.cu"],
+    "sage": ["inductive.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm_tc.cu", "spmm.cu"]}
 BACKWARD_SOURCES = ["backward.cu", "pack.cu", "spmm.cu", "ablation.cu"]
-WEIGHTED_SOURCES = ["weighted.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm_tc.cu"]
+WEIGHTED_SOURCES = ["weighted.cu", "pack.cu", "xnor_gemm.cu", "xnor_gemm_tc.cu", "spmm_tc.cu",
+                    "spmm.cu"]
 
 
 class ClockSampler:
@@ -648,7 +656,8 @@ def run_gpu(args, rank, world, local_rank):
         "cpu_baseline": cpu_baseline,
         "e2e": {"value": e2e_units / (e2e_max * 1e-3), "unit": "nodes/s",
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-        "gpu_launches": len(names) * args.steps,
+        "gpu_launches": (len(names) + tensor_core_aggregation(w) *
+                         standby_launches(w.N, nnz, w.K, w.hidden)) * args.steps,
         "clocks": clocks.summary(),
         "paper_context": {
             "cycle_ops_gcn": cost_model.cycle_ops(w.N, nnz // 2, dims, False),
@@ -766,7 +775,9 @@ def run_sweep(args, rank, world, local_rank):
         "cpu_baseline": None, "e2e": None,
         "note": "sweep point: one layer, kernel-level timing; no host-buffer run (the features "
                 "alone are up to 34 GB)",
-        "gpu_launches": 4 * args.steps, "clocks": clocks.summary(),
+        "gpu_launches": (4 + sweep_tensor_core_aggregation(w) *
+                         standby_launches(N, nnz, K, F)) * args.steps,
+        "clocks": clocks.summary(),
     }
     print(json.dumps(line), flush=True)
     return 0
@@ -1071,7 +1082,8 @@ def run_inductive(args, rank, world, local_rank):
                      "traffic_note": "DRAM bytes of one whole call (its 4 kernels)",
                      "peak_source": f"{peak_kind} MEASURED_PEAKS.json hbm_gbs",
                      "algorithmic_bytes": layer_bytes},
-        "cpu_baseline": None, "e2e": None, "gpu_launches": 4 * args.steps,
+        "cpu_baseline": None, "e2e": None,
+        "gpu_launches": (4 + planes * standby_launches(N, nnz, K, F)) * args.steps,
         "clocks": clocks.summary(),
     }
     print(json.dumps(line), flush=True)
@@ -1160,7 +1172,8 @@ def run_weighted(args, rank, world, local_rank):
                      "traffic_note": "DRAM bytes of one whole call (its 5 kernels)",
                      "peak_source": f"{peak_kind} MEASURED_PEAKS.json hbm_gbs",
                      "algorithmic_bytes": layer_bytes},
-        "cpu_baseline": None, "e2e": None, "gpu_launches": 5 * args.steps,
+        "cpu_baseline": None, "e2e": None,
+        "gpu_launches": (5 + planes * standby_launches(N, nnz, K, F)) * args.steps,
         "clocks": clocks.summary(),
     }
     print(json.dumps(line), flush=True)

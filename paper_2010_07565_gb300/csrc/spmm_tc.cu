@@ -20,8 +20,8 @@
 // byte per dot halves a staged row against fp16, which buys deeper rings and
 // half as many copies, for one permute and one packed fma per two dots. On
 // 232,965 nodes of mean degree 492 (114.8 M gathered rows): layer 1, 128
-// features, 2600 -> 1880 us (7.8 TB/s of 128-byte rows; issue 51 %, ALU and the
-// copies' latency bind); layer 2, 41 features, 1475 -> 1160 us. On 2^20 nodes of
+// features, 2600 -> 1590 us (9.2 TB/s of 128-byte rows; issue 57 %, ALU and the
+// copies' latency bind); layer 2, 41 features, 1475 -> 980 us. On 2^20 nodes of
 // mean degree 16, 64 features: 787 -> 464 us.
 //
 // A staged row is read with ldmatrix.trans as pairs of neighbouring features:

@@ -10,6 +10,7 @@ import oracle
 from gpu_helpers import check_sum, to_dev
 from paper_2010_07565_gb300 import binding as B
 from paper_2010_07565_gb300 import inputs
+from paper_2010_07565_gb300.runner import GCN2Forward, fused_kernel_names
 from test_gpu_byte_dots import planted_case, sampled
 
 pytestmark = pytest.mark.gpu
@@ -147,3 +148,20 @@ def test_row_scales_at_the_ends_of_fp32(cuda_device, power):
     err = np.abs(H.cpu().numpy()[rows].astype(np.float64) - ref["H"])
     # (the oracle sums the row scale in fp64; products below the normal range lose bits)
     assert (err <= (n + K) * (2.0 ** -23 * ref["absterm"] + 2.0 ** -149)).all()
+
+
+def test_forward_kernels_of_a_large_graph(cuda_device):
+    """The stand-by kernel is timed, and counted, with the aggregation it stands by for."""
+    N, K, Fh, Fo = 66003, 300, 64, 7
+    assert fused_kernel_names(N, K, Fh, Fo) == fused_kernel_names(3000, K, Fh, Fo)
+    c = inputs.layer_case(N, K, Fh, seed=4)
+    m = GCN2Forward(N, K, Fh, Fo, len(c["colidx"]), cuda_device)
+    m.load(X=to_dev(c["X"]), s=to_dev(c["s"]), t=to_dev(c["t"]), W1=to_dev(c["W"]),
+           W2=to_dev(inputs.weights(Fh, Fo, 5)), rowptr=to_dev(c["rowptr"]),
+           colidx=to_dev(c["colidx"]))
+    events = [torch.cuda.Event(enable_timing=True, external=True)
+              for _ in range(len(m.kernel_names) + 1)]
+    m.capture(events)
+    m.replay()
+    torch.cuda.synchronize()
+    assert all(a.elapsed_time(b) > 0 for a, b in zip(events, events[1:]))
